@@ -118,10 +118,10 @@ __global__ void __launch_bounds__(256) k_expec_dm(const typename Cplx<R>::T* __r
 //  * each Pauli string is Hermitian and h is real, so the contributions of i
 //    and i xor xy are complex conjugates: only indices with the highest bit
 //    of xy clear are visited, each counting 2 Re(i^eta q) h (-1)^{popc(i' & yz)}.
-// Arithmetic is double-float (qs_df.cuh): q and |alpha_i|^2 as error-free
-// FP32 dot products, every contribution added to one per-thread accumulator
-// with TwoSum, so the loop needs no FP64 instruction; each thread rounds its
-// sum to double once.  The imaginary part of the result is exactly zero.
+// Arithmetic is double-float (qs_df.cuh): products as error-free FP32 dot
+// products (complex64 parts as single floats), summed per term over a tile and
+// then times h into one per-thread accumulator with TwoSum, so the loop needs
+// no FP64 instruction; each thread rounds its sum to double once.  The imaginary part of the result is exactly zero.
 // A term as the kernel reads it from shared memory: h already split.
 struct TermDf {
   uint64_t xy, yz;
@@ -132,6 +132,44 @@ struct TermDf {
 struct GroupDf {
   uint64_t xy, hb;       // flip mask, its highest bit (0 for the diagonal run)
   int first, count;
+};
+
+// A group of at most kDirectTerms terms adds each term's own products into a
+// per-thread sum over the tile's E elements, which then takes one multiply by
+// the coefficient (2 products per element and term, plus 1 per tile); longer
+// groups form q once per element and add it per term (4 products per element,
+// 1 add per term).  The two cost the same at four terms.
+constexpr int kDirectTerms = 4;
+
+// c v as a double-float accumulation: floats (complex64 parts) have exact
+// two-term products, df pairs take the cross terms too
+__device__ __forceinline__ void prod_add(qsdf::dot_acc& a, float c, float v) {
+  const float p = c * v;
+  const float lo = qsdf::fmaf_(c, v, -p);
+  const float s2 = a.s + p;                     // TwoSum(s, p)
+  const float bb = s2 - a.s;
+  const float err = (a.s - (s2 - bb)) + (p - bb);
+  a.s = s2;
+  a.lo += lo + err;
+}
+__device__ __forceinline__ void prod_add(qsdf::dot_acc& a, qsdf::df c, qsdf::df v) { qsdf::dot_add(a, c, v); }
+__device__ __forceinline__ float flip(float x, bool neg) { return neg ? -x : x; }
+__device__ __forceinline__ qsdf::df flip(qsdf::df x, bool neg) { return neg ? qsdf::neg(x) : x; }
+__device__ __forceinline__ double flip(double x, bool neg) {
+  return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000 : 0), __double2loint(x));
+}
+// an amplitude part as the double-float kernel multiplies it
+template <typename R>
+struct PartOf;
+template <>
+struct PartOf<float> {
+  using T = float;
+  __device__ static T in(float x) { return x; }
+};
+template <>
+struct PartOf<double> {
+  using T = qsdf::df;
+  __device__ static T in(double x) { return qsdf::split(x); }
 };
 
 // Virtual tile positions handed out in increasing order: ctr[0] is the next
@@ -173,6 +211,7 @@ __global__ void __launch_bounds__(256) k_expec_sv(const typename Cplx<R>::T* __r
                                                   TileCounter tc) {
   using qsdf::df;
   using T2 = typename Cplx<R>::T;
+  using P = typename PartOf<R>::T;
   extern __shared__ unsigned char sm_raw[];
   TermDf* ts = reinterpret_cast<TermDf*>(sm_raw);
   GroupDf* gs = reinterpret_cast<GroupDf*>(ts + nterms);
@@ -210,7 +249,7 @@ __global__ void __launch_bounds__(256) k_expec_sv(const typename Cplx<R>::T* __r
     const uint64_t base = ordered_tile(vt, ord) * kTile;
     uint64_t iu[E];
     bool ok[E];
-    df ar[E], ai[E];
+    P ar[E], ai[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       iu[e] = base + (uint64_t)(e * 256 + threadIdx.x);
@@ -219,8 +258,8 @@ __global__ void __launch_bounds__(256) k_expec_sv(const typename Cplx<R>::T* __r
       a.x = 0;
       a.y = 0;
       if (ok[e]) a = psi[iu[e]];
-      ar[e] = to_df(a.x);
-      ai[e] = to_df(a.y);
+      ar[e] = PartOf<R>::in(a.x);
+      ai[e] = PartOf<R>::in(a.y);
     }
     for (int g = 0; g < ng; ++g) {
       const GroupDf G = gs[g];
@@ -228,8 +267,9 @@ __global__ void __launch_bounds__(256) k_expec_sv(const typename Cplx<R>::T* __r
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           if (!ok[e]) continue;
-          qsdf::dot_acc pa = qsdf::dot_first(ar[e], ar[e]);    // |alpha_i|^2
-          qsdf::dot_add(pa, ai[e], ai[e]);
+          qsdf::dot_acc pa{0.0f, 0.0f};                        // |alpha_i|^2
+          prod_add(pa, ar[e], ar[e]);
+          prod_add(pa, ai[e], ai[e]);
           const df p2 = qsdf::dot_result(pa);
           for (int n = G.first; n < G.first + G.count; ++n) {
             const bool neg = parity64(iu[e] & ts[n].yz);
@@ -248,19 +288,48 @@ __global__ void __launch_bounds__(256) k_expec_sv(const typename Cplx<R>::T* __r
         b[e].y = 0;
         if (vis[e]) b[e] = psi[iu[e] ^ G.xy];
       }
+      if (G.count <= kDirectTerms) {
+        P br[E], bi[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          br[e] = PartOf<R>::in(b[e].x);
+          bi[e] = PartOf<R>::in(b[e].y);
+        }
+        const uint64_t ip0 = (base + threadIdx.x) ^ G.xy;
+        for (int n = G.first; n < G.first + G.count; ++n) {
+          // 2 h (-1)^{popc(ip & yz)} Re(i^eta q), q = conj(a) b: eta 0 -> Re q, 1 -> -Im q, 2 -> -Re q, 3 -> Im q
+          const TermDf T = ts[n];
+          const bool n0 = parity64(ip0 & T.yz) != (T.eta == 1 || T.eta == 2);
+          qsdf::dot_acc t{0.0f, 0.0f};
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            if (!vis[e]) continue;
+            const bool neg = n0 != (bool)(__popc((unsigned)(e * 256) & (unsigned)T.yz) & 1);
+            if (T.eta & 1) {
+              prod_add(t, flip(ar[e], neg), bi[e]);
+              prod_add(t, flip(ai[e], !neg), br[e]);
+            } else {
+              prod_add(t, flip(ar[e], neg), br[e]);
+              prod_add(t, flip(ai[e], neg), bi[e]);
+            }
+          }
+          qsdf::dot_add(acc, df{2.0f * T.hh, 2.0f * T.hl}, qsdf::dot_result(t));   // exact scaling
+        }
+        continue;
+      }
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         if (!vis[e]) continue;
         const uint64_t ip = iu[e] ^ G.xy;
-        const df br = to_df(b[e].x), bi = to_df(b[e].y);
+        const P br = PartOf<R>::in(b[e].x), bi = PartOf<R>::in(b[e].y);
         // q = conj(a) b = (ar br + ai bi) + i (ar bi - ai br)
-        qsdf::dot_acc qa = qsdf::dot_first(ar[e], br);
-        qsdf::dot_add(qa, ai[e], bi);
-        qsdf::dot_acc qb = qsdf::dot_first(ar[e], bi);
-        qsdf::dot_add(qb, qsdf::neg(ai[e]), br);
+        qsdf::dot_acc qa{0.0f, 0.0f}, qb{0.0f, 0.0f};
+        prod_add(qa, ar[e], br);
+        prod_add(qa, ai[e], bi);
+        prod_add(qb, ar[e], bi);
+        prod_add(qb, flip(ai[e], true), br);
         const df qr = qsdf::dot_result(qa), qi = qsdf::dot_result(qb);
         for (int n = G.first; n < G.first + G.count; ++n) {
-          // 2 Re(i^eta q) (-1)^{popc(ip & yz)} h: eta 0 -> qr, 1 -> -qi, 2 -> -qr, 3 -> qi
           const int eta = ts[n].eta;
           const bool neg = parity64(ip & ts[n].yz) != (eta == 1 || eta == 2);
           const float s2 = neg ? -2.0f : 2.0f;                 // exact scaling
@@ -341,6 +410,29 @@ __global__ void __launch_bounds__(256) k_expec_sv_f64(const double2* __restrict_
       for (int e = 0; e < E; ++e) {
         vis[e] = ok[e] && !(iu[e] & G.hb);
         b[e] = vis[e] ? psi[iu[e] ^ G.xy] : make_double2(0.0, 0.0);
+      }
+      if (G.count <= kDirectTerms) {
+        const uint64_t ip0 = (base + threadIdx.x) ^ G.xy;
+        for (int n = G.first; n < G.first + G.count; ++n) {
+          // 2 h (-1)^{popc(ip & yz)} Re(i^eta q), q = conj(a) b: eta 0 -> Re q, 1 -> -Im q, 2 -> -Re q, 3 -> Im q
+          const PauliTerm T = ts[n];
+          const bool n0 = parity64(ip0 & T.yz) != (T.eta == 1 || T.eta == 2);
+          double t = 0.0;
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            if (!vis[e]) continue;
+            const bool neg = n0 != (bool)(__popc((unsigned)(e * 256) & (unsigned)T.yz) & 1);
+            if (T.eta & 1) {
+              t = fma(flip(a[e].x, neg), b[e].y, t);
+              t = fma(flip(a[e].y, !neg), b[e].x, t);
+            } else {
+              t = fma(flip(a[e].x, neg), b[e].x, t);
+              t = fma(flip(a[e].y, neg), b[e].y, t);
+            }
+          }
+          acc = fma(2.0 * T.h, t, acc);
+        }
+        continue;
       }
 #pragma unroll
       for (int e = 0; e < E; ++e) {
