@@ -87,17 +87,16 @@ typedef enum { QS_C64 = 0, QS_C128 = 1 } qs_prec;
  *     2^-53 |y| + 2^-54 max|x_k| max|m_k|.  So does a one-qubit unitary or
  *     Kraus map on a density matrix, applied as one two-target pass of
  *     conj(U) (x) U or of its superoperator on (t, t + N).
- *   - Dense gates with 3..5 targets (and two-target fused blocks) run on the
- *     bf16 tensor cores with eight
- *     exact 7-bit integer slices of 56-bit operands (rows and columns scaled
- *     by their largest exponent), exact FP32 level sums, one rounding.
- *   - Everything else (6-target dense gates, dephasing, superoperators,
+ *   - Dense gates with 3..6 targets (and two-target fused blocks) run on the
+ *     fp16 tensor cores with exact 8-bit integer slices: 55-bit amplitudes
+ *     (rows scaled by their largest exponent), 63-bit matrix entries (columns
+ *     scaled by theirs), exact FP32 level sums, one rounding.
+ *   - Everything else (dephasing, superoperators,
  *     norm, trace, expectation values, partial traces) is native FP64.
  * QS_ARITH_DF: double-float.  Amplitudes are split into float pairs (47-bit
  *   significands) and combined with error-free FP32 transformations; dense
- *   gates use seven 7-bit slices (49 bits).  Relative error per operation: a
- *   few units of 2^-46 for moduli in [2^-80, 2^128).  Somewhat faster than FX
- *   on dense gates, but narrower than IEEE double.
+ *   gates take the tensor-core path above.  Relative error per operation: a
+ *   few units of 2^-46 for moduli in [2^-80, 2^128): narrower than IEEE double.
  * QS_ARITH_F64: native FP64 throughout (FP64-pipe bound on GB300).
  * complex64 states ignore the setting. */
 typedef enum { QS_ARITH_DF = 0, QS_ARITH_F64 = 1, QS_ARITH_FX = 2 } qs_arith;

@@ -73,13 +73,14 @@ qs_status create(int nq, int ns, int is_density, qs_prec prec, void* d_amps, voi
   s->stream = static_cast<cudaStream_t>(stream);
   const size_t scratch = sizeof(double2) * (qsk::kPartials + 2);
   if (qsalloc::device(reinterpret_cast<void**>(&s->d_partials), scratch) != cudaSuccess ||
-      qsalloc::device(reinterpret_cast<void**>(&s->d_ring), kRingSlots * kSlotBytes) != cudaSuccess ||
+      qsalloc::device(reinterpret_cast<void**>(&s->d_ring), kRingSlots * kSlotBytes + qsk::kWideScratch) != cudaSuccess ||
       qsalloc::pinned(reinterpret_cast<void**>(&s->h_result), sizeof(double2) * 2) != cudaSuccess ||
       qsalloc::pinned(reinterpret_cast<void**>(&s->h_ring), kRingSlots * kSlotBytes) != cudaSuccess) {
     cudaGetLastError();
     release(s);
     return QS_ERR_OOM;
   }
+  s->d_wide = s->d_ring + kRingSlots * kSlotBytes;
   s->d_result = s->d_partials + qsk::kPartials;
   s->d_err = reinterpret_cast<int*>(s->d_partials + qsk::kPartials + 1);
   if (cudaMemset(s->d_err, 0, sizeof(int)) != cudaSuccess) {
@@ -331,10 +332,9 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
   // on the lowest free qubit
   const bool tc_n = n <= 5 && (n >= 3 || (n == 2 && nfree >= 1));
   const bool tc64 = s->prec == QS_C64 && s->tensor_cores && (tc_n || n == 6);   // 6: bf16x3 slices
-  // complex128: seven integer slices (49 bits) with double-float arithmetic,
-  // eight (56 bits) with block fixed point
+  // complex128 off the FP64 pipe: exact byte slices (55-bit amplitudes)
   const bool tc128 = s->prec == QS_C128 && (s->arith == QS_ARITH_DF || s->arith == QS_ARITH_FX) &&
-                     s->tensor_cores && tc_n;
+                     s->tensor_cores && (tc_n || n == 6);
   if (tc64 || tc128) {
     std::vector<int> kt(targs);
     if (n == 2) {
@@ -374,7 +374,7 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
     for (int i = 0; i < p.nhi; ++i) p.hi_ins[i] = (int8_t)hi[i];
     p.ntiles = 1ull << (s->ns - p.nhi);
     return cuda_status(tc64 ? qsk::launch_dense_tc(s->amps, p, s->stream)
-                            : qsk::launch_dense_ozaki(s->amps, p, s->arith == QS_ARITH_FX ? 8 : 7, s->stream));
+                            : qsk::launch_dense_ozaki(s->amps, p, s->d_wide, s->stream));
   }
   // Dense tile: P = targets u the lowest free qubits, |P| = min(kTileBits, free + n).
   const int g = std::min(qsk::kTileBits - n, nfree) < 0 ? 0 : std::min(qsk::kTileBits - n, nfree);

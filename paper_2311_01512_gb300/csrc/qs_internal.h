@@ -16,6 +16,7 @@ constexpr int kTileBits = 10;        // amplitudes staged per tile of the dense 
 constexpr int kReduceBlocks = 1216;  // 152 SMs x 8: fixed grid of the stage-one expectation and trace reductions
 constexpr int kNormBlocks = 4864;    // 152 SMs x 32: fixed grid of the norm, a pure stream over the state
 constexpr int kPartials = kNormBlocks;  // partial sums a handle holds (the larger grid)
+constexpr size_t kWideScratch = 295424;  // bytes of a handle's scratch for six-target gates (qs_tc_ozaki.cu)
 constexpr int kTermChunk = 2048;     // Pauli terms per device upload
 constexpr int kCostFeatures = 64;    // cost-model network: input features
 constexpr int kCostHidden = 64;      // hidden units per layer (two layers)
@@ -355,9 +356,9 @@ cudaError_t launch_group_fx(void* amps, int op, const GroupFxParams& p, cudaStre
 cudaError_t launch_dense_tc(void* amps, const TcParams& p, cudaStream_t st);
 // test of the bounded-wait path: a wait on an mbarrier nothing arrives at, given up after `polls` polls (qs_tc.cu)
 cudaError_t launch_test_wait_timeout(int* err, uint32_t polls, cudaStream_t st);
-// complex128 dense gates on the bf16 tensor cores, exact integer slices, 3 <= n <= 5 kernel targets (qs_tc_ozaki.cu);
-// slices: 7 (49-bit operands, with double-float arithmetic) or 8 (56-bit, with block fixed point)
-cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, int slices, cudaStream_t st);
+// complex128 dense gates on the fp16 tensor cores, exact byte slices, 3 <= n <= 6 kernel targets (qs_tc_ozaki.cu);
+// scratch: kWideScratch bytes of device memory used on st alone (six targets: the sliced matrix)
+cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st);
 cudaError_t launch_block_compose(const ComposeBlock* blocks, int nblocks, const ComposeInstr* instrs,
                                  const double* data, double* out, cudaStream_t st);
 // cost-model network (qs_mlp.cu)

@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(512, 1) k_dense_tc6(float2* __restrict__ psi, 
       for (int pr = 0; pr < 6; ++pr)
 #pragma unroll
         for (int kk = 0; kk < K / 16; ++kk)
-          mma_bf16(tmem + (pr == 0 ? 0u : (uint32_t)N), da + ((PS[pr] * SL + kk * 256) >> 4),
+          mma_f16(tmem + (pr == 0 ? 0u : (uint32_t)N), da + ((PS[pr] * SL + kk * 256) >> 4),
                    db + ((PT[pr] * SB + kk * 256) >> 4), idesc, (pr > 1 || kk != 0) ? 1u : 0u);
       mma_commit(mbar);
     }

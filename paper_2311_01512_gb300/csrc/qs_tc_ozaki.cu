@@ -1,50 +1,58 @@
-// Dense n-target gates (2 <= n <= 5) for complex128 states on the bf16 tensor
-// cores, with error-free integer slicing (the Ozaki scheme; the slicing and
-// its bounds are in qs_slices.cuh).
+// Dense n-target gates (2 <= n <= 6) for complex128 states on the fp16 tensor
+// cores, with error-free byte slicing (the Ozaki scheme; the slicing, its bounds
+// and the recombination are in qs_bytes.cuh).
 //
 // The group update alpha_kj -> sum_l m_jl alpha_kl (Sec. "Many-target gate",
 // Eq. (local many-target amplitude update)) over a tile of 128 groups is the
 // real GEMM C = A B, A[g, 2l + c'] the interleaved (re, im) amplitudes of group
 // g, B the realified matrix (B[2l, 2j] = Re m_jl, B[2l+1, 2j] = -Im m_jl,
 // B[2l, 2j+1] = Im m_jl, B[2l+1, 2j+1] = Re m_jl).  Each row of A (scaled by
-// its largest exponent) and each column of B is cut into KS = 7 or 8 balanced
-// digit slices; the slice products with s + t < KS run as tcgen05 kind::f16
+// its largest exponent) is cut into seven balanced bytes and each column of B
+// into eight; the 35 slice products with s + t <= 7 run as tcgen05 kind::f16
 // MMAs whose FP32 accumulation in tensor memory is exact, one accumulator per
 // level L = s + t; the epilogue recombines the levels in integers, converts
 // once to double and applies the two scales.  Two targets run as three: the
 // matrix is extended by an identity on one more (free) qubit, which changes
 // nothing in the result and fills the MMA's K = 16.
 //
-// The amplitude digits below the top one are stored offset by 192 (their
-// bf16 bit patterns are then two shifted fields and a constant); each tile's
-// accumulators start at P_L(n), minus the offset's contribution (192 times
-// the B column sums of the slices involved) plus, for K <= 32, the magic
-// 1.25 2^23 that leaves each level's integer in the low bits of its FP32
-// pattern.  One initialising MMA writes them: a constant A whose rows are
-// (1, 256, 65536, 0, ...) against a B whose column holds P = p0 + 256 p1 +
-// 65536 p2 in three bf16-exact parts.
+// The amplitude bytes are stored with an offset of 128 as fp16 subnormals.
+// Each tile's accumulators start at P_L(n), minus the offset's contribution
+// (plus the magic that leaves a level's integer in the low bits of its FP32
+// pattern, where it fits).  One initialising MMA writes them: a constant A
+// whose rows are (2^-24, 2^-16, 2^-8, 0, ...) against a B whose column holds
+// P = p0 + 256 p1 + 65536 p2 in three fp16-exact parts.
 //
-// Two kernels share these pieces.  k_dense_ozaki (below; five targets, and any
-// pass of fewer tiles than SMs) runs every phase in every thread;
-// k_dense_ozaki_ws (two to four targets) gives gathering and slicing, MMA
-// issue and the epilogue to separate warps (its own comment further down).
+// Why bytes: the kernels are bound by the integer pipe (a byte permute or a
+// logic operation per digit and pair, 64 a clock and SM), so what counts is the
+// integer instructions per amplitude.  Balanced 7-bit digits in bf16 (eight a
+// side) took about 95; byte-aligned digits need no shift per digit, no separate
+// top digit, one addition for rounding and balancing, and about 65.
+// Measured at 28 qubits, spread targets, per pass (the copy rate would take 1.27
+// ms): 3 targets 1.95 -> 1.50 ms, 4 targets 1.94 -> 1.50, 5 targets 3.32 -> 2.30,
+// 6 targets (native FP64 before) 110.6 -> 3.9.  Against extended precision the
+// relative error of an output vector fell from 7.7, 6.6, 7.6 and 37.5 to 6.7,
+// 6.1, 6.3 and 6.4 e-17.
 //
-// k_dense_ozaki's work mapping: thread (warp w, lane) owns row g = 32 (w mod 4) + lane (the
+// Four kernels share these pieces.  k_dense_ozaki_small (two to four targets,
+// passes of fewer tiles than SMs) runs every phase in every thread;
+// k_dense_ozaki_ws (two to four targets) and k_dense_ozaki5 give gathering and
+// slicing, MMA issue and the epilogue to separate warps; k_dense_ozaki6 walks
+// blocks of its product with the tile's amplitudes in registers.  The comments
+// of the last three stand with them.
+//
+// k_dense_ozaki_small's work mapping: thread (warp w, lane) owns row g = 32 (w mod 4) + lane (the
 // tensor-memory lane that warp may read) and the amplitudes l in
 // [c EPT, (c+1) EPT), c = w / 4, of that row, for the gather, the slicing and
 // the epilogue alike, so the row's exponent and base index stay in registers.
-// Pipeline per CTA (persistent, tiles c, c + grid, ...): the loads of the
-// next tile are issued right after the current tile's slices are written, so
-// they are in flight during the MMAs and the epilogue; with two buffers of
-// slices and accumulators (NBUF = 2) the epilogue of tile i - 1 would run
-// while the tensor cores work on tile i.  The row maxima of tile i + 1 are
-// taken after the epilogue, so a tile costs two CTA barriers.  Thread 0
-// issues the initialising MMA and then one MMA per A slice and K chunk,
-// against all the B slices it pairs with (see mma_tile).  Every wait is
-// bounded: on timeout the kernel records an error code, frees its tensor
-// memory and returns.
+// Per CTA (persistent, tiles c, c + grid, ...): the loads of the next tile are
+// issued right after the current tile's MMAs, so they are in flight during the
+// MMAs and the epilogue.  The row maxima of tile i + 1 are taken after the
+// epilogue, so a tile costs two CTA barriers.  Thread 0 issues the initialising
+// MMA and then one MMA per A slice and K chunk, against all the B slices it
+// pairs with (see mma_tile).  Every wait is bounded: on timeout the kernel
+// records an error code, frees its tensor memory and returns.
 #include "qs_device.cuh"
-#include "qs_slices.cuh"
+#include "qs_bytes.cuh"
 #include "qs_tc_ptx.cuh"
 
 namespace qsk {
@@ -59,26 +67,14 @@ __host__ __device__ constexpr uint32_t tmem_cols(uint32_t n) {
   return n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : (n <= 256 ? 256 : 512)));
 }
 
-// two floats holding small integers -> packed bf16 pair (lo in bits 0..15); exact
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+constexpr int kLv = qsby::kLevels;
+
+// fp16 bit pattern of a small integer
+__device__ __forceinline__ uint16_t half_bits(int v) {
+  uint16_t r;
+  asm("cvt.rn.f16.f32 %0, %1;" : "=h"(r) : "f"((float)v));
   return r;
 }
-
-// KS (7 or 8) digits of a double as floats
-template <int KS>
-__device__ __forceinline__ void digits(uint32_t hw, uint32_t lw, int emax, float* f) {
-  if constexpr (KS == 8)
-    qsoz::digit_floats_t8(qsoz::fixed_t8(hw, lw, emax), f);
-  else
-    qsoz::digit_floats_t(qsoz::fixed_t(hw, lw, emax), f);
-}
-
-// lower bound of a row or column exponent maximum: zeros and subnormals
-// (their implicit bit wrongly set) then shift out entirely
-template <int KS>
-__host__ __device__ constexpr int emax_floor() { return KS == 8 ? 58 : qsoz::kEmaxFloor; }
 
 // bounded wait on an mbarrier phase; true when it ran out
 __device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t parity) {
@@ -106,89 +102,71 @@ __device__ __forceinline__ double realified(const TcParams& p, int D, int k, int
 
 // All slice products of one tile.  B's slices lie back to back in shared
 // memory (slice t at t * bbytes), so for A slice s one MMA against the first
-// KS - s slices of B, with its accumulator starting at level s, adds A_s B_t
-// into level s + t for every t <= KS - 1 - s at once: each A slice is read once
+// 8 - s slices of B, with its accumulator starting at level s, adds A_s B_t
+// into level s + t for every t <= 7 - s at once: each A slice is read once
 // per 16-column K chunk.  Products wider than 256 columns are cut into
-// 256-column MMAs.  The first MMA (s = 0, first K chunk) initialises all
-// levels.  adesc / bdesc: descriptors of slice 0 of A and B; K chunks are
-// 256 bytes apart, 8-row groups of B kdim * 16 bytes (encoded address >> 4).
-template <int N, int KCH, int KS>
-__device__ __forceinline__ void mma_tile(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t abytes) {
+// 256-column MMAs.  adesc / bdesc: descriptors of slice 0 of A and B; K chunks
+// are 256 bytes apart, 8-row groups of B kdim * 16 bytes (encoded address >> 4).
+template <int N, int KCH>
+__device__ __forceinline__ void mma_tile(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc) {
   constexpr int K = 16 * KCH;
+  constexpr uint32_t abytes = kRows * K * 2;
 #pragma unroll
-  for (int s = 0; s < KS; ++s) {
+  for (int s = 0; s < qsby::kA; ++s) {
     constexpr int kMax = 256;
 #pragma unroll
-    for (int c0 = 0; c0 < (KS - s) * N; c0 += kMax) {
-      const int w = (KS - s) * N - c0 < kMax ? (KS - s) * N - c0 : kMax;
-      const uint32_t idesc = idesc_bf16(kRows, w);
+    for (int c0 = 0; c0 < (kLv - s) * N; c0 += kMax) {
+      const int w = (kLv - s) * N - c0 < kMax ? (kLv - s) * N - c0 : kMax;
+      const uint32_t idesc = idesc_f16(kRows, w);
 #pragma unroll
       for (int kk = 0; kk < KCH; ++kk)
-        mma_bf16(d_tmem + (uint32_t)(s * N + c0), adesc + ((s * abytes + kk * 256) >> 4),
-                 bdesc + (((uint32_t)c0 * K * 2 + kk * 256) >> 4), idesc, 1u);
+        mma_f16(d_tmem + (uint32_t)(s * N + c0), adesc + ((s * abytes + kk * 256) >> 4),
+                bdesc + (((uint32_t)c0 * K * 2 + kk * 256) >> 4), idesc, 1u);
     }
   }
 }
 
-
-// scale 2^(Ea + Eb - 2046 - 54) (seven slices) or 2^(Ea + Eb - 2046 - 53)
-// (eight: the recombined sum is kept divided by 2^8) with biased Ea, Eb
-template <int KS>
-__host__ __device__ constexpr int scale_off() { return KS == 8 ? 53 : 54; }
-
-// Per-CTA constants of a dense gate: the column exponent maxima of B (in
-// csc), B's digit slices, the initialising MMA's operands (A rows
-// (1, 256, 65536, 0, ...), B columns holding P_L(n) in three parts), the
-// target offsets of the group members and the row offsets of the tile.  Every
-// step runs over all (column, row) pairs of B at once, the maxima and the
-// digit column sums (colsum: KS x N ints) through shared-memory atomics, so
-// the setup is short next to one tile even for small states.
-template <int NT, int KS, bool kMagicPre>
-__device__ void tile_constants(const TcParams& p, unsigned char* b_dig, unsigned char* a_pre, unsigned char* b_pre,
-                               int* csc, int* colsum, uint64_t* toff, uint64_t* rowoff, int tid, int nthr) {
-  constexpr int D = 1 << NT, K = 2 * D, N = 2 * D, BBYTES = N * K * 2;
-  for (int n = tid; n < N; n += nthr) csc[n] = emax_floor<KS>();
-  for (int i = tid; i < KS * N; i += nthr) colsum[i] = 0;
-  __syncthreads();
-  // column fastest across threads: the lanes of a warp update different
-  // columns' maxima and sums (no same-address atomics)
-  for (int idx = tid; idx < N * K; idx += nthr) {
-    const int n = idx % N, k = idx / N;
-    atomicMax(csc + n, qsoz::biased_exp((uint32_t)__double2hiint(realified(p, D, k, n))));
-  }
-  __syncthreads();
-  for (int idx = tid; idx < N * K; idx += nthr) {
-    const int n = idx % N, k = idx / N;
-    const double v = realified(p, D, k, n);
-    float f[KS];
-    digits<KS>((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v), csc[n], f);
-    const uint32_t off = canon_off16(n, k, K);
+// The initialising MMA: every level column of the buffer at dcol starts at its P_L(n).
+template <int N>
+__device__ __forceinline__ void mma_start(uint32_t dcol, const unsigned char* a_pre, const unsigned char* b_pre) {
+  constexpr uint32_t LCOLS = kLv * N;
+  const uint64_t pad = smem_desc(smem_u32(a_pre), 128, 256), pbd = smem_desc(smem_u32(b_pre), 128, 256);
 #pragma unroll
-    for (int t = 0; t < KS; ++t) {
-      *reinterpret_cast<uint16_t*>(b_dig + t * BBYTES + off) = (uint16_t)(pack_bf16(f[t], 0.0f) & 0xFFFFu);
-      if (f[t] != 0.0f) atomicAdd(colsum + t * N + n, (int)f[t]);
-    }
+  for (uint32_t c0 = 0; c0 < LCOLS; c0 += 256) {
+    const uint32_t w = LCOLS - c0 < 256 ? LCOLS - c0 : 256;
+    mma_f16(dcol + c0, pad, pbd + ((c0 * 32) >> 4), idesc_f16(kRows, (int)w), 0u);
   }
-  __syncthreads();
-  // the start values P_L(n) = M - 192 sum_{t < L} colsum_t(n), one (L, n) per thread
-  for (int idx = tid; idx < KS * N; idx += nthr) {
-    const int L = idx / N, n = idx % N;
-    int corr = 0;
-    for (int t = 0; t < L; ++t) corr += colsum[t * N + n];
-    int pp[3];
-    qsoz::split_start((kMagicPre ? (int)qsoz::kPreMagic : 0) - qsoz::kDigitOffset * corr, pp);
-    const int col = L * N + n;
-#pragma unroll
-    for (int k = 0; k < 16; ++k)
-      *reinterpret_cast<uint16_t*>(b_pre + canon_off16(col, k, 16)) =
-          (uint16_t)(pack_bf16(k < 3 ? (float)pp[k] : 0.0f, 0.0f) & 0xFFFFu);
-  }
+}
+
+// Slice products of operands with K = 16 KCH columns.
+template <int N, int KCH>
+__device__ __forceinline__ void mma_products(uint32_t dcol, const unsigned char* A, const unsigned char* B) {
+  constexpr uint32_t sbo = KCH * 16 * 16;
+  mma_tile<N, KCH>(dcol, smem_desc(smem_u32(A), 128, sbo), smem_desc(smem_u32(B), 128, sbo));
+}
+
+// Rows (2^-24, 2^-16, 2^-8, 0, ...) of the initialising MMA's A.
+__device__ __forceinline__ void fill_start_rows(unsigned char* a_pre, int tid, int nthr) {
   for (int idx = tid; idx < kRows * 16; idx += nthr) {
     const int g = idx >> 4, k = idx & 15;
     *reinterpret_cast<uint16_t*>(a_pre + canon_off16(g, k, 16)) =
-        (uint16_t)(pack_bf16(k == 0 ? 1.0f : (k == 1 ? 256.0f : (k == 2 ? 65536.0f : 0.0f)), 0.0f) & 0xFFFFu);
+        (uint16_t)(k == 0 ? 0x0001 : (k == 1 ? 0x0100 : (k == 2 ? 0x1C00 : 0)));
   }
-  for (int j = tid; j < D; j += nthr) {
+}
+
+// The column of the initialising MMA's B that starts level column `col` at P.
+__device__ __forceinline__ void fill_start_column(unsigned char* b_pre, int col, int P) {
+  int pp[3];
+  qsby::split_start(P, pp);
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    *reinterpret_cast<uint16_t*>(b_pre + canon_off16(col, k, 16)) = k < 3 ? half_bits(pp[k]) : (uint16_t)0;
+}
+
+// Target offsets of the group members and row offsets of the tile.
+template <int NT>
+__device__ __forceinline__ void fill_offsets(const TcParams& p, uint64_t* toff, uint64_t* rowoff, int tid, int nthr) {
+  for (int j = tid; j < (1 << NT); j += nthr) {
     uint64_t off = 0;
 #pragma unroll
     for (int q = 0; q < NT; ++q)
@@ -206,71 +184,115 @@ __device__ void tile_constants(const TcParams& p, unsigned char* b_dig, unsigned
   }
 }
 
-// The initialising MMA (every level column of the buffer at dcol starts at its
-// P_L(n)) and the slice products of one tile; issued by one thread.
-template <int N, int KCH, int KS>
-__device__ __forceinline__ void mma_full_tile(uint32_t dcol, const unsigned char* a_pre, const unsigned char* b_pre,
-                                              const unsigned char* A, const unsigned char* b_dig) {
-  constexpr uint32_t LCOLS = KS * N;
-  constexpr uint32_t sbo = KCH * 16 * 16;
-  const uint64_t pad = smem_desc(smem_u32(a_pre), 128, 256), pbd = smem_desc(smem_u32(b_pre), 128, 256);
-#pragma unroll
-  for (uint32_t c0 = 0; c0 < LCOLS; c0 += 256) {
-    const uint32_t w = LCOLS - c0 < 256 ? LCOLS - c0 : 256;
-    mma_bf16(dcol + c0, pad, pbd + ((c0 * 32) >> 4), idesc_bf16(kRows, (int)w), 0u);
+// column exponent field -> the increment it adds to a result's exponent field
+__device__ __forceinline__ int column_scale(int field) { return field - ((2046 + qsby::kScale) << 20); }
+
+// Per-CTA constants of a dense gate: the column exponent fields of B (in
+// csc), B's digit slices, the initialising MMA's operands, the target offsets
+// of the group members and the row offsets of the tile.  Every step runs over
+// all (column, row) pairs of B at once, the maxima and the digit column sums
+// (colsum: 8 x N ints) through shared-memory atomics, so the setup is short
+// next to one tile even for small states.
+template <int NT>
+__device__ void tile_constants(const TcParams& p, unsigned char* b_dig, unsigned char* a_pre, unsigned char* b_pre,
+                               int* csc, int* colsum, uint64_t* toff, uint64_t* rowoff, int tid, int nthr) {
+  constexpr int D = 1 << NT, K = 2 * D, N = 2 * D, BBYTES = N * K * 2;
+  for (int n = tid; n < N; n += nthr) csc[n] = 0;
+  for (int i = tid; i < kLv * N; i += nthr) colsum[i] = 0;
+  __syncthreads();
+  // column fastest across threads: the lanes of a warp update different
+  // columns' maxima and sums (no same-address atomics)
+  for (int idx = tid; idx < N * K; idx += nthr) {
+    const int n = idx % N, k = idx / N;
+    atomicMax(csc + n, __double2hiint(realified(p, D, k, n)) & 0x7FFFFFFF);
   }
-  const uint64_t ad = smem_desc(smem_u32(A), 128, sbo), bd = smem_desc(smem_u32(b_dig), 128, sbo);
-  mma_tile<N, KCH, KS>(dcol, ad, bd, kRows * KCH * 16 * 2);
+  __syncthreads();
+  for (int idx = tid; idx < N * K; idx += nthr) {
+    const int n = idx % N, k = idx / N;
+    const double v = realified(p, D, k, n);
+    int d[qsby::kB];
+    qsby::digits_b((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v), qsby::row_field((uint32_t)csc[n]), d);
+    const uint32_t off = canon_off16(n, k, K);
+#pragma unroll
+    for (int t = 0; t < qsby::kB; ++t) {
+      *reinterpret_cast<uint16_t*>(b_dig + t * BBYTES + off) = half_bits(d[t]);
+      if (d[t] != 0) atomicAdd(colsum + n * kLv + t, d[t]);
+    }
+  }
+  fill_start_rows(a_pre, tid, nthr);
+  fill_offsets<NT>(p, toff, rowoff, tid, nthr);
+  __syncthreads();
+  for (int idx = tid; idx < kLv * N; idx += nthr) {
+    const int L = idx / N, n = idx % N;
+    fill_start_column(b_pre, L * N + n, qsby::start_value(L, K, colsum + n * kLv));
+  }
+  for (int n = tid; n < N; n += nthr) csc[n] = column_scale((int)qsby::row_field((uint32_t)csc[n]));
+}
+
+// one output: levels -> Q -> double, scaled by the row's and the column's powers of two
+template <int K>
+__device__ __forceinline__ double finish_output(const float* v, int egs, int scl) {
+  const double r = __ll2double_rn(qsby::combine<K>(v));
+  const int hi = __double2hiint(r);                // 0 only for r = 0, which stays 0
+  return __hiloint2double(hi != 0 ? hi + egs + scl : 0, __double2loint(r));
+}
+
+// fp16 operand words of four amplitudes (hi, lo words of re and im) at the 16-byte
+// column group `off` of every A slice
+__device__ __forceinline__ void store_slices(unsigned char* A, uint32_t off, uint32_t abytes, const uint32_t (*R)[4],
+                                             uint32_t ef1) {
+  uint32_t pk[4][qsby::kA];
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    qsby::packed_digits(qsby::bytes_of(R[e][0], R[e][1], ef1), qsby::bytes_of(R[e][2], R[e][3], ef1), pk[e]);
+#pragma unroll
+  for (int s = 0; s < qsby::kA; ++s)
+    *reinterpret_cast<uint4*>(A + s * abytes + off) = make_uint4(pk[0][s], pk[1][s], pk[2][s], pk[3][s]);
+}
+
+// largest high word without sign of an amplitude's parts
+__device__ __forceinline__ uint32_t max_abs(uint32_t m, const uint32_t* R) {
+  return max(m, max(R[0] & 0x7FFFFFFFu, R[2] & 0x7FFFFFFFu));
 }
 
 }  // namespace
 
-template <int NT, int THREADS, int NBUF, int CTAS, int KS>
-__global__ void __launch_bounds__(THREADS, CTAS) k_dense_ozaki(double2* __restrict__ psi, const __grid_constant__ TcParams p) {
-  constexpr int kS = KS;
+template <int NT, int THREADS, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS) k_dense_ozaki_small(double2* __restrict__ psi, const __grid_constant__ TcParams p) {
   constexpr int D = 1 << NT;
   constexpr int K = 2 * D, N = 2 * D;
   constexpr int CG = THREADS / kRows;         // threads per row
   constexpr int EPT = D / CG;                 // amplitudes per thread
   constexpr int CPW = 2 * EPT;                // accumulator columns per thread
   static_assert(EPT % 4 == 0, "four amplitudes per 16-byte slice store");
-  constexpr int ABYTES = kRows * K * 2;       // one bf16 digit slice of A
+  constexpr int ABYTES = kRows * K * 2;       // one digit slice of A
   constexpr int BBYTES = N * K * 2;
-  constexpr uint32_t LCOLS = kS * N;          // accumulator columns of one buffer
-  constexpr uint32_t TCOLS = tmem_cols(NBUF * LCOLS);
-  static_assert(NBUF * LCOLS <= 512, "tensor memory");
-  constexpr bool kMagicPre = K <= 32;         // accumulators start at the magic (no add in the epilogue)
-  constexpr uint32_t kMB = kMagicPre ? qsoz::kPreMagicBits : qsoz::kFaddMagicBits;
+  constexpr uint32_t LCOLS = kLv * N;         // accumulator columns
+  constexpr uint32_t TCOLS = tmem_cols(LCOLS);
+  static_assert(LCOLS <= 512, "tensor memory");
   constexpr int PREA = kRows * 32, PREB = (int)LCOLS * 32;   // initialising operands (K = 16)
   extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* a_dig = smem;                                        // NBUF x kS x ABYTES
-  unsigned char* b_dig = a_dig + NBUF * kS * ABYTES;                  // kS x BBYTES
-  unsigned char* a_pre = b_dig + kS * BBYTES;                         // PREA: rows (1, 256, 65536, 0...)
-  unsigned char* b_pre = a_pre + PREA;                                // PREB: (p0, p1, p2, 0...) per column
+  unsigned char* a_dig = smem;                                        // 7 x ABYTES
+  unsigned char* b_dig = a_dig + qsby::kA * ABYTES;                   // 8 x BBYTES
+  unsigned char* a_pre = b_dig + qsby::kB * BBYTES;                   // PREA
+  unsigned char* b_pre = a_pre + PREA;                                // PREB
   uint64_t* toff = reinterpret_cast<uint64_t*>(b_pre + PREB);         // D
   uint64_t* rowoff = toff + D;                                        // kRows
   uint64_t* tile_base = rowoff + kRows;                               // 2
-  uint64_t* mbar = tile_base + 2;                                     // 2
-  int* csc = reinterpret_cast<int*>(mbar + 2);                        // N: (column exponent - 2100) << 20
-  int* rowexp = csc + N;                                              // 2 x kRows: exponent field of the row maximum
-  int* colsum = rowexp + 2 * kRows;                                   // KS x N: digit column sums (setup)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(colsum + kS * N);
+  uint64_t* mbar = tile_base + 2;                                     // 1 (+ 1 pad)
+  int* csc = reinterpret_cast<int*>(mbar + 2);                        // N: exponent increment of a column
+  int* rowmax = csc + N;                                              // 2 x kRows: largest high word of a row
+  int* colsum = rowmax + 2 * kRows;                                   // N x 8: digit column sums (setup)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(colsum + kLv * N);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  tile_constants<NT, KS, kMagicPre>(p, b_dig, a_pre, b_pre, csc, colsum, toff, rowoff, tid, THREADS);
+  tile_constants<NT>(p, b_dig, a_pre, b_pre, csc, colsum, toff, rowoff, tid, THREADS);
   const int row_bits = p.tile_bits - NT;
-  for (int g = tid; g < kRows; g += THREADS) {
-    rowexp[g] = 0;
-    rowexp[kRows + g] = 0;
-  }
-  __syncthreads();
-  // column scales as exponent-field increments
-  for (int n = tid; n < N; n += THREADS) csc[n] = (int)((unsigned)(csc[n] - 2046 - scale_off<KS>()) << 20);
+  for (int g = tid; g < 2 * kRows; g += THREADS) rowmax[g] = 0;
   if (tid == 0) {
     tile_base[0] = insert_zeros(blockIdx.x, p.hi_ins, p.nhi) | p.ctrl_mask;
-#pragma unroll
-    for (int b = 0; b < NBUF; ++b) mbar_init(mbar + b, 1);      // one commit per tile
+    mbar_init(mbar, 1);                       // one commit per tile
   }
   if (warp == 0) {
     tmem_alloc(tmem_slot, TCOLS);
@@ -311,22 +333,21 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_dense_ozaki(double2* __restri
       R[i][3] = (uint32_t)__double2loint(v.y);
     }
   };
-  // row maximum of the exponents (the CG threads of a row are in different warps)
-  // (exponent fields compared in place: 0x7FF00000 of the high words)
+  // row maximum (the CG threads of a row are in different warps)
   auto row_max = [&](int slot) {
-    uint32_t em = (uint32_t)emax_floor<KS>() << 20;
+    uint32_t m = 0;
 #pragma unroll
-    for (int i = 0; i < EPT; ++i) em = max(em, max(R[i][0] & 0x7FF00000u, R[i][2] & 0x7FF00000u));
-    atomicMax(rowexp + slot * kRows + g, (int)em);
+    for (int i = 0; i < EPT; ++i) m = max_abs(m, R[i]);
+    atomicMax(rowmax + slot * kRows + g, (int)m);
   };
 
   // epilogue of one tile: levels -> exact integers -> doubles -> scatter
-  auto epilogue = [&](uint32_t tbuf, int egs, uint64_t rb) {
+  auto epilogue = [&](int egs, uint64_t rb) {
 #pragma unroll
     for (int cc = 0; cc < CPW; cc += 8) {
-      float v[kS][8];
+      float v[kLv][8];
 #pragma unroll
-      for (int L = 0; L < kS; ++L) tmem_ld8(tmem + tbuf + lane_addr + (uint32_t)(L * N + cg * CPW + cc), v[L]);
+      for (int L = 0; L < kLv; ++L) tmem_ld8(tmem + lane_addr + (uint32_t)(L * N + cg * CPW + cc), v[L]);
       tmem_wait_ld();
       if (row_ok) {
         const int4 s0 = *reinterpret_cast<const int4*>(csc + cg * CPW + cc);
@@ -335,13 +356,10 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_dense_ozaki(double2* __restri
         double o[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          uint32_t bits[kS];
+          float u[kLv];
 #pragma unroll
-          for (int L = 0; L < kS; ++L)
-            bits[L] = kMagicPre ? __float_as_uint(v[L][q]) : __float_as_uint(v[L][q] + 12582912.0f);
-          const double r = __ll2double_rn(qsoz::combine_pairs_u<KS, kMB>(bits));
-          const int hi = __double2hiint(r);                // 0 only for r = 0, which stays 0
-          o[q] = __hiloint2double(hi + (hi != 0 ? egs + scl[q] : 0), __double2loint(r));
+          for (int L = 0; L < kLv; ++L) u[L] = v[L][q];
+          o[q] = finish_output<K>(u, egs, scl[q]);
         }
 #pragma unroll
         for (int q = 0; q < 8; q += 2) psi[rb | tofs((cc + q) >> 1)] = make_double2(o[q], o[q + 1]);
@@ -356,63 +374,32 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_dense_ozaki(double2* __restri
     tile_base[1] = insert_zeros(blockIdx.x + gridDim.x, p.hi_ins, p.nhi) | p.ctrl_mask;
   __syncthreads();
 
-  uint32_t phases = 0;
+  uint32_t phase = 0;
   bool failed = false;
   int it = 0;
-  int eg_prev = 0;
-  uint64_t rb_prev = 0;
   for (uint64_t c = blockIdx.x; c < p.ntiles; c += gridDim.x, ++it) {
-    const int b = NBUF == 2 ? (it & 1) : 0;
     const int par = it & 1;                   // tile parity: row-maximum and base slots
     const uint64_t rb = tile_base[par] | roff;
     const bool has_next = c + gridDim.x < p.ntiles;
-    const int egs = rowexp[par * kRows + g];   // exponent field of the row maximum
-    const int eg = egs >> 20;
-    // digit slices of this thread's amplitudes, 16 bytes per slice and 4 amplitudes
-    unsigned char* A = a_dig + b * (kS * ABYTES);
+    const int egs = (int)qsby::row_field((uint32_t)rowmax[par * kRows + g]);   // exponent field of the row
 #pragma unroll
-    for (int i = 0; i < EPT; i += 4) {
-      uint32_t pk[4][kS];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const uint32_t* w = R[i + e];
-        const uint64_t tr = qsoz::fixed_ks<KS>(w[0], w[1], eg), ti = qsoz::fixed_ks<KS>(w[2], w[3], eg);
-        pk[e][0] = pack_bf16(qsoz::top_digit<KS>(tr), qsoz::top_digit<KS>(ti));
-        qsoz::packed_digits_fast<KS>(tr, ti, pk[e]);
-      }
-      const uint32_t off = canon_off16(g, 2 * (l0 + i), K);
-#pragma unroll
-      for (int s = 0; s < kS; ++s)
-        *reinterpret_cast<uint4*>(A + s * ABYTES + off) = make_uint4(pk[0][s], pk[1][s], pk[2][s], pk[3][s]);
-    }
+    for (int i = 0; i < EPT; i += 4)
+      store_slices(a_dig, canon_off16(g, 2 * (l0 + i), K), ABYTES, R + i, (uint32_t)egs + 0x100000u);
     fence_proxy_async();
     __syncthreads();
     if (tid == 0) {
       fence_after_sync();
-      const uint32_t dcol = tmem + (uint32_t)(b * LCOLS);
-      mma_full_tile<N, K / 16, KS>(dcol, a_pre, b_pre, A, b_dig);
-      mma_commit(mbar + b);
+      mma_start<N>(tmem, a_pre, b_pre);
+      mma_products<N, K / 16>(tmem, a_dig, b_dig);
+      mma_commit(mbar);
     }
-    if (cg == 0) rowexp[par * kRows + g] = 0;   // read by every thread of the row before the barrier
+    if (cg == 0) rowmax[par * kRows + g] = 0;   // read by every thread of the row before the barrier
     // loads of the next tile, in flight during the MMAs and the epilogue
     if (has_next) load_tile(tile_base[par ^ 1]);
-    bool timed_out = false;
-    if (NBUF == 2) {
-      if (it > 0) {
-        const int pb = b ^ 1;
-        timed_out = wait_phase(mbar + pb, (phases >> pb) & 1u);
-        phases ^= 1u << pb;
-        fence_after_sync();
-        epilogue((uint32_t)(pb * LCOLS), eg_prev, rb_prev);
-      }
-    } else {
-      timed_out = wait_phase(mbar, phases & 1u);
-      phases ^= 1u;
-      fence_after_sync();
-      epilogue(0u, egs, rb);
-    }
-    eg_prev = egs;
-    rb_prev = rb;
+    const bool timed_out = wait_phase(mbar, phase);
+    phase ^= 1u;
+    fence_after_sync();
+    epilogue(egs, rb);
     if (has_next) row_max(par ^ 1);
     if (tid == helper && c + 2 * (uint64_t)gridDim.x < p.ntiles)
       tile_base[par] = insert_zeros(c + 2 * (uint64_t)gridDim.x, p.hi_ins, p.nhi) | p.ctrl_mask;
@@ -421,50 +408,42 @@ __global__ void __launch_bounds__(THREADS, CTAS) k_dense_ozaki(double2* __restri
     fence_after_sync();
     if (failed) break;
   }
-  if (NBUF == 2 && !failed && it > 0) {
-    const int pb = (it - 1) & 1;
-    const bool timed_out = wait_phase(mbar + pb, (phases >> pb) & 1u);
-    fence_after_sync();
-    epilogue((uint32_t)(pb * LCOLS), eg_prev, rb_prev);
-    fence_before_sync();
-    failed = __syncthreads_or(timed_out) != 0;
-  }
   if (failed && tid == 0) atomicExch(p.err, 1);
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, TCOLS);
 }
 
-template <int NT, int THREADS, int NBUF, int CTAS, int kS>
-static cudaError_t dense_ozaki_nt(void* amps, const TcParams& p, cudaStream_t st) {
+template <int NT, int THREADS, int CTAS>
+static cudaError_t dense_ozaki_small(void* amps, const TcParams& p, cudaStream_t st) {
   constexpr int D = 1 << NT, K = 2 * D, N = 2 * D;
-  constexpr size_t smem = (size_t)NBUF * kS * (kRows * K * 2) + (size_t)kS * (N * K * 2) + kRows * 32 +
-                          (size_t)kS * N * 32 + 8 * (D + kRows + 4) + 4 * (N + 2 * kRows + kS * N) + 16;
+  constexpr size_t smem = (size_t)qsby::kA * (kRows * K * 2) + (size_t)qsby::kB * (N * K * 2) + kRows * 32 +
+                          (size_t)kLv * N * 32 + 8 * (D + kRows + 4) + 4 * (N + 2 * kRows + kLv * N) + 16;
   static_assert(smem * CTAS <= 227 * 1024, "shared memory");
-  static_assert(CTAS * tmem_cols(NBUF * kS * N) <= 512, "tensor memory");
+  static_assert(CTAS * tmem_cols(kLv * N) <= 512, "tensor memory");
   static bool attr_done = false;
   if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki<NT, THREADS, NBUF, CTAS, kS>,
+    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki_small<NT, THREADS, CTAS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
-  // for 3 and 4 targets, eight times the resident CTAs: the late ones even out
-  // the SMs' tile counts at the end of the pass (7% and 2% faster measured)
-  const uint64_t maxb = (uint64_t)num_sms() * CTAS * (NT <= 4 ? 8 : 1);
+  const uint64_t maxb = (uint64_t)num_sms() * CTAS;
   const unsigned g = (unsigned)(p.ntiles < maxb ? p.ntiles : maxb);
-  k_dense_ozaki<NT, THREADS, NBUF, CTAS, kS><<<g, THREADS, smem, st>>>(static_cast<double2*>(amps), p);
+  k_dense_ozaki_small<NT, THREADS, CTAS><<<g, THREADS, smem, st>>>(static_cast<double2*>(amps), p);
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// Warp-specialised form for two to four targets (K <= 32, so the accumulators
-// start at the magic and the epilogue reads level bit patterns directly).
-// Eight producer warps gather tiles with cp.async into a ring of S staging
-// slots (several tiles of loads in flight), take the row maxima (two threads
+// Warp-specialised form for two to four targets (K <= 32, so every level
+// starts at the magic and the epilogue reads level bit patterns directly).
+// A unit is one tile, or two for three targets (as many amplitudes a unit as
+// with four: one tile a unit, with four-deep rings, took 1.74 ms at 28 qubits
+// against 1.50).  Eight producer warps gather units with cp.async into a ring of
+// S staging slots (64 KB of loads in flight), take the row maxima (two threads
 // per row, one shuffle) and write the digit slices into a ring of NA operand
 // buffers; one thread issues the initialising MMA and the slice MMAs of each
-// tile into a ring of NTM tensor-memory buffers; eight epilogue warps (two per
-// lane quarter, each half of a row's columns) recombine, convert and store.
+// tile into a ring of NTM tensor-memory buffers; 16 epilogue warps (four per
+// lane quarter, each a part of a row's columns) recombine, convert and store.
 // Hand-offs are mbarriers: afull (producers -> MMA), aempty and accfull
 // (MMA completion -> producers, epilogue), tempty (epilogue -> MMA) and
 // mready (MMA thread -> epilogue, releasing onward the row exponents that the
@@ -476,7 +455,10 @@ static cudaError_t dense_ozaki_nt(void* amps, const TcParams& p, cudaStream_t st
 // and gives up when another role has.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int kWsE = 8, kWsP = 8;                   // epilogue and producer warps
+// epilogue and producer warps: with 8 and 8 the kernels waited for the epilogue
+// (28 qubits, 3 / 4 targets 1.76 / 1.52 ms as eight warps of eight columns at a
+// time, 1.91 / 1.65 of four; 16 warps 1.74 / 1.51)
+constexpr int kWsE = 16, kWsP = 8;
 constexpr int kWsThreads = 32 * (kWsE + kWsP + 1);  // and the MMA warp
 
 __device__ __forceinline__ bool wait_ring(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
@@ -494,23 +476,25 @@ __device__ __forceinline__ bool wait_ring_warp(uint64_t* bar, uint32_t parity, v
   return __any_sync(0xFFFFFFFFu, wait_ring(bar, parity, abort_flag)) != 0;
 }
 
-template <int NT, int KS>
+template <int NT>
 struct Ws {
   static constexpr int D = 1 << NT, K = 2 * D, N = 2 * D;
-  static constexpr int LCOLS = KS * N;
-  static constexpr int NTM = NT == 3 ? 4 : 2;        // accumulator buffers
+  static constexpr int RB = NT == 3 ? 2 : 1;         // 128-row tiles that go through the rings as one unit
+  static constexpr int LCOLS = kLv * N;              // accumulator columns of a tile
+  static constexpr int NTM = 2;                      // accumulator buffers
   static constexpr int TSTRIDE = 512 / NTM;          // their column stride
-  static constexpr int NA = NT == 3 ? 4 : 2;         // operand buffers
+  static constexpr int NA = 2;                       // operand buffers
   static constexpr int NM = NA + NTM;                // metadata slots
-  static constexpr int S = NT == 3 ? 4 : 2;          // staging slots (64 KB of loads in flight)
+  static constexpr int S = 2;                        // staging slots (64 KB of loads in flight)
   static constexpr int PT = 32 * kWsP;               // producer threads
-  static constexpr int EPP = D / 2;                  // amplitudes per producer thread (two per row)
-  static constexpr int EPE = D / 2;                  // amplitudes per epilogue thread (two per row)
+  static constexpr int EPP = D / 2;                  // amplitudes of a tile per producer thread (two per row)
+  static constexpr int EPE = RB * D / (kWsE / 4);    // amplitudes of a unit per epilogue thread
   static constexpr int ABYTES = kRows * K * 2, BBYTES = N * K * 2;
-  static constexpr int SLOT = PT * EPP * 16;
+  static constexpr int ABUF = RB * qsby::kA * ABYTES;   // operands of a unit
+  static constexpr int SLOT = RB * PT * EPP * 16;
   static constexpr size_t a_off = 0;
-  static constexpr size_t b_off = a_off + (size_t)NA * KS * ABYTES;
-  static constexpr size_t apre_off = b_off + (size_t)KS * BBYTES;
+  static constexpr size_t b_off = a_off + (size_t)NA * ABUF;
+  static constexpr size_t apre_off = b_off + (size_t)qsby::kB * BBYTES;
   static constexpr size_t bpre_off = apre_off + kRows * 32;
   static constexpr size_t stg_off = bpre_off + (size_t)LCOLS * 32;
   static constexpr size_t toff_off = stg_off + (size_t)S * SLOT;
@@ -518,21 +502,21 @@ struct Ws {
   static constexpr size_t bar_off = rowoff_off + 8 * kRows;
   static constexpr size_t csc_off = bar_off + 8 * (2 * NA + 2 * NTM + NM);
   static constexpr size_t ex_off = csc_off + 4 * N;
-  static constexpr size_t colsum_off = ex_off + 4 * (size_t)NM * kRows;
-  static constexpr size_t slot_off = colsum_off + 4 * (size_t)KS * N;
+  static constexpr size_t colsum_off = ex_off + 4 * (size_t)NM * RB * kRows;
+  static constexpr size_t slot_off = colsum_off + 4 * (size_t)kLv * N;
   static constexpr size_t bytes = slot_off + 16;
-  static_assert(LCOLS <= TSTRIDE && NTM * TSTRIDE <= 512, "tensor memory");
+  static_assert(RB * LCOLS <= TSTRIDE && NTM * TSTRIDE <= 512, "tensor memory");
   static_assert(bytes <= 227 * 1024, "shared memory");
   static_assert(K <= 32 && EPP % 4 == 0 && PT / kRows == 2, "mapping");
 };
 
 }  // namespace
 
-template <int NT, int KS>
+template <int NT>
 __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __restrict__ psi, const __grid_constant__ TcParams p) {
-  using W = Ws<NT, KS>;
+  using W = Ws<NT>;
   constexpr int K = W::K, N = W::N, NA = W::NA, NTM = W::NTM, NM = W::NM, S = W::S;
-  constexpr int EPP = W::EPP, EPE = W::EPE, PT = W::PT;
+  constexpr int EPP = W::EPP, EPE = W::EPE, PT = W::PT, RB = W::RB;
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* a_dig = smem + W::a_off;
   unsigned char* b_dig = smem + W::b_off;
@@ -553,7 +537,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + W::slot_off + 4);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  tile_constants<NT, KS, true>(p, b_dig, a_pre, b_pre, csc, colsum, toff, rowoff, tid, kWsThreads);
+  tile_constants<NT>(p, b_dig, a_pre, b_pre, csc, colsum, toff, rowoff, tid, kWsThreads);
   if (tid == 0) {
 #pragma unroll
     for (int j = 0; j < NA; ++j) {
@@ -574,109 +558,114 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
     tmem_relinquish();
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  fence_proxy_async();                        // B's slices and the initialising operands, for the MMAs
   fence_before_sync();
   __syncthreads();
   fence_after_sync();
-  for (int n = tid; n < N; n += kWsThreads) csc[n] = (int)((unsigned)(csc[n] - 2046 - scale_off<KS>()) << 20);
-  __syncthreads();
   const uint32_t tmem = *tmem_slot;
   const int row_bits = p.tile_bits - NT;
-  const uint64_t grid = gridDim.x;
-  // tile bases: x(c) = insert_zeros(c); x(c + d) = ((x(c) | hole) + insert_zeros(d)) & ~hole
+  const uint64_t grid = gridDim.x, nunits = p.ntiles / RB;
+  // unit u holds the tiles u RB + r, whose bases are x(u RB) | r rstep.
+  // x(c) = insert_zeros(c); x(c + d) = ((x(c) | hole) + insert_zeros(d)) & ~hole
   uint64_t hole = 0;
   for (int q = 0; q < p.nhi; ++q) hole |= 1ull << p.hi_ins[q];
-  const uint64_t gstep = insert_zeros(grid, p.hi_ins, p.nhi);
+  const uint64_t gstep = insert_zeros(grid * RB, p.hi_ins, p.nhi);
+  const uint64_t rstep = RB > 1 ? insert_zeros(1, p.hi_ins, p.nhi) : 0;
   auto step = [&](uint64_t x, uint64_t d) -> uint64_t { return ((x | hole) + d) & ~hole; };
 
   if (warp < kWsE) {
-    // ---- epilogue: row g (tensor-memory lane), amplitudes [eh EPE, (eh + 1) EPE) ----
-    const int q = warp & 3, eh = warp >> 2;
+    // ---- epilogue: row g (tensor-memory lane) of tile r, amplitudes [l0, l0 + EPE) ----
+    const int q = warp & 3;
+    constexpr int PER = kWsE / 4 / RB;        // threads per row
+    const int r = (warp >> 2) / PER, l0 = ((warp >> 2) % PER) * EPE;
     const int g = 32 * q + lane;
     const bool row_ok = g < (1 << row_bits);
     const uint32_t lane_addr = (uint32_t)(32 * q) << 16;
     uint64_t te[EPE];                         // byte offsets of this thread's amplitudes in a tile
 #pragma unroll
-    for (int i = 0; i < EPE; ++i) te[i] = (rowoff[g] | toff[eh * EPE + i]) << 4;
-    uint64_t xb = insert_zeros(blockIdx.x, p.hi_ins, p.nhi);
+    for (int i = 0; i < EPE; ++i) te[i] = (rowoff[g] | toff[l0 + i] | r * rstep) << 4;
+    uint64_t xb = insert_zeros(blockIdx.x * (uint64_t)RB, p.hi_ins, p.nhi);
     for (int i = 0;; ++i, xb = step(xb, gstep)) {
       const uint64_t c = blockIdx.x + (uint64_t)i * grid;
-      if (c >= p.ntiles) break;
+      if (c >= nunits) break;
       const int k = i % NTM, m = i % NM;
       if (wait_ring_warp(mready + m, (uint32_t)(i / NM) & 1u, abort_flag)) {
         *abort_flag = 1;
         break;
       }
-      const int egs = meta_ex[m * kRows + g];
+      const int egs = meta_ex[(m * RB + r) * kRows + g];
       char* tp = reinterpret_cast<char*>(psi) + ((xb | p.ctrl_mask) << 4);
       if (wait_ring_warp(accfull + k, (uint32_t)(i / NTM) & 1u, abort_flag)) {
         *abort_flag = 1;
         break;
       }
       fence_after_sync();
-      const uint32_t tb = tmem + (uint32_t)(k * W::TSTRIDE) + lane_addr + (uint32_t)(eh * 2 * EPE);
+      const uint32_t tb = tmem + (uint32_t)(k * W::TSTRIDE + r * W::LCOLS + 2 * l0) + lane_addr;
 #pragma unroll
-      for (int cc = 0; cc < 2 * EPE; cc += 8) {
-        float v[KS][8];
+      for (int cc = 0; cc < 2 * EPE; cc += 4) {
+        float v[kLv][4];
 #pragma unroll
-        for (int L = 0; L < KS; ++L) tmem_ld8(tb + (uint32_t)(L * N + cc), v[L]);
+        for (int L = 0; L < kLv; ++L) tmem_ld4(tb + (uint32_t)(L * N + cc), v[L]);
         tmem_wait_ld();
-        if (cc + 8 == 2 * EPE) {                // the buffer is read: hand it back to the MMA thread
+        if (cc + 4 == 2 * EPE) {                // the buffer is read: hand it back to the MMA thread
           fence_before_sync();
           __syncwarp();
           if (lane == 0) mbar_arrive(tempty + k);
         }
         if (row_ok) {
-          const int4 s0 = *reinterpret_cast<const int4*>(csc + eh * 2 * EPE + cc);
-          const int4 s1 = *reinterpret_cast<const int4*>(csc + eh * 2 * EPE + cc + 4);
-          const int scl[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-          double o[8];
+          const int4 s0 = *reinterpret_cast<const int4*>(csc + 2 * l0 + cc);
+          const int scl[4] = {s0.x, s0.y, s0.z, s0.w};
+          double o[4];
 #pragma unroll
-          for (int qq = 0; qq < 8; ++qq) {
-            uint32_t bits[KS];
+          for (int qq = 0; qq < 4; ++qq) {
+            float u[kLv];
 #pragma unroll
-            for (int L = 0; L < KS; ++L) bits[L] = __float_as_uint(v[L][qq]);
-            const double r = __ll2double_rn(qsoz::combine_pairs_u<KS, qsoz::kPreMagicBits>(bits));
-            const int hi = __double2hiint(r);   // 0 only for r = 0, which stays 0
-            o[qq] = __hiloint2double(hi != 0 ? hi + egs + scl[qq] : 0, __double2loint(r));
+            for (int L = 0; L < kLv; ++L) u[L] = v[L][qq];
+            o[qq] = finish_output<K>(u, egs, scl[qq]);
           }
 #pragma unroll
-          for (int qq = 0; qq < 8; qq += 2)
+          for (int qq = 0; qq < 4; qq += 2)
             *reinterpret_cast<double2*>(tp + te[(cc + qq) >> 1]) = make_double2(o[qq], o[qq + 1]);
         }
       }
     }
   } else if (warp < kWsE + kWsP) {
-    // ---- producers: row g, part h (amplitudes [h EPP, (h + 1) EPP)) ----
+    // ---- producers: row g of every tile of the unit, part h (amplitudes [h EPP, (h + 1) EPP)) ----
     const int pt = tid - 32 * kWsE, pw = pt >> 5;
-    const int g = 16 * pw + (lane >> 1), h = lane & 1;
+    // eight lanes (one 128-byte phase of a 16-byte store) hold eight rows of one
+    // column group, so the slice stores meet no bank twice
+    const int g = 16 * pw + (lane & 7) + 8 * (lane >> 4), h = (lane >> 3) & 1;
     const bool row_ok = g < (1 << row_bits);
     uint64_t tp[EPP];                         // byte offsets of this thread's amplitudes in a tile
 #pragma unroll
     for (int i = 0; i < EPP; ++i) tp[i] = (rowoff[g] | toff[h * EPP + i]) << 4;
     const uint32_t stg_addr = smem_u32(stg) + (uint32_t)pt * 16u;
     auto issue = [&](uint64_t x, int slot) {
-      const char* base = reinterpret_cast<const char*>(psi) + ((x | p.ctrl_mask) << 4);
 #pragma unroll
-      for (int i = 0; i < EPP; ++i)
-        cp_async16(stg_addr + (uint32_t)(slot * W::SLOT + i * PT * 16), row_ok ? (const void*)(base + tp[i]) : psi,
-                   row_ok ? 16u : 0u);
+      for (int r = 0; r < RB; ++r) {
+        const char* base = reinterpret_cast<const char*>(psi) + ((x | r * rstep | p.ctrl_mask) << 4);
+#pragma unroll
+        for (int i = 0; i < EPP; ++i)
+          cp_async16(stg_addr + (uint32_t)(slot * W::SLOT + (r * EPP + i) * PT * 16),
+                     row_ok ? (const void*)(base + tp[i]) : psi, row_ok ? 16u : 0u);
+      }
     };
-    uint64_t xi = insert_zeros(blockIdx.x, p.hi_ins, p.nhi);   // base of the next tile to issue
+    uint64_t xi = insert_zeros(blockIdx.x * (uint64_t)RB, p.hi_ins, p.nhi);   // base of the next tile to issue
 #pragma unroll
     for (int sl = 0; sl < S; ++sl) {
       const uint64_t c = blockIdx.x + (uint64_t)sl * grid;
-      if (c < p.ntiles) issue(xi, sl);
+      if (c < nunits) issue(xi, sl);
       cp_async_commit();
       xi = step(xi, gstep);
     }
     for (int i = 0;; ++i) {
       const uint64_t c = blockIdx.x + (uint64_t)i * grid;
-      if (c >= p.ntiles) break;
+      if (c >= nunits) break;
       const int slot = i % S, j = i % NA, m = i % NM;
       cp_async_wait<S - 1>();
-      uint32_t R[EPP][4];
+      uint32_t R[RB * EPP][4];
 #pragma unroll
-      for (int i2 = 0; i2 < EPP; ++i2) {
+      for (int i2 = 0; i2 < RB * EPP; ++i2) {
         uint4 v;
         asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
                      : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
@@ -686,15 +675,19 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
         R[i2][2] = v.w;
         R[i2][3] = v.z;
       }
-      // row maximum of the exponent fields (the row's other part is the neighbouring lane)
-      uint32_t em = (uint32_t)emax_floor<KS>() << 20;
+      // exponent fields of the rows (a row's other part is in lane xor 8)
+      uint32_t em[RB];
 #pragma unroll
-      for (int i2 = 0; i2 < EPP; ++i2) em = max(em, max(R[i2][0] & 0x7FF00000u, R[i2][2] & 0x7FF00000u));
-      em = max(em, __shfl_xor_sync(0xFFFFFFFFu, em, 1));
+      for (int r = 0; r < RB; ++r) {
+        em[r] = 0;
+#pragma unroll
+        for (int i2 = 0; i2 < EPP; ++i2) em[r] = max_abs(em[r], R[r * EPP + i2]);
+        em[r] = qsby::row_field(max(em[r], __shfl_xor_sync(0xFFFFFFFFu, em[r], 8)));
+      }
       // the slot's contents are in registers (used above): refill it S tiles ahead
       {
         const uint64_t c2 = c + (uint64_t)S * grid;
-        if (c2 < p.ntiles) issue(xi, slot);
+        if (c2 < nunits) issue(xi, slot);
         cp_async_commit();
         xi = step(xi, gstep);
       }
@@ -702,23 +695,14 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
         *abort_flag = 1;
         break;
       }
-      if (h == 0) meta_ex[m * kRows + g] = (int)em;
-      const int eg = (int)(em >> 20);
-      unsigned char* A = a_dig + j * (KS * W::ABYTES);
+      unsigned char* A = a_dig + j * W::ABUF;
 #pragma unroll
-      for (int i2 = 0; i2 < EPP; i2 += 4) {
-        uint32_t pk[4][KS];
+      for (int r = 0; r < RB; ++r) {
+        if (h == 0) meta_ex[(m * RB + r) * kRows + g] = (int)em[r];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const uint32_t* w = R[i2 + e];
-          const uint64_t tr = qsoz::fixed_ks<KS>(w[0], w[1], eg), ti = qsoz::fixed_ks<KS>(w[2], w[3], eg);
-          pk[e][0] = pack_bf16(qsoz::top_digit<KS>(tr), qsoz::top_digit<KS>(ti));
-          qsoz::packed_digits_fast<KS>(tr, ti, pk[e]);
-        }
-        const uint32_t off = canon_off16(g, 2 * (h * EPP + i2), K);
-#pragma unroll
-        for (int sl = 0; sl < KS; ++sl)
-          *reinterpret_cast<uint4*>(A + sl * W::ABYTES + off) = make_uint4(pk[0][sl], pk[1][sl], pk[2][sl], pk[3][sl]);
+        for (int i2 = 0; i2 < EPP; i2 += 4)
+          store_slices(A + r * qsby::kA * W::ABYTES, canon_off16(g, 2 * (h * EPP + i2), K), W::ABYTES, R + r * EPP + i2,
+                       em[r] + 0x100000u);
       }
       fence_proxy_async();
       __syncwarp();
@@ -730,7 +714,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
     int last = -1;
     for (int i = 0;; ++i) {
       const uint64_t c = blockIdx.x + (uint64_t)i * grid;
-      if (c >= p.ntiles) break;
+      if (c >= nunits) break;
       const int j = i % NA, k = i % NTM, m = i % NM;
       if (wait_ring(afull + j, (uint32_t)(i / NA) & 1u, abort_flag)) {
         *abort_flag = 1;
@@ -742,8 +726,12 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
         break;
       }
       fence_after_sync();
-      mma_full_tile<N, K / 16, KS>(tmem + (uint32_t)(k * W::TSTRIDE), a_pre, b_pre, a_dig + j * (KS * W::ABYTES),
-                                   b_dig);
+#pragma unroll
+      for (int r = 0; r < RB; ++r) {
+        const uint32_t dcol = tmem + (uint32_t)(k * W::TSTRIDE + r * W::LCOLS);
+        mma_start<N>(dcol, a_pre, b_pre);
+        mma_products<N, K / 16>(dcol, a_dig + j * W::ABUF + r * qsby::kA * W::ABYTES, b_dig);
+      }
       mma_commit(aempty + j);
       mma_commit(accfull + k);
       last = i;
@@ -758,45 +746,618 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <int NT, int KS>
+template <int NT>
 static cudaError_t dense_ozaki_ws(void* amps, const TcParams& p, cudaStream_t st) {
-  constexpr size_t smem = Ws<NT, KS>::bytes;
+  constexpr size_t smem = Ws<NT>::bytes;
   static bool attr_done = false;
   if (!attr_done) {
-    cudaError_t e =
-        cudaFuncSetAttribute(k_dense_ozaki_ws<NT, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki_ws<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr_done = true;
+  }
+  const uint64_t maxb = (uint64_t)num_sms(), nunits = p.ntiles / Ws<NT>::RB;
+  const unsigned g = (unsigned)(nunits < maxb ? nunits : maxb);
+  k_dense_ozaki_ws<NT><<<g, kWsThreads, smem, st>>>(static_cast<double2*>(amps), p);
+  return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// Five targets (K = N = 64), in two blocks of 32 columns of K and of N, warp
+// specialised.  16 producer warps (thread: row g, four amplitudes of each K
+// block, in registers; a block's registers are reloaded for the next tile as
+// soon as it is sliced) write one K block at a time into a ring of two operand
+// buffers (56 KB each).  One thread issues the MMAs, N block 0 over both K
+// blocks and then N block 1, into two accumulator buffers (256 columns each).
+// Eight epilogue warps (two per lane quarter) recombine, convert and store one
+// N block at a time.  B (64 KB) stays in shared memory.  So the MMAs on N block
+// 0 of a tile run behind the epilogue of the previous tile's N block 1, those
+// on N block 1 behind the epilogue of N block 0, and slicing behind both.
+//
+// Hand-offs are mbarriers: afull (producers -> MMA), aempty and accfull (MMA
+// completion), tempty (epilogue -> MMA) and mready (MMA thread -> epilogue,
+// releasing onward the row exponents that the producers wrote into one of four
+// metadata slots; a slot is rewritten four tiles later, after the slicing of
+// the tile before has waited for MMAs that waited for this tile's epilogue).
+// Row maxima go through shared memory and one barrier of the producer warps per
+// tile, which also carries the abort flag, so the producers leave together.
+// Every wait is bounded and gives up at once when another role has.
+// What bounds it: 10.3 thousand cycles per tile, of which the MMAs take 4.7 and
+// neither the integer pipe (51%) nor issue (48%) is full; the operand buffers
+// hold a single tile, so slicing the next one waits for the last MMAs on this
+// one.  A third buffer does not fit in shared memory.  Twelve epilogue warps in
+// place of eight (64 registers) took 2.53 ms against 2.30, and all phases in
+// the same 16 warps 3.05.
+// ---------------------------------------------------------------------------
+namespace {
+constexpr int kKnWarps = 16;                         // producer (five targets) or compute (six) warps
+constexpr int kKnC = 32 * kKnWarps;
+constexpr int kKnBlock = qsby::kB * 32 * 32 * 2;     // 16 KB: eight slices of a 32 x 32 block of B
+
+// barrier of those warps; true for all if any thread says so
+__device__ __forceinline__ bool compute_barrier_or(bool x) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n barrier.cta.red.or.pred p, 1, %2, q;\n"
+      " selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(r)
+      : "r"((uint32_t)x), "n"(kKnC)
+      : "memory");
+  return r != 0;
+}
+
+// bounded wait that gives up at once when another role has, and says so
+__device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  if (mbar_try_wait(bar, parity)) return false;
+  if (*abort_flag || wait_ring(bar, parity, abort_flag)) {
+    *abort_flag = 1;
+    return true;
+  }
+  return false;
+}
+
+// the same for a whole warp
+__device__ __forceinline__ bool wait_or_abort_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return __any_sync(0xFFFFFFFFu, wait_or_abort(bar, parity, abort_flag)) != 0;
+}
+
+// Epilogue of one N block (32 columns, accumulators at tb): a thread's row, NC of
+// its columns from column c0 of the block on; csc0: their scales; addr(a): where
+// amplitude a of those goes.  Hands the accumulators back on tempty once read.
+template <int K, int NC, typename Addr>
+__device__ __forceinline__ void epilogue_block(uint32_t tb, uint64_t* tempty, const int* csc0, int egs, bool row_ok,
+                                               int lane, const Addr& addr) {
+#pragma unroll
+  for (int cc = 0; cc < NC; cc += 4) {
+    float v[kLv][4];
+#pragma unroll
+    for (int L = 0; L < kLv; ++L) tmem_ld4(tb + (uint32_t)(L * 32 + cc), v[L]);
+    tmem_wait_ld();
+    if (cc + 4 == NC) {
+      fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty);
+    }
+    if (row_ok) {
+      const int4 s0 = *reinterpret_cast<const int4*>(csc0 + cc);
+      const int scl[4] = {s0.x, s0.y, s0.z, s0.w};
+      double o[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float u[kLv];
+#pragma unroll
+        for (int L = 0; L < kLv; ++L) u[L] = v[L][q];
+        o[q] = finish_output<K>(u, egs, scl[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; q += 2) *addr((cc + q) >> 1) = make_double2(o[q], o[q + 1]);
+    }
+  }
+}
+
+// the words of four amplitudes of a row (zeros beyond the last row)
+template <typename Addr>
+__device__ __forceinline__ void load_four(uint32_t (*R)[4], bool row_ok, const Addr& addr) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    double2 v = make_double2(0.0, 0.0);
+    if (row_ok) v = *addr(i);
+    R[i][0] = (uint32_t)__double2hiint(v.x);
+    R[i][1] = (uint32_t)__double2loint(v.x);
+    R[i][2] = (uint32_t)__double2hiint(v.y);
+    R[i][3] = (uint32_t)__double2loint(v.y);
+  }
+}
+
+// bits of the inserted (target, row and control) positions of a tile base
+__device__ __forceinline__ uint64_t hole_mask(const TcParams& p) {
+  uint64_t hole = 0;
+  for (int q = 0; q < p.nhi; ++q) hole |= 1ull << p.hi_ins[q];
+  return hole;
+}
+
+constexpr int kE5 = 8;                               // epilogue warps (two per lane quarter)
+struct W5 {
+  static constexpr int D = 32, K = 64, KB = 2, NM = 4;
+  static constexpr int THREADS = 32 * (kE5 + kKnWarps + 1);
+  static constexpr int ABYTES = kRows * 32 * 2, ABUF = qsby::kA * ABYTES;
+  static constexpr size_t b_off = 2 * (size_t)ABUF;
+  static constexpr size_t apre_off = b_off + (size_t)KB * KB * kKnBlock;
+  static constexpr size_t bpre_off = apre_off + kRows * 32;
+  static constexpr size_t toff_off = bpre_off + (size_t)KB * 8192;
+  static constexpr size_t rowoff_off = toff_off + 8 * D;
+  static constexpr size_t bar_off = rowoff_off + 8 * kRows;
+  static constexpr size_t csc_off = bar_off + 8 * 14;
+  static constexpr size_t max_off = csc_off + 4 * K;
+  static constexpr size_t ex_off = max_off + 4 * 3 * kRows;
+  static constexpr size_t colsum_off = ex_off + 4 * NM * kRows;
+  static constexpr size_t slot_off = colsum_off + 4 * (size_t)kLv * K;
+  static constexpr size_t bytes = slot_off + 16;
+  static_assert(bytes <= 227 * 1024, "shared memory");
+};
+}  // namespace
+
+__global__ void __launch_bounds__(W5::THREADS, 1)
+    k_dense_ozaki5(double2* __restrict__ psi, const __grid_constant__ TcParams p) {
+  using X = W5;
+  constexpr int D = X::D, K = X::K, KB = X::KB;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  unsigned char* a_dig = smem;
+  unsigned char* b_dig = smem + X::b_off;
+  unsigned char* a_pre = smem + X::apre_off;
+  unsigned char* b_pre = smem + X::bpre_off;
+  uint64_t* toff = reinterpret_cast<uint64_t*>(smem + X::toff_off);
+  uint64_t* rowoff = reinterpret_cast<uint64_t*>(smem + X::rowoff_off);
+  uint64_t* afull = reinterpret_cast<uint64_t*>(smem + X::bar_off);
+  uint64_t *aempty = afull + 2, *accfull = afull + 4, *tempty = afull + 6, *mready = afull + 8, *done = afull + 12;
+  int* csc = reinterpret_cast<int*>(smem + X::csc_off);
+  int* rowmax = reinterpret_cast<int*>(smem + X::max_off);       // 3 x kRows
+  int* meta_ex = reinterpret_cast<int*>(smem + X::ex_off);       // NM x kRows
+  int* colsum = reinterpret_cast<int*>(smem + X::colsum_off);    // K x 8 (setup)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + X::slot_off);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + X::slot_off + 4);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // B's slices in blocks of 32 x 32: block (K block, N block) at (kb KB + nb) 16 KB
+  for (int n = tid; n < K; n += X::THREADS) csc[n] = 0;
+  for (int i = tid; i < kLv * K; i += X::THREADS) colsum[i] = 0;
+  __syncthreads();
+  for (int idx = tid; idx < K * K; idx += X::THREADS)
+    atomicMax(csc + idx % K, __double2hiint(realified(p, D, idx / K, idx % K)) & 0x7FFFFFFF);
+  __syncthreads();
+  for (int idx = tid; idx < K * K; idx += X::THREADS) {
+    const int n = idx % K, k = idx / K;
+    const double v = realified(p, D, k, n);
+    int d[qsby::kB];
+    qsby::digits_b((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v), qsby::row_field((uint32_t)csc[n]), d);
+    unsigned char* blk = b_dig + ((k >> 5) * KB + (n >> 5)) * kKnBlock + canon_off16(n & 31, k & 31, 32);
+#pragma unroll
+    for (int t = 0; t < qsby::kB; ++t) {
+      *reinterpret_cast<uint16_t*>(blk + t * 2048) = half_bits(d[t]);
+      if (d[t] != 0) atomicAdd(colsum + n * kLv + t, d[t]);
+    }
+  }
+  __syncthreads();
+  for (int idx = tid; idx < kLv * K; idx += X::THREADS) {
+    const int L = idx / K, n = idx % K;
+    fill_start_column(b_pre + (n >> 5) * 8192, L * 32 + (n & 31), qsby::start_value(L, K, colsum + n * kLv));
+  }
+  for (int n = tid; n < K; n += X::THREADS) csc[n] = column_scale((int)qsby::row_field((uint32_t)csc[n]));
+  fill_start_rows(a_pre, tid, X::THREADS);
+  fill_offsets<5>(p, toff, rowoff, tid, X::THREADS);
+  for (int g = tid; g < 3 * kRows; g += X::THREADS) rowmax[g] = 0;
+  if (tid == 0) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(afull + b, kKnWarps);        // one arrival per producer warp
+      mbar_init(aempty + b, 1);
+      mbar_init(accfull + b, 1);
+      mbar_init(tempty + b, kE5);            // one arrival per epilogue warp
+    }
+#pragma unroll
+    for (int m = 0; m < X::NM; ++m) mbar_init(mready + m, 1);
+    mbar_init(done, 1);
+    *abort_flag = 0;
+  }
+  if (warp == 0) {
+    tmem_alloc(tmem_slot, 512);
+    tmem_relinquish();
+  }
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  fence_proxy_async();                        // B's slices and the initialising operands, for the MMAs
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+  const uint64_t grid = gridDim.x;
+  // tile bases: x(c) = insert_zeros(c); x(c + d) = ((x(c) | hole) + insert_zeros(d)) & ~hole
+  const uint64_t hole = hole_mask(p), gstep = insert_zeros(grid, p.hi_ins, p.nhi);
+  uint64_t xb = insert_zeros(blockIdx.x, p.hi_ins, p.nhi);
+
+  if (warp < kE5) {
+    // ---- epilogue: row g (tensor-memory lane), half h of each N block's columns ----
+    const int g = 32 * (warp & 3) + lane, h = warp >> 2;
+    const bool row_ok = g < (1 << (p.tile_bits - 5));
+    const uint32_t lane_addr = (uint32_t)(32 * (warp & 3)) << 16;
+    const uint64_t roff = rowoff[g] | p.ctrl_mask;
+    uint32_t it = 0;
+    bool bad = false;
+    for (uint64_t c = blockIdx.x; c < p.ntiles && !bad; c += grid, ++it, xb = ((xb | hole) + gstep) & ~hole) {
+      const uint32_t m = it % X::NM;
+      if (wait_or_abort_warp(mready + m, (it / X::NM) & 1u, abort_flag)) break;
+      const int egs = meta_ex[m * kRows + g];
+      const uint64_t rb = xb | roff;
+#pragma unroll
+      for (int nb = 0; nb < 2; ++nb) {
+        bad = wait_or_abort_warp(accfull + nb, it & 1u, abort_flag);
+        if (bad) break;
+        fence_after_sync();
+        epilogue_block<K, 16>(tmem + (uint32_t)(256 * nb + 16 * h) + lane_addr, tempty + nb, csc + 32 * nb + 16 * h, egs,
+                              row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 8 * h + a]); });
+      }
+    }
+  } else if (warp < kE5 + kKnWarps) {
+    // ---- producers: row g, amplitudes 16 kb + 4 cg + i (i < 4) of each K block ----
+    const int pw = warp - kE5, g = 32 * (pw & 3) + lane, cg = pw >> 2;
+    const bool row_ok = g < (1 << (p.tile_bits - 5));
+    const uint64_t roff = rowoff[g] | p.ctrl_mask;
+    const uint32_t a_addr = canon_off16(g, 8 * cg, 32);
+    uint32_t R[KB * 4][4];
+    uint64_t rb = xb | roff;
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb)
+      load_four(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
+    uint32_t it = 0;
+    bool bad = false;
+    for (uint64_t c = blockIdx.x; c < p.ntiles; c += grid, ++it) {
+      const uint32_t slot = it % 3;
+      uint32_t mx = 0;
+#pragma unroll
+      for (int i = 0; i < KB * 4; ++i) mx = max_abs(mx, R[i]);
+      atomicMax(rowmax + slot * kRows + g, (int)mx);   // the four threads of a row are in different warps
+      if (compute_barrier_or(bad || *abort_flag)) break;
+      const uint32_t ef = qsby::row_field((uint32_t)rowmax[slot * kRows + g]);   // exponent field of the row
+      if (cg == 0) {
+        // the previous tile's slot: read by every warp before this barrier, next
+        // written after the following one
+        rowmax[(slot == 0 ? 2 : slot - 1) * kRows + g] = 0;
+        meta_ex[(it % X::NM) * kRows + g] = (int)ef;
+      }
+      const bool has_next = c + grid < p.ntiles;
+      xb = ((xb | hole) + gstep) & ~hole;
+      rb = xb | roff;
+#pragma unroll
+      for (int kb = 0; kb < KB; ++kb) {
+        if (it > 0) bad |= wait_or_abort_warp(aempty + kb, (it - 1) & 1u, abort_flag);
+        store_slices(a_dig + kb * X::ABUF, a_addr, X::ABYTES, R + 4 * kb, ef + 0x100000u);
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(afull + kb);
+        if (has_next) load_four(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
+      }
+    }
+  } else if (lane == 0) {
+    // ---- MMA issue ----
+    uint32_t it = 0;
+    bool bad = false;
+    for (uint64_t c = blockIdx.x; c < p.ntiles && !bad; c += grid, ++it) {
+      for (int nb = 0; nb < 2 && !bad; ++nb) {
+        if (it > 0) bad = wait_or_abort(tempty + nb, (it - 1) & 1u, abort_flag);
+        if (bad) break;
+        fence_after_sync();
+        const uint32_t dcol = tmem + 256u * nb;
+        mma_start<32>(dcol, a_pre, b_pre + nb * 8192);
+        for (int kb = 0; kb < KB && !bad; ++kb) {
+          if (nb == 0) {
+            bad = wait_or_abort(afull + kb, it & 1u, abort_flag);
+            fence_after_sync();
+            if (kb == KB - 1) mbar_arrive(mready + it % X::NM);   // the producers' metadata, released onward
+          }
+          if (!bad) mma_products<32, 2>(dcol, a_dig + kb * X::ABUF, b_dig + (kb * KB + nb) * kKnBlock);
+          if (nb == 1) mma_commit(aempty + kb);
+        }
+        mma_commit(accfull + nb);
+      }
+    }
+    // every MMA is complete before the tensor memory is freed
+    mma_commit(done);
+    if (wait_phase(done, 0)) *abort_flag = 1;
+  }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  if (tid == 0 && *abort_flag) atomicExch(p.err, 1);
+  if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+static cudaError_t dense_ozaki5(void* amps, const TcParams& p, cudaStream_t st) {
+  static bool attr_done = false;
+  if (!attr_done) {
+    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki5, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W5::bytes);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
   const uint64_t maxb = (uint64_t)num_sms();
   const unsigned g = (unsigned)(p.ntiles < maxb ? p.ntiles : maxb);
-  k_dense_ozaki_ws<NT, KS><<<g, kWsThreads, smem, st>>>(static_cast<double2*>(amps), p);
+  k_dense_ozaki5<<<g, W5::THREADS, W5::bytes, st>>>(static_cast<double2*>(amps), p);
   return cudaGetLastError();
 }
 
-// Several independent single-buffered CTAs per SM, whose phases drift apart,
-// keep the SM busier than double buffering inside one CTA (measured at 30
-// qubits: 3 targets 10.3 ms as four 128-thread CTAs against 12.2 ms as two
-// double-buffered 256-thread CTAs; 4 targets 11.2 ms as two 256-thread CTAs
-// against 13.9 ms as one double-buffered 512-thread CTA).  Tensor memory
-// (seven levels of N columns per buffer) bounds the CTAs per SM.
+// ---------------------------------------------------------------------------
+// Six targets (K = N = 128), in four blocks of 32 columns of K and of N.  16
+// compute warps hold a tile's amplitudes in registers (thread: row g, four
+// amplitudes of each K block), slice one K block at a time into a ring of two
+// operand buffers, and recombine one N block at a time out of two accumulator
+// buffers.  Reading all inputs into registers first makes the update in place
+// safe.  One thread issues the MMAs: for a pair of N blocks, every K block
+// against both.  The second pair takes the K blocks in the order 3, 2, 1, 0, so
+// that two of its four are still in the operand buffers.  B's slices (256 KB)
+// do not fit in shared memory: a setup kernel (k_wide_matrix) writes them to the
+// handle's scratch, and another warp streams the 16 KB block of each (K, N) pair
+// from L2 into a ring of four slots with bulk copies.  Hand-offs as for five
+// targets, with bfull (bulk copy) and bempty (MMA completion) for B's slots.
+// Bound by the tensor cores (53% busy, two fifths of each tile's time being the
+// epilogues and slicing that share its 16 warps): 34.7 thousand cycles per tile.
+// ---------------------------------------------------------------------------
+namespace {
+// layout of the scratch that k_wide_matrix fills
+constexpr int kWideStart = 16 * kKnBlock;            // four start operands (N block) of 256 columns x 32 bytes
+constexpr int kWideScale = kWideStart + 4 * 8192;    // 128 column exponent increments
+static_assert(kWideScale + 4 * 128 <= (int)kWideScratch, "scratch of the six-target kernel");
+
+struct W6 {
+  static constexpr int D = 64, K = 128, KB = 4;
+  static constexpr int THREADS = kKnC + 64;
+  static constexpr int ABYTES = kRows * 32 * 2, ABUF = qsby::kA * ABYTES;
+  static constexpr size_t b_off = 2 * (size_t)ABUF;
+  static constexpr size_t apre_off = b_off + 4 * (size_t)kKnBlock;
+  static constexpr size_t bpre_off = apre_off + kRows * 32;
+  static constexpr size_t toff_off = bpre_off + (size_t)KB * 8192;
+  static constexpr size_t rowoff_off = toff_off + 8 * D;
+  static constexpr size_t bar_off = rowoff_off + 8 * kRows;
+  static constexpr size_t csc_off = bar_off + 8 * 18;
+  static constexpr size_t max_off = csc_off + 4 * K;
+  static constexpr size_t slot_off = max_off + 4 * 3 * kRows;
+  static constexpr size_t bytes = slot_off + 16;
+  static_assert(bytes <= 227 * 1024, "shared memory");
+};
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
+// K block of step j of pass np over K: the second pass goes back
+__device__ __forceinline__ int k_block(int np, int j) { return np ? W6::KB - 1 - j : j; }
+}  // namespace
+
+// One block per column of the realified six-target matrix, one thread per row:
+// digits into the 32 x 32 blocks of the scratch, start operands, column scale.
+__global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcParams p, unsigned char* __restrict__ out) {
+  constexpr int D = 64, K = 128;
+  __shared__ int mx, sums[kLv];
+  const int n = blockIdx.x, k = threadIdx.x;
+  if (k < kLv) sums[k] = 0;
+  if (k == 0) mx = 0;
+  __syncthreads();
+  const double v = realified(p, D, k, n);
+  atomicMax(&mx, __double2hiint(v) & 0x7FFFFFFF);
+  __syncthreads();
+  const uint32_t ef = qsby::row_field((uint32_t)mx);
+  int d[qsby::kB];
+  qsby::digits_b((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v), ef, d);
+  unsigned char* blk = out + ((k >> 5) * 4 + (n >> 5)) * kKnBlock + canon_off16(n & 31, k & 31, 32);
+#pragma unroll
+  for (int t = 0; t < qsby::kB; ++t) {
+    *reinterpret_cast<uint16_t*>(blk + t * 2048) = half_bits(d[t]);
+    atomicAdd(sums + t, d[t]);
+  }
+  __syncthreads();
+  if (k < kLv)
+    fill_start_column(out + kWideStart + (n >> 5) * 8192, k * 32 + (n & 31), qsby::start_value(k, K, sums));
+  if (k == 0) reinterpret_cast<int*>(out + kWideScale)[n] = column_scale((int)ef);
+}
+
+__global__ void __launch_bounds__(W6::THREADS, 1)
+    k_dense_ozaki6(double2* __restrict__ psi, const __grid_constant__ TcParams p, const unsigned char* __restrict__ wide) {
+  using X = W6;
+  constexpr int K = X::K, KB = X::KB, PAIRS = 2;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  unsigned char* a_dig = smem;
+  unsigned char* b_dig = smem + X::b_off;
+  unsigned char* a_pre = smem + X::apre_off;
+  unsigned char* b_pre = smem + X::bpre_off;
+  uint64_t* toff = reinterpret_cast<uint64_t*>(smem + X::toff_off);
+  uint64_t* rowoff = reinterpret_cast<uint64_t*>(smem + X::rowoff_off);
+  uint64_t* afull = reinterpret_cast<uint64_t*>(smem + X::bar_off);
+  uint64_t *aempty = afull + 2, *accfull = afull + 4, *tempty = afull + 6, *bfull = afull + 8, *bempty = afull + 12,
+           *done = afull + 16;
+  int* csc = reinterpret_cast<int*>(smem + X::csc_off);
+  int* rowmax = reinterpret_cast<int*>(smem + X::max_off);       // 3 x kRows
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + X::slot_off);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + X::slot_off + 4);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint4* src = reinterpret_cast<const uint4*>(wide + kWideStart);
+  for (int i = tid; i < KB * 8192 / 16; i += X::THREADS) reinterpret_cast<uint4*>(b_pre)[i] = src[i];
+  for (int n = tid; n < K; n += X::THREADS) csc[n] = reinterpret_cast<const int*>(wide + kWideScale)[n];
+  fill_start_rows(a_pre, tid, X::THREADS);
+  fill_offsets<6>(p, toff, rowoff, tid, X::THREADS);
+  for (int g = tid; g < 3 * kRows; g += X::THREADS) rowmax[g] = 0;
+  if (tid == 0) {
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(afull + b, kKnWarps);        // one arrival per compute warp
+      mbar_init(aempty + b, 1);
+      mbar_init(accfull + b, 1);
+      mbar_init(tempty + b, kKnWarps);
+    }
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      mbar_init(bfull + b, 1);
+      mbar_init(bempty + b, 1);
+    }
+    mbar_init(done, 1);
+    *abort_flag = 0;
+  }
+  if (warp == 0) {
+    tmem_alloc(tmem_slot, 512);
+    tmem_relinquish();
+  }
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  fence_proxy_async();                        // the initialising operands, for the MMAs
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+  const uint64_t grid = gridDim.x;
+  // tile bases: x(c) = insert_zeros(c); x(c + d) = ((x(c) | hole) + insert_zeros(d)) & ~hole
+  const uint64_t hole = hole_mask(p), gstep = insert_zeros(grid, p.hi_ins, p.nhi);
+
+  if (warp < kKnWarps) {
+    const int g = 32 * (warp & 3) + lane, cg = warp >> 2;         // row (tensor-memory lane), column group
+    const bool row_ok = g < (1 << (p.tile_bits - 6));
+    const uint64_t roff = rowoff[g] | p.ctrl_mask;
+    const uint32_t lane_addr = (uint32_t)(32 * (warp & 3)) << 16;
+    const uint32_t a_addr = canon_off16(g, 8 * cg, 32);
+    uint32_t R[KB * 4][4];                    // amplitudes 16 kb + 4 cg + i of the row, i < 4
+    uint32_t fills[2] = {0, 0}, reads[2] = {0, 0};   // uses of the operand and accumulator buffers so far
+    bool bad = false;
+    uint64_t xb = insert_zeros(blockIdx.x, p.hi_ins, p.nhi);
+    uint64_t rb = xb | roff;
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb)
+      load_four(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
+    uint32_t it = 0;
+    for (uint64_t c = blockIdx.x; c < p.ntiles; c += grid, ++it) {
+      const uint32_t slot = it % 3;
+      uint32_t mx = 0;
+#pragma unroll
+      for (int i = 0; i < KB * 4; ++i) mx = max_abs(mx, R[i]);
+      atomicMax(rowmax + slot * kRows + g, (int)mx);   // the four threads of a row are in different warps
+      if (compute_barrier_or(bad || *abort_flag)) break;
+      const uint32_t ef = qsby::row_field((uint32_t)rowmax[slot * kRows + g]);   // exponent field of the row
+      // the previous tile's slot: read by every warp before this barrier, next
+      // written after the following one
+      if (cg == 0) rowmax[(slot == 0 ? 2 : slot - 1) * kRows + g] = 0;
+      const bool has_next = c + grid < p.ntiles;
+      xb = ((xb | hole) + gstep) & ~hole;
+      const uint64_t rb_next = xb | roff;
+#pragma unroll
+      for (int np = 0; np < PAIRS; ++np) {
+#pragma unroll
+        for (int j = 0; j < KB; ++j) {
+          if (np > 0 && j < 2) continue;      // still in the operand buffers
+          const int kb = k_block(np, j), b = kb & 1;
+          if (fills[b] > 0) bad |= wait_or_abort_warp(aempty + b, (fills[b] - 1) & 1u, abort_flag);
+          ++fills[b];
+          store_slices(a_dig + b * X::ABUF, a_addr, X::ABYTES, R + 4 * kb, ef + 0x100000u);
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(afull + b);
+          // the last use of these registers in this tile
+          if (has_next && (np > 0 || kb >= 2))
+            load_four(R + 4 * kb, row_ok, [&](int i) { return psi + (rb_next | toff[16 * kb + 4 * cg + i]); });
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int nb = 2 * np + h;
+          bad |= wait_or_abort_warp(accfull + h, reads[h] & 1u, abort_flag);
+          ++reads[h];
+          fence_after_sync();
+          epilogue_block<K, 8>(tmem + (uint32_t)(256 * h + 8 * cg) + lane_addr, tempty + h, csc + 32 * nb + 8 * cg, (int)ef,
+                               row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 4 * cg + a]); });
+        }
+      }
+      rb = rb_next;
+    }
+  } else if (warp == kKnWarps && lane == 0) {
+    // ---- MMA issue ----
+    uint32_t fills[2] = {0, 0}, writes[2] = {0, 0}, nblk = 0;
+    bool bad = false;
+    for (uint64_t c = blockIdx.x; c < p.ntiles && !bad; c += grid)
+      for (int np = 0; np < PAIRS && !bad; ++np)
+        for (int j = 0; j < KB && !bad; ++j) {
+          const int kb = k_block(np, j), b = kb & 1;
+          if (np == 0 || j >= 2) {
+            bad = wait_or_abort(afull + b, fills[b] & 1u, abort_flag);
+            ++fills[b];
+          }
+          for (int h = 0; h < 2 && !bad; ++h) {
+            const uint32_t dcol = tmem + 256u * h;
+            if (j == 0) {
+              if (writes[h] > 0) bad = wait_or_abort(tempty + h, (writes[h] - 1) & 1u, abort_flag);
+              ++writes[h];
+            }
+            const uint32_t slot = nblk & 3u;
+            if (!bad) bad = wait_or_abort(bfull + slot, (nblk >> 2) & 1u, abort_flag);
+            if (bad) break;
+            ++nblk;
+            fence_after_sync();
+            if (j == 0) mma_start<32>(dcol, a_pre, b_pre + (2 * np + h) * 8192);
+            mma_products<32, 2>(dcol, a_dig + b * X::ABUF, b_dig + slot * kKnBlock);
+            mma_commit(bempty + slot);
+            if (j == KB - 1) mma_commit(accfull + h);
+          }
+          // the buffer is free unless the next pass starts with it
+          if (np > 0 || j < 2) mma_commit(aempty + b);
+        }
+    // every MMA is complete before the tensor memory is freed
+    mma_commit(done);
+    if (wait_phase(done, 0)) *abort_flag = 1;
+  } else if (warp == kKnWarps + 1 && lane == 0) {
+    // ---- B blocks, in the order of the MMA thread ----
+    uint32_t nblk = 0;
+    bool bad = false;
+    for (uint64_t c = blockIdx.x; c < p.ntiles && !bad; c += grid)
+      for (int np = 0; np < PAIRS && !bad; ++np)
+        for (int j = 0; j < KB && !bad; ++j)
+          for (int h = 0; h < 2; ++h, ++nblk) {
+            const uint32_t slot = nblk & 3u;
+            if (nblk >= 4) bad = wait_or_abort(bempty + slot, ((nblk >> 2) - 1) & 1u, abort_flag);
+            if (bad) break;
+            bulk_load(smem_u32(b_dig) + slot * kKnBlock, wide + (k_block(np, j) * KB + 2 * np + h) * kKnBlock, kKnBlock,
+                      bfull + slot);
+          }
+    // every copy has arrived before the CTA ends (the last fill of each slot)
+    for (uint32_t s = 0; s < 4; ++s) {
+      const uint32_t f = nblk > s ? (nblk - s + 3) / 4 : 0;       // fills of slot s
+      if (f > 0 && wait_phase(bfull + s, (f - 1) & 1u)) *abort_flag = 1;
+    }
+  }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  if (tid == 0 && *abort_flag) atomicExch(p.err, 1);
+  if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+static cudaError_t dense_ozaki6(void* amps, const TcParams& p, void* scratch, cudaStream_t st) {
+  static bool attr_done = false;
+  if (!attr_done) {
+    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki6, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W6::bytes);
+    if (e != cudaSuccess) return e;
+    attr_done = true;
+  }
+  unsigned char* wide = static_cast<unsigned char*>(scratch);
+  k_wide_matrix<<<W6::K, W6::K, 0, st>>>(p, wide);
+  const uint64_t maxb = (uint64_t)num_sms();
+  const unsigned g = (unsigned)(p.ntiles < maxb ? p.ntiles : maxb);
+  k_dense_ozaki6<<<g, W6::THREADS, W6::bytes, st>>>(static_cast<double2*>(amps), p, wide);
+  return cudaGetLastError();
+}
+
 // Passes of fewer tiles than SMs (small states) go to the single-CTA kernels,
 // whose setup is lighter than the warp-specialised kernel's (one tile per CTA
 // leaves nothing to pipeline).
-cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, int slices, cudaStream_t st) {
+cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st) {
   const bool small = p.ntiles < (uint64_t)num_sms();
-  if (slices == 8) {
-    switch (p.n) {
-      case 3: return small ? dense_ozaki_nt<3, 128, 1, 4, 8>(amps, p, st) : dense_ozaki_ws<3, 8>(amps, p, st);
-      case 4: return small ? dense_ozaki_nt<4, 256, 1, 2, 8>(amps, p, st) : dense_ozaki_ws<4, 8>(amps, p, st);
-      case 5: return dense_ozaki_nt<5, 512, 1, 1, 8>(amps, p, st);
-      default: return cudaErrorInvalidValue;
-    }
-  }
   switch (p.n) {
-    case 3: return small ? dense_ozaki_nt<3, 128, 1, 4, 7>(amps, p, st) : dense_ozaki_ws<3, 7>(amps, p, st);
-    case 4: return small ? dense_ozaki_nt<4, 256, 1, 2, 7>(amps, p, st) : dense_ozaki_ws<4, 7>(amps, p, st);
-    case 5: return dense_ozaki_nt<5, 512, 1, 1, 7>(amps, p, st);
+    case 3: return small ? dense_ozaki_small<3, 128, 4>(amps, p, st) : dense_ozaki_ws<3>(amps, p, st);
+    case 4: return small ? dense_ozaki_small<4, 256, 2>(amps, p, st) : dense_ozaki_ws<4>(amps, p, st);
+    case 5: return dense_ozaki5(amps, p, st);
+    case 6: return dense_ozaki6(amps, p, scratch, st);
     default: return cudaErrorInvalidValue;
   }
 }

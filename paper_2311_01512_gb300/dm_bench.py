@@ -170,7 +170,7 @@ def large(qs, wl, torch, peak_gbs, reps=1):
         ex_ms = e0.elapsed_time(e1)
     out = {"workload": "15-qubit density matrix (30-qubit Choi vector, 16 GiB), 400 ops",
            "arithmetic": "complex128, the default block fixed point (two-target passes on the CUDA cores, "
-                         "3-5-target passes as eight slices on the tensor cores)",
+                         "3-6-target passes as byte slices on the tensor cores)",
            "runs": reps, "ms_total": total_ms, "ms_runs": totals, "gb_total": total_bytes / 1e9,
            "gbs": total_bytes / total_ms / 1e6,
            "frac_of_peak": (total_bytes / total_ms / 1e6) / peak_gbs if peak_gbs else None,

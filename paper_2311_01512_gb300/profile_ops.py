@@ -2,7 +2,7 @@
 size, in the default complex128 arithmetic (block fixed point): one-target
 gate, 3-qubit diagonal, weight-6 Pauli gadget, a Z-only (phase) gadget, dense
 gates on 2 targets (CUDA cores, block fixed point) and on 3, 4 and 5 targets
-(bf16 tensor cores, eight integer slices), and a 5-target dense gate on a
+(fp16 tensor cores, byte slices), and a 5-target dense gate on a
 complex64 state (tf32 tensor cores), each repeated.
 
     python -m paper_2311_01512_gb300.profile_ops --qubits 28 --reps 3
@@ -51,7 +51,8 @@ import numpy as np
 # launch order of one repetition -> the bench's kernel family names
 _FAMILIES = {"k_gate1_fx": ["k_gate1"], "k_diag_fx": ["k_diag"], "k_gadget_fx": ["k_gadget"],
              "k_phase_fx": ["k_phase"], "k_gate2_fx": ["k_dense<2>"], "k_dense_ozaki_ws<3": ["k_dense<3>"],
-             "k_dense_ozaki_ws<4": ["k_dense<4>"], "k_dense_ozaki<5": ["k_dense<5>"], "k_dense_tc<5": ["c64 k_dense<5>"]}
+             "k_dense_ozaki_ws<4": ["k_dense<4>"], "k_dense_ozaki<5": ["k_dense<5>"],
+             "k_dense_ozaki5": ["k_dense<5>"], "k_dense_tc<5": ["c64 k_dense<5>"]}
 
 
 def summarize_traffic(paths, qubits, scale_to, out):
