@@ -73,14 +73,13 @@ qs_status create(int nq, int ns, int is_density, qs_prec prec, void* d_amps, voi
   s->stream = static_cast<cudaStream_t>(stream);
   const size_t scratch = sizeof(double2) * (qsk::kPartials + 2);
   if (qsalloc::device(reinterpret_cast<void**>(&s->d_partials), scratch) != cudaSuccess ||
-      qsalloc::device(reinterpret_cast<void**>(&s->d_ring), kRingSlots * kSlotBytes + qsk::kWideScratch) != cudaSuccess ||
+      qsalloc::device(reinterpret_cast<void**>(&s->d_ring), kRingSlots * kSlotBytes) != cudaSuccess ||
       qsalloc::pinned(reinterpret_cast<void**>(&s->h_result), sizeof(double2) * 2) != cudaSuccess ||
       qsalloc::pinned(reinterpret_cast<void**>(&s->h_ring), kRingSlots * kSlotBytes) != cudaSuccess) {
     cudaGetLastError();
     release(s);
     return QS_ERR_OOM;
   }
-  s->d_wide = s->d_ring + kRingSlots * kSlotBytes;
   s->d_result = s->d_partials + qsk::kPartials;
   s->d_err = reinterpret_cast<int*>(s->d_partials + qsk::kPartials + 1);
   if (cudaMemset(s->d_err, 0, sizeof(int)) != cudaSuccess) {
@@ -109,6 +108,7 @@ struct qs_program {
   std::vector<void*> chunks;      // device arena, never moved (the graph holds its addresses)
   size_t used = 0, cap = 0;       // in the last chunk
   cudaStream_t side = nullptr;    // uploads during recording (outside the capture)
+  std::vector<std::vector<unsigned char>> staged;  // their host copies, until the recording ends
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
 };
@@ -137,8 +137,12 @@ qs_status rec_put(qs_program* p, const void* host, size_t bytes, const void** de
   *slot = -1;
   void* d = rec_alloc(p, bytes);
   if (!d) return QS_ERR_OOM;
-  if (cudaMemcpyAsync(d, host, bytes, cudaMemcpyHostToDevice, p->side) != cudaSuccess ||
-      cudaStreamSynchronize(p->side) != cudaSuccess)
+  try {
+    p->staged.emplace_back(static_cast<const unsigned char*>(host), static_cast<const unsigned char*>(host) + bytes);
+  } catch (const std::bad_alloc&) {
+    return QS_ERR_OOM;
+  }
+  if (cudaMemcpyAsync(d, p->staged.back().data(), bytes, cudaMemcpyHostToDevice, p->side) != cudaSuccess)
     return QS_ERR_CUDA;
   *dev = d;
   return QS_OK;
@@ -146,6 +150,7 @@ qs_status rec_put(qs_program* p, const void* host, size_t bytes, const void** de
 
 void program_free(qs_program* p) {
   if (!p) return;
+  if (p->side) cudaStreamSynchronize(p->side);
   if (p->exec) cudaGraphExecDestroy(p->exec);
   if (p->graph) cudaGraphDestroy(p->graph);
   for (void* c : p->chunks) cudaFree(c);
@@ -188,6 +193,26 @@ qs_status ring_take(qs_state* s, size_t bytes, void** dev, int* slot) {
   return QS_OK;
 }
 
+// The same over as many consecutive slots as `bytes` needs, [*first, *first + *count).
+qs_status ring_take_run(qs_state* s, size_t bytes, void** dev, int* first, int* count) {
+  if (s->rec) {
+    *first = -1;
+    *count = 0;
+    *dev = rec_alloc(s->rec, bytes);
+    return *dev ? QS_OK : QS_ERR_OOM;
+  }
+  const int n = (int)((bytes + kSlotBytes - 1) / kSlotBytes);
+  if (n > kRingSlots) return QS_ERR_ARG;
+  const int k = s->ring_next + n <= kRingSlots ? s->ring_next : 0;
+  s->ring_next = (k + n) % kRingSlots;
+  for (int j = k; j < k + n; ++j)
+    if (cudaEventSynchronize(s->ring_ev[j]) != cudaSuccess) return QS_ERR_CUDA;
+  *dev = s->d_ring + (size_t)k * kSlotBytes;
+  *first = k;
+  *count = n;
+  return QS_OK;
+}
+
 qs_status ring_done(qs_state* s, int slot) {
   if (slot < 0) return QS_OK;      // arena data of a recorded program: nothing to release
   return cuda_status(cudaEventRecord(s->ring_ev[slot], s->stream));
@@ -227,6 +252,18 @@ qsk::FxPart fx_part(double v, int em) {
   return qsk::FxPart{q.h, q.l};
 }
 bool is_fx(const qs_state* s) { return s->prec == QS_C128 && s->arith == QS_ARITH_FX; }
+
+// Passes over at most 2^kSmallDenseBits[n] amplitudes (n targets) take
+// launch_dense_fx instead of the tensor-core kernels.  Measured, us a pass in
+// a replayed program, one thread per amplitude / tensor cores:
+//   2 targets (fused blocks) 2^20 13.2 / 18.3; 3 targets 2^19 11.5 / 12.8, 2^20
+//   22.8 / 15.9; 4 targets 2^17 7.0 / 11.7, 2^18 12.4 / 11.2; 5 targets 2^17
+//   16.9 / 19.8, 2^18 30.8 / 19.8.
+constexpr int kSmallDenseBits[6] = {0, 0, 20, 19, 17, 17};
+// The same for launch_dense_digits (density matrices).  Measured as above: 3
+// targets 2^16 7.5 us (tensor cores 11), 4 targets 2^14 6.1 (10.3) and 2^16 15.3
+// (10.5), 5 targets 2^14 13.3 (19.8) and 2^16 50.
+constexpr int kSmallDigitBits[6] = {0, 0, 16, 16, 14, 14};
 
 // One dense or one-target gate pass on storage positions (already shifted).
 qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vector<int>& targs, const double* host_mat,
@@ -335,6 +372,30 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
   // complex128 off the FP64 pipe: exact byte slices (55-bit amplitudes)
   const bool tc128 = s->prec == QS_C128 && (s->arith == QS_ARITH_DF || s->arith == QS_ARITH_FX) &&
                      s->tensor_cores && (tc_n || n == 6);
+  // complex128 passes over few amplitudes, 2..5 targets: off the tensor cores
+  // (density matrices in block fixed point keep the arithmetic that these
+  // passes had there)
+  const bool digits = s->is_density && s->arith == QS_ARITH_FX;
+  if (tc128 && n <= 5 && nfree + n <= (digits ? kSmallDigitBits : kSmallDenseBits)[n]) {
+    qsk::DenseFxParams p{};
+    p.mat = static_cast<const double*>(dev_mat);
+    p.conj = conj;
+    p.ctrl_mask = cmask;
+    std::vector<int> kt(targs), ins(ctrls);
+    if (digits && n == 2) kt.push_back(__builtin_ctzll(~fixed));
+    p.n = (int)kt.size();
+    p.nmat = n;
+    for (int q = 0; q < p.n; ++q) {
+      p.tpos[q] = (int8_t)kt[q];
+      ins.push_back(kt[q]);
+    }
+    std::sort(ins.begin(), ins.end());
+    p.nins = (int)ins.size();
+    for (int q = 0; q < p.nins; ++q) p.ins[q] = (int8_t)ins[q];
+    p.ngroups = 1ull << (s->ns - p.nins);
+    return cuda_status(digits ? qsk::launch_dense_digits(s->amps, p, s->stream)
+                              : qsk::launch_dense_fx(s->amps, p, s->stream));
+  }
   if (tc64 || tc128) {
     std::vector<int> kt(targs);
     if (n == 2) {
@@ -373,8 +434,19 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
     p.nhi = (int)hi.size();
     for (int i = 0; i < p.nhi; ++i) p.hi_ins[i] = (int8_t)hi[i];
     p.ntiles = 1ull << (s->ns - p.nhi);
-    return cuda_status(tc64 ? qsk::launch_dense_tc(s->amps, p, s->stream)
-                            : qsk::launch_dense_ozaki(s->amps, p, s->d_wide, s->stream));
+    if (tc64) return cuda_status(qsk::launch_dense_tc(s->amps, p, s->stream));
+    if (n < 6) return cuda_status(qsk::launch_dense_ozaki(s->amps, p, nullptr, s->stream));
+    // six targets: the sliced matrix goes through scratch in the ring
+    void* wide = nullptr;
+    int first = -1, count = 0;
+    qs_status st = ring_take_run(s, qsk::kWideScratch, &wide, &first, &count);
+    if (st != QS_OK) return st;
+    st = cuda_status(qsk::launch_dense_ozaki(s->amps, p, wide, s->stream));
+    for (int j = 0; j < count; ++j) {
+      const qs_status st2 = ring_done(s, first + j);
+      if (st == QS_OK) st = st2;
+    }
+    return st;
   }
   // Dense tile: P = targets u the lowest free qubits, |P| = min(kTileBits, free + n).
   const int g = std::min(qsk::kTileBits - n, nfree) < 0 ? 0 : std::min(qsk::kTileBits - n, nfree);
@@ -452,6 +524,33 @@ qs_status gadget_pass(qs_state* s, const std::vector<int>& targs, const int* pau
     return cuda_status(qsk::launch_gadget_df(s->amps, q, s->stream));
   }
   return cuda_status(qsk::launch_gadget(s->prec, s->amps, p, s->stream));
+}
+
+// S = sum_m conj(K_m) (x) K_m of n-qubit operators in device memory (FP64, on the
+// device), applied as one 2n-target pass on t u (t + N): matrix bit q on t[q], bit
+// n + q on t[q] + N (Sec. "Kraus map").  While recording, S is formed once on the
+// program's side stream, outside the capture: its operators are constants of the
+// program, and a replay then takes one launch instead of two.
+qs_status superop_pass(qs_state* s, const std::vector<int>& t, const double* kraus, int num_ops) {
+  const int n = (int)t.size();
+  const size_t kbytes = sizeof(double) * 2 * (size_t(1) << (2 * n)) * (size_t)num_ops;
+  const void* dk = nullptr;
+  void* dsup = nullptr;
+  int slot_k = -1, slot_s = -1;
+  qs_status st = ring_put(s, kraus, kbytes, &dk, &slot_k);
+  if (st != QS_OK) return st;
+  st = ring_take(s, sizeof(double) * 2 * ((size_t)1 << (4 * n)), &dsup, &slot_s);
+  if (st == QS_OK)
+    st = cuda_status(qsk::launch_superop(static_cast<const double*>(dk), num_ops, n, static_cast<double*>(dsup),
+                                         s->rec ? s->rec->side : s->stream));
+  if (st == QS_OK) {
+    std::vector<int> tt(t);
+    for (int q = 0; q < n; ++q) tt.push_back(t[q] + s->nq);
+    st = gate_pass(s, {}, tt, nullptr, dsup, 0);
+  }
+  const qs_status a = ring_done(s, slot_k);
+  const qs_status b = slot_s >= 0 ? ring_done(s, slot_s) : QS_OK;
+  return st != QS_OK ? st : (a != QS_OK ? a : b);
 }
 
 qs_status reduce_to_host(qs_state* s, double* out) {
@@ -632,34 +731,18 @@ qs_status qs_apply_ctrl_multi_target(qs_state* s, const int* ctrls, int nctrl, c
     qsh::superop1(mat, 1, sup);
     return gate_pass(s, {}, {t[0], t[0] + s->nq}, sup, nullptr, 0);
   }
+  // Density matrix, uncontrolled two-target unitary on the tensor-core path:
+  // U on t and U^* on t + N in one 4-target pass of conj(U) (x) U, the
+  // superoperator of the one-operator Kraus map {U} (Sec. "Kraus map"), which
+  // reads and writes the Choi vector once instead of twice.
+  const bool tc = s->tensor_cores && (s->prec == QS_C64 || s->arith == QS_ARITH_DF || s->arith == QS_ARITH_FX);
+  if (s->is_density && nctrl == 0 && ntarg == 2 && tc) return superop_pass(s, t, mat, 1);
   const size_t mat_bytes = sizeof(double) * 2 * (size_t(1) << (2 * ntarg));
   const void* dmat = nullptr;
   int slot = -1;
   if (ntarg > 1) {
     st = ring_put(s, mat, mat_bytes, &dmat, &slot);
     if (st != QS_OK) return st;
-  }
-  // Density matrix, uncontrolled two-target unitary on the tensor-core path:
-  // U on t and U^* on t + N in one 4-target pass of conj(U) (x) U, the
-  // superoperator of the one-operator Kraus map {U} (Sec. "Kraus map"), which
-  // reads and writes the Choi vector once instead of twice.
-  const bool tc = s->tensor_cores && (s->prec == QS_C64 || s->arith == QS_ARITH_DF || s->arith == QS_ARITH_FX);
-  if (s->is_density && nctrl == 0 && ntarg == 2 && tc) {
-    void* dsup = nullptr;
-    int slot_s = -1;
-    st = ring_take(s, sizeof(double) * 2 * 256, &dsup, &slot_s);
-    if (st == QS_OK)
-      st = cuda_status(qsk::launch_superop(static_cast<const double*>(dmat), 1, 2, static_cast<double*>(dsup),
-                                           s->stream));
-    if (st == QS_OK) {
-      std::vector<int> t4(t);
-      for (int q = 0; q < 2; ++q) t4.push_back(t[q] + s->nq);
-      st = gate_pass(s, {}, t4, nullptr, dsup, 0);
-    }
-    const qs_status a = slot_s >= 0 ? ring_done(s, slot_s) : QS_OK;
-    const qs_status b = ring_done(s, slot);
-    if (st == QS_OK) st = a != QS_OK ? a : b;
-    return st;
   }
   st = gate_pass(s, c, t, mat, dmat, 0);
   if (st == QS_OK && s->is_density) {
@@ -786,25 +869,7 @@ qs_status qs_apply_kraus(qs_state* s, const int* targs, int n, const double* kra
     qsh::superop1(kraus, num_ops, sup);
     return gate_pass(s, {}, {targs[0], targs[0] + s->nq}, sup, nullptr, 0);
   }
-  const void* dk = nullptr;
-  void* dsup = nullptr;
-  int slot_k = -1, slot_s = -1;
-  st = ring_put(s, kraus, kbytes, &dk, &slot_k);
-  if (st != QS_OK) return st;
-  st = ring_take(s, sizeof(double) * 2 * ((size_t)1 << (4 * n)), &dsup, &slot_s);
-  if (st == QS_OK)
-    st = cuda_status(qsk::launch_superop(static_cast<const double*>(dk), num_ops, n, static_cast<double*>(dsup),
-                                         s->stream));
-  if (st == QS_OK) {
-    // S on t u (t + N): matrix bit q on t[q], bit n + q on t[q] + N (Sec. "Kraus map")
-    std::vector<int> t(targs, targs + n);
-    for (int q = 0; q < n; ++q) t.push_back(targs[q] + s->nq);
-    st = gate_pass(s, {}, t, nullptr, dsup, 0);
-  }
-  const qs_status a = ring_done(s, slot_k);
-  const qs_status b = slot_s >= 0 ? ring_done(s, slot_s) : QS_OK;
-  if (st == QS_OK) st = a != QS_OK ? a : b;
-  return st;
+  return superop_pass(s, std::vector<int>(targs, targs + n), kraus, num_ops);
 }
 
 namespace {
@@ -1061,6 +1126,14 @@ qs_status qs_record_end(qs_state* s, qs_program** out) {
     return QS_ERR_CUDA;
   }
   p->graph = g;
+  // uploads and superoperators on the side stream are complete before any replay
+  if (cudaStreamSynchronize(p->side) != cudaSuccess) {
+    cudaGetLastError();
+    program_free(p);
+    return QS_ERR_CUDA;
+  }
+  p->staged.clear();
+  p->staged.shrink_to_fit();
   if (cudaGraphInstantiate(&p->exec, g, 0) != cudaSuccess) {
     cudaGetLastError();
     program_free(p);

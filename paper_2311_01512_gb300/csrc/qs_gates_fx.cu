@@ -150,6 +150,86 @@ __global__ void __launch_bounds__(256) k_gate2_fx(double2* __restrict__ psi, con
 }
 
 // ---------------------------------------------------------------------------
+// Dense gate on NT = 2..5 targets of a small state (Sec. "Many-target gate"),
+// one thread per amplitude.  The 2^NT threads of a group (lanes of one warp)
+// convert their own amplitude with the group's largest exponent and exchange the
+// parts through shared memory; thread j sums row j of the matrix, whose parts
+// every block prepares in shared memory with one exponent per row, laid out by
+// column so that the lanes of a group read consecutive words.  The 2^(NT+1) real
+// terms of an output go four at a time through the accumulators of qs_fx.cuh;
+// the partial sums are added shifted down by NT - 2 bits (|V| stays below 2^63
+// as in the two-target kernel), so the error is at most
+//   2^-53 |y| + (7 2^(NT+1) + 2^(2 NT - 2) + 8) 2^-60 max|x_k| max|m_k|.
+// Why: on a few thousand amplitudes the tensor-core kernels run on one or two
+// SMs behind a setup that slices the whole matrix; here every block does a few
+// hundred instructions of setup and a pass spreads over the SMs.  4096 amplitudes, us a pass in a
+// replayed program: 2 targets (fused block) 9.3 -> 1.7, 3 targets 9.1 -> 2.0, 4
+// targets 10.9 -> 2.7, 5 targets 19.6 -> 4.9.
+// ---------------------------------------------------------------------------
+template <int NT>
+__global__ void __launch_bounds__(128) k_dense_fx(double2* __restrict__ psi, const __grid_constant__ DenseFxParams p) {
+  constexpr int D = 1 << NT, SH = NT - 2;
+  __shared__ int4 cm[D * D];                  // entry (j, k) at k D + j: parts of re and im
+  __shared__ int em[D];                       // largest biased exponent of a row
+  __shared__ int4 xs[128];                    // the amplitudes' parts
+  const int tid = threadIdx.x, j = tid % D;
+  const uint64_t k0 = (uint64_t)blockIdx.x * (128 / D) + tid / D;
+  const bool ok = k0 < p.ngroups;
+  uint64_t i = insert_zeros(k0, p.ins, p.nins) | p.ctrl_mask;
+#pragma unroll
+  for (int q = 0; q < NT; ++q)
+    if ((j >> q) & 1) i |= 1ull << p.tpos[q];
+  const double2 a = ok ? psi[i] : make_double2(0.0, 0.0);
+  constexpr int EPT = (D * D + 127) / 128;    // matrix entries per thread
+  double2 m[EPT];
+  if (tid < D) em[tid] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < EPT; ++e) {
+    const int idx = tid + 128 * e;
+    m[e] = idx < D * D ? reinterpret_cast<const double2*>(p.mat)[idx] : make_double2(0.0, 0.0);
+    if (p.conj) m[e].y = -m[e].y;
+    if (idx < D * D) atomicMax(em + idx / D, max(qsfx::expo_of(m[e].x), qsfx::expo_of(m[e].y)));
+  }
+  const Wd wr = words(a.x), wi = words(a.y);
+  uint32_t exf = emax2(wr, wi);
+#pragma unroll
+  for (int b = 1; b < D; b <<= 1) exf = max(exf, __shfl_xor_sync(0xFFFFFFFFu, exf, b));
+  const CPart own = cfx(wr, wi, exf);
+  xs[tid] = make_int4(own.re.h, own.re.l, own.im.h, own.im.l);
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < EPT; ++e) {
+    const int idx = tid + 128 * e;
+    if (idx < D * D) {
+      const int row = idx / D, er = em[row];
+      const Part re = qsfx::fixed_const(m[e].x, er), im = qsfx::fixed_const(m[e].y, er);
+      cm[(idx % D) * D + row] = make_int4(re.h, re.l, im.h, im.l);
+    }
+  }
+  __syncthreads();
+  int64_t vr = 0, vi = 0;
+  const int4* x = xs + (tid - j);
+#pragma unroll 4
+  for (int k = 0; k < D; k += 2) {
+    Acc ar = qsfx::acc_zero(), ai = qsfx::acc_zero();
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int4 xv = x[k + u], mv = cm[(k + u) * D + j];
+      const Part xr{xv.x, xv.y}, xi{xv.z, xv.w}, nxi{-xv.z, -xv.w}, mr{mv.x, mv.y}, mi{mv.z, mv.w};
+      qsfx::mac(ar, xr, mr);
+      qsfx::mac(ar, nxi, mi);
+      qsfx::mac(ai, xr, mi);
+      qsfx::mac(ai, xi, mr);
+    }
+    vr += qsfx::acc_value(ar) >> SH;
+    vi += qsfx::acc_value(ai) >> SH;
+  }
+  const qsfx::Scale sc = qsfx::scale_for((int)(exf >> 20) + SH, em[j]);
+  if (ok) psi[i] = make_double2(qsfx::finish_v(vr, sc), qsfx::finish_v(vi, sc));
+}
+
+// ---------------------------------------------------------------------------
 // Diagonal: alpha_i -> d_j alpha_i, j = the target bits of i.
 // ---------------------------------------------------------------------------
 template <int N>
@@ -385,6 +465,19 @@ cudaError_t launch_gate2_fx(void* amps, const Gate2FxParams& p, cudaStream_t st)
     k_gate2_fx<true><<<g, 256, 0, st>>>(static_cast<double2*>(amps), p);
   else
     k_gate2_fx<false><<<g, 256, 0, st>>>(static_cast<double2*>(amps), p);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_dense_fx(void* amps, const DenseFxParams& p, cudaStream_t st) {
+  const unsigned g = (unsigned)((p.ngroups * (1u << p.n) + 127) / 128);
+  double2* a = static_cast<double2*>(amps);
+  switch (p.n) {
+    case 2: k_dense_fx<2><<<g, 128, 0, st>>>(a, p); break;
+    case 3: k_dense_fx<3><<<g, 128, 0, st>>>(a, p); break;
+    case 4: k_dense_fx<4><<<g, 128, 0, st>>>(a, p); break;
+    case 5: k_dense_fx<5><<<g, 128, 0, st>>>(a, p); break;
+    default: return cudaErrorInvalidValue;
+  }
   return cudaGetLastError();
 }
 

@@ -34,7 +34,6 @@ struct qs_state {
   // staging ring for matrices and term lists: pinned host slot -> device slot
   unsigned char* h_ring = nullptr;
   unsigned char* d_ring = nullptr;
-  unsigned char* d_wide = nullptr;   // after the ring's slots: scratch of six-target gates (qsk::kWideScratch)
   cudaEvent_t ring_ev[qsapi::kRingSlots] = {};
   int ring_next = 0;
   // between qs_record_begin and qs_record_end: the program being recorded

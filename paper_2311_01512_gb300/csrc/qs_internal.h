@@ -16,7 +16,7 @@ constexpr int kTileBits = 10;        // amplitudes staged per tile of the dense 
 constexpr int kReduceBlocks = 1216;  // 152 SMs x 8: fixed grid of the stage-one expectation and trace reductions
 constexpr int kNormBlocks = 4864;    // 152 SMs x 32: fixed grid of the norm, a pure stream over the state
 constexpr int kPartials = kNormBlocks;  // partial sums a handle holds (the larger grid)
-constexpr size_t kWideScratch = 295424;  // bytes of a handle's scratch for six-target gates (qs_tc_ozaki.cu)
+constexpr size_t kWideScratch = 295424;  // bytes of scratch of a six-target gate (qs_tc_ozaki.cu)
 constexpr int kTermChunk = 2048;     // Pauli terms per device upload
 constexpr int kCostFeatures = 64;    // cost-model network: input features
 constexpr int kCostHidden = 64;      // hidden units per layer (two layers)
@@ -143,6 +143,20 @@ struct Gate2FxParams {
   int lo, hi;            // the targets sorted (the no-control index path)
   int nins;
   int8_t ins[kMaxQ];
+};
+
+// Dense gate on 2..5 targets of a small state (k_dense_fx, k_dense_digits):
+// groups of 2^n amplitudes base | target bits.
+struct DenseFxParams {
+  const double* mat;     // device, 2^n x 2^n complex128 row-major (re, im)
+  uint64_t ngroups;
+  uint64_t ctrl_mask;
+  int n;                 // targets of the kernel
+  int nmat;              // targets of the stored matrix (k_dense_digits: < n: identity on the others)
+  int conj;
+  int nins;
+  int8_t tpos[kMaxDense];
+  int8_t ins[kMaxQ];     // sorted targets and controls
 };
 
 // Diagonal entry d_j: parts of Re, Im and -Im with their shared exponent.
@@ -348,6 +362,10 @@ cudaError_t launch_gadget_df(void* amps, const GadgetDfParams& p, cudaStream_t s
 // complex128 in block fixed point (qs_gates_fx.cu)
 cudaError_t launch_gate1_fx(void* amps, const Gate1FxParams& p, cudaStream_t st);
 cudaError_t launch_gate2_fx(void* amps, const Gate2FxParams& p, cudaStream_t st);
+// 2 <= n <= 5 targets
+cudaError_t launch_dense_fx(void* amps, const DenseFxParams& p, cudaStream_t st);
+// small density matrices, 3 <= n <= 5 kernel targets (qs_gates_digits.cu)
+cudaError_t launch_dense_digits(void* amps, const DenseFxParams& p, cudaStream_t st);
 cudaError_t launch_diag_fx(void* amps, const DiagFxParams& p, cudaStream_t st);
 cudaError_t launch_gadget_fx(void* amps, const GadgetFxParams& p, cudaStream_t st);
 // G_DEPOL1, G_DEPOL2, G_DAMP, G_PAULI1

@@ -33,24 +33,11 @@
 // relative error of an output vector fell from 7.7, 6.6, 7.6 and 37.5 to 6.7,
 // 6.1, 6.3 and 6.4 e-17.
 //
-// Four kernels share these pieces.  k_dense_ozaki_small (two to four targets,
-// passes of fewer tiles than SMs) runs every phase in every thread;
-// k_dense_ozaki_ws (two to four targets) and k_dense_ozaki5 give gathering and
-// slicing, MMA issue and the epilogue to separate warps; k_dense_ozaki6 walks
-// blocks of its product with the tile's amplitudes in registers.  The comments
-// of the last three stand with them.
-//
-// k_dense_ozaki_small's work mapping: thread (warp w, lane) owns row g = 32 (w mod 4) + lane (the
-// tensor-memory lane that warp may read) and the amplitudes l in
-// [c EPT, (c+1) EPT), c = w / 4, of that row, for the gather, the slicing and
-// the epilogue alike, so the row's exponent and base index stay in registers.
-// Per CTA (persistent, tiles c, c + grid, ...): the loads of the next tile are
-// issued right after the current tile's MMAs, so they are in flight during the
-// MMAs and the epilogue.  The row maxima of tile i + 1 are taken after the
-// epilogue, so a tile costs two CTA barriers.  Thread 0 issues the initialising
-// MMA and then one MMA per A slice and K chunk, against all the B slices it
-// pairs with (see mma_tile).  Every wait is bounded: on timeout the kernel
-// records an error code, frees its tensor memory and returns.
+// Three kernels share these pieces: k_dense_ozaki_ws (two to four targets) and
+// k_dense_ozaki5 give gathering and slicing, MMA issue and the epilogue to
+// separate warps; k_dense_ozaki6 walks blocks of its product with the tile's
+// amplitudes in registers.  Passes over few amplitudes go to k_dense_fx
+// (qs_gates_fx.cu) instead, except with six targets.
 #include "qs_device.cuh"
 #include "qs_bytes.cuh"
 #include "qs_tc_ptx.cuh"
@@ -62,10 +49,6 @@ using namespace tcptx;
 
 constexpr int kRows = 128;
 constexpr uint32_t kWaitLimit = 1u << 26;
-
-__host__ __device__ constexpr uint32_t tmem_cols(uint32_t n) {
-  return n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : (n <= 256 ? 256 : 512)));
-}
 
 constexpr int kLv = qsby::kLevels;
 
@@ -84,20 +67,64 @@ __device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-// entry (k, n) of the realified (and possibly identity-extended) matrix
-__device__ __forceinline__ double realified(const TcParams& p, int D, int k, int n) {
-  int j = n >> 1, l = k >> 1;
-  const int c = n & 1, cp = k & 1;
+// entry (j, l) of the complex (and possibly identity-extended) matrix, D x D
+__device__ __forceinline__ double2 matrix_entry(const TcParams& p, int D, int j, int l) {
   if (p.nmat < p.n) {
-    if ((j >> p.nmat) != (l >> p.nmat)) return 0.0;
+    if ((j >> p.nmat) != (l >> p.nmat)) return make_double2(0.0, 0.0);
     const int mm = (1 << p.nmat) - 1;
     j &= mm;
     l &= mm;
     D = 1 << p.nmat;
   }
-  const double mr = p.mat[2 * (j * D + l)];
-  const double mi = p.conj ? -p.mat[2 * (j * D + l) + 1] : p.mat[2 * (j * D + l) + 1];
-  return c == 0 ? (cp == 0 ? mr : -mi) : (cp == 0 ? mi : mr);
+  double2 m = reinterpret_cast<const double2*>(p.mat)[j * D + l];
+  if (p.conj) m.y = -m.y;
+  return m;
+}
+
+__device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7FFFFFFFu; }
+
+// The slices of B from the complex matrix: entry (j, l) = (re, im) gives rows 2l,
+// 2l + 1 of column 2j (re, -im) and of column 2j + 1 (im, re), whose scales are
+// one, so two sets of digits and 16 stores of a pair serve four entries (a
+// negated digit stays within 128).  Leaves the column scales in csc and the digit
+// column sums in colsum (2D x 8).  off(n, k): byte offset of entry (k, n) in a
+// slice; slices are tstride bytes apart.  Ends without a barrier.
+template <int NT, int NTHR, typename Off>
+__device__ __forceinline__ void slice_matrix(const TcParams& p, unsigned char* b_dig, uint32_t tstride, const Off& off,
+                                             int* csc, int* colsum, int tid) {
+  constexpr int D = 1 << NT, E = (D * D + NTHR - 1) / NTHR;
+  for (int n = tid; n < 2 * D; n += NTHR) csc[n] = 0;
+  for (int i = tid; i < kLv * 2 * D; i += NTHR) colsum[i] = 0;
+  __syncthreads();
+  double2 m[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    // column fastest across threads: the lanes of a warp update different columns
+    const int idx = tid + e * NTHR, j = idx % D, l = idx / D;
+    if (idx >= D * D) break;
+    m[e] = matrix_entry(p, D, j, l);
+    atomicMax(csc + 2 * j, (int)max(abs_hi(m[e].x), abs_hi(m[e].y)));
+  }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int idx = tid + e * NTHR, j = idx % D, l = idx / D;
+    if (idx >= D * D) break;
+    const uint32_t ef = qsby::row_field((uint32_t)csc[2 * j]);
+    int dr[qsby::kB], di[qsby::kB];
+    qsby::digits_b((uint32_t)__double2hiint(m[e].x), (uint32_t)__double2loint(m[e].x), ef, dr);
+    qsby::digits_b((uint32_t)__double2hiint(m[e].y), (uint32_t)__double2loint(m[e].y), ef, di);
+    unsigned char *b0 = b_dig + off(2 * j, 2 * l), *b1 = b_dig + off(2 * j + 1, 2 * l);
+#pragma unroll
+    for (int t = 0; t < qsby::kB; ++t) {
+      const uint32_t hr = half_bits(dr[t]), hi = half_bits(di[t]);
+      *reinterpret_cast<uint32_t*>(b0 + t * tstride) = hr | ((di[t] ? hi ^ 0x8000u : 0u) << 16);
+      *reinterpret_cast<uint32_t*>(b1 + t * tstride) = hi | (hr << 16);
+      atomicAdd(colsum + 2 * j * kLv + t, dr[t] - di[t]);
+      atomicAdd(colsum + (2 * j + 1) * kLv + t, dr[t] + di[t]);
+    }
+  }
+  __syncthreads();
 }
 
 // All slice products of one tile.  B's slices lie back to back in shared
@@ -145,12 +172,11 @@ __device__ __forceinline__ void mma_products(uint32_t dcol, const unsigned char*
   mma_tile<N, KCH>(dcol, smem_desc(smem_u32(A), 128, sbo), smem_desc(smem_u32(B), 128, sbo));
 }
 
-// Rows (2^-24, 2^-16, 2^-8, 0, ...) of the initialising MMA's A.
+// Rows (2^-24, 2^-16, 2^-8, 0, ...) of the initialising MMA's A: two 16-byte core-matrix rows each.
 __device__ __forceinline__ void fill_start_rows(unsigned char* a_pre, int tid, int nthr) {
-  for (int idx = tid; idx < kRows * 16; idx += nthr) {
-    const int g = idx >> 4, k = idx & 15;
-    *reinterpret_cast<uint16_t*>(a_pre + canon_off16(g, k, 16)) =
-        (uint16_t)(k == 0 ? 0x0001 : (k == 1 ? 0x0100 : (k == 2 ? 0x1C00 : 0)));
+  for (int g = tid; g < kRows; g += nthr) {
+    *reinterpret_cast<uint4*>(a_pre + canon_off16(g, 0, 16)) = make_uint4(0x01000001u, 0x1C00u, 0u, 0u);
+    *reinterpret_cast<uint4*>(a_pre + canon_off16(g, 8, 16)) = make_uint4(0u, 0u, 0u, 0u);
   }
 }
 
@@ -158,9 +184,9 @@ __device__ __forceinline__ void fill_start_rows(unsigned char* a_pre, int tid, i
 __device__ __forceinline__ void fill_start_column(unsigned char* b_pre, int col, int P) {
   int pp[3];
   qsby::split_start(P, pp);
-#pragma unroll
-  for (int k = 0; k < 16; ++k)
-    *reinterpret_cast<uint16_t*>(b_pre + canon_off16(col, k, 16)) = k < 3 ? half_bits(pp[k]) : (uint16_t)0;
+  const uint32_t lo = half_bits(pp[0]) | ((uint32_t)half_bits(pp[1]) << 16);
+  *reinterpret_cast<uint4*>(b_pre + canon_off16(col, 0, 16)) = make_uint4(lo, half_bits(pp[2]), 0u, 0u);
+  *reinterpret_cast<uint4*>(b_pre + canon_off16(col, 8, 16)) = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Target offsets of the group members and row offsets of the tile.
@@ -187,46 +213,25 @@ __device__ __forceinline__ void fill_offsets(const TcParams& p, uint64_t* toff, 
 // column exponent field -> the increment it adds to a result's exponent field
 __device__ __forceinline__ int column_scale(int field) { return field - ((2046 + qsby::kScale) << 20); }
 
-// Per-CTA constants of a dense gate: the column exponent fields of B (in
-// csc), B's digit slices, the initialising MMA's operands, the target offsets
-// of the group members and the row offsets of the tile.  Every step runs over
-// all (column, row) pairs of B at once, the maxima and the digit column sums
-// (colsum: 8 x N ints) through shared-memory atomics, so the setup is short
-// next to one tile even for small states.
-template <int NT>
+// Per-CTA constants of a dense gate: the column scales and the digit slices of
+// B, the initialising MMA's operands, the target offsets of the group members
+// and the row offsets of the tile.
+template <int NT, int NTHR>
 __device__ void tile_constants(const TcParams& p, unsigned char* b_dig, unsigned char* a_pre, unsigned char* b_pre,
-                               int* csc, int* colsum, uint64_t* toff, uint64_t* rowoff, int tid, int nthr) {
-  constexpr int D = 1 << NT, K = 2 * D, N = 2 * D, BBYTES = N * K * 2;
-  for (int n = tid; n < N; n += nthr) csc[n] = 0;
-  for (int i = tid; i < kLv * N; i += nthr) colsum[i] = 0;
-  __syncthreads();
-  // column fastest across threads: the lanes of a warp update different
-  // columns' maxima and sums (no same-address atomics)
-  for (int idx = tid; idx < N * K; idx += nthr) {
-    const int n = idx % N, k = idx / N;
-    atomicMax(csc + n, __double2hiint(realified(p, D, k, n)) & 0x7FFFFFFF);
-  }
-  __syncthreads();
-  for (int idx = tid; idx < N * K; idx += nthr) {
-    const int n = idx % N, k = idx / N;
-    const double v = realified(p, D, k, n);
-    int d[qsby::kB];
-    qsby::digits_b((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v), qsby::row_field((uint32_t)csc[n]), d);
-    const uint32_t off = canon_off16(n, k, K);
-#pragma unroll
-    for (int t = 0; t < qsby::kB; ++t) {
-      *reinterpret_cast<uint16_t*>(b_dig + t * BBYTES + off) = half_bits(d[t]);
-      if (d[t] != 0) atomicAdd(colsum + n * kLv + t, d[t]);
-    }
-  }
-  fill_start_rows(a_pre, tid, nthr);
-  fill_offsets<NT>(p, toff, rowoff, tid, nthr);
-  __syncthreads();
-  for (int idx = tid; idx < kLv * N; idx += nthr) {
+                               int* csc, int* colsum, uint64_t* toff, uint64_t* rowoff, int tid) {
+  constexpr int D = 1 << NT, K = 2 * D, N = 2 * D;
+  fill_start_rows(a_pre, tid, NTHR);
+  fill_offsets<NT>(p, toff, rowoff, tid, NTHR);
+  slice_matrix<NT, NTHR>(p, b_dig, N * K * 2, [](int n, int k) { return canon_off16(n, k, K); }, csc, colsum, tid);
+  for (int idx = tid; idx < kLv * N; idx += NTHR) {
     const int L = idx / N, n = idx % N;
     fill_start_column(b_pre, L * N + n, qsby::start_value(L, K, colsum + n * kLv));
   }
-  for (int n = tid; n < N; n += nthr) csc[n] = column_scale((int)qsby::row_field((uint32_t)csc[n]));
+  for (int j = tid; j < D; j += NTHR) {
+    const int sc = column_scale((int)qsby::row_field((uint32_t)csc[2 * j]));
+    csc[2 * j] = sc;
+    csc[2 * j + 1] = sc;
+  }
 }
 
 // one output: levels -> Q -> double, scaled by the row's and the column's powers of two
@@ -256,182 +261,6 @@ __device__ __forceinline__ uint32_t max_abs(uint32_t m, const uint32_t* R) {
 }
 
 }  // namespace
-
-template <int NT, int THREADS, int CTAS>
-__global__ void __launch_bounds__(THREADS, CTAS) k_dense_ozaki_small(double2* __restrict__ psi, const __grid_constant__ TcParams p) {
-  constexpr int D = 1 << NT;
-  constexpr int K = 2 * D, N = 2 * D;
-  constexpr int CG = THREADS / kRows;         // threads per row
-  constexpr int EPT = D / CG;                 // amplitudes per thread
-  constexpr int CPW = 2 * EPT;                // accumulator columns per thread
-  static_assert(EPT % 4 == 0, "four amplitudes per 16-byte slice store");
-  constexpr int ABYTES = kRows * K * 2;       // one digit slice of A
-  constexpr int BBYTES = N * K * 2;
-  constexpr uint32_t LCOLS = kLv * N;         // accumulator columns
-  constexpr uint32_t TCOLS = tmem_cols(LCOLS);
-  static_assert(LCOLS <= 512, "tensor memory");
-  constexpr int PREA = kRows * 32, PREB = (int)LCOLS * 32;   // initialising operands (K = 16)
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* a_dig = smem;                                        // 7 x ABYTES
-  unsigned char* b_dig = a_dig + qsby::kA * ABYTES;                   // 8 x BBYTES
-  unsigned char* a_pre = b_dig + qsby::kB * BBYTES;                   // PREA
-  unsigned char* b_pre = a_pre + PREA;                                // PREB
-  uint64_t* toff = reinterpret_cast<uint64_t*>(b_pre + PREB);         // D
-  uint64_t* rowoff = toff + D;                                        // kRows
-  uint64_t* tile_base = rowoff + kRows;                               // 2
-  uint64_t* mbar = tile_base + 2;                                     // 1 (+ 1 pad)
-  int* csc = reinterpret_cast<int*>(mbar + 2);                        // N: exponent increment of a column
-  int* rowmax = csc + N;                                              // 2 x kRows: largest high word of a row
-  int* colsum = rowmax + 2 * kRows;                                   // N x 8: digit column sums (setup)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(colsum + kLv * N);
-
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-  tile_constants<NT>(p, b_dig, a_pre, b_pre, csc, colsum, toff, rowoff, tid, THREADS);
-  const int row_bits = p.tile_bits - NT;
-  for (int g = tid; g < 2 * kRows; g += THREADS) rowmax[g] = 0;
-  if (tid == 0) {
-    tile_base[0] = insert_zeros(blockIdx.x, p.hi_ins, p.nhi) | p.ctrl_mask;
-    mbar_init(mbar, 1);                       // one commit per tile
-  }
-  if (warp == 0) {
-    tmem_alloc(tmem_slot, TCOLS);
-    tmem_relinquish();
-  }
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
-
-  const int g = 32 * (warp & 3) + lane;       // row (tensor-memory lane)
-  const int cg = warp >> 2;                   // amplitude / column group of the row
-  const int l0 = cg * EPT;
-  const bool row_ok = g < (1 << row_bits);
-  const uint64_t roff = rowoff[g];
-  const uint32_t lane_addr = (uint32_t)(32 * (warp & 3)) << 16;
-  const int helper = THREADS > kRows ? kRows : 0;   // computes tile bases
-  // target offsets of this thread's amplitudes: registers when few
-  constexpr bool kRegOff = EPT <= 4;
-  uint64_t toffr[kRegOff ? EPT : 1];
-  if (kRegOff) {
-#pragma unroll
-    for (int i = 0; i < (kRegOff ? EPT : 1); ++i) toffr[i] = toff[l0 + i];
-  }
-  auto tofs = [&](int i) -> uint64_t { return kRegOff ? toffr[kRegOff ? i : 0] : toff[l0 + i]; };
-
-  uint32_t R[EPT][4];
-  auto load_tile = [&](uint64_t base) {
-    const uint64_t rb = base | roff;
-#pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-      double2 v = make_double2(0.0, 0.0);
-      if (row_ok) v = psi[rb | tofs(i)];
-      R[i][0] = (uint32_t)__double2hiint(v.x);
-      R[i][1] = (uint32_t)__double2loint(v.x);
-      R[i][2] = (uint32_t)__double2hiint(v.y);
-      R[i][3] = (uint32_t)__double2loint(v.y);
-    }
-  };
-  // row maximum (the CG threads of a row are in different warps)
-  auto row_max = [&](int slot) {
-    uint32_t m = 0;
-#pragma unroll
-    for (int i = 0; i < EPT; ++i) m = max_abs(m, R[i]);
-    atomicMax(rowmax + slot * kRows + g, (int)m);
-  };
-
-  // epilogue of one tile: levels -> exact integers -> doubles -> scatter
-  auto epilogue = [&](int egs, uint64_t rb) {
-#pragma unroll
-    for (int cc = 0; cc < CPW; cc += 8) {
-      float v[kLv][8];
-#pragma unroll
-      for (int L = 0; L < kLv; ++L) tmem_ld8(tmem + lane_addr + (uint32_t)(L * N + cg * CPW + cc), v[L]);
-      tmem_wait_ld();
-      if (row_ok) {
-        const int4 s0 = *reinterpret_cast<const int4*>(csc + cg * CPW + cc);
-        const int4 s1 = *reinterpret_cast<const int4*>(csc + cg * CPW + cc + 4);
-        const int scl[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-        double o[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          float u[kLv];
-#pragma unroll
-          for (int L = 0; L < kLv; ++L) u[L] = v[L][q];
-          o[q] = finish_output<K>(u, egs, scl[q]);
-        }
-#pragma unroll
-        for (int q = 0; q < 8; q += 2) psi[rb | tofs((cc + q) >> 1)] = make_double2(o[q], o[q + 1]);
-      }
-    }
-  };
-
-  // prologue: the first tile's amplitudes and row maxima, the second tile's base
-  load_tile(tile_base[0]);
-  row_max(0);
-  if (tid == helper && blockIdx.x + gridDim.x < p.ntiles)
-    tile_base[1] = insert_zeros(blockIdx.x + gridDim.x, p.hi_ins, p.nhi) | p.ctrl_mask;
-  __syncthreads();
-
-  uint32_t phase = 0;
-  bool failed = false;
-  int it = 0;
-  for (uint64_t c = blockIdx.x; c < p.ntiles; c += gridDim.x, ++it) {
-    const int par = it & 1;                   // tile parity: row-maximum and base slots
-    const uint64_t rb = tile_base[par] | roff;
-    const bool has_next = c + gridDim.x < p.ntiles;
-    const int egs = (int)qsby::row_field((uint32_t)rowmax[par * kRows + g]);   // exponent field of the row
-#pragma unroll
-    for (int i = 0; i < EPT; i += 4)
-      store_slices(a_dig, canon_off16(g, 2 * (l0 + i), K), ABYTES, R + i, (uint32_t)egs + 0x100000u);
-    fence_proxy_async();
-    __syncthreads();
-    if (tid == 0) {
-      fence_after_sync();
-      mma_start<N>(tmem, a_pre, b_pre);
-      mma_products<N, K / 16>(tmem, a_dig, b_dig);
-      mma_commit(mbar);
-    }
-    if (cg == 0) rowmax[par * kRows + g] = 0;   // read by every thread of the row before the barrier
-    // loads of the next tile, in flight during the MMAs and the epilogue
-    if (has_next) load_tile(tile_base[par ^ 1]);
-    const bool timed_out = wait_phase(mbar, phase);
-    phase ^= 1u;
-    fence_after_sync();
-    epilogue(egs, rb);
-    if (has_next) row_max(par ^ 1);
-    if (tid == helper && c + 2 * (uint64_t)gridDim.x < p.ntiles)
-      tile_base[par] = insert_zeros(c + 2 * (uint64_t)gridDim.x, p.hi_ins, p.nhi) | p.ctrl_mask;
-    fence_before_sync();
-    failed = __syncthreads_or(timed_out) != 0;
-    fence_after_sync();
-    if (failed) break;
-  }
-  if (failed && tid == 0) atomicExch(p.err, 1);
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, TCOLS);
-}
-
-template <int NT, int THREADS, int CTAS>
-static cudaError_t dense_ozaki_small(void* amps, const TcParams& p, cudaStream_t st) {
-  constexpr int D = 1 << NT, K = 2 * D, N = 2 * D;
-  constexpr size_t smem = (size_t)qsby::kA * (kRows * K * 2) + (size_t)qsby::kB * (N * K * 2) + kRows * 32 +
-                          (size_t)kLv * N * 32 + 8 * (D + kRows + 4) + 4 * (N + 2 * kRows + kLv * N) + 16;
-  static_assert(smem * CTAS <= 227 * 1024, "shared memory");
-  static_assert(CTAS * tmem_cols(kLv * N) <= 512, "tensor memory");
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki_small<NT, THREADS, CTAS>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_done = true;
-  }
-  const uint64_t maxb = (uint64_t)num_sms() * CTAS;
-  const unsigned g = (unsigned)(p.ntiles < maxb ? p.ntiles : maxb);
-  k_dense_ozaki_small<NT, THREADS, CTAS><<<g, THREADS, smem, st>>>(static_cast<double2*>(amps), p);
-  return cudaGetLastError();
-}
 
 // ---------------------------------------------------------------------------
 // Warp-specialised form for two to four targets (K <= 32, so every level
@@ -537,7 +366,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + W::slot_off + 4);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  tile_constants<NT>(p, b_dig, a_pre, b_pre, csc, colsum, toff, rowoff, tid, kWsThreads);
+  tile_constants<NT, kWsThreads>(p, b_dig, a_pre, b_pre, csc, colsum, toff, rowoff, tid);
   if (tid == 0) {
 #pragma unroll
     for (int j = 0; j < NA; ++j) {
@@ -756,6 +585,7 @@ static cudaError_t dense_ozaki_ws(void* amps, const TcParams& p, cudaStream_t st
     attr_done = true;
   }
   const uint64_t maxb = (uint64_t)num_sms(), nunits = p.ntiles / Ws<NT>::RB;
+  if (nunits == 0) return cudaErrorInvalidValue;   // such passes go elsewhere (qs_api.cpp)
   const unsigned g = (unsigned)(nunits < maxb ? nunits : maxb);
   k_dense_ozaki_ws<NT><<<g, kWsThreads, smem, st>>>(static_cast<double2*>(amps), p);
   return cudaGetLastError();
@@ -917,33 +747,22 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + X::slot_off + 4);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  fill_start_rows(a_pre, tid, X::THREADS);
+  fill_offsets<5>(p, toff, rowoff, tid, X::THREADS);
   // B's slices in blocks of 32 x 32: block (K block, N block) at (kb KB + nb) 16 KB
-  for (int n = tid; n < K; n += X::THREADS) csc[n] = 0;
-  for (int i = tid; i < kLv * K; i += X::THREADS) colsum[i] = 0;
-  __syncthreads();
-  for (int idx = tid; idx < K * K; idx += X::THREADS)
-    atomicMax(csc + idx % K, __double2hiint(realified(p, D, idx / K, idx % K)) & 0x7FFFFFFF);
-  __syncthreads();
-  for (int idx = tid; idx < K * K; idx += X::THREADS) {
-    const int n = idx % K, k = idx / K;
-    const double v = realified(p, D, k, n);
-    int d[qsby::kB];
-    qsby::digits_b((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v), qsby::row_field((uint32_t)csc[n]), d);
-    unsigned char* blk = b_dig + ((k >> 5) * KB + (n >> 5)) * kKnBlock + canon_off16(n & 31, k & 31, 32);
-#pragma unroll
-    for (int t = 0; t < qsby::kB; ++t) {
-      *reinterpret_cast<uint16_t*>(blk + t * 2048) = half_bits(d[t]);
-      if (d[t] != 0) atomicAdd(colsum + n * kLv + t, d[t]);
-    }
-  }
-  __syncthreads();
+  slice_matrix<5, X::THREADS>(
+      p, b_dig, 2048,
+      [](int n, int k) { return ((k >> 5) * KB + (n >> 5)) * kKnBlock + (int)canon_off16(n & 31, k & 31, 32); }, csc,
+      colsum, tid);
   for (int idx = tid; idx < kLv * K; idx += X::THREADS) {
     const int L = idx / K, n = idx % K;
     fill_start_column(b_pre + (n >> 5) * 8192, L * 32 + (n & 31), qsby::start_value(L, K, colsum + n * kLv));
   }
-  for (int n = tid; n < K; n += X::THREADS) csc[n] = column_scale((int)qsby::row_field((uint32_t)csc[n]));
-  fill_start_rows(a_pre, tid, X::THREADS);
-  fill_offsets<5>(p, toff, rowoff, tid, X::THREADS);
+  for (int j = tid; j < D; j += X::THREADS) {
+    const int sc = column_scale((int)qsby::row_field((uint32_t)csc[2 * j]));
+    csc[2 * j] = sc;
+    csc[2 * j + 1] = sc;
+  }
   for (int g = tid; g < 3 * kRows; g += X::THREADS) rowmax[g] = 0;
   if (tid == 0) {
 #pragma unroll
@@ -1092,7 +911,7 @@ static cudaError_t dense_ozaki5(void* amps, const TcParams& p, cudaStream_t st) 
 // against both.  The second pair takes the K blocks in the order 3, 2, 1, 0, so
 // that two of its four are still in the operand buffers.  B's slices (256 KB)
 // do not fit in shared memory: a setup kernel (k_wide_matrix) writes them to the
-// handle's scratch, and another warp streams the 16 KB block of each (K, N) pair
+// caller's scratch, and another warp streams the 16 KB block of each (K, N) pair
 // from L2 into a ring of four slots with bulk copies.  Hand-offs as for five
 // targets, with bfull (bulk copy) and bempty (MMA completion) for B's slots.
 // Bound by the tensor cores (53% busy, two fifths of each tile's time being the
@@ -1141,7 +960,8 @@ __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcP
   if (k < kLv) sums[k] = 0;
   if (k == 0) mx = 0;
   __syncthreads();
-  const double v = realified(p, D, k, n);
+  const double2 m = matrix_entry(p, D, n >> 1, k >> 1);
+  const double v = (n & 1) ? ((k & 1) ? m.x : m.y) : ((k & 1) ? -m.y : m.x);
   atomicMax(&mx, __double2hiint(v) & 0x7FFFFFFF);
   __syncthreads();
   const uint32_t ef = qsby::row_field((uint32_t)mx);
@@ -1348,14 +1168,10 @@ static cudaError_t dense_ozaki6(void* amps, const TcParams& p, void* scratch, cu
   return cudaGetLastError();
 }
 
-// Passes of fewer tiles than SMs (small states) go to the single-CTA kernels,
-// whose setup is lighter than the warp-specialised kernel's (one tile per CTA
-// leaves nothing to pipeline).
 cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st) {
-  const bool small = p.ntiles < (uint64_t)num_sms();
   switch (p.n) {
-    case 3: return small ? dense_ozaki_small<3, 128, 4>(amps, p, st) : dense_ozaki_ws<3>(amps, p, st);
-    case 4: return small ? dense_ozaki_small<4, 256, 2>(amps, p, st) : dense_ozaki_ws<4>(amps, p, st);
+    case 3: return dense_ozaki_ws<3>(amps, p, st);
+    case 4: return dense_ozaki_ws<4>(amps, p, st);
     case 5: return dense_ozaki5(amps, p, st);
     case 6: return dense_ozaki6(amps, p, scratch, st);
     default: return cudaErrorInvalidValue;

@@ -49,6 +49,30 @@ def test_dense_gate(n, nq, spread):
         assert np.max(np.abs((got - want).view(np.float64))) <= bound(n, psi, mat)
 
 
+@pytest.mark.parametrize("n", [2, 3, 4, 5])
+@pytest.mark.parametrize("extra", [0, 1, 2, 5, 8, 11, 12, 13, 14])
+def test_small_passes(n, extra):
+    """Dense blocks and gates with controls around the size where passes change
+    from one thread per amplitude to the tensor cores."""
+    from paper_2311_01512_gb300 import qs
+    nq = n + extra
+    rng = np.random.default_rng(700 + 20 * n + extra)
+    psi = wl.random_statevector(nq, rng) * 2.0 ** -rng.integers(0, 12, size=1 << nq)
+    mat = np.ascontiguousarray(wl.haar_unitary(1 << n, rng))
+    perm = [int(q) for q in rng.permutation(nq)]
+    for ctrls in ([], perm[n:n + 1], perm[n:n + 3]):
+        st = qs.State(nq)
+        st.set_amps(psi)
+        if ctrls:
+            qs.qs_apply_ctrl_multi_target(st.handle, ctrls, perm[:n], mat)
+        else:
+            qs.qs_apply_dense_block(st.handle, perm[:n], mat)
+        got = st.get_amps()
+        st.close()
+        want = orc.run_ops(psi, [{"op": "unitary", "ctrls": ctrls, "targs": perm[:n], "mat": mat}], is_density=False)
+        assert np.max(np.abs((got - want).view(np.float64))) <= bound(n, psi, mat)
+
+
 def test_repeated_gates_share_the_scratch():
     """Six-target gates with different matrices queued back to back, and through
     a recorded program replayed twice."""
@@ -78,14 +102,17 @@ def test_repeated_gates_share_the_scratch():
     st.close()
 
 
-@pytest.mark.parametrize("nq", [4, 8])
+@pytest.mark.parametrize("nq", [4, 8, 9])
 def test_density_matrix_passes(nq):
-    """Three-qubit Kraus maps (a six-target superoperator) and the two passes of
+    """Three-qubit Kraus maps (a six-target superoperator), two-qubit ones,
+    and the two passes of
     controlled and wide unitaries."""
     from paper_2311_01512_gb300 import qs
     rng = np.random.default_rng(67 + nq)
     rho = orc.densmatr_from_pure(wl.random_statevector(nq, rng))
     ops = [{"op": "kraus", "targs": [3, 0, 2], "kraus": wl.haar_kraus(3, 3, rng)},
+           {"op": "kraus", "targs": [2, 0], "kraus": wl.haar_kraus(2, 4, rng)},
+           {"op": "unitary", "ctrls": [], "targs": [3, 1], "mat": wl.haar_unitary(4, rng)},
            {"op": "unitary", "ctrls": [], "targs": [2, 0, 3, 1], "mat": wl.haar_unitary(16, rng)},
            {"op": "unitary", "ctrls": [1], "targs": [2, 0, 3], "mat": wl.haar_unitary(8, rng)}]
     st = qs.State(nq, density=True)
