@@ -2,10 +2,11 @@
 // their own circuits, run by one persistent kernel launch (qs_batch_kernels.cu)
 // that is captured once in a CUDA graph and replayed.
 //
-// Scheduling: states are ordered by estimated work (amplitudes x operations),
+// Scheduling: states are ordered by estimated work (amplitudes x operation costs),
 // largest first, and CTAs take them from a shared counter, so the long states
 // start early and the short ones fill the gaps (longest-processing-time
-// order).  The launch shape (threads per CTA, CTAs per SM, and with it the
+// order).  A state with more than a CTA's share of the work would outlast the
+// rest; such heavy states are shared by the CTAs of a cluster.  The launch shape (threads per CTA, CTAs per SM, and with it the
 // largest state kept in shared memory) is chosen by timing every candidate on
 // the batch itself.
 //
@@ -49,6 +50,7 @@ struct qs_batch {
   long num_segs = 0;
   int wide = 0;                 // some operation is dense on 3 or 4 targets
   int threads = 256, ctas = 0, smem_qubits = -1;
+  int cluster = 1, nheavy = 0;  // heavy states (first in the order) are shared by clusters of CTAs
   cudaStream_t capture_stream = nullptr;  // own stream for recording (the caller's may be the legacy stream)
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -149,6 +151,7 @@ int smem_qubits_for(qs_prec prec, int ctas_per_sm) {
 // ---- segment plans (for one tile size L) ------------------------------------
 struct Plan {
   int L = -1;
+  int cluster = 1;                    // CTAs that share a heavy state
   std::vector<qsk::BatchState> states;
   std::vector<qsk::BatchSeg> segs;
   std::vector<qsk::BatchXlat> xlat;   // parallel to the operations
@@ -164,12 +167,21 @@ struct Plan {
   }
 };
 
-// Segments of every state larger than 2^L amplitudes (qs_batch_plan.h).
-void build_plan(Plan& P, int L, const std::vector<int>& nq, const std::vector<qsk::BatchState>& base,
-                const std::vector<qsk::BatchOp>& ops) {
+// Least qubits of a heavy state: eight tiles (the largest cluster) of 2^8 amplitudes.
+constexpr int kHeavyMinQubits = 11;
+
+// Segments of every state larger than 2^L amplitudes (qs_batch_plan.h); with
+// clusters, heavy states in tiles small enough for one per CTA of a cluster.
+void build_plan(Plan& P, int L, int cluster, const std::vector<int>& nq, const std::vector<char>& heavy,
+                const std::vector<qsk::BatchState>& base, const std::vector<qsk::BatchOp>& ops) {
   P.L = L;
+  P.cluster = cluster;
   P.states = base;
-  qsbatch::build_segments(L, nq, P.states, ops, P.segs, P.xlat);
+  std::vector<int> Ls(nq.size(), L);
+  if (cluster > 1)
+    for (size_t s = 0; s < nq.size(); ++s)
+      if (heavy[s]) Ls[s] = std::min(L, nq[s] - (31 - __builtin_clz((unsigned)cluster)));
+  qsbatch::build_segments(Ls, nq, P.states, ops, P.segs, P.xlat);
 }
 
 bool upload_plan(Plan& P) {
@@ -402,16 +414,32 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
   b->wide = 0;
   for (const auto& op : ops)
     if (op.kind == 0 && op.n > 2) b->wide = 1;
+  const int sms = qsk::num_sms();
+  // work per state; heavy: more than one CTA's share at two CTAs per SM
+  std::vector<double> work(S);
+  double total = 0.0;
+  for (int s = 0; s < S; ++s) {
+    double c = 1.0;
+    for (const auto& op : b->progs[s]) c += qsbatch::op_cost(op);
+    work[s] = c * (double)(1ull << b->nq[s]);
+    total += work[s];
+  }
+  std::vector<char> heavy(S, 0);
+  int nheavy = 0;
+  for (int s = 0; s < S; ++s)
+    if (b->nq[s] >= kHeavyMinQubits && work[s] > total / (2 * sms)) {
+      heavy[s] = 1;
+      ++nheavy;
+    }
   std::vector<int> order(S);
   for (int s = 0; s < S; ++s) order[s] = s;
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-    return ((double)(1ull << b->nq[x]) * (1 + b->progs[x].size())) >
-           ((double)(1ull << b->nq[y]) * (1 + b->progs[y].size()));
+    return heavy[x] != heavy[y] ? heavy[x] > heavy[y] : work[x] > work[y];
   });
   if (qsalloc::device(reinterpret_cast<void**>(&b->d_order), sizeof(int) * S) != cudaSuccess ||
       qsalloc::device(reinterpret_cast<void**>(&b->d_ops), sizeof(qsk::BatchOp) * std::max<size_t>(1, ops.size())) != cudaSuccess ||
       qsalloc::device(reinterpret_cast<void**>(&b->d_consts), sizeof(double) * std::max<size_t>(1, consts.size())) != cudaSuccess ||
-      qsalloc::device(reinterpret_cast<void**>(&b->d_counter), sizeof(int)) != cudaSuccess) {
+      qsalloc::device(reinterpret_cast<void**>(&b->d_counter), 2 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     free_device(b);
     return QS_ERR_OOM;
@@ -424,29 +452,36 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
     free_device(b);
     return QS_ERR_CUDA;
   }
-  // launch-shape candidates: (threads, CTAs per SM); each shared-memory size
-  // (tile size) has its own segment plan
-  const int sms = qsk::num_sms();
+  // launch-shape candidates; each shared-memory size (tile size) has its own
+  // segment plan, with and without heavy states shared by clusters
   if (qsk::batch_set_max_smem(200 * 1024) != cudaSuccess) {
     cudaGetLastError();
     return QS_ERR_CUDA;
   }
-  std::vector<std::pair<int, int>> cands;
-  if (autotune)
-    cands = {{128, 4}, {256, 2}, {256, 4}, {512, 1}, {512, 2}};
-  else
-    cands = {{256, 2}};
+  struct Shape {
+    int threads, per_sm, cluster;
+  };
+  std::vector<Shape> cands;
+  if (autotune) {
+    cands = {{128, 4, 1}, {256, 2, 1}, {256, 4, 1}, {512, 1, 1}, {512, 2, 1}};
+    // 512 complex64 states of 10-17 qubits: 1.54 ms without clusters, 1.22-1.38
+    // in clusters of 2 and 4, 1.68 of 8; 256 complex128 states, a quarter of them
+    // density matrices: 7.69, 3.75, 1.91 and 1.82 ms
+    if (nheavy) cands.insert(cands.end(), {{512, 1, 2}, {512, 1, 4}, {256, 2, 4}, {256, 2, 8}});
+  } else {
+    cands = {{256, 2, nheavy ? 4 : 1}};
+  }
   std::vector<Plan> plans;
   plans.reserve(cands.size());       // pointers into it stay valid
-  auto plan_for = [&](int L) -> Plan* {
+  auto plan_for = [&](int L, int cluster) -> Plan* {
     for (auto& P : plans)
-      if (P.L == L) return &P;
+      if (P.L == L && P.cluster == cluster) return &P;
     plans.emplace_back();
-    build_plan(plans.back(), L, b->nq, states, ops);
+    build_plan(plans.back(), L, cluster, b->nq, heavy, states, ops);
     return &plans.back();
   };
   for (const auto& c : cands) {
-    Plan* P = plan_for(smem_qubits_for(b->prec, c.second));
+    Plan* P = plan_for(smem_qubits_for(b->prec, c.per_sm), c.cluster);
     if (!P->d_states && !upload_plan(*P)) {
       for (auto& Q : plans) Q.release();
       free_device(b);
@@ -459,12 +494,22 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
   float best = 1e30f;
   int best_plan = -1;
   for (const auto& c : cands) {
-    const int sq = smem_qubits_for(b->prec, c.second);
-    Plan* P = plan_for(sq);
-    if (cudaMemsetAsync(b->d_counter, 0, sizeof(int), b->stream) != cudaSuccess) return QS_ERR_CUDA;
+    const int sq = smem_qubits_for(b->prec, c.per_sm);
+    Plan* P = plan_for(sq, c.cluster);
+    const int nh = c.cluster > 1 ? nheavy : 0;
+    int ctas = sms * c.per_sm;
+    if (c.cluster > 1) {
+      int n = 0;
+      if (qsk::batch_max_clusters(b->prec, c.threads, sq, b->wide, c.cluster, &n) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        continue;
+      }
+      ctas = n * c.cluster;
+    }
+    if (cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(int), b->stream) != cudaSuccess) return QS_ERR_CUDA;
     cudaEventRecord(e0, b->stream);
-    if (qsk::launch_batch(b->prec, b->pool, P->d_states, b->d_order, S, b->d_ops, b->d_consts, P->d_segs,
-                          P->d_xlat, b->d_counter, c.first, sms * c.second, sq, b->wide, b->stream) != cudaSuccess) {
+    if (qsk::launch_batch(b->prec, b->pool, P->d_states, b->d_order, S, nh, b->d_ops, b->d_consts, P->d_segs, P->d_xlat,
+                          b->d_counter, c.threads, ctas, sq, b->wide, c.cluster, b->stream) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -474,9 +519,11 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
     cudaEventElapsedTime(&ms, e0, e1);
     if (ms < best) {
       best = ms;
-      b->threads = c.first;
-      b->ctas = sms * c.second;
+      b->threads = c.threads;
+      b->ctas = ctas;
       b->smem_qubits = sq;
+      b->cluster = c.cluster;
+      b->nheavy = nh;
       best_plan = (int)(P - plans.data());
     }
   }
@@ -498,10 +545,11 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
     cudaGetLastError();
     return QS_ERR_CUDA;
   }
-  cudaError_t e = cudaMemsetAsync(b->d_counter, 0, sizeof(int), b->capture_stream);
+  cudaError_t e = cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(int), b->capture_stream);
   if (e == cudaSuccess)
-    e = qsk::launch_batch(b->prec, b->pool, b->d_states, b->d_order, S, b->d_ops, b->d_consts, b->d_segs, b->d_xlat,
-                          b->d_counter, b->threads, b->ctas, b->smem_qubits, b->wide, b->capture_stream);
+    e = qsk::launch_batch(b->prec, b->pool, b->d_states, b->d_order, S, b->nheavy, b->d_ops, b->d_consts, b->d_segs,
+                          b->d_xlat, b->d_counter, b->threads, b->ctas, b->smem_qubits, b->wide, b->cluster,
+                          b->capture_stream);
   cudaGraph_t g = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(b->capture_stream, &g);
   if (e != cudaSuccess || e2 != cudaSuccess || !g) {

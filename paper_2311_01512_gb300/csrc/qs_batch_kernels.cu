@@ -3,7 +3,8 @@
 // work counter (states ordered largest first) and applies that state's whole
 // program with only block-level synchronisation between operations: in shared
 // memory when the state fits, otherwise in place in global memory (small states
-// stay in L2).  No CTA ever waits for another one.
+// stay in L2).  Only the CTAs of a cluster, which the hardware schedules
+// together, wait for one another, on the heavy states that they share.
 //
 // Operations (the statevector gates of Sec. "One-target gate", "Many-control
 // one-target gate", "Many-target gate", "Phase gadget", "Pauli gadget"):
@@ -12,6 +13,8 @@
 // lowered unitaries to their two passes and channels to superoperators
 // (dense operations on t and t + N).  complex64 states compute in FP32,
 // complex128 states in double-float (qs_df.cuh).
+#include <cooperative_groups.h>
+
 #include "qs_device.cuh"
 #include "qs_df.cuh"
 
@@ -311,19 +314,21 @@ __device__ __forceinline__ void op_pair(P* a, uint32_t i, uint32_t j, const Gad<
 // Out of line, so its registers do not weigh on the other operations.
 template <int NT, typename P, typename K>
 __device__ __noinline__ void dense_sweep(P* a, uint32_t groups, InsMasks ins, uint32_t ctrl, uint32_t tb0,
-                                         uint32_t tb1, uint32_t tb2, uint32_t tb3, const K* kc) {
+                                         uint32_t tb1, uint32_t tb2, uint32_t tb3, const K* kc, uint32_t lane,
+                                         uint32_t lanes) {
   const uint32_t tb[4] = {tb0, tb1, tb2, tb3};
-  for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x)
+  for (uint32_t g = lane; g < groups; g += lanes)
     op_denseN<NT>(a, insert_zeros_m(g, ins) | ctrl, tb, kc);
 }
 
 // ---- one operation on a whole state held at `a` (shared or global) ---------
-// kc: the operation's constants (load_consts).
+// kc: the operation's constants (load_consts); lane, lanes: this thread's index among
+// those that share the operation, and their number.
 // WIDE: the batch has dense operations on 3 or 4 targets (superoperators of
 // density-matrix channels); without them the kernel carries no call to the
 // out-of-line sweeps, whose call sites cost the narrow kernel registers.
 template <bool WIDE, typename P, typename K>
-__device__ void apply_op(P* a, int nq, const BatchOp& op, const K* kc) {
+__device__ void apply_op(P* a, int nq, const BatchOp& op, const K* kc, uint32_t lane, uint32_t lanes) {
   const uint32_t dim = 1u << nq;
   const int kind = op.kind, n = op.n;
   if (kind == 0) {
@@ -335,12 +340,12 @@ __device__ void apply_op(P* a, int nq, const BatchOp& op, const K* kc) {
       K m[8];   // in registers for the sweep (its stores may alias shared memory)
 #pragma unroll
       for (int i = 0; i < 8; ++i) m[i] = kc[i];
-      for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x) {
+      for (uint32_t g = lane; g < groups; g += lanes) {
         const uint32_t base = insert_zeros_m(g, ins) | ctrl;
         op_dense1(a, base, base | b0, m);
       }
     } else if (n == 2) {
-      for (uint32_t g = threadIdx.x; g < groups; g += blockDim.x) {
+      for (uint32_t g = lane; g < groups; g += lanes) {
         const uint32_t base = insert_zeros_m(g, ins) | ctrl;
         const uint32_t idx[4] = {base, base | b0, base | b1, base | b0 | b1};
         op_dense2(a, idx, kc);
@@ -348,13 +353,13 @@ __device__ void apply_op(P* a, int nq, const BatchOp& op, const K* kc) {
     } else if constexpr (WIDE) {
       const uint32_t tb2 = 1u << op.t[2], tb3 = n > 3 ? 1u << op.t[3] : 0u;
       if (n == 3)
-        dense_sweep<3>(a, groups, ins, ctrl, b0, b1, tb2, tb3, kc);
+        dense_sweep<3>(a, groups, ins, ctrl, b0, b1, tb2, tb3, kc, lane, lanes);
       else
-        dense_sweep<4>(a, groups, ins, ctrl, b0, b1, tb2, tb3, kc);
+        dense_sweep<4>(a, groups, ins, ctrl, b0, b1, tb2, tb3, kc, lane, lanes);
     }
   } else if (kind == 1) {
     const int t0 = op.t[0], t1 = n > 1 ? op.t[1] : 0, t2 = n > 2 ? op.t[2] : 0;
-    for (uint32_t i = threadIdx.x; i < dim; i += blockDim.x) {
+    for (uint32_t i = lane; i < dim; i += lanes) {
       int j = (int)((i >> t0) & 1u);
       if (n > 1) j |= (int)((i >> t1) & 1u) << 1;
       if (n > 2) j |= (int)((i >> t2) & 1u) << 2;
@@ -364,10 +369,10 @@ __device__ void apply_op(P* a, int nq, const BatchOp& op, const K* kc) {
     const auto G = make_gad(kc);
     const uint32_t xy = op.xy, yz = op.yz;
     if (xy == 0) {
-      for (uint32_t i = threadIdx.x; i < dim; i += blockDim.x) op_phase(a, i, G, __popc(i & yz) & 1);
+      for (uint32_t i = lane; i < dim; i += lanes) op_phase(a, i, G, __popc(i & yz) & 1);
     } else {
       const int q = (op.eta + 1) & 3, h = op.h;
-      for (uint32_t k = threadIdx.x; k < (dim >> 1); k += blockDim.x) {
+      for (uint32_t k = lane; k < (dim >> 1); k += lanes) {
         const uint32_t i = ((k >> h) << (h + 1)) | (k & ((1u << h) - 1));
         const uint32_t j = i ^ xy;
         op_pair(a, i, j, G, __popc(i & yz) & 1, __popc(j & yz) & 1, q);
@@ -408,9 +413,9 @@ __device__ void apply_tile_op(P* a, int L, const BatchOp& op, const BatchXlat& x
     } else if constexpr (WIDE) {
       const uint32_t tb2 = 1u << x.lt[2], tb3 = n > 3 ? 1u << x.lt[3] : 0u;
       if (n == 3)
-        dense_sweep<3>(a, groups, ins, ctrl, b0, b1, tb2, tb3, kc);
+        dense_sweep<3>(a, groups, ins, ctrl, b0, b1, tb2, tb3, kc, threadIdx.x, blockDim.x);
       else
-        dense_sweep<4>(a, groups, ins, ctrl, b0, b1, tb2, tb3, kc);
+        dense_sweep<4>(a, groups, ins, ctrl, b0, b1, tb2, tb3, kc, threadIdx.x, blockDim.x);
     }
   } else if (kind == 1) {
     int jfix = 0, lt[3] = {-1, -1, -1};
@@ -441,131 +446,208 @@ __device__ void apply_tile_op(P* a, int L, const BatchOp& op, const BatchXlat& x
   }
 }
 
+// The block's shared memory besides the tile.
+template <typename T2>
+struct BatchShared {
+  uint32_t tl[128], th[128];
+  KT<T2> k[2][kMaxConsts];  // constants of the current and the next operation
+};
+
+// A state's segments, shared by `parts` CTAs of which this is number `part`:
+// tiles part, part + parts, ...; sync() after each segment (and each operation
+// of a global-memory segment) orders the CTAs.  A tiled segment loads each tile
+// (one 16-byte or 8-byte gather per amplitude through two 128-entry offset
+// tables; the five lowest qubits are always tile qubits, so a warp reads 32
+// consecutive amplitudes), applies the segment's operations to it and writes it
+// back.
+template <bool WIDE, typename T2, typename Sync>
+__device__ __forceinline__ void run_segments(T2* __restrict__ g, const BatchState& st, const BatchOp* __restrict__ ops,
+                                             const double* __restrict__ consts, const BatchSeg* __restrict__ segs,
+                                             const BatchXlat* __restrict__ xlat, typename SmemOf<T2>::T* sm,
+                                             BatchShared<T2>& sh, uint32_t part, uint32_t parts, const Sync& sync) {
+  using SM = SmemOf<T2>;
+  const uint32_t dim = 1u << st.nq;
+  for (int sg = st.first_seg; sg < st.first_seg + st.nsegs; ++sg) {
+    const BatchSeg S = segs[sg];
+    if (S.L == 0) {
+      load_consts<T2>(ops[S.first_op], consts, sh.k[0]);
+      __syncthreads();
+      for (int k = 0; k < S.nops; ++k) {
+        apply_op<WIDE>(g, st.nq, ops[S.first_op + k], sh.k[k & 1], part * blockDim.x + threadIdx.x, parts * blockDim.x);
+        if (k + 1 < S.nops) load_consts<T2>(ops[S.first_op + k + 1], consts, sh.k[(k + 1) & 1]);
+        sync();
+      }
+      continue;
+    }
+    const int L = S.L, hi = L - 7;                  // 8 <= L <= 14
+    uint32_t qmask = 0;
+    for (int b = 0; b < L; ++b) qmask |= 1u << S.q[b];
+    for (int j = threadIdx.x; j < 128; j += blockDim.x) {
+      uint32_t tl = 0, th = 0;
+      for (int b = 0; b < 7; ++b)
+        if ((j >> b) & 1) tl |= 1u << S.q[b];
+      for (int b = 0; b < hi; ++b)
+        if ((j >> b) & 1) th |= 1u << S.q[7 + b];
+      sh.tl[j] = tl;
+      sh.th[j] = th;
+    }
+    __syncthreads();
+    const uint32_t fmask = (dim - 1) & ~qmask;       // the other qubits: the tile number, deposited
+    const uint32_t ntiles = dim >> L, tdim = 1u << L;
+    for (uint32_t tile = part; tile < ntiles; tile += parts) {
+      uint32_t base = 0;
+      {
+        uint32_t m = fmask, t = tile;
+        while (m) {
+          const uint32_t low = m & (~m + 1u);
+          if (t & 1u) base |= low;
+          m ^= low;
+          t >>= 1;
+        }
+      }
+      for (uint32_t i = threadIdx.x; i < tdim; i += blockDim.x) sm[i] = SM::in(g[base | sh.tl[i & 127u] | sh.th[i >> 7]]);
+      load_consts<T2>(ops[S.first_op], consts, sh.k[0]);
+      __syncthreads();
+      for (int k = 0; k < S.nops; ++k) {
+        apply_tile_op<WIDE>(sm, L, ops[S.first_op + k], xlat[S.first_op + k], base, sh.k[k & 1]);
+        if (k + 1 < S.nops) load_consts<T2>(ops[S.first_op + k + 1], consts, sh.k[(k + 1) & 1]);
+        __syncthreads();
+      }
+      for (uint32_t i = threadIdx.x; i < tdim; i += blockDim.x) g[base | sh.tl[i & 127u] | sh.th[i >> 7]] = SM::out(sm[i]);
+      __syncthreads();
+    }
+    if (parts > 1) sync();
+  }
+}
+
 }  // namespace
 
-// One CTA per state at a time.  States of at most smem_qubits qubits are
-// copied to shared memory, run there, and copied back.  Larger states run
-// segment by segment: a tiled segment loads each tile (one 16-byte or 8-byte
-// gather per amplitude through two 128-entry offset tables; the five lowest
-// qubits are always tile qubits, so a warp reads 32 consecutive amplitudes),
-// applies the segment's operations to it and writes it back.
-template <typename T2, bool WIDE>
-__global__ void __launch_bounds__(512, sizeof(T2) == 8 ? 2 : 1)
+// CTAs take states from work counters, largest first.  CL: the CTAs of a
+// cluster first share the heavy states (order[0 .. nheavy)), each taking a part
+// of every segment's tiles with a cluster barrier between segments; those states
+// alone would outlast the rest of the batch on one CTA each.  Then (and without
+// clusters throughout) each CTA takes one state at a time: a state of at most
+// smem_qubits qubits is copied to shared memory, run there, and copied back, a
+// larger one runs segment by segment.  Without
+// clusters a batch took as long as its largest state on one CTA: 256 complex128
+// states of 10-16 storage qubits 7.69 ms, with clusters of eight 1.82 (the
+// autotuner picks the size).
+template <typename T2, bool WIDE, bool CL>
+__global__ void __launch_bounds__(512, sizeof(T2) == 8 && !CL ? 2 : 1)
     k_batch(T2* __restrict__ pool, const BatchState* __restrict__ states, const int* __restrict__ order, int nstates,
-            const BatchOp* __restrict__ ops, const double* __restrict__ consts, const BatchSeg* __restrict__ segs,
-            const BatchXlat* __restrict__ xlat, int* __restrict__ counter, int smem_qubits) {
+            int nheavy, const BatchOp* __restrict__ ops, const double* __restrict__ consts,
+            const BatchSeg* __restrict__ segs, const BatchXlat* __restrict__ xlat, int* __restrict__ counters,
+            int smem_qubits) {
   using SM = SmemOf<T2>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   typename SM::T* sm = reinterpret_cast<typename SM::T*>(smem_raw);
   __shared__ int s_work;
-  __shared__ uint32_t s_tl[128], s_th[128];
-  __shared__ KT<T2> s_k[2][kMaxConsts];  // constants of the current and the next operation
+  __shared__ BatchShared<T2> sh;
+  namespace cg = cooperative_groups;
+  bool shared_phase = CL;
   while (true) {
-    if (threadIdx.x == 0) s_work = atomicAdd(counter, 1);
-    __syncthreads();
-    const int w = s_work;
-    __syncthreads();
-    if (w >= nstates) break;
+    uint32_t part = 0, parts = 1;
+    int w;
+    if (CL && shared_phase) {
+      const cg::cluster_group cl = cg::this_cluster();
+      part = cl.block_rank();
+      parts = cl.num_blocks();
+      if (part == 0 && threadIdx.x == 0) s_work = atomicAdd(counters + 1, 1);
+      cl.sync();
+      w = *cl.map_shared_rank(&s_work, 0);
+      cl.sync();
+      if (w >= nheavy) {
+        shared_phase = false;
+        continue;
+      }
+    } else {
+      if (threadIdx.x == 0) s_work = nheavy + atomicAdd(counters, 1);
+      __syncthreads();
+      w = s_work;
+      __syncthreads();
+      if (w >= nstates) break;
+    }
     const BatchState st = states[order[w]];
     T2* g = pool + st.offset;
-    const uint32_t dim = 1u << st.nq;
-    if (st.nq <= smem_qubits) {
+    if (parts == 1 && st.nq <= smem_qubits) {
+      const uint32_t dim = 1u << st.nq;
       for (uint32_t i = threadIdx.x; i < dim; i += blockDim.x) sm[i] = SM::in(g[i]);
-      if (st.nops > 0) load_consts<T2>(ops[st.first_op], consts, s_k[0]);
+      if (st.nops > 0) load_consts<T2>(ops[st.first_op], consts, sh.k[0]);
       __syncthreads();
       for (int k = 0; k < st.nops; ++k) {
-        apply_op<WIDE>(sm, st.nq, ops[st.first_op + k], s_k[k & 1]);
-        if (k + 1 < st.nops) load_consts<T2>(ops[st.first_op + k + 1], consts, s_k[(k + 1) & 1]);
+        apply_op<WIDE>(sm, st.nq, ops[st.first_op + k], sh.k[k & 1], threadIdx.x, blockDim.x);
+        if (k + 1 < st.nops) load_consts<T2>(ops[st.first_op + k + 1], consts, sh.k[(k + 1) & 1]);
         __syncthreads();
       }
       for (uint32_t i = threadIdx.x; i < dim; i += blockDim.x) g[i] = SM::out(sm[i]);
       __syncthreads();
       continue;
     }
-    for (int sg = st.first_seg; sg < st.first_seg + st.nsegs; ++sg) {
-      const BatchSeg S = segs[sg];
-      if (S.L == 0) {
-        load_consts<T2>(ops[S.first_op], consts, s_k[0]);
+    run_segments<WIDE>(g, st, ops, consts, segs, xlat, sm, sh, part, parts, [&]() {
+      if (CL && parts > 1)
+        cg::this_cluster().sync();
+      else
         __syncthreads();
-        for (int k = 0; k < S.nops; ++k) {
-          apply_op<WIDE>(g, st.nq, ops[S.first_op + k], s_k[k & 1]);
-          if (k + 1 < S.nops) load_consts<T2>(ops[S.first_op + k + 1], consts, s_k[(k + 1) & 1]);
-          __syncthreads();
-        }
-        continue;
-      }
-      const int L = S.L, hi = L - 7;                  // 8 <= L <= 14
-      uint32_t qmask = 0;
-      for (int b = 0; b < L; ++b) qmask |= 1u << S.q[b];
-      for (int j = threadIdx.x; j < 128; j += blockDim.x) {
-        uint32_t tl = 0, th = 0;
-        for (int b = 0; b < 7; ++b)
-          if ((j >> b) & 1) tl |= 1u << S.q[b];
-        for (int b = 0; b < hi; ++b)
-          if ((j >> b) & 1) th |= 1u << S.q[7 + b];
-        s_tl[j] = tl;
-        s_th[j] = th;
-      }
-      __syncthreads();
-      const uint32_t fmask = (dim - 1) & ~qmask;       // the other qubits: the tile number, deposited
-      const uint32_t ntiles = dim >> L, tdim = 1u << L;
-      for (uint32_t tile = 0; tile < ntiles; ++tile) {
-        uint32_t base = 0;
-        {
-          uint32_t m = fmask, t = tile;
-          while (m) {
-            const uint32_t low = m & (~m + 1u);
-            if (t & 1u) base |= low;
-            m ^= low;
-            t >>= 1;
-          }
-        }
-        for (uint32_t i = threadIdx.x; i < tdim; i += blockDim.x)
-          sm[i] = SM::in(g[base | s_tl[i & 127u] | s_th[i >> 7]]);
-        load_consts<T2>(ops[S.first_op], consts, s_k[0]);
-        __syncthreads();
-        for (int k = 0; k < S.nops; ++k) {
-          apply_tile_op<WIDE>(sm, L, ops[S.first_op + k], xlat[S.first_op + k], base, s_k[k & 1]);
-          if (k + 1 < S.nops) load_consts<T2>(ops[S.first_op + k + 1], consts, s_k[(k + 1) & 1]);
-          __syncthreads();
-        }
-        for (uint32_t i = threadIdx.x; i < tdim; i += blockDim.x)
-          g[base | s_tl[i & 127u] | s_th[i >> 7]] = SM::out(sm[i]);
-        __syncthreads();
-      }
-    }
+    });
   }
 }
 
+namespace {
+template <typename T2>
+const void* batch_kernel(bool wide, bool cl) {
+  if (wide) return cl ? (const void*)k_batch<T2, true, true> : (const void*)k_batch<T2, true, false>;
+  return cl ? (const void*)k_batch<T2, false, true> : (const void*)k_batch<T2, false, false>;
+}
+const void* batch_kernel(qs_prec prec, bool wide, bool cl) {
+  return prec == QS_C128 ? batch_kernel<double2>(wide, cl) : batch_kernel<float2>(wide, cl);
+}
+size_t batch_smem(qs_prec prec, int smem_qubits) {
+  return (smem_qubits >= 0 ? (size_t(1) << smem_qubits) : 0) * (prec == QS_C128 ? 16 : 8);
+}
+void batch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int threads, int ctas, size_t smem, int cluster,
+                  cudaStream_t st) {
+  cfg = cudaLaunchConfig_t{};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)cluster;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+}
+}  // namespace
+
 cudaError_t batch_set_max_smem(int bytes) {
-  for (const void* f : {(const void*)k_batch<double2, false>, (const void*)k_batch<double2, true>,
-                        (const void*)k_batch<float2, false>, (const void*)k_batch<float2, true>}) {
-    const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-  }
+  for (qs_prec prec : {QS_C64, QS_C128})
+    for (int v = 0; v < 4; ++v) {
+      const cudaError_t e = cudaFuncSetAttribute(batch_kernel(prec, v & 1, v & 2),
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+      if (e != cudaSuccess) return e;
+    }
   return cudaSuccess;
 }
 
+// Clusters of `cluster` CTAs that are resident at once.
+cudaError_t batch_max_clusters(qs_prec prec, int threads, int smem_qubits, int wide, int cluster, int* n) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  batch_config(cfg, &attr, threads, cluster, batch_smem(prec, smem_qubits), cluster, nullptr);
+  return cudaOccupancyMaxActiveClusters(n, batch_kernel(prec, wide != 0, true), &cfg);
+}
+
 // No attribute calls here: this launch is also recorded into a CUDA graph.
-cudaError_t launch_batch(qs_prec prec, void* pool, const BatchState* states, const int* order, int nstates,
+// counters: two zeroed ints; ctas a multiple of cluster (1: no clusters, nheavy 0).
+cudaError_t launch_batch(qs_prec prec, void* pool, const BatchState* states, const int* order, int nstates, int nheavy,
                          const BatchOp* ops, const double* consts, const BatchSeg* segs, const BatchXlat* xlat,
-                         int* counter, int threads, int ctas, int smem_qubits, int wide, cudaStream_t st) {
-  const size_t smem = (smem_qubits >= 0 ? (size_t(1) << smem_qubits) : 0) * (prec == QS_C128 ? 16 : 8);
-  double2* p128 = static_cast<double2*>(pool);
-  float2* p64 = static_cast<float2*>(pool);
-  if (prec == QS_C128 && wide)
-    k_batch<double2, true><<<ctas, threads, smem, st>>>(p128, states, order, nstates, ops, consts, segs, xlat, counter,
-                                                        smem_qubits);
-  else if (prec == QS_C128)
-    k_batch<double2, false><<<ctas, threads, smem, st>>>(p128, states, order, nstates, ops, consts, segs, xlat,
-                                                         counter, smem_qubits);
-  else if (wide)
-    k_batch<float2, true><<<ctas, threads, smem, st>>>(p64, states, order, nstates, ops, consts, segs, xlat, counter,
-                                                       smem_qubits);
-  else
-    k_batch<float2, false><<<ctas, threads, smem, st>>>(p64, states, order, nstates, ops, consts, segs, xlat, counter,
-                                                        smem_qubits);
-  return cudaGetLastError();
+                         int* counters, int threads, int ctas, int smem_qubits, int wide, int cluster, cudaStream_t st) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr;
+  batch_config(cfg, &attr, threads, ctas, batch_smem(prec, smem_qubits), cluster, st);
+  void* args[] = {&pool, &states, &order, &nstates, &nheavy, &ops, &consts, &segs, &xlat, &counters, &smem_qubits};
+  const cudaError_t e = cudaLaunchKernelExC(&cfg, batch_kernel(prec, wide != 0, cluster > 1), args);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace qsk

@@ -74,13 +74,13 @@ inline qsk::BatchXlat translate(const qsk::BatchOp& op, uint32_t qmask) {
   return x;
 }
 
-// Segments of every state larger than 2^L amplitudes (states[s].first_seg and
-// nsegs are set; xlat gets one entry per operation).  Greedy: an operation
+// Segments of every state larger than 2^Ls[s] amplitudes, its tile size
+// (states[s].first_seg and nsegs are set; xlat gets one entry per operation).  Greedy: an operation
 // joins the open segment while the union of pairing qubits and the five
 // lowest qubits stays within L; an operation that alone exceeds it runs in
 // global memory (a segment with L = 0).  The tile qubits are that union,
 // filled up with the lowest remaining qubits.
-inline void build_segments(int L, const std::vector<int>& nq, std::vector<qsk::BatchState>& states,
+inline void build_segments(const std::vector<int>& Ls, const std::vector<int>& nq, std::vector<qsk::BatchState>& states,
                            const std::vector<qsk::BatchOp>& ops, std::vector<qsk::BatchSeg>& segs,
                            std::vector<qsk::BatchXlat>& xlat) {
   segs.clear();
@@ -89,6 +89,7 @@ inline void build_segments(int L, const std::vector<int>& nq, std::vector<qsk::B
     qsk::BatchState& st = states[s];
     st.first_seg = (int)segs.size();
     st.nsegs = 0;
+    const int L = Ls[s];
     if (nq[s] <= L) continue;
     const uint32_t low = (1u << std::min(5, nq[s])) - 1u;
     auto emit = [&](int first, int n, uint32_t U, bool tiled) {
@@ -129,6 +130,21 @@ inline void build_segments(int L, const std::vector<int>& nq, std::vector<qsk::B
     if (cnt) emit(k0, cnt, U, true);
     st.nsegs = (int)segs.size() - st.first_seg;
   }
+}
+
+// One tile size for every state.
+inline void build_segments(int L, const std::vector<int>& nq, std::vector<qsk::BatchState>& states,
+                           const std::vector<qsk::BatchOp>& ops, std::vector<qsk::BatchSeg>& segs,
+                           std::vector<qsk::BatchXlat>& xlat) {
+  build_segments(std::vector<int>(nq.size(), L), nq, states, ops, segs, xlat);
+}
+
+// Relative cost of an operation per amplitude of its state, for the order and
+// the split of the work: a dense update on n targets does 2^n multiply-adds per
+// amplitude that the controls leave, on top of moving it.
+inline double op_cost(const qsk::BatchOp& op) {
+  if (op.kind != 0) return 1.0;
+  return (0.5 + 0.5 * (1 << op.n)) / (1u << popc32(op.ctrl));
 }
 
 // ---- superoperators on the Choi vector (Sec. "Kraus map") -------------------

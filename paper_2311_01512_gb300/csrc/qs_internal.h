@@ -389,9 +389,10 @@ cudaError_t launch_mlp_adam(float* params, const float* grad, float* m, float* v
                             cudaStream_t st);
 int num_sms();  // multiprocessors of the current device (cached)
 cudaError_t batch_set_max_smem(int bytes);
-cudaError_t launch_batch(qs_prec prec, void* pool, const BatchState* states, const int* order, int nstates,
+cudaError_t batch_max_clusters(qs_prec prec, int threads, int smem_qubits, int wide, int cluster, int* n);
+cudaError_t launch_batch(qs_prec prec, void* pool, const BatchState* states, const int* order, int nstates, int nheavy,
                          const BatchOp* ops, const double* consts, const BatchSeg* segs, const BatchXlat* xlat,
-                         int* counter, int threads, int ctas, int smem_qubits, int wide, cudaStream_t st);
+                         int* counters, int threads, int ctas, int smem_qubits, int wide, int cluster, cudaStream_t st);
 cudaError_t launch_group(qs_prec prec, void* amps, int op, const GroupParams& p, cudaStream_t st);
 // complex128 channels in double-float arithmetic: G_DEPOL1, G_DEPOL2, G_DAMP, G_PAULI1 (qs_gates_df.cu)
 cudaError_t launch_group_df(void* amps, int op, const GroupParams& p, cudaStream_t st);
