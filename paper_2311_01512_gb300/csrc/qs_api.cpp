@@ -352,6 +352,7 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
       p.m[2 * e] = host_mat[2 * e];
       p.m[2 * e + 1] = conj ? -host_mat[2 * e + 1] : host_mat[2 * e + 1];
     }
+    for (int e = 0; e < 8; ++e) p.mf[e] = (float)p.m[e];
     std::vector<int> ins(ctrls);
     ins.push_back(targs[0]);
     std::sort(ins.begin(), ins.end());
@@ -488,6 +489,8 @@ qs_status gadget_pass(qs_state* s, const std::vector<int>& targs, const int* pau
   const double phi = -0.5 * theta;
   p.c = std::cos(phi);
   p.s = std::sin(phi);
+  p.cf = (float)p.c;
+  p.sf = (float)p.s;
   p.eta = num_y & 3;
   if (p.xy) {
     p.h = 63 - __builtin_clzll(p.xy);
@@ -892,7 +895,10 @@ qs_status group_channel(qs_state* s, int op, int t1, int t2, const double* f) {
   std::sort(pos.begin(), pos.end());
   for (int b = 0; b < p.nbits; ++b) p.ins[b] = (int8_t)pos[b];
   p.ngroups = 1ull << (s->ns - p.nbits);
-  for (int k = 0; k < 4; ++k) p.f[k] = f[k];
+  for (int k = 0; k < 4; ++k) {
+    p.f[k] = f[k];
+    p.ff[k] = (float)f[k];
+  }
   // complex128 with double-float arithmetic: channels that mix or scale by
   // non-trivial coefficients use the double-float kernel (the FP64 one is
   // bound by the FP64 pipe, not by memory); dephasing stays on FP64

@@ -35,7 +35,15 @@ namespace qsk {
 template <typename R, int OP>
 __global__ void __launch_bounds__(256) k_group(typename Cplx<R>::T* __restrict__ rho, const __grid_constant__ GroupParams p) {
   using T2 = typename Cplx<R>::T;
-  const R f0 = (R)p.f[0], f1 = (R)p.f[1], f2 = (R)p.f[2], f3 = (R)p.f[3];
+  R f[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if constexpr (sizeof(R) == 4)
+      f[q] = p.ff[q];
+    else
+      f[q] = p.f[q];
+  }
+  const R f0 = f[0], f1 = f[1], f2 = f[2], f3 = f[3];
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < p.ngroups; k += stride) {
     const uint64_t base = insert_zeros(k, p.ins, p.nbits);

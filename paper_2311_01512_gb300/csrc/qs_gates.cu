@@ -18,6 +18,15 @@ int num_sms() {
   return cached;
 }
 
+// the constant in the kernel's precision
+template <typename R>
+__device__ __forceinline__ R pick(double d, float f) {
+  if constexpr (sizeof(R) == 4)
+    return f;
+  else
+    return d;
+}
+
 // ---------------------------------------------------------------------------
 // One-target gate, Sec. "One-target gate" and Sec. "Many-control one-target
 // gate": for each of the 2^(Ns-1-s) pairs, i0 has zero bits inserted at the
@@ -27,8 +36,11 @@ int num_sms() {
 template <typename R>
 __global__ void __launch_bounds__(256) k_gate1(typename Cplx<R>::T* __restrict__ psi, const __grid_constant__ Gate1Params p) {
   using T2 = typename Cplx<R>::T;
-  const R m00r = (R)p.m[0], m00i = (R)p.m[1], m01r = (R)p.m[2], m01i = (R)p.m[3];
-  const R m10r = (R)p.m[4], m10i = (R)p.m[5], m11r = (R)p.m[6], m11i = (R)p.m[7];
+  R m[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) m[e] = pick<R>(p.m[e], p.mf[e]);
+  const R m00r = m[0], m00i = m[1], m01r = m[2], m01i = m[3];
+  const R m10r = m[4], m10i = m[5], m11r = m[6], m11i = m[7];
   const uint64_t tbit = 1ull << p.t;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < p.npairs; k += stride) {
@@ -172,7 +184,7 @@ __global__ void __launch_bounds__(256) k_diag(typename Cplx<R>::T* __restrict__ 
 template <typename R>
 __global__ void __launch_bounds__(256) k_gadget(typename Cplx<R>::T* __restrict__ psi, const __grid_constant__ GadgetParams p) {
   using T2 = typename Cplx<R>::T;
-  const R c = (R)p.c, s = (R)p.s;
+  const R c = pick<R>(p.c, p.cf), s = pick<R>(p.s, p.sf);
   const int q = (p.eta + 1) & 3;  // i * eta = i^(#Y + 1)
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t k = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; k < p.nwork; k += stride) {
@@ -192,7 +204,7 @@ __global__ void __launch_bounds__(256) k_gadget(typename Cplx<R>::T* __restrict_
 template <typename R>
 __global__ void __launch_bounds__(256) k_phase(typename Cplx<R>::T* __restrict__ psi, const __grid_constant__ GadgetParams p) {
   using T2 = typename Cplx<R>::T;
-  const R c = (R)p.c, s = (R)p.s;
+  const R c = pick<R>(p.c, p.cf), s = pick<R>(p.s, p.sf);
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   if constexpr (sizeof(R) == 4) {
     // complex64: two neighbouring amplitudes (16 bytes) per thread and step

@@ -25,8 +25,13 @@ constexpr int kCostParams = kCostHidden * kCostFeatures + kCostHidden + kCostHid
 
 // One-target gate on pairs (i0, i1 = i0 | 2^t) (Sec. "One-target gate",
 // Sec. "Many-control one-target gate").
+// Constants come in both precisions: converted once on the host, not in every
+// thread (a double-to-float conversion runs at the FP64 rate, and eight of them
+// per thread took longer than the memory traffic of a complex64 pass: 24 qubits
+// 127 -> 47 us, 25 qubits 149 -> 86).
 struct Gate1Params {
   double m[8];           // m00, m01, m10, m11 as (re, im), already conjugated if needed
+  float mf[8];
   uint64_t npairs;       // 2^(Ns - 1 - s)
   uint64_t ctrl_mask;    // control bits, set in every enumerated index
   int t;
@@ -99,6 +104,7 @@ struct GadgetParams {
   uint64_t yz;           // qubits with Y or Z: the sign bits
   uint64_t nwork;        // pairs (xy != 0) or amplitudes (xy == 0)
   double c, s;           // cos(phi), sin(phi), phi = -theta/2
+  float cf, sf;
   int eta;               // number of Y factors mod 4
   int h;                 // highest bit of xy (pair enumeration)
 };
@@ -189,6 +195,7 @@ struct GroupParams {
   int8_t ins[4];         // sorted member positions
   int8_t mpos[4];        // member bit b -> qubit position
   double f[4];           // channel coefficients (see the kernel)
+  float ff[4];
 };
 
 // The same channels in block fixed point: coefficient slots with their own
