@@ -265,6 +265,25 @@ constexpr int kSmallDenseBits[6] = {0, 0, 20, 19, 17, 17};
 // (10.5), 5 targets 2^14 13.3 (19.8) and 2^16 50.
 constexpr int kSmallDigitBits[6] = {0, 0, 16, 16, 14, 14};
 
+// Whether a dense pass of n targets and nctrl controls runs off the tensor cores
+// because it covers few amplitudes, and on which kernel: complex128, 2..5
+// targets.  Density matrices in block fixed point keep the arithmetic that these
+// passes had on the tensor cores (digits).
+enum SmallRoute { SMALL_NO, SMALL_FX, SMALL_DIGITS };
+SmallRoute small_route(const qs_state* s, int n, int nctrl) {
+  const int nfree = s->ns - n - nctrl;
+  if (s->prec != QS_C128 || s->arith == QS_ARITH_F64 || !s->tensor_cores || n < 2 || n > 5 || (n == 2 && nfree < 1))
+    return SMALL_NO;
+  const bool digits = s->is_density && s->arith == QS_ARITH_FX;
+  if (nfree + n > (digits ? kSmallDigitBits : kSmallDenseBits)[n]) return SMALL_NO;
+  return digits ? SMALL_DIGITS : SMALL_FX;
+}
+
+// Whether gate_pass reads the matrix from device memory (it takes the host's otherwise).
+bool needs_device_matrix(const qs_state* s, int n, int nctrl) {
+  return n > 1 && !(n == 2 && is_fx(s)) && small_route(s, n, nctrl) == SMALL_NO;
+}
+
 // One dense or one-target gate pass on storage positions (already shifted).
 qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vector<int>& targs, const double* host_mat,
                     const void* dev_mat, int conj, bool force_dense) {
@@ -373,11 +392,8 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
   // complex128 off the FP64 pipe: exact byte slices (55-bit amplitudes)
   const bool tc128 = s->prec == QS_C128 && (s->arith == QS_ARITH_DF || s->arith == QS_ARITH_FX) &&
                      s->tensor_cores && (tc_n || n == 6);
-  // complex128 passes over few amplitudes, 2..5 targets: off the tensor cores
-  // (density matrices in block fixed point keep the arithmetic that these
-  // passes had there)
-  const bool digits = s->is_density && s->arith == QS_ARITH_FX;
-  if (tc128 && n <= 5 && nfree + n <= (digits ? kSmallDigitBits : kSmallDenseBits)[n]) {
+  if (const SmallRoute route = small_route(s, n, (int)ctrls.size())) {
+    const bool digits = route == SMALL_DIGITS;
     qsk::DenseFxParams p{};
     p.mat = static_cast<const double*>(dev_mat);
     p.conj = conj;
@@ -394,8 +410,9 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
     p.nins = (int)ins.size();
     for (int q = 0; q < p.nins; ++q) p.ins[q] = (int8_t)ins[q];
     p.ngroups = 1ull << (s->ns - p.nins);
-    return cuda_status(digits ? qsk::launch_dense_digits(s->amps, p, s->stream)
-                              : qsk::launch_dense_fx(s->amps, p, s->stream));
+    const double* hm = dev_mat ? nullptr : host_mat;
+    return cuda_status(digits ? qsk::launch_dense_digits(s->amps, p, hm, s->stream)
+                              : qsk::launch_dense_fx(s->amps, p, hm, s->stream));
   }
   if (tc64 || tc128) {
     std::vector<int> kt(targs);
@@ -529,13 +546,22 @@ qs_status gadget_pass(qs_state* s, const std::vector<int>& targs, const int* pau
   return cuda_status(qsk::launch_gadget(s->prec, s->amps, p, s->stream));
 }
 
-// S = sum_m conj(K_m) (x) K_m of n-qubit operators in device memory (FP64, on the
-// device), applied as one 2n-target pass on t u (t + N): matrix bit q on t[q], bit
+// Two-qubit maps of at most this many operators (a channel needs no more than 16)
+// on small states have their 256 entries formed on the host, some microseconds.
+constexpr int kHostSuperopOps = 16;
+
+// S = sum_m conj(K_m) (x) K_m of n-qubit operators (FP64, on the device except for
+// small states), applied as one 2n-target pass on t u (t + N): matrix bit q on t[q], bit
 // n + q on t[q] + N (Sec. "Kraus map").  While recording, S is formed once on the
 // program's side stream, outside the capture: its operators are constants of the
 // program, and a replay then takes one launch instead of two.
 qs_status superop_pass(qs_state* s, const std::vector<int>& t, const double* kraus, int num_ops) {
   const int n = (int)t.size();
+  if (n == 2 && num_ops <= kHostSuperopOps && !needs_device_matrix(s, 4, 0)) {
+    double sup[512];
+    qsh::superop2(kraus, num_ops, sup);
+    return gate_pass(s, {}, {t[0], t[1], t[0] + s->nq, t[1] + s->nq}, sup, nullptr, 0);
+  }
   const size_t kbytes = sizeof(double) * 2 * (size_t(1) << (2 * n)) * (size_t)num_ops;
   const void* dk = nullptr;
   void* dsup = nullptr;
@@ -743,7 +769,7 @@ qs_status qs_apply_ctrl_multi_target(qs_state* s, const int* ctrls, int nctrl, c
   const size_t mat_bytes = sizeof(double) * 2 * (size_t(1) << (2 * ntarg));
   const void* dmat = nullptr;
   int slot = -1;
-  if (ntarg > 1) {
+  if (needs_device_matrix(s, ntarg, nctrl)) {
     st = ring_put(s, mat, mat_bytes, &dmat, &slot);
     if (st != QS_OK) return st;
   }

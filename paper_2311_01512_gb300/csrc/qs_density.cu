@@ -161,8 +161,8 @@ __global__ void k_superop(const double* __restrict__ kraus, int num_ops, int n, 
     const double* km = kraus + (size_t)2 * m * d2;
     const double ar = km[2 * (i * d + j)], ai = -km[2 * (i * d + j) + 1];  // conj(K[i, j])
     const double br = km[2 * (k * d + l)], bi = km[2 * (k * d + l) + 1];   // K[k, l]
-    sr += ar * br - ai * bi;
-    si += ar * bi + ai * br;
+    sr += fma(ar, br, -(ai * bi));   // in this form on the host too (qs_superop1.h)
+    si += fma(ar, bi, ai * br);
   }
   sup[2 * e] = sr;
   sup[2 * e + 1] = si;

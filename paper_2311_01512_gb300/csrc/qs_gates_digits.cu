@@ -20,6 +20,8 @@
 // Why: on 4096 amplitudes the tensor-core kernel ran two tiles on two SMs behind
 // a setup that slices the whole matrix.  4096 amplitudes, four targets, us a
 // pass in a replayed program: 10.9 -> 4.3.
+#include <cstring>
+
 #include "qs_device.cuh"
 #include "qs_slices.cuh"
 
@@ -55,9 +57,10 @@ struct DigitSmem {
 
 }  // namespace
 
-template <int NT>
+template <int NT, typename Mat>
 __global__ void __launch_bounds__(kDigitThreads) k_dense_digits(double2* __restrict__ psi,
-                                                                const __grid_constant__ DenseFxParams p) {
+                                                                const __grid_constant__ DenseFxParams p,
+                                                                const __grid_constant__ Mat mat) {
   using S = DigitSmem<NT>;
   constexpr int D = S::D;
   extern __shared__ __align__(16) float sm[];
@@ -81,7 +84,7 @@ __global__ void __launch_bounds__(kDigitThreads) k_dense_digits(double2* __restr
     m[e] = make_double2(0.0, 0.0);
     // an identity on the targets beyond the stored matrix
     if (idx < D * D && (row >> p.nmat) == (l >> p.nmat))
-      m[e] = reinterpret_cast<const double2*>(p.mat)[((row & mm) << p.nmat) + (l & mm)];
+      m[e] = mat.m[((row & mm) << p.nmat) + (l & mm)];
     if (p.conj) m[e].y = -m[e].y;
   }
   for (int n = tid; n < D; n += kDigitThreads) cexp[n] = kExpFloor;
@@ -138,25 +141,33 @@ __global__ void __launch_bounds__(kDigitThreads) k_dense_digits(double2* __restr
   if (ok) reinterpret_cast<double*>(psi)[2 * i + c] = o;
 }
 
-template <int NT>
-static cudaError_t dense_digits(void* amps, const DenseFxParams& p, cudaStream_t st) {
+template <int NT, typename Mat>
+static cudaError_t dense_digits(void* amps, const DenseFxParams& p, const Mat& mat, cudaStream_t st) {
   static bool attr_done = false;
   if (!attr_done) {
-    const cudaError_t e = cudaFuncSetAttribute(k_dense_digits<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaError_t e = cudaFuncSetAttribute(k_dense_digits<NT, Mat>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)DigitSmem<NT>::bytes);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
   const unsigned g = (unsigned)((p.ngroups + DigitSmem<NT>::G - 1) / DigitSmem<NT>::G);
-  k_dense_digits<NT><<<g, kDigitThreads, DigitSmem<NT>::bytes, st>>>(static_cast<double2*>(amps), p);
+  k_dense_digits<NT, Mat><<<g, kDigitThreads, DigitSmem<NT>::bytes, st>>>(static_cast<double2*>(amps), p, mat);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dense_digits(void* amps, const DenseFxParams& p, cudaStream_t st) {
+template <int NT>
+static cudaError_t dense_digits_n(void* amps, const DenseFxParams& p, const double* host_mat, cudaStream_t st) {
+  if (!host_mat) return dense_digits<NT>(amps, p, MatPtr{reinterpret_cast<const double2*>(p.mat)}, st);
+  MatArg<NT> m;
+  std::memcpy(&m, host_mat, sizeof(double2) << (2 * p.nmat));
+  return dense_digits<NT>(amps, p, m, st);
+}
+
+cudaError_t launch_dense_digits(void* amps, const DenseFxParams& p, const double* host_mat, cudaStream_t st) {
   switch (p.n) {
-    case 3: return dense_digits<3>(amps, p, st);
-    case 4: return dense_digits<4>(amps, p, st);
-    case 5: return dense_digits<5>(amps, p, st);
+    case 3: return dense_digits_n<3>(amps, p, host_mat, st);
+    case 4: return dense_digits_n<4>(amps, p, host_mat, st);
+    case 5: return dense_digits_n<5>(amps, p, host_mat, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -3,6 +3,8 @@
 // double.  Same operations and index enumeration as qs_gates.cu and
 // qs_density.cu: one- and two-target gates with controls, diagonals, Pauli
 // and phase gadgets, and the density-matrix channels that mix amplitudes.
+#include <cstring>
+
 #include "qs_device.cuh"
 #include "qs_fx.cuh"
 
@@ -166,8 +168,9 @@ __global__ void __launch_bounds__(256) k_gate2_fx(double2* __restrict__ psi, con
 // replayed program: 2 targets (fused block) 9.3 -> 1.7, 3 targets 9.1 -> 2.0, 4
 // targets 10.9 -> 2.7, 5 targets 19.6 -> 4.9.
 // ---------------------------------------------------------------------------
-template <int NT>
-__global__ void __launch_bounds__(128) k_dense_fx(double2* __restrict__ psi, const __grid_constant__ DenseFxParams p) {
+template <int NT, typename Mat>
+__global__ void __launch_bounds__(128) k_dense_fx(double2* __restrict__ psi, const __grid_constant__ DenseFxParams p,
+                                                  const __grid_constant__ Mat mat) {
   constexpr int D = 1 << NT, SH = NT - 2;
   __shared__ int4 cm[D * D];                  // entry (j, k) at k D + j: parts of re and im
   __shared__ int em[D];                       // largest biased exponent of a row
@@ -187,7 +190,7 @@ __global__ void __launch_bounds__(128) k_dense_fx(double2* __restrict__ psi, con
 #pragma unroll
   for (int e = 0; e < EPT; ++e) {
     const int idx = tid + 128 * e;
-    m[e] = idx < D * D ? reinterpret_cast<const double2*>(p.mat)[idx] : make_double2(0.0, 0.0);
+    m[e] = idx < D * D ? mat.m[idx] : make_double2(0.0, 0.0);
     if (p.conj) m[e].y = -m[e].y;
     if (idx < D * D) atomicMax(em + idx / D, max(qsfx::expo_of(m[e].x), qsfx::expo_of(m[e].y)));
   }
@@ -468,14 +471,25 @@ cudaError_t launch_gate2_fx(void* amps, const Gate2FxParams& p, cudaStream_t st)
   return cudaGetLastError();
 }
 
-cudaError_t launch_dense_fx(void* amps, const DenseFxParams& p, cudaStream_t st) {
-  const unsigned g = (unsigned)((p.ngroups * (1u << p.n) + 127) / 128);
+template <int NT>
+static void dense_fx(double2* a, const DenseFxParams& p, const double* host_mat, cudaStream_t st) {
+  const unsigned g = (unsigned)(((p.ngroups << NT) + 127) / 128);
+  if (host_mat) {
+    MatArg<NT> m;
+    std::memcpy(&m, host_mat, sizeof(m));
+    k_dense_fx<NT, MatArg<NT>><<<g, 128, 0, st>>>(a, p, m);
+  } else {
+    k_dense_fx<NT, MatPtr><<<g, 128, 0, st>>>(a, p, MatPtr{reinterpret_cast<const double2*>(p.mat)});
+  }
+}
+
+cudaError_t launch_dense_fx(void* amps, const DenseFxParams& p, const double* host_mat, cudaStream_t st) {
   double2* a = static_cast<double2*>(amps);
   switch (p.n) {
-    case 2: k_dense_fx<2><<<g, 128, 0, st>>>(a, p); break;
-    case 3: k_dense_fx<3><<<g, 128, 0, st>>>(a, p); break;
-    case 4: k_dense_fx<4><<<g, 128, 0, st>>>(a, p); break;
-    case 5: k_dense_fx<5><<<g, 128, 0, st>>>(a, p); break;
+    case 2: dense_fx<2>(a, p, host_mat, st); break;
+    case 3: dense_fx<3>(a, p, host_mat, st); break;
+    case 4: dense_fx<4>(a, p, host_mat, st); break;
+    case 5: dense_fx<5>(a, p, host_mat, st); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

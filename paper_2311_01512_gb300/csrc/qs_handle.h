@@ -50,8 +50,9 @@ qs_status ring_put(qs_state* s, const void* host, size_t bytes, const void** dev
 qs_status ring_take(qs_state* s, size_t bytes, void** dev, int* slot);
 qs_status ring_done(qs_state* s, int slot);
 // One dense-gate pass on storage positions (already shifted for the conjugate
-// pass of a density matrix).  host_mat is needed only for one-target gates
-// unless force_dense; dev_mat (complex128, row-major) for more targets.
+// pass of a density matrix).  The matrix (complex128, row-major) is host_mat for one
+// target unless force_dense, and for what needs_device_matrix leaves out; dev_mat
+// for the rest, and for any pass of two and more targets.
 qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vector<int>& targs, const double* host_mat,
                     const void* dev_mat, int conj, bool force_dense = false);
 qs_status gadget_pass(qs_state* s, const std::vector<int>& targs, const int* paulis, double theta);

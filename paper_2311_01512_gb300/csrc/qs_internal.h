@@ -154,7 +154,7 @@ struct Gate2FxParams {
 // Dense gate on 2..5 targets of a small state (k_dense_fx, k_dense_digits):
 // groups of 2^n amplitudes base | target bits.
 struct DenseFxParams {
-  const double* mat;     // device, 2^n x 2^n complex128 row-major (re, im)
+  const double* mat;     // device, 2^nmat x 2^nmat complex128 row-major (re, im); not used with a host matrix
   uint64_t ngroups;
   uint64_t ctrl_mask;
   int n;                 // targets of the kernel
@@ -163,6 +163,19 @@ struct DenseFxParams {
   int nins;
   int8_t tpos[kMaxDense];
   int8_t ins[kMaxQ];     // sorted targets and controls
+};
+
+// The matrix as a kernel argument of its own: a device pointer, or the entries
+// themselves (at most 16 KB).  A small state's pass with its matrix in the
+// arguments needs no copy before it: measured at 2^10 amplitudes, us a call, with
+// the copy / without: 3 targets 7.0 / 3.4, 4 targets 11.5 / 3.7, 5 targets 12.6 /
+// 9.1; two-qubit Kraus map of four operators (host superoperator) 16.9 / 4.4.
+struct MatPtr {
+  const double2* m;
+};
+template <int N>
+struct MatArg {
+  double2 m[1 << (2 * N)];
 };
 
 // Diagonal entry d_j: parts of Re, Im and -Im with their shared exponent.
@@ -369,10 +382,10 @@ cudaError_t launch_gadget_df(void* amps, const GadgetDfParams& p, cudaStream_t s
 // complex128 in block fixed point (qs_gates_fx.cu)
 cudaError_t launch_gate1_fx(void* amps, const Gate1FxParams& p, cudaStream_t st);
 cudaError_t launch_gate2_fx(void* amps, const Gate2FxParams& p, cudaStream_t st);
-// 2 <= n <= 5 targets
-cudaError_t launch_dense_fx(void* amps, const DenseFxParams& p, cudaStream_t st);
+// 2 <= n <= 5 targets; host_mat: the matrix, if it is not at p.mat
+cudaError_t launch_dense_fx(void* amps, const DenseFxParams& p, const double* host_mat, cudaStream_t st);
 // small density matrices, 3 <= n <= 5 kernel targets (qs_gates_digits.cu)
-cudaError_t launch_dense_digits(void* amps, const DenseFxParams& p, cudaStream_t st);
+cudaError_t launch_dense_digits(void* amps, const DenseFxParams& p, const double* host_mat, cudaStream_t st);
 cudaError_t launch_diag_fx(void* amps, const DiagFxParams& p, cudaStream_t st);
 cudaError_t launch_gadget_fx(void* amps, const GadgetFxParams& p, cudaStream_t st);
 // G_DEPOL1, G_DEPOL2, G_DAMP, G_PAULI1

@@ -1,7 +1,9 @@
-// Superoperator of a one-qubit Kraus map, formed on the host (no CUDA
+// Superoperators of one- and two-qubit Kraus maps, formed on the host (no CUDA
 // dependency, so the host check tests/host/superop1_check.cpp compiles it
 // with g++ alone).
 #pragma once
+
+#include <cmath>
 
 namespace qsh {
 
@@ -22,6 +24,28 @@ inline void superop1(const double* kraus, int num_ops, double* sup) {
         sup[2 * (4 * r + c)] += ar * br - ai * bi;
         sup[2 * (4 * r + c) + 1] += ar * bi + ai * br;
       }
+  }
+}
+
+// The same of two-qubit operators (4x4) as a 16x16 matrix, row 4 i + k, column
+// 4 j + l, with the operations of the device superoperator kernel one by one (a
+// fused multiply-add on a product, operators added in order), so that both
+// give the same bits.  sup: 512 doubles (256 complex, row-major).
+inline void superop2(const double* kraus, int num_ops, double* sup) {
+  for (int e = 0; e < 512; ++e) sup[e] = 0.0;
+  for (int m = 0; m < num_ops; ++m) {
+    const double* K = kraus + 32 * m;
+    for (int i = 0; i < 4; ++i)
+      for (int k = 0; k < 4; ++k)
+        for (int j = 0; j < 4; ++j) {
+          const double ar = K[2 * (4 * i + j)], ai = -K[2 * (4 * i + j) + 1];
+          double* out = sup + 2 * (16 * (4 * i + k) + 4 * j);
+          for (int l = 0; l < 4; ++l) {
+            const double br = K[2 * (4 * k + l)], bi = K[2 * (4 * k + l) + 1];
+            out[2 * l] += std::fma(ar, br, -(ai * bi));
+            out[2 * l + 1] += std::fma(ar, bi, ai * br);
+          }
+        }
   }
 }
 

@@ -122,3 +122,30 @@ def test_density_matrix_passes(nq):
     got = st.get_amps()
     st.close()
     assert np.max(np.abs(got - orc.run_ops(rho, ops, is_density=True))) < 1e-14
+
+
+@pytest.mark.parametrize("arith", ["fx", "df"])
+@pytest.mark.parametrize("nq", [2, 4, 7, 8])
+def test_two_qubit_superoperator_host_and_device(nq, arith):
+    """Kraus maps of at most 16 operators on small states have their superoperator
+    formed on the host, the same map with zero operators appended on the device:
+    the same operations, hence equal results; and the map against the oracle."""
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(1600 + nq)
+    states, w = wl.random_mixed_state_vectors(nq, 3, rng)
+    beta = sum(wi * orc.densmatr_from_pure(s) for wi, s in zip(w, states))
+    for m in (1, 4, 16):
+        kraus = list(wl.haar_kraus(2, m, rng))
+        zeros = [np.zeros((4, 4), dtype=np.complex128)] * (17 - m)
+        t = [int(q) for q in rng.permutation(nq)[:2]]
+        got = []
+        for ops in (kraus, kraus + zeros):
+            dm = qs.State(nq, density=True, prec=qs.QS_C128)
+            qs.qs_set_arithmetic(dm.handle, qs.QS_ARITH_FX if arith == "fx" else qs.QS_ARITH_DF)
+            dm.set_amps(beta)
+            qs.qs_apply_kraus(dm.handle, t, ops)
+            got.append(dm.get_amps())
+            dm.close()
+        assert np.array_equal(got[0], got[1])
+        want = orc.densmatr_apply_kraus(beta, t, kraus)
+        assert np.max(np.abs((got[0] - want).view(np.float64))) <= bound(4, beta, orc.superoperator(kraus))
