@@ -582,9 +582,10 @@ qs_status superop_pass(qs_state* s, const std::vector<int>& t, const double* kra
   return st != QS_OK ? st : (a != QS_OK ? a : b);
 }
 
-qs_status reduce_to_host(qs_state* s, double* out) {
-  if (cudaMemcpyAsync(s->h_result, s->d_result, sizeof(double2), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
-    return QS_ERR_CUDA;
+// The reduction queued on the state's stream has written its result to h_result
+// (pinned memory that the kernels store to: on a 10-qubit norm the copy back from
+// the device that this replaces and the grids of small states were 25 of 40 us).
+qs_status result_from_host(qs_state* s, double* out) {
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) return QS_ERR_CUDA;
   out[0] = s->h_result[0].x;
   out[1] = s->h_result[0].y;
@@ -1075,35 +1076,43 @@ qs_status qs_expec_pauli_sum(const qs_state* cs, const int* paulis, const double
     if (st != QS_OK) return st;
     const auto* dt = static_cast<const qsk::PauliTerm*>(dterms);
     cudaError_t e;
-    if (s->is_density)
-      e = qsk::launch_expec_dm(s->prec, s->amps, s->nq, dt, cnt, s->d_partials, s->stream);
-    else if (first < ndiag)
+    int grid = 0;
+    if (s->is_density) {
+      grid = qsk::expec_dm_blocks(s->nq, cnt);
+      const bool alone = grid == 1 && cnt == num_terms;
+      e = qsk::launch_expec_dm(s->prec, s->amps, s->nq, dt, cnt, alone ? s->h_result : s->d_partials, s->stream);
+      if (alone) grid = 0;
+    } else if (first < ndiag) {
+      grid = qsk::expec_sv_diag_blocks(s->nq);
       e = qsk::launch_expec_sv_diag(s->prec, s->amps, s->nq, dt, cnt, s->d_partials, s->stream,
                                        s->arith != QS_ARITH_DF);
-    else
+    } else {
       e = qsk::launch_expec_sv(s->prec, s->amps, s->nq, dt, cnt, s->d_partials, s->stream, s->arith != QS_ARITH_DF,
-                               qsk::make_tile_order(terms.data() + first, cnt));
-    if (e == cudaSuccess) e = qsk::launch_reduce_final(s->d_partials, s->d_result, first > 0, s->stream);
+                               qsk::make_tile_order(terms.data() + first, cnt), &grid);
+    }
+    if (e == cudaSuccess && grid > 0)
+      e = qsk::launch_reduce_final(s->d_partials, s->d_result, first > 0, s->stream, grid, s->h_result);
     first += cnt;
     st = ring_done(s, slot);
     if (e != cudaSuccess) return QS_ERR_CUDA;
     if (st != QS_OK) return st;
   }
-  return reduce_to_host(s, out);
+  return result_from_host(s, out);
 }
 
 qs_status qs_calc_norm_or_trace(const qs_state* cs, double* out) {
   if (cs && cs->rec) return QS_ERR_ARG;   // not while recording
   qs_state* s = const_cast<qs_state*>(cs);
   if (!s || !out) return QS_ERR_ARG;
-  cudaError_t e = s->is_density ? qsk::launch_trace(s->prec, s->amps, s->nq, s->d_partials, s->stream)
-                                : qsk::launch_norm(s->prec, s->amps, s->ns, s->d_partials, s->stream,
-                                                   s->arith != QS_ARITH_DF);
-  if (e == cudaSuccess)
-    e = qsk::launch_reduce_final(s->d_partials, s->d_result, 0, s->stream,
-                                 s->is_density ? qsk::kReduceBlocks : qsk::kNormBlocks);
+  const int grid = s->is_density ? qsk::trace_blocks(s->nq) : qsk::norm_blocks(s->prec, s->ns);
+  double2* part = grid == 1 ? s->h_result : s->d_partials;
+  cudaError_t e = s->is_density
+                      ? qsk::launch_trace(s->prec, s->amps, s->nq, part, s->stream)
+                      : qsk::launch_norm(s->prec, s->amps, s->ns, part, s->stream, s->arith != QS_ARITH_DF);
+  if (e == cudaSuccess && grid > 1)
+    e = qsk::launch_reduce_final(s->d_partials, s->d_result, 0, s->stream, grid, s->h_result);
   if (e != cudaSuccess) return QS_ERR_CUDA;
-  return reduce_to_host(s, out);
+  return result_from_host(s, out);
 }
 
 qs_status qs_synchronize(const qs_state* s) {

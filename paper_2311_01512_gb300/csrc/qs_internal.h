@@ -13,8 +13,8 @@ namespace qsk {
 constexpr int kMaxQ = QS_MAX_STORAGE_QUBITS;
 constexpr int kMaxDense = QS_MAX_DENSE_TARGETS;
 constexpr int kTileBits = 10;        // amplitudes staged per tile of the dense kernel: 2^10
-constexpr int kReduceBlocks = 1216;  // 152 SMs x 8: fixed grid of the stage-one expectation and trace reductions
-constexpr int kNormBlocks = 4864;    // 152 SMs x 32: fixed grid of the norm, a pure stream over the state
+constexpr int kReduceBlocks = 1216;  // 152 SMs x 8: largest grid of the stage-one expectation and trace reductions
+constexpr int kNormBlocks = 4864;    // 152 SMs x 32: largest grid of the norm, a pure stream over the state
 constexpr int kPartials = kNormBlocks;  // partial sums a handle holds (the larger grid)
 constexpr size_t kWideScratch = 295424;  // bytes of scratch of a six-target gate (qs_tc_ozaki.cu)
 constexpr int kTermChunk = 2048;     // Pauli terms per device upload
@@ -426,21 +426,28 @@ cudaError_t launch_init_zero(qs_prec prec, void* amps, int ns, cudaStream_t st);
 // bytes (a multiple of 16) from src (device-accessible, 16-byte aligned) to dst
 cudaError_t launch_copy16(void* dst, const void* src, size_t bytes, cudaStream_t st);
 
-// Reductions: stage one writes kReduceBlocks complex128 partial sums, stage two
-// sums them in a fixed order into result[0] (added to result[0] if accumulate).
+// Reductions: stage one writes one complex128 partial sum a block, stage two
+// sums them in a fixed order into result[0] (added to result[0] if accumulate) and,
+// if given, into *host (pinned host memory).  The stage-one grid is norm_blocks()
+// and the like for the same arguments; a lone block's partial sum is the result.
 // f64: complex128 products and sums in native FP64 (FP64 and block fixed-point
 // arithmetic) instead of double-float.
+int norm_blocks(qs_prec prec, int ns);
+int trace_blocks(int nq);
+int expec_dm_blocks(int nq, int nterms);
+int expec_sv_diag_blocks(int nq);
 cudaError_t launch_norm(qs_prec prec, const void* amps, int ns, double2* partials, cudaStream_t st, bool f64);
 cudaError_t launch_trace(qs_prec prec, const void* amps, int nq, double2* partials, cudaStream_t st);
 cudaError_t launch_expec_dm(qs_prec prec, const void* amps, int nq, const PauliTerm* terms,
                             int nterms, double2* partials, cudaStream_t st);
-// order: from make_tile_order on the same terms (host copy)
+// order: from make_tile_order on the same terms (host copy); partials has
+// kReduceBlocks slots, *grid is set to the blocks launched
 cudaError_t launch_expec_sv(qs_prec prec, const void* amps, int nq, const PauliTerm* terms,
-                            int nterms, double2* partials, cudaStream_t st, bool f64, const TileOrder& order);
+                            int nterms, double2* partials, cudaStream_t st, bool f64, const TileOrder& order, int* grid);
 // the diagonal (I/Z) terms of a statevector Pauli sum by warp Walsh-Hadamard transforms; N >= 5
 cudaError_t launch_expec_sv_diag(qs_prec prec, const void* amps, int nq, const PauliTerm* terms, int nterms,
                                  double2* partials, cudaStream_t st, bool f64);
 cudaError_t launch_reduce_final(const double2* partials, double2* result, int accumulate, cudaStream_t st,
-                                int nblocks = kReduceBlocks);
+                                int nblocks, double2* host);
 
 }  // namespace qsk

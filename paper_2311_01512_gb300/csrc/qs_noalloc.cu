@@ -103,10 +103,11 @@ extern "C" qs_status qs_expec_pauli_sum_noalloc(const void* d_amps, int num_qubi
   if (cudaMemcpyAsync(d_terms, terms, sizeof(qsk::PauliTerm) * (size_t)num_terms, cudaMemcpyHostToDevice, stream) !=
       cudaSuccess)
     return QS_ERR_CUDA;
+  int grid = qsk::expec_dm_blocks(num_qubits, num_terms);
   cudaError_t e = is_density ? qsk::launch_expec_dm(prec, d_amps, num_qubits, d_terms, num_terms, d_partials, stream)
                              : qsk::launch_expec_sv(prec, d_amps, num_qubits, d_terms, num_terms, d_partials, stream, true,
-                                                    qsk::make_tile_order(terms, num_terms));
-  if (e == cudaSuccess) e = qsk::launch_reduce_final(d_partials, d_result, 0, stream);
+                                                    qsk::make_tile_order(terms, num_terms), &grid);
+  if (e == cudaSuccess) e = qsk::launch_reduce_final(d_partials, d_result, 0, stream, grid, nullptr);
   double2 result;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&result, d_result, sizeof(double2), cudaMemcpyDeviceToHost, stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(stream);

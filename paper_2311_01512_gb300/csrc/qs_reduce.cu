@@ -1,7 +1,10 @@
 // Reductions: norm, trace, and Pauli-sum expectation values.  Stage one runs
-// a fixed grid (kNormBlocks for the norm, kReduceBlocks for the others), each
-// block writing one complex128 partial sum; stage two adds the partials in a
-// fixed order, so results do not depend on scheduling.
+// a grid of at most kNormBlocks (the norm) or kReduceBlocks blocks (the others),
+// each block writing one complex128 partial sum; stage two adds the partials in a
+// fixed order, so results do not depend on scheduling.  Work that needs fewer
+// blocks launches fewer: a work item has the same block and thread at any grid that
+// covers the work in one sweep, and the blocks left out would write zeros, so the
+// sums are the same.
 #include "qs_device.cuh"
 #include "qs_df.cuh"
 
@@ -596,7 +599,7 @@ static cudaError_t launch_diag(const void* amps, int nq, const PauliTerm* terms,
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
-  k_expec_sv_diag<R, U><<<kReduceBlocks, 256, sizeof(ZTermDf) * (size_t)nterms, st>>>(
+  k_expec_sv_diag<R, U><<<expec_sv_diag_blocks(nq), 256, sizeof(ZTermDf) * (size_t)nterms, st>>>(
       static_cast<const typename Cplx<R>::T*>(amps), nq, terms, nterms, partials);
   return cudaGetLastError();
 }
@@ -616,11 +619,12 @@ cudaError_t launch_expec_sv_diag(qs_prec prec, const void* amps, int nq, const P
       attr_done = true;
     }
     const size_t sm = sizeof(ZTerm64) * (size_t)nterms;
+    const int g = expec_sv_diag_blocks(nq);
     if (nq >= 7)
-      k_expec_sv_diag_f64<4><<<kReduceBlocks, 256, sm, st>>>(static_cast<const double2*>(amps), nq, terms, nterms,
+      k_expec_sv_diag_f64<4><<<g, 256, sm, st>>>(static_cast<const double2*>(amps), nq, terms, nterms,
                                                               partials);
     else
-      k_expec_sv_diag_f64<1><<<kReduceBlocks, 256, sm, st>>>(static_cast<const double2*>(amps), nq, terms, nterms,
+      k_expec_sv_diag_f64<1><<<g, 256, sm, st>>>(static_cast<const double2*>(amps), nq, terms, nterms,
                                                               partials);
     return cudaGetLastError();
   }
@@ -633,7 +637,8 @@ cudaError_t launch_expec_sv_diag(qs_prec prec, const void* amps, int nq, const P
 
 // Stage two: one block of 1024 threads; thread j adds partials j, j + 1024, ...
 __global__ void __launch_bounds__(1024) k_reduce_final(const double2* __restrict__ partials, int n,
-                                                       double2* __restrict__ result, int accumulate) {
+                                                       double2* __restrict__ result, int accumulate,
+                                                       double2* __restrict__ host) {
   double sr = 0.0, si = 0.0;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
     sr += partials[j].x;
@@ -641,63 +646,72 @@ __global__ void __launch_bounds__(1024) k_reduce_final(const double2* __restrict
   }
   const double2 s = block_sum(make_double2(sr, si));
   if (threadIdx.x == 0) {
-    if (accumulate) {
-      result[0].x += s.x;
-      result[0].y += s.y;
-    } else {
-      result[0] = s;
-    }
+    double2 r = s;
+    if (accumulate) r = make_double2(result[0].x + s.x, result[0].y + s.y);
+    result[0] = r;
+    if (host) *host = r;
   }
 }
 
-// Stage-one kernels always run exactly kReduceBlocks blocks; blocks with no
-// work write a zero partial.
+// Blocks of 256 threads for `items` work items, at most cap.
+static int blocks_for(uint64_t items, int cap) {
+  const uint64_t b = (items + 255) / 256;
+  return b < (uint64_t)cap ? (int)b : cap;
+}
+
+int norm_blocks(qs_prec prec, int ns) {
+  const uint64_t n = 1ull << ns;
+  return blocks_for(prec == QS_C64 && ns > 0 ? n / 2 : n, kNormBlocks);   // complex64: two amplitudes a thread
+}
+int trace_blocks(int nq) { return blocks_for(1ull << nq, kReduceBlocks); }
+int expec_dm_blocks(int nq, int nterms) { return blocks_for((uint64_t)nterms << nq, kReduceBlocks); }
+// a thread of the diagonal-term kernels takes four amplitudes (one below 7 qubits)
+int expec_sv_diag_blocks(int nq) { return blocks_for((1ull << nq) / (nq >= 7 ? 4 : 1), kReduceBlocks); }
+
 cudaError_t launch_norm(qs_prec prec, const void* amps, int ns, double2* partials, cudaStream_t st, bool f64) {
   const uint64_t n = 1ull << ns;
+  const int g = norm_blocks(prec, ns);
   if (prec == QS_C128 && f64)
-    k_norm_f64<<<kNormBlocks, 256, 0, st>>>(static_cast<const double2*>(amps), n, partials);
+    k_norm_f64<<<g, 256, 0, st>>>(static_cast<const double2*>(amps), n, partials);
   else if (prec == QS_C128)
-    k_norm<double><<<kNormBlocks, 256, 0, st>>>(static_cast<const double2*>(amps), n, partials);
+    k_norm<double><<<g, 256, 0, st>>>(static_cast<const double2*>(amps), n, partials);
   else
-    k_norm<float><<<kNormBlocks, 256, 0, st>>>(static_cast<const float2*>(amps), n, partials);
+    k_norm<float><<<g, 256, 0, st>>>(static_cast<const float2*>(amps), n, partials);
   return cudaGetLastError();
 }
 
 cudaError_t launch_trace(qs_prec prec, const void* amps, int nq, double2* partials, cudaStream_t st) {
+  const int g = trace_blocks(nq);
   if (prec == QS_C128)
-    k_trace<double><<<kReduceBlocks, 256, 0, st>>>(static_cast<const double2*>(amps), nq, partials);
+    k_trace<double><<<g, 256, 0, st>>>(static_cast<const double2*>(amps), nq, partials);
   else
-    k_trace<float><<<kReduceBlocks, 256, 0, st>>>(static_cast<const float2*>(amps), nq, partials);
+    k_trace<float><<<g, 256, 0, st>>>(static_cast<const float2*>(amps), nq, partials);
   return cudaGetLastError();
 }
 
 cudaError_t launch_expec_dm(qs_prec prec, const void* amps, int nq, const PauliTerm* terms, int nterms,
                             double2* partials, cudaStream_t st) {
+  const int g = expec_dm_blocks(nq, nterms);
   if (prec == QS_C128)
-    k_expec_dm<double><<<kReduceBlocks, 256, 0, st>>>(static_cast<const double2*>(amps), nq, terms, nterms,
-                                                      partials);
+    k_expec_dm<double><<<g, 256, 0, st>>>(static_cast<const double2*>(amps), nq, terms, nterms, partials);
   else
-    k_expec_dm<float><<<kReduceBlocks, 256, 0, st>>>(static_cast<const float2*>(amps), nq, terms, nterms,
-                                                     partials);
+    k_expec_dm<float><<<g, 256, 0, st>>>(static_cast<const float2*>(amps), nq, terms, nterms, partials);
   return cudaGetLastError();
 }
 
-// Blocks of the statevector expectation kernels: as many as are resident at
-// once (at most kReduceBlocks), so that the blocks walk consecutive virtual
-// tiles together and a coset of the tile order is processed while it is in
-// L2.  The other partial slots are zeroed (the final sum stays in a fixed
-// order for a given kernel and GPU).
-// The last partial slot holds the kernels' TileCounter (zeroed here with the
-// unused slots, and zero again when the kernel ends), so the grid is at most
-// kReduceBlocks - 1.
+// Blocks of the statevector expectation kernels: as many as have a tile, and at
+// most as many as are resident at once (and kReduceBlocks - 1), so that the blocks
+// walk consecutive virtual tiles together and a coset of the tile order is
+// processed while it is in L2.  The last partial slot holds the kernels' TileCounter
+// (zeroed here, and zero again when the kernel ends).
 template <typename K>
-static cudaError_t resident_grid(K kernel, size_t smem, double2* partials, cudaStream_t st, unsigned* grid) {
+static cudaError_t resident_grid(K kernel, size_t smem, int nq, double2* partials, cudaStream_t st, int* grid) {
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 256, smem);
   if (e != cudaSuccess) return e;
   const int g = per_sm > 0 ? per_sm * num_sms() : 1;
-  *grid = (unsigned)(g < kReduceBlocks - 1 ? g : kReduceBlocks - 1);
-  return cudaMemsetAsync(partials + *grid, 0, sizeof(double2) * (kReduceBlocks - *grid), st);
+  *grid = blocks_for(1ull << (nq > 2 ? nq - 2 : 0), g < kReduceBlocks - 1 ? g : kReduceBlocks - 1);
+  return cudaMemsetAsync(partials + kReduceBlocks - 1, 0, sizeof(double2), st);
 }
 
 static TileCounter tile_counter(double2* partials) {
@@ -706,7 +720,7 @@ static TileCounter tile_counter(double2* partials) {
 
 template <typename R, int E>
 static cudaError_t expec_sv_u(const void* amps, int nq, const PauliTerm* terms, int nterms, double2* partials,
-                              cudaStream_t st, const TileOrder& ord) {
+                              cudaStream_t st, const TileOrder& ord, int* grid) {
   static bool attr_done = false;
   if (!attr_done) {
     const cudaError_t e = cudaFuncSetAttribute(k_expec_sv<R, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -715,16 +729,15 @@ static cudaError_t expec_sv_u(const void* amps, int nq, const PauliTerm* terms, 
     attr_done = true;
   }
   const size_t smem = (sizeof(TermDf) + sizeof(GroupDf)) * (size_t)nterms;
-  unsigned grid = kReduceBlocks;
-  const cudaError_t e = resident_grid(k_expec_sv<R, E>, smem, partials, st, &grid);
+  const cudaError_t e = resident_grid(k_expec_sv<R, E>, smem, nq, partials, st, grid);
   if (e != cudaSuccess) return e;
-  k_expec_sv<R, E><<<grid, 256, smem, st>>>(static_cast<const typename Cplx<R>::T*>(amps), nq, terms, nterms,
+  k_expec_sv<R, E><<<*grid, 256, smem, st>>>(static_cast<const typename Cplx<R>::T*>(amps), nq, terms, nterms,
                                             partials, ord, tile_counter(partials));
   return cudaGetLastError();
 }
 
 cudaError_t launch_expec_sv(qs_prec prec, const void* amps, int nq, const PauliTerm* terms, int nterms,
-                            double2* partials, cudaStream_t st, bool f64, const TileOrder& ord) {
+                            double2* partials, cudaStream_t st, bool f64, const TileOrder& ord, int* grid) {
   static_assert(256 * 4 == (1 << kExpecTileBits), "tiles of the expectation kernels");
   if (nterms > kTermChunk) return cudaErrorInvalidValue;
   if (prec == QS_C128 && f64) {
@@ -736,22 +749,21 @@ cudaError_t launch_expec_sv(qs_prec prec, const void* amps, int nq, const PauliT
       if (e != cudaSuccess) return e;
       attr_done = true;
     }
-    unsigned grid = kReduceBlocks;
-    const cudaError_t e = resident_grid(k_expec_sv_f64<4>, per * (size_t)nterms, partials, st, &grid);
+    const cudaError_t e = resident_grid(k_expec_sv_f64<4>, per * (size_t)nterms, nq, partials, st, grid);
     if (e != cudaSuccess) return e;
-    k_expec_sv_f64<4><<<grid, 256, per * (size_t)nterms, st>>>(static_cast<const double2*>(amps), nq, terms, nterms,
+    k_expec_sv_f64<4><<<*grid, 256, per * (size_t)nterms, st>>>(static_cast<const double2*>(amps), nq, terms, nterms,
                                                                 partials, ord, tile_counter(partials));
     return cudaGetLastError();
   }
   // tiles of 1024 amplitudes (28 qubits, 8 random terms: 6.9 ms against 7.5
   // and 8.0 ms for tiles of 512 and 2048)
-  return prec == QS_C128 ? expec_sv_u<double, 4>(amps, nq, terms, nterms, partials, st, ord)
-                         : expec_sv_u<float, 4>(amps, nq, terms, nterms, partials, st, ord);
+  return prec == QS_C128 ? expec_sv_u<double, 4>(amps, nq, terms, nterms, partials, st, ord, grid)
+                         : expec_sv_u<float, 4>(amps, nq, terms, nterms, partials, st, ord, grid);
 }
 
 cudaError_t launch_reduce_final(const double2* partials, double2* result, int accumulate, cudaStream_t st,
-                                int nblocks) {
-  k_reduce_final<<<1, 1024, 0, st>>>(partials, nblocks, result, accumulate);
+                                int nblocks, double2* host) {
+  k_reduce_final<<<1, 1024, 0, st>>>(partials, nblocks, result, accumulate, host);
   return cudaGetLastError();
 }
 
