@@ -25,7 +25,8 @@
  *     keeps it alive until qs_destroy.  The pointer must be 256-byte aligned.
  *   - each handle owns a little library memory: a device scratch area for
  *     reductions and a pinned staging ring for gate matrices.  It is allocated
- *     by qs_create_* and freed by qs_destroy.
+ *     by qs_create_* and given up by qs_destroy; up to four such areas stay
+ *     for the next handles of their device until the last handle is destroyed.
  *   - host arrays passed to any call are read before the call returns; the
  *     caller may reuse them at once.
  *

@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -46,15 +47,115 @@ bool injected_failure() {
   return true;
 }
 
-void release(qs_state* s) {
-  if (!s) return;
-  if (s->d_partials) cudaFree(s->d_partials);
-  if (s->d_ring) cudaFree(s->d_ring);
-  if (s->h_result) cudaFreeHost(s->h_result);
-  if (s->h_ring) cudaFreeHost(s->h_ring);
-  for (auto& ev : s->ring_ev)
+// A handle's memory: reduction scratch and error word, staging ring and its events.
+struct HandleScratch {
+  int device = 0;
+  double2* d_partials = nullptr;
+  unsigned char* d_ring = nullptr;
+  double2* h_result = nullptr;
+  unsigned char* h_ring = nullptr;
+  cudaEvent_t ring_ev[kRingSlots] = {};
+};
+
+void free_scratch(const HandleScratch& c) {
+  if (c.d_partials) cudaFree(c.d_partials);
+  if (c.d_ring) cudaFree(c.d_ring);
+  if (c.h_result) cudaFreeHost(c.h_result);
+  if (c.h_ring) cudaFreeHost(c.h_ring);
+  for (auto ev : c.ring_ev)
     if (ev) cudaEventDestroy(ev);
+}
+
+// Memory of destroyed handles, kept for the next ones of the same device while any
+// handle is alive (at most kIdleScratch of them, 2.2 MB each; all given back with
+// the last handle): allocating and freeing it takes 370 us, so a program that takes
+// reduced density matrices of a small state spent most of its time there.  A
+// handle's stream has been waited for when its memory arrives here, so any stream
+// and thread may use it next.
+constexpr size_t kIdleScratch = 4;
+std::mutex g_scratch_mutex;
+std::vector<HandleScratch> g_scratch_idle;
+int g_scratch_handles = 0;   // handles alive
+
+// Memory of an earlier handle for a new one, if there is any.
+bool take_scratch(int device, HandleScratch* out) {
+  std::lock_guard<std::mutex> lock(g_scratch_mutex);
+  for (size_t i = 0; i < g_scratch_idle.size(); ++i)
+    if (g_scratch_idle[i].device == device) {
+      *out = g_scratch_idle[i];
+      g_scratch_idle.erase(g_scratch_idle.begin() + (ptrdiff_t)i);
+      return true;
+    }
+  return false;
+}
+
+// One handle fewer (`alive`: it had been counted); its memory is kept (if `idle`:
+// no work that uses it is left) or freed.
+void give_scratch(const HandleScratch& c, bool idle, bool alive) {
+  std::vector<HandleScratch> gone;
+  {
+    std::lock_guard<std::mutex> lock(g_scratch_mutex);
+    if (alive) --g_scratch_handles;
+    bool keep = false;
+    if (idle && g_scratch_handles > 0 && g_scratch_idle.size() < kIdleScratch) {
+      try {
+        g_scratch_idle.push_back(c);
+        keep = true;
+      } catch (const std::bad_alloc&) {
+      }
+    }
+    if (g_scratch_handles == 0) gone.swap(g_scratch_idle);
+    if (keep) return;
+  }
+  for (const auto& g : gone) free_scratch(g);
+  free_scratch(c);
+}
+
+// idle: nothing on the GPU uses the handle's memory any more
+void release(qs_state* s, bool idle) {
+  if (!s) return;
+  HandleScratch c;
+  c.device = s->device;
+  c.d_partials = s->d_partials;
+  c.d_ring = s->d_ring;
+  c.h_result = s->h_result;
+  c.h_ring = s->h_ring;
+  std::copy(s->ring_ev, s->ring_ev + kRingSlots, c.ring_ev);
+  give_scratch(c, idle, true);
   delete s;
+}
+
+// The four allocations and the events of a handle; *out is complete or freed.
+qs_status make_scratch(int device, HandleScratch* out) {
+  HandleScratch c;
+  if (take_scratch(device, &c)) {
+    for (int i = 0; i < 4; ++i)              // the allocations it stands for may be made to fail
+      if (injected_failure()) {
+        give_scratch(c, true, false);
+        return QS_ERR_OOM;
+      }
+  } else {
+    c.device = device;
+    if (qsalloc::device(reinterpret_cast<void**>(&c.d_partials), sizeof(double2) * (qsk::kPartials + 2)) != cudaSuccess ||
+        qsalloc::device(reinterpret_cast<void**>(&c.d_ring), kRingSlots * kSlotBytes) != cudaSuccess ||
+        qsalloc::pinned(reinterpret_cast<void**>(&c.h_result), sizeof(double2) * 2) != cudaSuccess ||
+        qsalloc::pinned(reinterpret_cast<void**>(&c.h_ring), kRingSlots * kSlotBytes) != cudaSuccess) {
+      cudaGetLastError();
+      free_scratch(c);
+      return QS_ERR_OOM;
+    }
+    for (auto& ev : c.ring_ev)
+      if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
+        free_scratch(c);
+        return QS_ERR_CUDA;
+      }
+  }
+  if (cudaMemset(c.d_partials + qsk::kPartials + 1, 0, sizeof(int)) != cudaSuccess) {   // the error word
+    free_scratch(c);
+    return QS_ERR_CUDA;
+  }
+  *out = c;
+  return QS_OK;
 }
 
 qs_status create(int nq, int ns, int is_density, qs_prec prec, void* d_amps, void* stream, qs_state** out) {
@@ -71,26 +172,24 @@ qs_status create(int nq, int ns, int is_density, qs_prec prec, void* d_amps, voi
   s->is_density = is_density;
   s->prec = prec;
   s->stream = static_cast<cudaStream_t>(stream);
-  const size_t scratch = sizeof(double2) * (qsk::kPartials + 2);
-  if (qsalloc::device(reinterpret_cast<void**>(&s->d_partials), scratch) != cudaSuccess ||
-      qsalloc::device(reinterpret_cast<void**>(&s->d_ring), kRingSlots * kSlotBytes) != cudaSuccess ||
-      qsalloc::pinned(reinterpret_cast<void**>(&s->h_result), sizeof(double2) * 2) != cudaSuccess ||
-      qsalloc::pinned(reinterpret_cast<void**>(&s->h_ring), kRingSlots * kSlotBytes) != cudaSuccess) {
-    cudaGetLastError();
-    release(s);
-    return QS_ERR_OOM;
+  // without a device (or driver) the first allocation reports it
+  if (cudaGetDevice(&s->device) != cudaSuccess) cudaGetLastError();
+  HandleScratch c;
+  const qs_status st = make_scratch(s->device, &c);
+  if (st != QS_OK) {
+    delete s;
+    return st;
   }
+  s->d_partials = c.d_partials;
+  s->d_ring = c.d_ring;
+  s->h_result = c.h_result;
+  s->h_ring = c.h_ring;
+  std::copy(c.ring_ev, c.ring_ev + kRingSlots, s->ring_ev);
   s->d_result = s->d_partials + qsk::kPartials;
   s->d_err = reinterpret_cast<int*>(s->d_partials + qsk::kPartials + 1);
-  if (cudaMemset(s->d_err, 0, sizeof(int)) != cudaSuccess) {
-    release(s);
-    return QS_ERR_CUDA;
-  }
-  for (auto& ev : s->ring_ev) {
-    if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
-      release(s);
-      return QS_ERR_CUDA;
-    }
+  {
+    std::lock_guard<std::mutex> lock(g_scratch_mutex);
+    ++g_scratch_handles;
   }
   *out = s;
   return QS_OK;
@@ -665,7 +764,7 @@ qs_status qs_create_densmatr(int num_qubits, qs_prec prec, void* d_amps, void* c
 qs_status qs_destroy(qs_state* state) {
   if (!state || state->rec) return QS_ERR_ARG;
   const cudaError_t e = cudaStreamSynchronize(state->stream);
-  release(state);
+  release(state, e == cudaSuccess);
   return cuda_status(e);
 }
 
@@ -1029,7 +1128,7 @@ qs_status qs_partial_trace(const qs_state* in, const int* targs, int n, void* d_
   p.nout = 1ull << (2 * m);
   st = cuda_status(qsk::launch_ptrace(in->prec, in->amps, d_out_amps, p, in->stream));
   if (st != QS_OK) {
-    release(o);
+    release(o, true);
     return st;
   }
   *out = o;

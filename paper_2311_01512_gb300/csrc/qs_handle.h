@@ -27,6 +27,7 @@ struct qs_state {
   int tensor_cores = 1;  // complex64 dense gates with 3..5 targets on tcgen05
   int* d_err = nullptr;  // device error word (bounded waits that ran out)
   cudaStream_t stream = nullptr;
+  int device = 0;
   // reduction scratch (device) and its pinned host mirror
   double2* d_partials = nullptr;
   double2* d_result = nullptr;

@@ -125,6 +125,9 @@ QS_PLAN_GREEDY = 1
 QS_PLAN_COST = 2
 
 NOALLOC_MAX_TERMS = 256
+
+_C_DOUBLE = ctypes.c_double
+_C128 = np.dtype(np.complex128)
 for _name, (_res, _args) in SIGNATURES.items():
     _fn = getattr(_lib, _name)
     _fn.restype = _res
@@ -150,6 +153,8 @@ def _ints(xs):
 
 def _doubles(arr):
     """complex or real array -> contiguous float64 buffer (kept alive by the caller)."""
+    if type(arr) is np.ndarray and arr.dtype is _C128 and arr.size and arr.flags.c_contiguous and arr.flags.writeable:
+        return arr, (_C_DOUBLE * (2 * arr.size)).from_buffer(arr)     # the array itself
     a = np.asarray(arr)
     if np.iscomplexobj(a):
         a = np.ascontiguousarray(a, dtype=np.complex128).view(np.float64)
