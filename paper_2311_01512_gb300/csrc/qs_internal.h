@@ -8,6 +8,10 @@
 
 #include "qs.h"
 
+namespace qstile {
+struct TilePass;
+}
+
 namespace qsk {
 
 constexpr int kMaxQ = QS_MAX_STORAGE_QUBITS;
@@ -425,6 +429,9 @@ cudaError_t launch_dm_from_pure(qs_prec prec, void* rho, const void* psi, int nq
 cudaError_t launch_init_zero(qs_prec prec, void* amps, int ns, cudaStream_t st);
 // bytes (a multiple of 16) from src (device-accessible, 16-byte aligned) to dst
 cudaError_t launch_copy16(void* dst, const void* src, size_t bytes, cudaStream_t st);
+
+// one tile pass of a complex64 state (qs_tile.h)
+cudaError_t launch_tile_pass(void* amps, const qstile::TilePass& p, cudaStream_t st);
 
 // Reductions: stage one writes one complex128 partial sum a block, stage two
 // sums them in a fixed order into result[0] (added to result[0] if accumulate) and,

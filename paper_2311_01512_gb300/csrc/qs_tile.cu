@@ -1,0 +1,234 @@
+// Tile passes of planned complex64 circuits (qs_tile.h): one block per tile reads
+// 2^12 amplitudes into shared memory, runs the pass's sweeps and writes them back.
+//
+// What bounds it: instruction issue (2.6 of 4 a clock), then the FP32 pipe; a pass
+// by itself costs one read and one write of the state (1.27 ms at 29 qubits), and
+// for 16 amplitudes a sweep adds 16 shared loads, 16 stores and some 50 index
+// instructions a thread, a one-target gate 128 multiply-adds, a two-target gate
+// 256, a gadget 64 and 15 for signs.  150 random gates at 29 qubits, 17 passes: 48
+// ms, against 97 (blocks of six qubits) to 127 (of three) in dense blocks.
+// Four 256-thread blocks a multiprocessor (64 registers a thread): one block's
+// sweeps run while the others' loads and stores are in flight (tiles of 2^13 with
+// two 512-thread blocks, 15 passes: 49.7 ms).  Matrices come from shared memory:
+// indexed reads of the constant bank took 82 ms.
+#include "qs_device.cuh"
+#include "qs_internal.h"
+#include "qs_tile.h"
+
+namespace qsk {
+namespace {
+
+using namespace qstile;
+
+constexpr int kTileThreads = 1 << kThreadBits;
+constexpr size_t kTileSmem = (sizeof(float2) << kPassBits) + sizeof(float) * kMaxCoef;
+
+// Entries e and e + 1 of a complex matrix at shared address u (16-byte aligned).
+// Volatile: loaded where they are used, so that a matrix is not kept in 32
+// registers beside the 32 of the amplitudes.
+__device__ __forceinline__ float4 entries(uint32_t u, int e) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(u + 8 * e));
+  return v;
+}
+
+// ok: bit r = the controls are set at register r (C; otherwise they are everywhere)
+template <int K, bool C>
+__device__ __forceinline__ void gate1(float2 (&a)[kSweepAmps], uint32_t u, uint32_t ok) {
+  const float4 m0 = entries(u, 0), m1 = entries(u, 2);
+#pragma unroll
+  for (int r = 0; r < kSweepAmps; ++r) {
+    if (r >> K & 1) continue;
+    if (C && !(ok >> r & 1u)) continue;
+    const float2 x = a[r], y = a[r | 1 << K];
+    a[r] = make_float2(m0.x * x.x - m0.y * x.y + m0.z * y.x - m0.w * y.y, m0.x * x.y + m0.y * x.x + m0.z * y.y + m0.w * y.x);
+    a[r | 1 << K] =
+        make_float2(m1.x * x.x - m1.y * x.y + m1.z * y.x - m1.w * y.y, m1.x * x.y + m1.y * x.x + m1.z * y.y + m1.w * y.x);
+  }
+}
+
+template <int K0, int K1, bool C>
+__device__ __forceinline__ void gate2(float2 (&a)[kSweepAmps], uint32_t u, uint32_t ok) {
+#pragma unroll
+  for (int r = 0; r < kSweepAmps; ++r) {
+    if ((r >> K0 & 1) || (r >> K1 & 1)) continue;
+    if (C && !(ok >> r & 1u)) continue;
+    float2 v[4];
+#pragma unroll
+    for (int l = 0; l < 4; ++l) v[l] = a[r | (l & 1) << K0 | (l >> 1) << K1];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float4 p = entries(u, 4 * j);
+      float2 o = make_float2(p.x * v[0].x, p.x * v[0].y);
+      o = make_float2(fmaf(-p.y, v[0].y, o.x), fmaf(p.y, v[0].x, o.y));
+      o = make_float2(fmaf(p.z, v[1].x, o.x), fmaf(p.z, v[1].y, o.y));
+      o = make_float2(fmaf(-p.w, v[1].y, o.x), fmaf(p.w, v[1].x, o.y));
+      const float4 q = entries(u, 4 * j + 2);
+      o = make_float2(fmaf(q.x, v[2].x, o.x), fmaf(q.x, v[2].y, o.y));
+      o = make_float2(fmaf(-q.y, v[2].y, o.x), fmaf(q.y, v[2].x, o.y));
+      o = make_float2(fmaf(q.z, v[3].x, o.x), fmaf(q.z, v[3].y, o.y));
+      o = make_float2(fmaf(-q.w, v[3].y, o.x), fmaf(q.w, v[3].x, o.y));
+      a[r | (j & 1) << K0 | (j >> 1) << K1] = o;
+    }
+  }
+}
+
+template <bool C>
+__device__ __forceinline__ void dense(float2 (&a)[kSweepAmps], const TileOp& op, uint32_t u, uint32_t ok) {
+  if (op.kind == OP_GATE1) {
+    if (op.k == 0) gate1<0, C>(a, u, ok);
+    if (op.k == 1) gate1<1, C>(a, u, ok);
+    if (op.k == 2) gate1<2, C>(a, u, ok);
+    if (op.k == 3) gate1<3, C>(a, u, ok);
+  } else {
+    if (op.k == 0) gate2<0, 1, C>(a, u, ok);
+    if (op.k == 1) gate2<0, 2, C>(a, u, ok);
+    if (op.k == 2) gate2<0, 3, C>(a, u, ok);
+    if (op.k == 3) gate2<1, 2, C>(a, u, ok);
+    if (op.k == 4) gate2<1, 3, C>(a, u, ok);
+    if (op.k == 5) gate2<2, 3, C>(a, u, ok);
+  }
+}
+
+// a_r <- c a_r + s_r i^IM a_{r ^ M}; s_r = s with its sign changed by the parity of
+// r & y (the sign of register 0 is in s already)
+template <int M, bool IM>
+__device__ __forceinline__ void gadget(float2 (&a)[kSweepAmps], float c, uint32_t s, uint32_t y) {
+  uint32_t t[kSweepAmps];
+  t[0] = s;
+#pragma unroll
+  for (int r = 1; r < kSweepAmps; ++r) {
+    const int low = r & -r, b = low == 1 ? 0 : low == 2 ? 1 : low == 4 ? 2 : 3;
+    t[r] = t[r ^ low] ^ (y >> b & 1u) << 31;
+  }
+#pragma unroll
+  for (int r = 0; r < kSweepAmps; ++r) {
+    const int q = r ^ M;
+    if (q < r) continue;
+    const float sr = __uint_as_float(t[r]), sq = __uint_as_float(t[q]);
+    const float2 x = a[r], y2 = a[q];
+    a[r] = IM ? make_float2(c * x.x - sr * y2.y, c * x.y + sr * y2.x) : make_float2(c * x.x + sr * y2.x, c * x.y + sr * y2.y);
+    if (q != r)
+      a[q] = IM ? make_float2(c * y2.x - sq * x.y, c * y2.y + sq * x.x) : make_float2(c * y2.x + sq * x.x, c * y2.y + sq * x.y);
+  }
+}
+
+// (Separate ifs, not a switch: joins of two paths keep the amplitudes in their
+// registers, a join of many made the compiler spill 900 bytes.)
+template <int M>
+__device__ __forceinline__ void gadget_m(float2 (&a)[kSweepAmps], uint32_t k, float c, uint32_t s, uint32_t y) {
+  if (k == M) gadget<M, false>(a, c, s, y);
+  if (k == (M | 16)) gadget<M, true>(a, c, s, y);
+}
+
+template <int M>
+__device__ __forceinline__ void gadget_4m(float2 (&a)[kSweepAmps], uint32_t k, float c, uint32_t s, uint32_t y) {
+  if ((k & 12) != M) return;
+  gadget_m<M>(a, k, c, s, y);
+  gadget_m<M + 1>(a, k, c, s, y);
+  gadget_m<M + 2>(a, k, c, s, y);
+  gadget_m<M + 3>(a, k, c, s, y);
+}
+
+__device__ __forceinline__ uint64_t thread_offset(const TilePass& p, uint32_t tid) {
+  uint64_t off = 0;
+  for (int j = 0; j < p.ntrun; ++j) off += (uint64_t)(tid & p.trun[j].mask) * p.trun[j].mul;
+  return off;
+}
+
+__global__ void __launch_bounds__(kTileThreads, 4) k_tile_pass(float2* __restrict__ psi, const __grid_constant__ TilePass p) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  float* coef = reinterpret_cast<float*>(sm + (sizeof(float2) << kPassBits));
+  const uint32_t tid = threadIdx.x;
+  uint64_t tb = 0;
+  for (int j = 0; j < p.nbrun; ++j) tb += (uint64_t)(blockIdx.x & p.brun[j].mask) * p.brun[j].mul;
+  {
+    float2* const mine = psi + (tb + thread_offset(p, tid));   // tile index r << kThreadBits | tid is at mine[p.off[r]]
+    const uint32_t home = slot(tid) * 8;
+    float2 v[kSweepAmps];
+#pragma unroll
+    for (int r = 0; r < kSweepAmps; ++r) v[r] = mine[p.off[r]];
+    for (uint32_t e = tid; e < p.ncoef; e += kTileThreads) coef[e] = p.coef[e];
+#pragma unroll
+    for (int r = 0; r < kSweepAmps; ++r)
+      *reinterpret_cast<float2*>(sm + (home ^ slot((uint32_t)r << kThreadBits) * 8)) = v[r];
+  }
+  __syncthreads();
+  for (uint32_t s = 0; s < p.nsweeps; ++s) {
+    const TileSweep& w = p.sweep[s];
+    uint32_t base = 0;
+#pragma unroll
+    for (int b = 0; b < kThreadBits; ++b) base += (tid >> b & 1u) * w.mul[b];
+    const uint32_t addr = slot(base) * 8;
+    float2 a[kSweepAmps];
+#pragma unroll
+    for (int r = 0; r < kSweepAmps; ++r) a[r] = *reinterpret_cast<const float2*>(sm + (addr ^ w.csw[r]));
+    const uint32_t end = w.first + w.count;
+    for (uint32_t o = w.first; o < end; ++o) {
+      const TileOp& op = p.op[o];
+      if (op.kind <= OP_GATE2) {
+        if ((tb & op.cg) != op.cg) continue;
+        const uint32_t fixed = op.cl & ~op.creg;
+        if ((base & fixed) != fixed) continue;
+        const uint32_t u = (uint32_t)__cvta_generic_to_shared(coef) + 4 * op.coef;
+        if (!op.creg) {
+          dense<false>(a, op, u, 0);
+        } else {
+          uint32_t ok = 0;
+#pragma unroll
+          for (int r = 0; r < kSweepAmps; ++r) ok |= (((base ^ w.comb[r]) & op.cl) == op.cl ? 1u : 0u) << r;
+          dense<true>(a, op, u, ok);
+        }
+      }
+      if (op.kind == OP_GADGET) {
+        const uint32_t flip = (uint32_t)(__popcll(tb & op.yzg) + __popc(base & op.yzl)) << 31;
+        const uint32_t sb = __float_as_uint(op.s) ^ flip;
+        gadget_4m<0>(a, op.k, op.c, sb, op.sgn);
+        gadget_4m<4>(a, op.k, op.c, sb, op.sgn);
+        gadget_4m<8>(a, op.k, op.c, sb, op.sgn);
+        gadget_4m<12>(a, op.k, op.c, sb, op.sgn);
+      }
+      if (op.kind == OP_DIAG) {
+        uint32_t j = 0;
+        for (uint32_t q = 0; q < op.nd; ++q) {
+          const uint32_t d = op.dpos[q];
+          j |= ((d & 0x80u) ? (uint32_t)(tb >> (d & 0x7fu)) & 1u : base >> d & 1u) << q;
+        }
+        const float2* dg = reinterpret_cast<const float2*>(coef + op.coef);
+#pragma unroll
+        for (int r = 0; r < kSweepAmps; ++r) {
+          const float2 d = dg[j ^ op.jr[r]], x = a[r];
+          a[r] = make_float2(d.x * x.x - d.y * x.y, d.x * x.y + d.y * x.x);
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kSweepAmps; ++r) *reinterpret_cast<float2*>(sm + (addr ^ w.csw[r])) = a[r];
+    __syncthreads();
+  }
+  // (computed again instead of kept over the sweeps: registers)
+  uint32_t t2;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(t2));
+  float2* const mine = psi + (tb + thread_offset(p, t2));
+  const uint32_t home = slot(t2) * 8;
+#pragma unroll
+  for (int r = 0; r < kSweepAmps; ++r)
+    mine[p.off[r]] = *reinterpret_cast<const float2*>(sm + (home ^ slot((uint32_t)r << kThreadBits) * 8));
+}
+
+}  // namespace
+
+cudaError_t launch_tile_pass(void* amps, const qstile::TilePass& p, cudaStream_t st) {
+  static bool attr_done = false;
+  if (!attr_done) {
+    const cudaError_t e = cudaFuncSetAttribute(k_tile_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem);
+    if (e != cudaSuccess) return e;
+    attr_done = true;
+  }
+  k_tile_pass<<<(unsigned)p.ntiles, kTileThreads, kTileSmem, st>>>(static_cast<float2*>(amps), p);
+  return cudaGetLastError();
+}
+
+}  // namespace qsk
