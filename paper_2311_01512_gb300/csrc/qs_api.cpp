@@ -522,6 +522,15 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
       fixed |= 1ull << f;
     }
     const int nk = (int)kt.size();
+    // complex128 kernels take their targets in ascending order, so that a thread's
+    // neighbouring amplitudes are neighbours in memory when the lowest target is qubit 0
+    std::vector<int> order(kt.size());
+    for (int q = 0; q < nk; ++q) order[(size_t)q] = q;
+    if (tc128) std::sort(order.begin(), order.end(), [&](int x, int y) { return kt[(size_t)x] < kt[(size_t)y]; });
+    {
+      const std::vector<int> given(kt);
+      for (int q = 0; q < nk; ++q) kt[(size_t)q] = given[(size_t)order[(size_t)q]];
+    }
     // tensor-core tile: 128 groups, P = kernel targets u the 7 lowest free qubits
     const int g = std::min(7, s->ns - nk - (int)ctrls.size());
     std::vector<int> P(kt);
@@ -541,6 +550,7 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
     p.tile_bits = (int)P.size();
     for (int b = 0; b < p.tile_bits; ++b) p.P[b] = (int8_t)P[b];
     for (int q = 0; q < nk; ++q) {
+      p.mbit[q] = (int8_t)order[(size_t)q];
       p.tslot[q] = (int8_t)(std::find(P.begin(), P.end(), kt[q]) - P.begin());
       p.tslot_mask |= 1u << p.tslot[q];
       p.tpos[q] = (int8_t)kt[q];

@@ -90,6 +90,7 @@ struct TcParams {
   uint32_t tslot_mask;   // bits of P that are targets
   int8_t tslot[kMaxDense];
   int8_t tpos[kMaxDense];
+  int8_t mbit[kMaxDense];   // matrix bit of kernel target q (complex128: targets ascend, the matrix keeps its order)
   int8_t P[16];
   int8_t hi_ins[kMaxQ];
 };

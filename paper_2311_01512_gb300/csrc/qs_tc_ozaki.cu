@@ -68,7 +68,12 @@ __device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t parity) {
 }
 
 // entry (j, l) of the complex (and possibly identity-extended) matrix, D x D
-__device__ __forceinline__ double2 matrix_entry(const TcParams& p, int D, int j, int l) {
+__device__ __forceinline__ double2 matrix_entry(const TcParams& p, int D, int jk, int lk) {
+  int j = 0, l = 0;                               // kernel targets -> matrix bits
+  for (int q = 0; q < p.n; ++q) {
+    j |= (jk >> q & 1) << p.mbit[q];
+    l |= (lk >> q & 1) << p.mbit[q];
+  }
   if (p.nmat < p.n) {
     if ((j >> p.nmat) != (l >> p.nmat)) return make_double2(0.0, 0.0);
     const int mm = (1 << p.nmat) - 1;
@@ -255,6 +260,12 @@ __device__ __forceinline__ void store_slices(unsigned char* A, uint32_t off, uin
     *reinterpret_cast<uint4*>(A + s * abytes + off) = make_uint4(pk[0][s], pk[1][s], pk[2][s], pk[3][s]);
 }
 
+// two neighbouring amplitudes (32-byte aligned)
+__device__ __forceinline__ void store_pair(void* at, const double* o) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(at), "d"(o[0]), "d"(o[1]), "d"(o[2]), "d"(o[3])
+               : "memory");
+}
+
 // largest high word without sign of an amplitude's parts
 __device__ __forceinline__ uint32_t max_abs(uint32_t m, const uint32_t* R) {
   return max(m, max(R[0] & 0x7FFFFFFFu, R[2] & 0x7FFFFFFFu));
@@ -341,7 +352,7 @@ struct Ws {
 
 }  // namespace
 
-template <int NT>
+template <int NT, bool PAIRS>
 __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __restrict__ psi, const __grid_constant__ TcParams p) {
   using W = Ws<NT>;
   constexpr int K = W::K, N = W::N, NA = W::NA, NTM = W::NTM, NM = W::NM, S = W::S;
@@ -452,9 +463,13 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
             for (int L = 0; L < kLv; ++L) u[L] = v[L][qq];
             o[qq] = finish_output<K>(u, egs, scl[qq]);
           }
+          if (PAIRS) {
+            store_pair(tp + te[cc >> 1], o);
+          } else {
 #pragma unroll
-          for (int qq = 0; qq < 4; qq += 2)
-            *reinterpret_cast<double2*>(tp + te[(cc + qq) >> 1]) = make_double2(o[qq], o[qq + 1]);
+            for (int qq = 0; qq < 4; qq += 2)
+              *reinterpret_cast<double2*>(tp + te[(cc + qq) >> 1]) = make_double2(o[qq], o[qq + 1]);
+          }
         }
       }
     }
@@ -465,9 +480,16 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
     // column group, so the slice stores meet no bank twice
     const int g = 16 * pw + (lane & 7) + 8 * (lane >> 4), h = (lane >> 3) & 1;
     const bool row_ok = g < (1 << row_bits);
-    uint64_t tp[EPP];                         // byte offsets of this thread's amplitudes in a tile
+    // Neighbours in pairs: lanes 2 i and 2 i + 1 copy each other's halves of a sector.
+    // Copy i of a lane is amplitude (i & ~1) | (lane & 1) of the row of lane
+    // (lane & ~1) | (i & 1), and goes to that thread's place: (i' PT + pt') 16 with
+    // i' - i = pt - pt' = (lane & 1) - (i & 1).
+    const int odd = lane & 1;
+    const uint32_t swap[2] = {PAIRS ? (uint32_t)(odd * (PT - 1) * 16) : 0u, PAIRS ? (uint32_t)((odd - 1) * (PT - 1) * 16) : 0u};
+    uint64_t tp[EPP];                         // byte offsets in a tile of the amplitudes that this thread copies
 #pragma unroll
-    for (int i = 0; i < EPP; ++i) tp[i] = (rowoff[g] | toff[h * EPP + i]) << 4;
+    for (int i = 0; i < EPP; ++i)
+      tp[i] = PAIRS ? (rowoff[(g & ~1) | (i & 1)] | toff[h * EPP + ((i & ~1) | odd)]) << 4 : (rowoff[g] | toff[h * EPP + i]) << 4;
     const uint32_t stg_addr = smem_u32(stg) + (uint32_t)pt * 16u;
     auto issue = [&](uint64_t x, int slot) {
 #pragma unroll
@@ -475,7 +497,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
         const char* base = reinterpret_cast<const char*>(psi) + ((x | r * rstep | p.ctrl_mask) << 4);
 #pragma unroll
         for (int i = 0; i < EPP; ++i)
-          cp_async16(stg_addr + (uint32_t)(slot * W::SLOT + (r * EPP + i) * PT * 16),
+          cp_async16(stg_addr + swap[i & 1] + (uint32_t)(slot * W::SLOT + (r * EPP + i) * PT * 16),
                      row_ok ? (const void*)(base + tp[i]) : psi, row_ok ? 16u : 0u);
       }
     };
@@ -492,6 +514,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
       if (c >= nunits) break;
       const int slot = i % S, j = i % NA, m = i % NM;
       cp_async_wait<S - 1>();
+      if (PAIRS) __syncwarp();                // the other lane's copies, too
       uint32_t R[RB * EPP][4];
 #pragma unroll
       for (int i2 = 0; i2 < RB * EPP; ++i2) {
@@ -514,6 +537,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
         em[r] = qsby::row_field(max(em[r], __shfl_xor_sync(0xFFFFFFFFu, em[r], 8)));
       }
       // the slot's contents are in registers (used above): refill it S tiles ahead
+      if (PAIRS) __syncwarp();
       {
         const uint64_t c2 = c + (uint64_t)S * grid;
         if (c2 < nunits) issue(xi, slot);
@@ -575,19 +599,19 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-template <int NT>
+template <int NT, bool PAIRS>
 static cudaError_t dense_ozaki_ws(void* amps, const TcParams& p, cudaStream_t st) {
   constexpr size_t smem = Ws<NT>::bytes;
   static bool attr_done = false;
   if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki_ws<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki_ws<NT, PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
   const uint64_t maxb = (uint64_t)num_sms(), nunits = p.ntiles / Ws<NT>::RB;
   if (nunits == 0) return cudaErrorInvalidValue;   // such passes go elsewhere (qs_api.cpp)
   const unsigned g = (unsigned)(nunits < maxb ? nunits : maxb);
-  k_dense_ozaki_ws<NT><<<g, kWsThreads, smem, st>>>(static_cast<double2*>(amps), p);
+  k_dense_ozaki_ws<NT, PAIRS><<<g, kWsThreads, smem, st>>>(static_cast<double2*>(amps), p);
   return cudaGetLastError();
 }
 
@@ -653,7 +677,7 @@ __device__ __forceinline__ bool wait_or_abort_warp(uint64_t* bar, uint32_t parit
 // Epilogue of one N block (32 columns, accumulators at tb): a thread's row, NC of
 // its columns from column c0 of the block on; csc0: their scales; addr(a): where
 // amplitude a of those goes.  Hands the accumulators back on tempty once read.
-template <int K, int NC, typename Addr>
+template <int K, int NC, bool PAIRS, typename Addr>
 __device__ __forceinline__ void epilogue_block(uint32_t tb, uint64_t* tempty, const int* csc0, int egs, bool row_ok,
                                                int lane, const Addr& addr) {
 #pragma unroll
@@ -678,23 +702,48 @@ __device__ __forceinline__ void epilogue_block(uint32_t tb, uint64_t* tempty, co
         for (int L = 0; L < kLv; ++L) u[L] = v[L][q];
         o[q] = finish_output<K>(u, egs, scl[q]);
       }
+      if (PAIRS) {
+        store_pair(addr(cc >> 1), o);
+      } else {
 #pragma unroll
-      for (int q = 0; q < 4; q += 2) *addr((cc + q) >> 1) = make_double2(o[q], o[q + 1]);
+        for (int q = 0; q < 4; q += 2) *addr((cc + q) >> 1) = make_double2(o[q], o[q + 1]);
+      }
     }
   }
 }
 
-// the words of four amplitudes of a row (zeros beyond the last row)
-template <typename Addr>
+// Two neighbouring amplitudes at once.  With qubit 0 a target, an amplitude by itself
+// uses half of a 32-byte sector, and its other half is read or written again by the
+// thread's next access.
+__device__ __forceinline__ void load_pair(const double2* at, double2* v) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(v[0].x), "=d"(v[0].y), "=d"(v[1].x), "=d"(v[1].y)
+               : "l"(at)
+               : "memory");
+}
+
+// the words of four amplitudes of a row (zeros beyond the last row); PAIRS: amplitudes
+// 0, 1 and 2, 3 are neighbours in memory
+template <bool PAIRS, typename Addr>
 __device__ __forceinline__ void load_four(uint32_t (*R)[4], bool row_ok, const Addr& addr) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    double2 v = make_double2(0.0, 0.0);
-    if (row_ok) v = *addr(i);
-    R[i][0] = (uint32_t)__double2hiint(v.x);
-    R[i][1] = (uint32_t)__double2loint(v.x);
-    R[i][2] = (uint32_t)__double2hiint(v.y);
-    R[i][3] = (uint32_t)__double2loint(v.y);
+  for (int i = 0; i < 4; i += 2) {
+    double2 v[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+    if (row_ok) {
+      if (PAIRS) {
+        load_pair(addr(i), v);
+      } else {
+        v[0] = *addr(i);
+        v[1] = *addr(i + 1);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      R[i + e][0] = (uint32_t)__double2hiint(v[e].x);
+      R[i + e][1] = (uint32_t)__double2loint(v[e].x);
+      R[i + e][2] = (uint32_t)__double2hiint(v[e].y);
+      R[i + e][3] = (uint32_t)__double2loint(v[e].y);
+    }
   }
 }
 
@@ -726,6 +775,7 @@ struct W5 {
 };
 }  // namespace
 
+template <bool PAIRS>
 __global__ void __launch_bounds__(W5::THREADS, 1)
     k_dense_ozaki5(double2* __restrict__ psi, const __grid_constant__ TcParams p) {
   using X = W5;
@@ -810,7 +860,7 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
         bad = wait_or_abort_warp(accfull + nb, it & 1u, abort_flag);
         if (bad) break;
         fence_after_sync();
-        epilogue_block<K, 16>(tmem + (uint32_t)(256 * nb + 16 * h) + lane_addr, tempty + nb, csc + 32 * nb + 16 * h, egs,
+        epilogue_block<K, 16, PAIRS>(tmem + (uint32_t)(256 * nb + 16 * h) + lane_addr, tempty + nb, csc + 32 * nb + 16 * h, egs,
                               row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 8 * h + a]); });
       }
     }
@@ -824,7 +874,7 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
     uint64_t rb = xb | roff;
 #pragma unroll
     for (int kb = 0; kb < KB; ++kb)
-      load_four(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
+      load_four<PAIRS>(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
     uint32_t it = 0;
     bool bad = false;
     for (uint64_t c = blockIdx.x; c < p.ntiles; c += grid, ++it) {
@@ -851,7 +901,7 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(afull + kb);
-        if (has_next) load_four(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
+        if (has_next) load_four<PAIRS>(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
       }
     }
   } else if (lane == 0) {
@@ -888,16 +938,17 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
+template <bool PAIRS>
 static cudaError_t dense_ozaki5(void* amps, const TcParams& p, cudaStream_t st) {
   static bool attr_done = false;
   if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki5, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W5::bytes);
+    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki5<PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W5::bytes);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
   const uint64_t maxb = (uint64_t)num_sms();
   const unsigned g = (unsigned)(p.ntiles < maxb ? p.ntiles : maxb);
-  k_dense_ozaki5<<<g, W5::THREADS, W5::bytes, st>>>(static_cast<double2*>(amps), p);
+  k_dense_ozaki5<PAIRS><<<g, W5::THREADS, W5::bytes, st>>>(static_cast<double2*>(amps), p);
   return cudaGetLastError();
 }
 
@@ -979,10 +1030,11 @@ __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcP
   if (k == 0) reinterpret_cast<int*>(out + kWideScale)[n] = column_scale((int)ef);
 }
 
+template <bool PAIRS>
 __global__ void __launch_bounds__(W6::THREADS, 1)
     k_dense_ozaki6(double2* __restrict__ psi, const __grid_constant__ TcParams p, const unsigned char* __restrict__ wide) {
   using X = W6;
-  constexpr int K = X::K, KB = X::KB, PAIRS = 2;
+  constexpr int K = X::K, KB = X::KB, NPASS = 2;
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* a_dig = smem;
   unsigned char* b_dig = smem + X::b_off;
@@ -1048,7 +1100,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
     uint64_t rb = xb | roff;
 #pragma unroll
     for (int kb = 0; kb < KB; ++kb)
-      load_four(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
+      load_four<PAIRS>(R + 4 * kb, row_ok, [&](int i) { return psi + (rb | toff[16 * kb + 4 * cg + i]); });
     uint32_t it = 0;
     for (uint64_t c = blockIdx.x; c < p.ntiles; c += grid, ++it) {
       const uint32_t slot = it % 3;
@@ -1065,7 +1117,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
       xb = ((xb | hole) + gstep) & ~hole;
       const uint64_t rb_next = xb | roff;
 #pragma unroll
-      for (int np = 0; np < PAIRS; ++np) {
+      for (int np = 0; np < NPASS; ++np) {
 #pragma unroll
         for (int j = 0; j < KB; ++j) {
           if (np > 0 && j < 2) continue;      // still in the operand buffers
@@ -1078,7 +1130,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
           if (lane == 0) mbar_arrive(afull + b);
           // the last use of these registers in this tile
           if (has_next && (np > 0 || kb >= 2))
-            load_four(R + 4 * kb, row_ok, [&](int i) { return psi + (rb_next | toff[16 * kb + 4 * cg + i]); });
+            load_four<PAIRS>(R + 4 * kb, row_ok, [&](int i) { return psi + (rb_next | toff[16 * kb + 4 * cg + i]); });
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -1086,7 +1138,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
           bad |= wait_or_abort_warp(accfull + h, reads[h] & 1u, abort_flag);
           ++reads[h];
           fence_after_sync();
-          epilogue_block<K, 8>(tmem + (uint32_t)(256 * h + 8 * cg) + lane_addr, tempty + h, csc + 32 * nb + 8 * cg, (int)ef,
+          epilogue_block<K, 8, PAIRS>(tmem + (uint32_t)(256 * h + 8 * cg) + lane_addr, tempty + h, csc + 32 * nb + 8 * cg, (int)ef,
                                row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 4 * cg + a]); });
         }
       }
@@ -1097,7 +1149,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
     uint32_t fills[2] = {0, 0}, writes[2] = {0, 0}, nblk = 0;
     bool bad = false;
     for (uint64_t c = blockIdx.x; c < p.ntiles && !bad; c += grid)
-      for (int np = 0; np < PAIRS && !bad; ++np)
+      for (int np = 0; np < NPASS && !bad; ++np)
         for (int j = 0; j < KB && !bad; ++j) {
           const int kb = k_block(np, j), b = kb & 1;
           if (np == 0 || j >= 2) {
@@ -1131,7 +1183,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
     uint32_t nblk = 0;
     bool bad = false;
     for (uint64_t c = blockIdx.x; c < p.ntiles && !bad; c += grid)
-      for (int np = 0; np < PAIRS && !bad; ++np)
+      for (int np = 0; np < NPASS && !bad; ++np)
         for (int j = 0; j < KB && !bad; ++j)
           for (int h = 0; h < 2; ++h, ++nblk) {
             const uint32_t slot = nblk & 3u;
@@ -1153,10 +1205,11 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
+template <bool PAIRS>
 static cudaError_t dense_ozaki6(void* amps, const TcParams& p, void* scratch, cudaStream_t st) {
   static bool attr_done = false;
   if (!attr_done) {
-    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki6, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W6::bytes);
+    cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki6<PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W6::bytes);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
@@ -1164,18 +1217,29 @@ static cudaError_t dense_ozaki6(void* amps, const TcParams& p, void* scratch, cu
   k_wide_matrix<<<W6::K, W6::K, 0, st>>>(p, wide);
   const uint64_t maxb = (uint64_t)num_sms();
   const unsigned g = (unsigned)(p.ntiles < maxb ? p.ntiles : maxb);
-  k_dense_ozaki6<<<g, W6::THREADS, W6::bytes, st>>>(static_cast<double2*>(amps), p, wide);
+  k_dense_ozaki6<PAIRS><<<g, W6::THREADS, W6::bytes, st>>>(static_cast<double2*>(amps), p, wide);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st) {
+template <bool PAIRS>
+static cudaError_t dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st) {
   switch (p.n) {
-    case 3: return dense_ozaki_ws<3>(amps, p, st);
-    case 4: return dense_ozaki_ws<4>(amps, p, st);
-    case 5: return dense_ozaki5(amps, p, st);
-    case 6: return dense_ozaki6(amps, p, scratch, st);
+    case 3: return dense_ozaki_ws<3, PAIRS>(amps, p, st);
+    case 4: return dense_ozaki_ws<4, PAIRS>(amps, p, st);
+    case 5: return dense_ozaki5<PAIRS>(amps, p, st);
+    case 6: return dense_ozaki6<PAIRS>(amps, p, scratch, st);
     default: return cudaErrorInvalidValue;
   }
+}
+
+// With qubit 0 a target, amplitudes 2 i and 2 i + 1 of a row are neighbours in memory:
+// they move together (32 bytes, a whole sector).  28 qubits, ms, one by one / in
+// pairs: 3, 4, 5, 6 targets on qubits 0, 1, ...: 2.50 / 2.27, 3.01 / 2.34, 3.32 / 2.73, 5.03 / 4.33; on
+// qubit 0 and high ones: 1.94 / 1.71, 1.99 / 1.77, 2.25 / 2.20, 3.92 / 3.86.  Other
+// passes keep the plain form: the exchange costs the producers up to 8% there.
+cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st) {
+  if (p.tpos[0] == 0 && p.tile_bits > p.n) return dense_ozaki<true>(amps, p, scratch, st);
+  return dense_ozaki<false>(amps, p, scratch, st);
 }
 
 }  // namespace qsk
