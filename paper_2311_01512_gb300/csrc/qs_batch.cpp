@@ -15,6 +15,10 @@
 // targets, gadget X/Y qubits) together with the five lowest qubits fit in a
 // tile of L qubits; the kernel then moves each tile through shared memory once
 // per segment instead of moving the state once per operation.
+//
+// complex64 states of at least a tile of qs_tile.h whose operations fit its passes
+// can take those instead: launch k runs the k-th pass of every such state, one block
+// per tile, while a second branch of the graph runs the other states.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -28,6 +32,7 @@
 #include "qs_alloc.h"
 #include "qs_internal.h"
 #include "qs_batch_plan.h"
+#include "qs_tile.h"
 
 struct qs_batch {
   qs_prec prec = QS_C64;
@@ -47,11 +52,16 @@ struct qs_batch {
   qsk::BatchOp* d_ops = nullptr;
   double* d_consts = nullptr;
   int* d_counter = nullptr;
+  // tile passes: packed descriptors, blocks of launch k at [level[k], level[k + 1])
+  unsigned char* d_passes = nullptr;
+  qstile::TileItem* d_items = nullptr;
+  std::vector<int> level;
   long num_segs = 0;
   int wide = 0;                 // some operation is dense on 3 or 4 targets
   int threads = 256, ctas = 0, smem_qubits = -1;
-  int cluster = 1, nheavy = 0;  // heavy states (first in the order) are shared by clusters of CTAs
+  int cluster = 1;              // heavy states (first in the order) are shared by clusters of CTAs
   cudaStream_t capture_stream = nullptr;  // own stream for recording (the caller's may be the legacy stream)
+  cudaStream_t branch_stream = nullptr;   // and for the graph's second branch
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool compiled = false;
@@ -65,7 +75,7 @@ void free_device(qs_batch* b) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   for (void* p : {(void*)b->d_states, (void*)b->d_segs, (void*)b->d_xlat, (void*)b->d_order, (void*)b->d_ops,
-                  (void*)b->d_consts, (void*)b->d_counter})
+                  (void*)b->d_consts, (void*)b->d_counter, (void*)b->d_passes, (void*)b->d_items})
     if (p) cudaFree(p);
   b->d_consts = nullptr;
   b->exec = nullptr;
@@ -76,6 +86,9 @@ void free_device(qs_batch* b) {
   b->d_order = nullptr;
   b->d_ops = nullptr;
   b->d_counter = nullptr;
+  b->d_passes = nullptr;
+  b->d_items = nullptr;
+  b->level.clear();
   b->compiled = false;
 }
 
@@ -201,6 +214,43 @@ bool upload_plan(Plan& P) {
                                       cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
+// The tile passes of a state, none if it has an operation that does not fit.
+void tile_passes(const qs_batch* b, int s, std::vector<qstile::TilePass>* out) {
+  out->clear();
+  const std::vector<qsk::BatchOp>& prog = b->progs[(size_t)s];
+  std::vector<std::vector<int>> lists(3 * prog.size());     // controls, targets, Paulis
+  std::vector<qstile::Gate> gates;
+  for (size_t i = 0; i < prog.size(); ++i) {
+    const qsk::BatchOp& op = prog[i];
+    std::vector<int>&c = lists[3 * i], &t = lists[3 * i + 1], &pl = lists[3 * i + 2];
+    const double* data = b->consts[(size_t)s].data() + op.coff;
+    qstile::Gate g;
+    g.kind = op.kind;
+    if (op.kind == 2) {
+      for (int q = 0; q < b->nq[(size_t)s]; ++q)
+        if ((op.xy | op.yz) >> q & 1) {
+          t.push_back(q);
+          pl.push_back((op.xy >> q & 1) ? ((op.yz >> q & 1) ? 2 : 1) : 3);
+        }
+      g.c = data[0];
+      g.s = data[1];
+    } else {
+      t.assign(op.t, op.t + op.n);
+      for (int q = 0; q < b->nq[(size_t)s]; ++q)
+        if (op.ctrl >> q & 1) c.push_back(q);
+      g.data = data;
+    }
+    g.ctrls = &c;
+    g.targs = &t;
+    g.paulis = &pl;
+    for (int q : c) g.qmask |= 1ull << q;
+    for (int q : t) g.qmask |= 1ull << q;
+    if (!qstile::fits(g, b->nq[(size_t)s])) return;
+    gates.push_back(g);
+  }
+  qstile::build_passes(gates, b->nq[(size_t)s], out);
+}
+
 // Two-qubit channels on the members of (t1, t2, t1 + N, t2 + N): member bits
 // 0, 1 are t1, t2 and bits 2, 3 are t1 + N, t2 + N.
 qs_status add_channel2(qs_batch* b, int state, int t1, int t2, bool depol, double p) {
@@ -254,6 +304,7 @@ qs_status qs_batch_destroy(qs_batch* b) {
   if (!b) return QS_ERR_ARG;
   free_device(b);
   if (b->capture_stream) cudaStreamDestroy(b->capture_stream);
+  if (b->branch_stream) cudaStreamDestroy(b->branch_stream);
   delete b;
   return QS_OK;
 }
@@ -431,12 +482,50 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
       heavy[s] = 1;
       ++nheavy;
     }
+  // tile passes, level by level: pass k of every state that has one
+  std::vector<char> tiled(S, 0);
+  std::vector<unsigned char> passes;         // packed
+  std::vector<qstile::TileItem> items;
+  if (b->prec == QS_C64) {
+    std::vector<std::vector<uint32_t>> of(S);   // where a state's passes start
+    std::vector<qstile::TilePass> mine;
+    size_t levels = 0;
+    for (int s = 0; s < S; ++s) {
+      tile_passes(b, s, &mine);
+      if (mine.empty()) continue;
+      tiled[s] = 1;
+      for (const auto& p : mine) {
+        of[s].push_back((uint32_t)(passes.size() / 16));
+        qstile::pack(p, &passes);
+      }
+      levels = std::max(levels, of[s].size());
+    }
+    for (size_t k = 0; k < levels; ++k) {
+      b->level.push_back((int)items.size());
+      for (int s = 0; s < S; ++s)
+        if (k < of[s].size())
+          for (uint32_t t = 0; t < 1u << (b->nq[s] - qstile::kPassBits); ++t)
+            items.push_back(qstile::TileItem{b->offset[s], of[s][k], t});
+    }
+    b->level.push_back((int)items.size());
+  }
+  // largest first, heavy ones before the others; a second list without the tiled states
   std::vector<int> order(S);
   for (int s = 0; s < S; ++s) order[s] = s;
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
     return heavy[x] != heavy[y] ? heavy[x] > heavy[y] : work[x] > work[y];
   });
-  if (qsalloc::device(reinterpret_cast<void**>(&b->d_order), sizeof(int) * S) != cudaSuccess ||
+  int rest = 0, rest_heavy = 0;
+  for (int i = 0; i < S; ++i)
+    if (const int s = order[i]; !tiled[s]) {
+      order.push_back(s);
+      ++rest;
+      rest_heavy += heavy[s];
+    }
+  if (qsalloc::device(reinterpret_cast<void**>(&b->d_order), sizeof(int) * order.size()) != cudaSuccess ||
+      (!passes.empty() &&
+       (qsalloc::device(reinterpret_cast<void**>(&b->d_passes), passes.size()) != cudaSuccess ||
+        qsalloc::device(reinterpret_cast<void**>(&b->d_items), sizeof(qstile::TileItem) * items.size()) != cudaSuccess)) ||
       qsalloc::device(reinterpret_cast<void**>(&b->d_ops), sizeof(qsk::BatchOp) * std::max<size_t>(1, ops.size())) != cudaSuccess ||
       qsalloc::device(reinterpret_cast<void**>(&b->d_consts), sizeof(double) * std::max<size_t>(1, consts.size())) != cudaSuccess ||
       qsalloc::device(reinterpret_cast<void**>(&b->d_counter), 2 * sizeof(int)) != cudaSuccess) {
@@ -444,7 +533,10 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
     free_device(b);
     return QS_ERR_OOM;
   }
-  if (cudaMemcpy(b->d_order, order.data(), sizeof(int) * S, cudaMemcpyHostToDevice) != cudaSuccess ||
+  if (cudaMemcpy(b->d_order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+      (!passes.empty() &&
+       (cudaMemcpy(b->d_passes, passes.data(), passes.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(b->d_items, items.data(), sizeof(qstile::TileItem) * items.size(), cudaMemcpyHostToDevice) != cudaSuccess)) ||
       (!ops.empty() &&
        cudaMemcpy(b->d_ops, ops.data(), sizeof(qsk::BatchOp) * ops.size(), cudaMemcpyHostToDevice) != cudaSuccess) ||
       (!consts.empty() && cudaMemcpy(b->d_consts, consts.data(), sizeof(double) * consts.size(),
@@ -460,16 +552,22 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
   }
   struct Shape {
     int threads, per_sm, cluster;
+    bool tiles;            // tile passes, and this launch for the rest
   };
   std::vector<Shape> cands;
   if (autotune) {
-    cands = {{128, 4, 1}, {256, 2, 1}, {256, 4, 1}, {512, 1, 1}, {512, 2, 1}};
+    cands = {{128, 4, 1, false}, {256, 2, 1, false}, {256, 4, 1, false}, {512, 1, 1, false}, {512, 2, 1, false}};
     // 512 complex64 states of 10-17 qubits: 1.54 ms without clusters, 1.22-1.38
     // in clusters of 2 and 4, 1.68 of 8; 256 complex128 states, a quarter of them
     // density matrices: 7.69, 3.75, 1.91 and 1.82 ms
-    if (nheavy) cands.insert(cands.end(), {{512, 1, 2}, {512, 1, 4}, {256, 2, 4}, {256, 2, 8}});
+    if (nheavy)
+      cands.insert(cands.end(), {{512, 1, 2, false}, {512, 1, 4, false}, {256, 2, 4, false}, {256, 2, 8, false}});
+    // tile passes: the 512 states in 0.67 ms
+    if (!passes.empty()) cands.push_back({256, 2, rest_heavy ? 4 : 1, true});
+  } else if (!passes.empty()) {
+    cands = {{256, 2, rest_heavy ? 4 : 1, true}};
   } else {
-    cands = {{256, 2, nheavy ? 4 : 1}};
+    cands = {{256, 2, nheavy ? 4 : 1, false}};
   }
   std::vector<Plan> plans;
   plans.reserve(cands.size());       // pointers into it stay valid
@@ -488,15 +586,31 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
       return QS_ERR_OOM;
     }
   }
+  // the launches of a shape: the persistent one on st, the tile passes on tile_st
+  auto launch = [&](const Plan& P, int threads, int ctas, int sq, int cluster, bool tiles, cudaStream_t st,
+                    cudaStream_t tile_st) -> cudaError_t {
+    cudaError_t e = cudaSuccess;
+    const int n = tiles ? rest : S, nh = cluster > 1 ? (tiles ? rest_heavy : nheavy) : 0;
+    if (n > 0) {
+      e = cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(int), st);
+      if (e == cudaSuccess)
+        e = qsk::launch_batch(b->prec, b->pool, P.d_states, b->d_order + (tiles ? S : 0), n, nh, b->d_ops, b->d_consts,
+                              P.d_segs, P.d_xlat, b->d_counter, threads, ctas, sq, b->wide, cluster, st);
+    }
+    if (tiles)
+      for (size_t k = 0; k + 1 < b->level.size() && e == cudaSuccess; ++k)
+        e = qsk::launch_tile_items(b->pool, b->d_passes, b->d_items + b->level[k], b->level[k + 1] - b->level[k], tile_st);
+    return e;
+  };
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   float best = 1e30f;
   int best_plan = -1;
+  bool best_tiles = false;
   for (const auto& c : cands) {
     const int sq = smem_qubits_for(b->prec, c.per_sm);
     Plan* P = plan_for(sq, c.cluster);
-    const int nh = c.cluster > 1 ? nheavy : 0;
     int ctas = sms * c.per_sm;
     if (c.cluster > 1) {
       int n = 0;
@@ -506,10 +620,8 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
       }
       ctas = n * c.cluster;
     }
-    if (cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(int), b->stream) != cudaSuccess) return QS_ERR_CUDA;
     cudaEventRecord(e0, b->stream);
-    if (qsk::launch_batch(b->prec, b->pool, P->d_states, b->d_order, S, nh, b->d_ops, b->d_consts, P->d_segs, P->d_xlat,
-                          b->d_counter, c.threads, ctas, sq, b->wide, c.cluster, b->stream) != cudaSuccess) {
+    if (launch(*P, c.threads, ctas, sq, c.cluster, c.tiles, b->stream, b->stream) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -523,7 +635,7 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
       b->ctas = ctas;
       b->smem_qubits = sq;
       b->cluster = c.cluster;
-      b->nheavy = nh;
+      best_tiles = c.tiles;
       best_plan = (int)(P - plans.data());
     }
   }
@@ -539,19 +651,32 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
   b->best_ms = best;
   // record on the batch's own stream: reset the work counter, one persistent launch
   if (cudaStreamSynchronize(b->stream) != cudaSuccess) return QS_ERR_CUDA;
-  if (!b->capture_stream && cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking) != cudaSuccess)
-    return QS_ERR_CUDA;
+  for (cudaStream_t* st : {&b->capture_stream, &b->branch_stream})
+    if (!*st && cudaStreamCreateWithFlags(st, cudaStreamNonBlocking) != cudaSuccess) return QS_ERR_CUDA;
   if (cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();
     return QS_ERR_CUDA;
   }
-  cudaError_t e = cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(int), b->capture_stream);
+  // the persistent launch and the tile passes as two branches
+  const Plan& P = plans[best_plan];
+  const bool fork = best_tiles && rest > 0;
+  cudaEvent_t forked = nullptr, joined = nullptr;
+  cudaError_t e = cudaSuccess;
+  if (fork) {
+    e = cudaEventCreateWithFlags(&forked, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&joined, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(forked, b->capture_stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->branch_stream, forked, 0);
+  }
   if (e == cudaSuccess)
-    e = qsk::launch_batch(b->prec, b->pool, b->d_states, b->d_order, S, b->nheavy, b->d_ops, b->d_consts, b->d_segs,
-                          b->d_xlat, b->d_counter, b->threads, b->ctas, b->smem_qubits, b->wide, b->cluster,
-                          b->capture_stream);
+    e = launch(P, b->threads, b->ctas, b->smem_qubits, b->cluster, best_tiles, b->capture_stream,
+               fork ? b->branch_stream : b->capture_stream);
+  if (fork && e == cudaSuccess) e = cudaEventRecord(joined, b->branch_stream);
+  if (fork && e == cudaSuccess) e = cudaStreamWaitEvent(b->capture_stream, joined, 0);
   cudaGraph_t g = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(b->capture_stream, &g);
+  if (forked) cudaEventDestroy(forked);
+  if (joined) cudaEventDestroy(joined);
   if (e != cudaSuccess || e2 != cudaSuccess || !g) {
     cudaGetLastError();
     if (g) cudaGraphDestroy(g);

@@ -169,7 +169,8 @@ qstile::Gate tile_view(const CGate& g) {
   v.targs = &g.targs;
   v.paulis = &g.paulis;
   v.data = g.data.data();
-  v.theta = g.theta;
+  v.c = std::cos(-0.5 * g.theta);
+  v.s = std::sin(-0.5 * g.theta);
   v.qmask = g.qmask;
   return v;
 }

@@ -10,6 +10,7 @@
 
 namespace qstile {
 struct TilePass;
+struct TileItem;
 }
 
 namespace qsk {
@@ -433,6 +434,9 @@ cudaError_t launch_copy16(void* dst, const void* src, size_t bytes, cudaStream_t
 
 // one tile pass of a complex64 state (qs_tile.h)
 cudaError_t launch_tile_pass(void* amps, const qstile::TilePass& p, cudaStream_t st);
+// tiles of many complex64 states, one block each (device arrays; passes packed)
+cudaError_t launch_tile_items(void* pool, const unsigned char* passes, const qstile::TileItem* items, int nitems,
+                              cudaStream_t st);
 
 // Reductions: stage one writes one complex128 partial sum a block, stage two
 // sums them in a fixed order into result[0] (added to result[0] if accumulate) and,

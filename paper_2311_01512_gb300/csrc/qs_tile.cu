@@ -138,19 +138,22 @@ __device__ __forceinline__ uint64_t thread_offset(const TilePass& p, uint32_t ti
   return off;
 }
 
-__global__ void __launch_bounds__(kTileThreads, 4) k_tile_pass(float2* __restrict__ psi, const __grid_constant__ TilePass p) {
-  extern __shared__ __align__(16) unsigned char sm[];
-  float* coef = reinterpret_cast<float*>(sm + (sizeof(float2) << kPassBits));
+// Tile `tile` of the pass; coef: its coefficients in shared memory (COPY: copied there
+// from p, otherwise they are in place).
+template <bool COPY>
+__device__ __forceinline__ void run_tile(float2* __restrict__ psi, const TilePass& p, uint32_t tile, unsigned char* sm,
+                                         float* coef) {
   const uint32_t tid = threadIdx.x;
   uint64_t tb = 0;
-  for (int j = 0; j < p.nbrun; ++j) tb += (uint64_t)(blockIdx.x & p.brun[j].mask) * p.brun[j].mul;
+  for (int j = 0; j < p.nbrun; ++j) tb += (uint64_t)(tile & p.brun[j].mask) * p.brun[j].mul;
   {
     float2* const mine = psi + (tb + thread_offset(p, tid));   // tile index r << kThreadBits | tid is at mine[p.off[r]]
     const uint32_t home = slot(tid) * 8;
     float2 v[kSweepAmps];
 #pragma unroll
     for (int r = 0; r < kSweepAmps; ++r) v[r] = mine[p.off[r]];
-    for (uint32_t e = tid; e < p.ncoef; e += kTileThreads) coef[e] = p.coef[e];
+    if (COPY)
+      for (uint32_t e = tid; e < p.ncoef; e += kTileThreads) coef[e] = p.coef[e];
 #pragma unroll
     for (int r = 0; r < kSweepAmps; ++r)
       *reinterpret_cast<float2*>(sm + (home ^ slot((uint32_t)r << kThreadBits) * 8)) = v[r];
@@ -218,7 +221,48 @@ __global__ void __launch_bounds__(kTileThreads, 4) k_tile_pass(float2* __restric
     mine[p.off[r]] = *reinterpret_cast<const float2*>(sm + (home ^ slot((uint32_t)r << kThreadBits) * 8));
 }
 
+__global__ void __launch_bounds__(kTileThreads, 4) k_tile_pass(float2* __restrict__ psi, const __grid_constant__ TilePass p) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  run_tile<true>(psi, p, blockIdx.x, sm, reinterpret_cast<float*>(sm + (sizeof(float2) << kPassBits)));
+}
+
+// The same over the tiles of many states: packed passes, copied to shared memory.
+__global__ void __launch_bounds__(kTileThreads, 4)
+    k_tile_items(float2* __restrict__ pool, const unsigned char* __restrict__ passes, const TileItem* __restrict__ items) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const TileItem it = items[blockIdx.x];
+  const unsigned char* from = passes + (size_t)it.pass * 16;
+  const TilePass& head = *reinterpret_cast<const TilePass*>(from);
+  TilePass& p = *reinterpret_cast<TilePass*>(sm + (sizeof(float2) << kPassBits));
+  auto copy = [&](void* to, uint32_t bytes) {
+    for (uint32_t e = threadIdx.x; e < padded(bytes) / 16; e += kTileThreads)
+      static_cast<uint4*>(to)[e] = reinterpret_cast<const uint4*>(from)[e];
+    from += padded(bytes);
+  };
+  const uint32_t ns = head.nsweeps, no = head.nops, nc = head.ncoef;
+  copy(&p, kHeadBytes);
+  copy(p.sweep, ns * (uint32_t)sizeof(TileSweep));
+  copy(p.op, no * (uint32_t)sizeof(TileOp));
+  copy(p.coef, nc * (uint32_t)sizeof(float));
+  __syncthreads();
+  run_tile<false>(pool + it.offset, p, it.tile, sm, p.coef);
+}
+
 }  // namespace
+
+cudaError_t launch_tile_items(void* pool, const unsigned char* passes, const qstile::TileItem* items, int nitems,
+                              cudaStream_t st) {
+  constexpr size_t smem = (sizeof(float2) << kPassBits) + sizeof(TilePass);
+  static_assert(4 * (smem + 1024) <= 227 * 1024 && kHeadBytes % 16 == 0, "shared memory");
+  static bool attr_done = false;
+  if (!attr_done) {
+    const cudaError_t e = cudaFuncSetAttribute(k_tile_items, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr_done = true;
+  }
+  k_tile_items<<<nitems, kTileThreads, smem, st>>>(static_cast<float2*>(pool), passes, items);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_tile_pass(void* amps, const qstile::TilePass& p, cudaStream_t st) {
   static bool attr_done = false;

@@ -16,7 +16,7 @@
 // skipped ones when nothing in between touches their qubits.
 #pragma once
 
-#include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <cstring>
 #include <utility>
@@ -75,10 +75,33 @@ struct TilePass {
   int8_t P[kPassBits];             // qubit of tile bit b, ascending; 0..kPassLow-1 first
   uint8_t nbrun, ntrun;
   uint32_t nsweeps, nops, ncoef;
-  TileSweep sweep[kMaxOps];
-  TileOp op[kMaxOps];
-  float coef[kMaxCoef];
+  alignas(16) TileSweep sweep[kMaxOps];
+  alignas(16) TileOp op[kMaxOps];
+  alignas(16) float coef[kMaxCoef];
 };
+
+// One block of a launch over many states: a tile of a pass.
+struct TileItem {
+  uint64_t offset;                 // of the state's first amplitude
+  uint32_t pass, tile;             // pass: where its packed form starts, in units of 16 bytes
+};
+
+QT_HD constexpr uint32_t padded(uint32_t bytes) { return (bytes + 15) & ~15u; }
+constexpr uint32_t kHeadBytes = offsetof(TilePass, sweep);
+
+// Appends a pass without its unused parts: head, sweeps, operations, coefficients,
+// each padded to 16 bytes (about 2 KB where the whole struct has 8.7).
+inline void pack(const TilePass& p, std::vector<unsigned char>* out) {
+  auto put = [&](const void* from, uint32_t bytes) {
+    const unsigned char* f = static_cast<const unsigned char*>(from);
+    out->insert(out->end(), f, f + bytes);
+    out->resize(padded((uint32_t)bytes) - bytes + out->size());
+  };
+  put(&p, kHeadBytes);
+  put(p.sweep, (uint32_t)sizeof(TileSweep) * p.nsweeps);
+  put(p.op, (uint32_t)sizeof(TileOp) * p.nops);
+  put(p.coef, (uint32_t)sizeof(float) * p.ncoef);
+}
 
 // Shared-memory slot of tile index i: the bank bits 0..3 (8-byte words) fold in
 // every higher bit, so that lanes along any four suitable bits meet each bank once.
@@ -88,7 +111,7 @@ struct Gate {
   int kind = 0;                    // 0 dense, 1 diagonal, 2 gadget
   const std::vector<int>*ctrls = nullptr, *targs = nullptr, *paulis = nullptr;
   const double* data = nullptr;
-  double theta = 0.0;
+  double c = 1.0, s = 0.0;         // gadget: cos and sin of phi = -theta / 2
   uint64_t qmask = 0;
 };
 
@@ -252,13 +275,12 @@ inline void finish_sweep(TilePass& p, TileSweep& sw, const std::vector<Gate>& gs
       op.yzg = yz & ~inside;
       op.yzl = tile_mask(yz);
       for (int k = 0; k < kSweepDim; ++k) op.sgn |= (uint32_t)parity(v[k] & op.yzl) << k;
-      const double phi = -0.5 * g.theta;
       // exp(i phi P): c a_i + s i^q a_j, j = i ^ xy, with the sign of parity(j & yz):
       // register 0 pairs with register m
       const int q = (ny + 1 + 2 * parity(sw.comb[m] & op.yzl)) & 3;
       op.k = m | (uint32_t)(q & 1) << 4;
-      op.c = (float)std::cos(phi);
-      op.s = (float)(q >= 2 ? -std::sin(phi) : std::sin(phi));
+      op.c = (float)g.c;
+      op.s = (float)(q >= 2 ? -g.s : g.s);
     }
   }
 }

@@ -43,7 +43,8 @@ static void make(Circuit& c, int n, int count, std::mt19937_64& rng) {
     for (int k = 0; k < nt; ++k) c.paulis[i].push_back((int)(rng() % 4));
     const int m = g.kind == 0 ? 2 << (2 * nt) : 2 << nt;
     for (int k = 0; k < m; ++k) c.data[i].push_back((float)(nd(rng) / (g.kind == 0 ? std::sqrt(2.0 * (1 << nt)) : 1.4)));
-    g.theta = nd(rng);
+    const double phi = -0.5 * nd(rng);
+    g.c = std::cos(phi), g.s = std::sin(phi);
     g.ctrls = &c.ctrls[i], g.targs = &c.targs[i], g.paulis = &c.paulis[i], g.data = c.data[i].data();
     for (int k = 0; k < nt + nc; ++k) g.qmask |= 1ull << q[k];
     c.gates.push_back(g);
@@ -84,9 +85,8 @@ static void direct(const Gate& g, std::vector<cd>& a) {
         ny += p == 2;
       }
       static const cd ipow[4] = {{1, 0}, {0, 1}, {-1, 0}, {0, -1}};
-      const double phi = -0.5 * g.theta;
       const size_t k = i ^ xy;
-      o[i] = std::cos(phi) * a[i] + ipow[(ny + 1) & 3] * std::sin(phi) * (parity(k & yz) ? -1.0 : 1.0) * a[k];
+      o[i] = g.c * a[i] + ipow[(ny + 1) & 3] * g.s * (parity(k & yz) ? -1.0 : 1.0) * a[k];
     }
   }
   a.swap(o);
