@@ -36,8 +36,8 @@ ARITH_CODE = {"fx": 2, "df": 0, "f64": 1}     # qs_arith
 DTYPE = {
     "fx": ("c128 storage; arithmetic at least FP64: one- and two-target gates, diagonals and gadgets in 60-bit "
            "block fixed point with exact integer products and one rounding per output (error <= 2^-53 |y| + "
-           "2^-55 max|x| max|m|, 2^-54 for the two-target gates' eight terms), 3-5-target gates as eight exact "
-           "7-bit slices (56-bit operands) on the bf16 tensor cores"),
+           "2^-55 max|x| max|m|, 2^-54 for the two-target gates' eight terms), 3-6-target gates as exact "
+           "byte slices (55-bit amplitudes, 62-bit matrices) on the fp16 tensor cores"),
     "df": "c128 storage, double-float (2xf32, 47-bit) arithmetic",
     "f64": "c128 storage, native f64 arithmetic",
 }
@@ -70,7 +70,7 @@ def parse_args(argv=None):
     ap.add_argument("--fused-max-block", type=int, default=6,
                     help="widest fused block the cost-model planner may form (6 on complex64; complex128 stops at 5)")
     ap.add_argument("--fused-prec", choices=("c64", "c128"), default="c64",
-                    help="precision of the fused form: complex64 (3xTF32 blocks) or complex128 (bf16 integer slices)")
+                    help="precision of the fused form: complex64 (3xTF32 blocks) or complex128 (fp16 byte slices)")
     ap.add_argument("--detail", default="", help="write per-kernel-family statistics to this JSON file")
     ap.add_argument("--cpu-sample", type=int, default=0, help=argparse.SUPPRESS)
     return ap.parse_args(argv)

@@ -269,8 +269,10 @@ qs_status qs_expec_pauli_sum(const qs_state* state, const int* paulis, const dou
  * at most max_block_qubits (<= QS_MAX_DENSE_TARGETS) qubits.  Each block of
  * two or more gates is composed on the device into one dense matrix in FP64
  * and applied as a single dense gate (tensor cores for complex64 blocks of
- * 3..5 qubits, the handle's complex128 arithmetic otherwise); a one-gate block
- * runs that gate's own kernel.  Not in the paper: this groups the paper's
+ * 3..6 qubits, the handle's complex128 arithmetic otherwise); a one-gate block
+ * runs that gate's own kernel.  Where it is faster, complex64 statevectors take
+ * runs of blocks gate by gate in shared-memory tiles (the plan has to hold a
+ * fused block; matrices are FP32 there, products and sums FP32).  Not in the paper: this groups the paper's
  * many-target gate updates (Sec. "Many-target gate") so that each pass over
  * the state does more work.  The applied operation is the same up to rounding.
  * ------------------------------------------------------------------------ */
