@@ -562,7 +562,7 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
     // density matrices: 7.69, 3.75, 1.91 and 1.82 ms
     if (nheavy)
       cands.insert(cands.end(), {{512, 1, 2, false}, {512, 1, 4, false}, {256, 2, 4, false}, {256, 2, 8, false}});
-    // tile passes: the 512 states in 0.67 ms
+    // tile passes: the 512 states in 0.61 ms
     if (!passes.empty()) cands.push_back({256, 2, rest_heavy ? 4 : 1, true});
   } else if (!passes.empty()) {
     cands = {{256, 2, rest_heavy ? 4 : 1, true}};

@@ -176,9 +176,9 @@ qstile::Gate tile_view(const CGate& g) {
 }
 
 // Time of a gate inside a tile pass, in passes over the state (96 gates of a kind
-// at 27 qubits, us a gate over the 316 of a read and a write: one target 62, two
-// targets 107, gadgets 53, diagonals 60).
-double tile_cost(const CGate& g) { return g.kind == 0 ? (g.targs.size() == 1 ? 0.2 : 0.34) : g.kind == 1 ? 0.19 : 0.17; }
+// at 27 qubits, us a gate over the 316 of a read and a write: one target 52, two
+// targets 111, gadgets 52, diagonals 62).
+double tile_cost(const CGate& g) { return g.kind == 0 ? (g.targs.size() == 1 ? 0.16 : 0.35) : g.kind == 1 ? 0.19 : 0.17; }
 
 // Time of a block on its own kernel: a dense block is bound by its operand
 // preparation from four qubits on (29 qubits, ms: 3 qubits 1.28, 4 1.57, 5 1.63, 6
@@ -192,8 +192,8 @@ double block_cost(const qs_circuit* c, const CBlock& b) {
 // Finds the plan's runs of blocks that complex64 statevectors take in tile passes.
 // A block stays a block if a gate of it does not fit a tile, or if it has so many
 // gates that one dense pass is faster than the gates in a tile (96 gates on six
-// qubits: 1.8 ms in four blocks, 5.9 ms in tile passes at 27 qubits; 96 gates on
-// all qubits: 22 ms and 7.6 ms for gadgets, 6.4 and 6.3 for one-target gates).
+// qubits: 1.8 ms in four blocks, 4.9 ms in tile passes at 27 qubits; 96 gates on
+// all qubits: 22 ms and 7.6 ms for gadgets, 6.4 and 5.1 for one-target gates).
 // From the smallest state that has a tile on, fewer launches win too (150 gates at
 // 13 qubits: 0.62 ms and 0.13).
 void find_runs(qs_circuit* c) {

@@ -1,16 +1,17 @@
 // Tile passes of planned complex64 circuits (qs_tile.h): one block per tile reads
 // 2^12 amplitudes into shared memory, runs the pass's sweeps and writes them back.
 //
-// What bounds it: instruction issue (2.6 of 4 a clock), then the FP32 pipe; a pass
-// by itself costs one read and one write of the state (1.27 ms at 29 qubits), and
-// for 16 amplitudes a sweep adds 16 shared loads, 16 stores and some 50 index
-// instructions a thread, a one-target gate 128 multiply-adds, a two-target gate
-// 256, a gadget 64 and 15 for signs.  150 random gates at 29 qubits, 17 passes: 48
-// ms, against 97 (blocks of six qubits) to 127 (of three) in dense blocks.
+// What bounds it: instruction issue (about two thirds of the slots), then the FP32
+// pipe; a pass by itself costs one read and one write of the state (1.27 ms at 29
+// qubits), and for 16 amplitudes a sweep adds 16 shared loads, 16 stores and some 50
+// index instructions a thread, a one-target gate 64 packed multiply-adds and 32 moves,
+// a two-target gate 128 and 32, a gadget 64 (32 with an odd number of Y) and 15 for
+// signs.  150 random gates at 29 qubits, 17 passes: 44.6 ms, 48.0 with one operation an
+// instruction, against 97 (blocks of six qubits) to 127 (of three) in dense blocks.
 // Four 256-thread blocks a multiprocessor (64 registers a thread): one block's
 // sweeps run while the others' loads and stores are in flight (tiles of 2^13 with
-// two 512-thread blocks, 15 passes: 49.7 ms).  Matrices come from shared memory:
-// indexed reads of the constant bank took 82 ms.
+// two 512-thread blocks, 15 passes: 49.7 against 48.0 ms).  Matrices come from shared
+// memory: indexed reads of the constant bank took 82 ms.
 #include "qs_device.cuh"
 #include "qs_internal.h"
 #include "qs_tile.h"
@@ -23,29 +24,42 @@ using namespace qstile;
 constexpr int kTileThreads = 1 << kThreadBits;
 constexpr size_t kTileSmem = (sizeof(float2) << kPassBits) + sizeof(float) * kMaxCoef;
 
-// Entries e and e + 1 of a complex matrix at shared address u (16-byte aligned).
-// Volatile: loaded where they are used, so that a matrix is not kept in 32
-// registers beside the 32 of the amplitudes.
-__device__ __forceinline__ float4 entries(uint32_t u, int e) {
-  float4 v;
-  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(u + 8 * e));
-  return v;
+// Two FP32 operations at once on a (re, im) pair.
+__device__ __forceinline__ unsigned long long& bits(float2& v) { return reinterpret_cast<unsigned long long&>(v); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(bits(d)) : "l"(bits(a)), "l"(bits(b)));
+  return d;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(bits(d)) : "l"(bits(a)), "l"(bits(b)), "l"(bits(c)));
+  return d;
+}
+
+// Entry e of a matrix at shared address u: (re, re) and (-im, im).  Volatile:
+// loaded where it is used, so that a matrix is not kept in registers beside the 32 of
+// the amplitudes.
+struct Entry {
+  float2 r, i;
+};
+__device__ __forceinline__ Entry entry(uint32_t u, int e) {
+  Entry m;
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(bits(m.r)), "=l"(bits(m.i)) : "r"(u + 16 * e));
+  return m;
 }
 
 // ok: bit r = the controls are set at register r (C; otherwise they are everywhere)
 template <int K, bool C>
 __device__ __forceinline__ void gate1(float2 (&a)[kSweepAmps], uint32_t u, uint32_t ok) {
-  const float4 m0 = entries(u, 0), m1 = entries(u, 2);
+  const Entry m0 = entry(u, 0), m1 = entry(u, 1), m2 = entry(u, 2), m3 = entry(u, 3);
 #pragma unroll
   for (int r = 0; r < kSweepAmps; ++r) {
     if (r >> K & 1) continue;
     if (C && !(ok >> r & 1u)) continue;
-    const float2 x = a[r], y = a[r | 1 << K];
-    a[r] = make_float2(m0.x * x.x - m0.y * x.y + m0.z * y.x - m0.w * y.y, m0.x * x.y + m0.y * x.x + m0.z * y.y + m0.w * y.x);
-    a[r | 1 << K] =
-        make_float2(m1.x * x.x - m1.y * x.y + m1.z * y.x - m1.w * y.y, m1.x * x.y + m1.y * x.x + m1.z * y.y + m1.w * y.x);
+    const float2 x = a[r], y = a[r | 1 << K], xs = make_float2(x.y, x.x), ys = make_float2(y.y, y.x);
+    a[r] = fma2(m1.i, ys, fma2(m1.r, y, fma2(m0.i, xs, mul2(m0.r, x))));
+    a[r | 1 << K] = fma2(m3.i, ys, fma2(m3.r, y, fma2(m2.i, xs, mul2(m2.r, x))));
   }
 }
 
@@ -55,23 +69,19 @@ __device__ __forceinline__ void gate2(float2 (&a)[kSweepAmps], uint32_t u, uint3
   for (int r = 0; r < kSweepAmps; ++r) {
     if ((r >> K0 & 1) || (r >> K1 & 1)) continue;
     if (C && !(ok >> r & 1u)) continue;
-    float2 v[4];
+    float2 o[4];
 #pragma unroll
-    for (int l = 0; l < 4; ++l) v[l] = a[r | (l & 1) << K0 | (l >> 1) << K1];
+    for (int l = 0; l < 4; ++l) {
+      const float2 v = a[r | (l & 1) << K0 | (l >> 1) << K1], vs = make_float2(v.y, v.x);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float4 p = entries(u, 4 * j);
-      float2 o = make_float2(p.x * v[0].x, p.x * v[0].y);
-      o = make_float2(fmaf(-p.y, v[0].y, o.x), fmaf(p.y, v[0].x, o.y));
-      o = make_float2(fmaf(p.z, v[1].x, o.x), fmaf(p.z, v[1].y, o.y));
-      o = make_float2(fmaf(-p.w, v[1].y, o.x), fmaf(p.w, v[1].x, o.y));
-      const float4 q = entries(u, 4 * j + 2);
-      o = make_float2(fmaf(q.x, v[2].x, o.x), fmaf(q.x, v[2].y, o.y));
-      o = make_float2(fmaf(-q.y, v[2].y, o.x), fmaf(q.y, v[2].x, o.y));
-      o = make_float2(fmaf(q.z, v[3].x, o.x), fmaf(q.z, v[3].y, o.y));
-      o = make_float2(fmaf(-q.w, v[3].y, o.x), fmaf(q.w, v[3].x, o.y));
-      a[r | (j & 1) << K0 | (j >> 1) << K1] = o;
+      for (int j = 0; j < 4; ++j) {
+        const Entry m = entry(u, 4 * j + l);
+        o[j] = l == 0 ? mul2(m.r, v) : fma2(m.r, v, o[j]);
+        o[j] = fma2(m.i, vs, o[j]);
+      }
     }
+#pragma unroll
+    for (int l = 0; l < 4; ++l) a[r | (l & 1) << K0 | (l >> 1) << K1] = o[l];
   }
 }
 
@@ -108,10 +118,15 @@ __device__ __forceinline__ void gadget(float2 (&a)[kSweepAmps], float c, uint32_
     const int q = r ^ M;
     if (q < r) continue;
     const float sr = __uint_as_float(t[r]), sq = __uint_as_float(t[q]);
-    const float2 x = a[r], y2 = a[q];
-    a[r] = IM ? make_float2(c * x.x - sr * y2.y, c * x.y + sr * y2.x) : make_float2(c * x.x + sr * y2.x, c * x.y + sr * y2.y);
-    if (q != r)
-      a[q] = IM ? make_float2(c * y2.x - sq * x.y, c * y2.y + sq * x.x) : make_float2(c * y2.x + sq * x.x, c * y2.y + sq * x.y);
+    const float2 x = a[r], z = a[q];
+    if (IM) {
+      a[r] = make_float2(c * x.x - sr * z.y, c * x.y + sr * z.x);
+      if (q != r) a[q] = make_float2(c * z.x - sq * x.y, c * z.y + sq * x.x);
+    } else {
+      const float2 cc = make_float2(c, c);
+      a[r] = fma2(make_float2(sr, sr), z, mul2(cc, x));
+      if (q != r) a[q] = fma2(make_float2(sq, sq), x, mul2(cc, z));
+    }
   }
 }
 

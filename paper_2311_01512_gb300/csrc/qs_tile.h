@@ -37,7 +37,7 @@ constexpr int kSweepDim = 4;
 constexpr int kSweepAmps = 1 << kSweepDim;
 constexpr int kThreadBits = kPassBits - kSweepDim;
 constexpr int kMaxOps = 24;
-constexpr int kMaxCoef = 768;
+constexpr int kMaxCoef = 1024;
 
 enum { OP_GATE1 = 0, OP_GATE2 = 1, OP_GADGET = 2, OP_DIAG = 3 };
 
@@ -126,8 +126,9 @@ inline uint64_t flips(const Gate& g) {
   return m;
 }
 
+// Floats of a gate's coefficients: a matrix entry is (re, re, -im, im).
 inline int coefs(const Gate& g) {
-  return g.kind == 0 ? (g.targs->size() == 1 ? 8 : 32) : g.kind == 1 ? 2 << g.targs->size() : 0;
+  return g.kind == 0 ? 4 << (2 * g.targs->size()) : g.kind == 1 ? 2 << g.targs->size() : 0;
 }
 
 // Whether tile passes of a state of nq qubits can hold the gate.
@@ -141,6 +142,12 @@ inline int parity(uint64_t x) { return __builtin_popcountll(x) & 1; }
 
 // Bank bits of a tile index.
 inline uint32_t bank(uint32_t i) { return slot(i) & 15u; }
+
+inline void put_entry(float* d, const double* m) {
+  d[0] = d[1] = (float)m[0];
+  d[2] = (float)-m[1];
+  d[3] = (float)m[1];
+}
 
 // The sweep of the pass's ops [first, first + count) and their directions
 // (unit vectors of dense targets in `unit`, gadget masks in `masks`; `ctl`: tile bits
@@ -237,7 +244,7 @@ inline void finish_sweep(TilePass& p, TileSweep& sw, const std::vector<Gate>& gs
       if (n == 1) {
         op.kind = OP_GATE1;
         op.k = (uint32_t)__builtin_ctz(reg(1u << loc[(*g.targs)[0]]));
-        for (int e = 0; e < 8; ++e) d[e] = (float)g.data[e];
+        for (int e = 0; e < 4; ++e) put_entry(d + 4 * e, g.data + 2 * e);
       } else {
         op.kind = OP_GATE2;
         int k0 = __builtin_ctz(reg(1u << loc[(*g.targs)[0]])), k1 = __builtin_ctz(reg(1u << loc[(*g.targs)[1]]));
@@ -246,8 +253,7 @@ inline void finish_sweep(TilePass& p, TileSweep& sw, const std::vector<Gate>& gs
         op.k = (uint32_t)(k0 == 0 ? k1 - 1 : k0 == 1 ? k1 + 1 : 5);   // 01 02 03 12 13 23
         auto perm = [&](int j) { return sw2 ? (j & 1) << 1 | j >> 1 : j; };
         for (int j = 0; j < 4; ++j)
-          for (int l = 0; l < 4; ++l)
-            for (int c = 0; c < 2; ++c) d[2 * (4 * j + l) + c] = (float)g.data[2 * (4 * perm(j) + perm(l)) + c];
+          for (int l = 0; l < 4; ++l) put_entry(d + 4 * (4 * j + l), g.data + 2 * (4 * perm(j) + perm(l)));
       }
       p.ncoef += (uint32_t)coefs(g);
     } else if (g.kind == 1) {

@@ -92,6 +92,11 @@ static void direct(const Gate& g, std::vector<cd>& a) {
   a.swap(o);
 }
 
+static cd entry(const float* d, int e) {
+  d += 4 * e;
+  return d[0] == d[1] && d[2] == -d[3] ? cd(d[0], d[3]) : cd(NAN, NAN);
+}
+
 static int run(const TilePass& p, std::vector<cd>& psi) {
   constexpr uint32_t kAmps = 1u << kPassBits, kThreads = 1u << kThreadBits;
   if (p.ncoef > kMaxCoef || p.nops > kMaxOps || p.nsweeps > kMaxOps) return fault("limits");
@@ -136,14 +141,14 @@ static int run(const TilePass& p, std::vector<cd>& psi) {
             if (op.kind <= OP_GATE2 && ((tb & op.cg) != op.cg || ((base ^ w.comb[r]) & op.cl) != op.cl)) continue;
             if (op.kind == OP_GATE1) {
               const int j = r >> op.k & 1, r0 = r & ~(1 << op.k);
-              v[r] = cd(d[4 * j], d[4 * j + 1]) * old[r0] + cd(d[4 * j + 2], d[4 * j + 3]) * old[r0 | 1 << op.k];
+              v[r] = entry(d, 2 * j) * old[r0] + entry(d, 2 * j + 1) * old[r0 | 1 << op.k];
             } else if (op.kind == OP_GATE2) {
               static const int K0[6] = {0, 0, 0, 1, 1, 2}, K1[6] = {1, 2, 3, 2, 3, 3};
               const int k0 = K0[op.k], k1 = K1[op.k], j = (r >> k0 & 1) | (r >> k1 & 1) << 1;
               const int r0 = r & ~(1 << k0) & ~(1 << k1);
               v[r] = 0;
               for (int l = 0; l < 4; ++l)
-                v[r] += cd(d[2 * (4 * j + l)], d[2 * (4 * j + l) + 1]) * old[r0 | (l & 1) << k0 | (l >> 1) << k1];
+                v[r] += entry(d, 4 * j + l) * old[r0 | (l & 1) << k0 | (l >> 1) << k1];
             } else if (op.kind == OP_GADGET) {
               const int sg = parity(tb & op.yzg) ^ parity(base & op.yzl) ^ parity(op.sgn & (uint32_t)r);
               const double f = sg ? -op.s : op.s;
