@@ -17,7 +17,7 @@ bench's kernel families and stamped with the kernel sources' digest:
         --scale-to 30 --out profiles/dram_traffic.json
 
 With --dense-times it instead times complex128 dense gates (block fixed
-point: the two-target CUDA-core kernel, eight-slice tensor-core kernels for
+point: the two-target CUDA-core kernel, byte-slice tensor-core kernels for
 three to five targets) on a state of --qubits qubits at
 three placements per target count (lowest qubits, spread, highest qubits)
 and one controlled case, each the median of --reps CUDA-event timings after
