@@ -214,9 +214,9 @@ bool upload_plan(Plan& P) {
                                       cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
-// The tile passes of a state, none if it has an operation that does not fit.
-void tile_passes(const qs_batch* b, int s, std::vector<qstile::TilePass>* out) {
-  out->clear();
+// Appends the packed tile passes of a state and where each starts (in units of 16
+// bytes); nothing if it has an operation that does not fit.
+void tile_passes(const qs_batch* b, int s, std::vector<unsigned char>* out, std::vector<uint32_t>* at) {
   const std::vector<qsk::BatchOp>& prog = b->progs[(size_t)s];
   std::vector<std::vector<int>> lists(3 * prog.size());     // controls, targets, Paulis
   std::vector<qstile::Gate> gates;
@@ -248,7 +248,10 @@ void tile_passes(const qs_batch* b, int s, std::vector<qstile::TilePass>* out) {
     if (!qstile::fits(g, b->nq[(size_t)s])) return;
     gates.push_back(g);
   }
-  qstile::build_passes(gates, b->nq[(size_t)s], out);
+  qstile::build_passes(gates, b->nq[(size_t)s], [&](const qstile::TilePass& p) {
+    at->push_back((uint32_t)(out->size() / 16));
+    qstile::pack(p, out);
+  });
 }
 
 // Two-qubit channels on the members of (t1, t2, t1 + N, t2 + N): member bits
@@ -487,27 +490,28 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
   std::vector<unsigned char> passes;         // packed
   std::vector<qstile::TileItem> items;
   if (b->prec == QS_C64) {
-    std::vector<std::vector<uint32_t>> of(S);   // where a state's passes start
-    std::vector<qstile::TilePass> mine;
-    size_t levels = 0;
-    for (int s = 0; s < S; ++s) {
-      tile_passes(b, s, &mine);
-      if (mine.empty()) continue;
-      tiled[s] = 1;
-      for (const auto& p : mine) {
-        of[s].push_back((uint32_t)(passes.size() / 16));
-        qstile::pack(p, &passes);
+    try {
+      std::vector<std::vector<uint32_t>> of(S);   // where a state's passes start
+      size_t levels = 0;
+      for (int s = 0; s < S; ++s) {
+        tile_passes(b, s, &passes, &of[s]);
+        tiled[s] = !of[s].empty();
+        levels = std::max(levels, of[s].size());
       }
-      levels = std::max(levels, of[s].size());
-    }
-    for (size_t k = 0; k < levels; ++k) {
+      for (size_t k = 0; k < levels; ++k) {
+        b->level.push_back((int)items.size());
+        for (int s = 0; s < S; ++s)
+          if (k < of[s].size())
+            for (uint32_t t = 0; t < 1u << (b->nq[s] - qstile::kPassBits); ++t)
+              items.push_back(qstile::TileItem{b->offset[s], of[s][k], t});
+      }
       b->level.push_back((int)items.size());
-      for (int s = 0; s < S; ++s)
-        if (k < of[s].size())
-          for (uint32_t t = 0; t < 1u << (b->nq[s] - qstile::kPassBits); ++t)
-            items.push_back(qstile::TileItem{b->offset[s], of[s][k], t});
+    } catch (const std::bad_alloc&) {             // without tile passes
+      passes.clear();
+      items.clear();
+      b->level.clear();
+      std::fill(tiled.begin(), tiled.end(), 0);
     }
-    b->level.push_back((int)items.size());
   }
   // largest first, heavy ones before the others; a second list without the tiled states
   std::vector<int> order(S);

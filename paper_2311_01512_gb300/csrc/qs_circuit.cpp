@@ -45,7 +45,8 @@ struct CBlock {
 // A run of blocks [first, last) that complex64 statevectors take in tile passes.
 struct TileRun {
   size_t first = 0, last = 0;
-  std::vector<qstile::TilePass> passes;
+  std::vector<unsigned char> passes;   // packed
+  std::vector<size_t> at;              // where each starts
 };
 
 int popc64(uint64_t x) { return __builtin_popcountll(x); }
@@ -223,9 +224,12 @@ void find_runs(qs_circuit* c) {
       TileRun r;
       r.first = bi;
       r.last = e;
-      qstile::build_passes(gates, c->nq, &r.passes);
+      qstile::build_passes(gates, c->nq, [&](const qstile::TilePass& p) {
+        r.at.push_back(r.passes.size());
+        qstile::pack(p, &r.passes);
+      });
       // a pass's own read and write are half hidden behind the gates
-      cost_tiles = std::max(cost_tiles + 0.5 * (double)r.passes.size(), (double)r.passes.size());
+      cost_tiles = std::max(cost_tiles + 0.5 * (double)r.at.size(), (double)r.at.size());
       if (cost_tiles < cost_blocks) c->runs.push_back(std::move(r));
     }
     bi = e > bi ? e : bi + 1;
@@ -574,8 +578,11 @@ qs_status qs_circuit_apply(qs_circuit* c, qs_state* s) {
   size_t run = 0;
   for (size_t bi = 0; bi < c->blocks.size(); ++bi) {
     if (tiles && run < c->runs.size() && c->runs[run].first == bi) {
-      for (const auto& p : c->runs[run].passes)
+      qstile::TilePass p{};
+      for (const size_t at : c->runs[run].at) {
+        qstile::unpack(c->runs[run].passes.data() + at, &p);
         if (qsk::launch_tile_pass(s->amps, p, s->stream) != cudaSuccess) return QS_ERR_CUDA;
+      }
       bi = c->runs[run++].last - 1;
       continue;
     }

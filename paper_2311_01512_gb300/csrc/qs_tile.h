@@ -103,6 +103,18 @@ inline void pack(const TilePass& p, std::vector<unsigned char>* out) {
   put(p.coef, (uint32_t)sizeof(float) * p.ncoef);
 }
 
+// The pass packed at `from`.
+inline void unpack(const unsigned char* from, TilePass* p) {
+  auto get = [&](void* to, uint32_t bytes) {
+    std::memcpy(to, from, bytes);
+    from += padded(bytes);
+  };
+  get(p, kHeadBytes);
+  get(p->sweep, (uint32_t)sizeof(TileSweep) * p->nsweeps);
+  get(p->op, (uint32_t)sizeof(TileOp) * p->nops);
+  get(p->coef, (uint32_t)sizeof(float) * p->ncoef);
+}
+
 // Shared-memory slot of tile index i: the bank bits 0..3 (8-byte words) fold in
 // every higher bit, so that lanes along any four suitable bits meet each bank once.
 QT_HD constexpr uint32_t slot(uint32_t i) { return i ^ (((i >> 4) ^ (i >> 8) ^ (i >> 12)) & 15u); }
@@ -291,33 +303,38 @@ inline void finish_sweep(TilePass& p, TileSweep& sw, const std::vector<Gate>& gs
   }
 }
 
-// Passes that apply the gates (each fits()) in an equivalent order.
-inline void build_passes(const std::vector<Gate>& gates, int nq, std::vector<TilePass>* out) {
-  std::vector<int> left;
+// Passes that apply the gates (each fits()) in an equivalent order, handed to emit one
+// by one.
+template <typename Emit>
+inline void build_passes(const std::vector<Gate>& gates, int nq, const Emit& emit) {
+  std::vector<int> left, rest;              // left: from `begin` on
+  size_t begin = 0;
   for (int i = 0; i < (int)gates.size(); ++i) left.push_back(i);
-  while (!left.empty()) {
-    std::vector<int> take, rest;
+  const uint64_t all = (1ull << nq) - 1;
+  while (begin < left.size()) {
+    std::vector<int> take;
     uint64_t tile = (1ull << kPassLow) - 1, blocked = 0;
     int ncoef = 0;
-    for (int i : left) {
-      const Gate& g = gates[i];
+    rest.clear();
+    // until a gate skipped before blocks every qubit
+    size_t at = begin;
+    for (; at < left.size() && blocked != all && (int)take.size() < kMaxOps; ++at) {
+      const Gate& g = gates[left[at]];
       const uint64_t t = tile | flips(g);
-      if (!(g.qmask & blocked) && __builtin_popcountll(t) <= kPassBits && (int)take.size() < kMaxOps &&
-          ncoef + coefs(g) <= kMaxCoef) {
-        take.push_back(i);
+      if (!(g.qmask & blocked) && __builtin_popcountll(t) <= kPassBits && ncoef + coefs(g) <= kMaxCoef) {
+        take.push_back(left[at]);
         tile = t;
         ncoef += coefs(g);
       } else {
         blocked |= g.qmask;
-        rest.push_back(i);
-        // gates without qubits (global phases) never block and always commute
+        rest.push_back(left[at]);
       }
     }
-    left.swap(rest);
+    begin = at - rest.size();               // the skipped gates, then those not looked at
+    for (size_t i = 0; i < rest.size(); ++i) left[begin + i] = rest[i];
     for (int q = 0; __builtin_popcountll(tile) < kPassBits; ++q) tile |= 1ull << q;
-    out->emplace_back();
-    TilePass& p = out->back();
-    std::memset(&p, 0, sizeof(p));
+    TilePass p;
+    std::memset(static_cast<void*>(&p), 0, sizeof(p));
     p.ntiles = 1ull << (nq - kPassBits);
     std::vector<uint32_t> loc(64, 0);
     for (int q = 0, b = 0; q < nq; ++q)
@@ -397,6 +414,7 @@ inline void build_passes(const std::vector<Gate>& gates, int nq, std::vector<Til
       p.nops = (uint32_t)gs.size();
       finish_sweep(p, sw, gs, loc, unit, masks, ctl);
     }
+    emit(p);
   }
 }
 

@@ -186,7 +186,16 @@ int main() {
       if (!fits(g, n)) return fault("fits");
       direct(g, a);
     }
-    build_passes(c.gates, n, &passes);
+    std::vector<unsigned char> packed;
+    std::vector<size_t> at;
+    build_passes(c.gates, n, [&](const TilePass& p) {
+      at.push_back(packed.size());
+      pack(p, &packed);
+    });
+    for (size_t a : at) {
+      passes.emplace_back();
+      unpack(packed.data() + a, &passes.back());
+    }
     size_t ops = 0;
     for (const TilePass& p : passes) {
       ops += p.nops;
