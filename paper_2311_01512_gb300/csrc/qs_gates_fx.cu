@@ -159,9 +159,14 @@ __global__ void __launch_bounds__(256) k_gate2_fx(double2* __restrict__ psi, con
 // every block prepares in shared memory with one exponent per row, laid out by
 // column so that the lanes of a group read consecutive words.  The 2^(NT+1) real
 // terms of an output go four at a time through the accumulators of qs_fx.cuh;
-// the partial sums are added shifted down by NT - 2 bits (|V| stays below 2^63
-// as in the two-target kernel), so the error is at most
-//   2^-53 |y| + (7 2^(NT+1) + 2^(2 NT - 2) + 8) 2^-60 max|x_k| max|m_k|.
+// the partial sums are added shifted down by NT - 2 bits, rounded to nearest.  |V| stays
+// below 2^63: it is at most 2^(NT-1) 4 (2^60 - 2^7) / 2^(NT-2) = 2^63 - 2^10, and the
+// dropped products, floors and roundings add less than 20.  The error is at most
+//   2^-53 |y| + (2^(NT+4) + 2^(2 NT - 2) [NT > 2]) 2^-60 max|x_k| max|m_k|:
+// 7 units a term and 4 an accumulator's floor, as in the two-target kernel, and half a
+// unit of 2^(NT-2) for each of the 2^(NT-1) shifts.  Rows of Haar unitaries, of the
+// outputs' rms (exact reference): 4.8, 4.8, 4.9 and 5.1e-17 for 2 to 5 targets, no
+// one-sided part (rounded down the shifts left 1.2e-16 at five).
 // Why: on a few thousand amplitudes the tensor-core kernels run on one or two
 // SMs behind a setup that slices the whole matrix; here every block does a few
 // hundred instructions of setup and a pass spreads over the SMs.  4096 amplitudes, us a pass in a
@@ -225,8 +230,8 @@ __global__ void __launch_bounds__(128) k_dense_fx(double2* __restrict__ psi, con
       qsfx::mac(ai, xr, mi);
       qsfx::mac(ai, xi, mr);
     }
-    vr += qsfx::acc_value(ar) >> SH;
-    vi += qsfx::acc_value(ai) >> SH;
+    vr += qsfx::partial(ar, SH);
+    vi += qsfx::partial(ai, SH);
   }
   const qsfx::Scale sc = qsfx::scale_for((int)(exf >> 20) + SH, em[j]);
   if (ok) psi[i] = make_double2(qsfx::finish_v(vr, sc), qsfx::finish_v(vi, sc));
