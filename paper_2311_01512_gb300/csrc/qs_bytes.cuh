@@ -153,6 +153,22 @@ QS_HD void split_start(int P, int* p) {
   p[0] = r - 256 * p[1];
 }
 
+// A result is Q as a double times 2^(inc / 2^20).  Adding inc to the exponent field
+// does it where no nonzero Q (1 <= |Q| < 2^62) leaves the normal numbers:
+constexpr int kMinInc = -(1022 << 20), kMaxInc = (2046 - 1023 - 62) << 20;
+QS_HD double add_inc(double r, int inc) {
+  uint32_t hw, lw;
+  qsdf::d2w(r, hw, lw);                          // hw is 0 only for r = 0, which stays 0
+  return qsdf::w2d(hw != 0 ? hw + (uint32_t)inc : 0u, lw);
+}
+// Elsewhere two factors (|inc| < 2^31, so both are normal numbers): the first product
+// is exact where the result is below it, so the result is rounded once, to a subnormal
+// number, 0 or infinity where it has to be.
+QS_HD double mul_inc(double r, int inc) {
+  const int e = inc >> 20, e1 = e / 2;
+  return r * qsdf::w2d((uint32_t)(1023 + e1) << 20, 0u) * qsdf::w2d((uint32_t)(1023 + e - e1) << 20, 0u);
+}
+
 QS_HD uint32_t fbits(float v) { return qsdf::f2u(v); }
 QS_HD int to_int(float v) { return (int)v; }   // exact integers
 

@@ -22,6 +22,7 @@
 // pass in a replayed program: 10.9 -> 4.3.
 #include <cstring>
 
+#include "qs_bytes.cuh"
 #include "qs_device.cuh"
 #include "qs_slices.cuh"
 
@@ -136,8 +137,9 @@ __global__ void __launch_bounds__(kDigitThreads) k_dense_digits(double2* __restr
 #pragma unroll
   for (int L = 0; L < 8; ++L) bits[L] = __float_as_uint(lv[L]);
   const double r = __ll2double_rn(qsoz::combine_pairs_u<8, qsoz::kFaddMagicBits>(bits));
-  const int hi = __double2hiint(r);                          // 0 only for r = 0, which stays 0
-  const double o = __hiloint2double(hi != 0 ? hi + (er + cexp[j] - 2046 - 53) * (1 << 20) : 0, __double2loint(r));
+  const int inc = (er + cexp[j] - 2046 - 53) * (1 << 20);
+  const bool rare = inc < qsby::kMinInc || inc > qsby::kMaxInc;
+  const double o = rare ? qsby::mul_inc(r, inc) : qsby::add_inc(r, inc);
   if (ok) reinterpret_cast<double*>(psi)[2 * i + c] = o;
 }
 

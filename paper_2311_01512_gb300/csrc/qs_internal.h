@@ -21,7 +21,7 @@ constexpr int kTileBits = 10;        // amplitudes staged per tile of the dense 
 constexpr int kReduceBlocks = 1216;  // 152 SMs x 8: largest grid of the stage-one expectation and trace reductions
 constexpr int kNormBlocks = 4864;    // 152 SMs x 32: largest grid of the norm, a pure stream over the state
 constexpr int kPartials = kNormBlocks;  // partial sums a handle holds (the larger grid)
-constexpr size_t kWideScratch = 295424;  // bytes of scratch of a six-target gate (qs_tc_ozaki.cu)
+constexpr size_t kWideScratch = 295936;  // bytes of scratch of a six-target gate (qs_tc_ozaki.cu)
 constexpr int kTermChunk = 2048;     // Pauli terms per device upload
 constexpr int kCostFeatures = 64;    // cost-model network: input features
 constexpr int kCostHidden = 64;      // hidden units per layer (two layers)

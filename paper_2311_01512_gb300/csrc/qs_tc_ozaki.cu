@@ -216,15 +216,33 @@ __device__ __forceinline__ void fill_offsets(const TcParams& p, uint64_t* toff, 
 }
 
 // column exponent field -> the increment it adds to a result's exponent field
-__device__ __forceinline__ int column_scale(int field) { return field - ((2046 + qsby::kScale) << 20); }
+__host__ __device__ constexpr int column_scale(int field) {
+  return (field - (1024 << 20)) - ((1022 + qsby::kScale) << 20);   // in steps within 32 bits
+}
+
+// Row exponent fields [lim[0], lim[1]] whose results can have their exponent fields
+// added (qsby::add_inc) in every column that is not all zeros.  The limits start at
+// those of a column of exponent 0; limit_rows takes in a column's (csc: its largest
+// high word, scale: its increment).
+__device__ __forceinline__ void start_row_limits(int* lim) {
+  constexpr int one = column_scale(1023 << 20);
+  lim[0] = qsby::kMinInc - one;
+  lim[1] = qsby::kMaxInc - one;
+}
+__device__ __forceinline__ void limit_rows(int* lim, int csc, int scale) {
+  if (csc == 0) return;
+  atomicMax(lim, qsby::kMinInc - scale);
+  atomicMin(lim + 1, qsby::kMaxInc - max(scale, qsby::kMaxInc - 0x7FFFFFFF));
+}
 
 // Per-CTA constants of a dense gate: the column scales and the digit slices of
 // B, the initialising MMA's operands, the target offsets of the group members
 // and the row offsets of the tile.
 template <int NT, int NTHR>
 __device__ void tile_constants(const TcParams& p, unsigned char* b_dig, unsigned char* a_pre, unsigned char* b_pre,
-                               int* csc, int* colsum, uint64_t* toff, uint64_t* rowoff, int tid) {
+                               int* csc, int* lim, int* colsum, uint64_t* toff, uint64_t* rowoff, int tid) {
   constexpr int D = 1 << NT, K = 2 * D, N = 2 * D;
+  if (tid == 0) start_row_limits(lim);
   fill_start_rows(a_pre, tid, NTHR);
   fill_offsets<NT>(p, toff, rowoff, tid, NTHR);
   slice_matrix<NT, NTHR>(p, b_dig, N * K * 2, [](int n, int k) { return canon_off16(n, k, K); }, csc, colsum, tid);
@@ -233,18 +251,33 @@ __device__ void tile_constants(const TcParams& p, unsigned char* b_dig, unsigned
     fill_start_column(b_pre, L * N + n, qsby::start_value(L, K, colsum + n * kLv));
   }
   for (int j = tid; j < D; j += NTHR) {
-    const int sc = column_scale((int)qsby::row_field((uint32_t)csc[2 * j]));
+    const int mx = csc[2 * j], sc = column_scale((int)qsby::row_field((uint32_t)mx));
+    limit_rows(lim, mx, sc);
     csc[2 * j] = sc;
     csc[2 * j + 1] = sc;
   }
 }
 
-// one output: levels -> Q -> double, scaled by the row's and the column's powers of two
+// Four outputs: levels -> Q -> double, scaled by the row's and the columns' powers of
+// two.  rare: the row's exponent is beyond the limits.
 template <int K>
-__device__ __forceinline__ double finish_output(const float* v, int egs, int scl) {
-  const double r = __ll2double_rn(qsby::combine<K>(v));
-  const int hi = __double2hiint(r);                // 0 only for r = 0, which stays 0
-  return __hiloint2double(hi != 0 ? hi + egs + scl : 0, __double2loint(r));
+__device__ __forceinline__ void finish_outputs(const float (*v)[4], int egs, const int* csc, bool rare, double* o) {
+  const int4 s = *reinterpret_cast<const int4*>(csc);
+  const int inc[4] = {egs + s.x, egs + s.y, egs + s.z, egs + s.w};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float u[kLv];
+#pragma unroll
+    for (int L = 0; L < kLv; ++L) u[L] = v[L][q];
+    o[q] = __ll2double_rn(qsby::combine<K>(u));
+  }
+  if (rare) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o[q] = qsby::mul_inc(o[q], inc[q]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o[q] = qsby::add_inc(o[q], inc[q]);
+  }
 }
 
 // fp16 operand words of four amplitudes (hi, lo words of re and im) at the 16-byte
@@ -344,6 +377,7 @@ struct Ws {
   static constexpr size_t ex_off = csc_off + 4 * N;
   static constexpr size_t colsum_off = ex_off + 4 * (size_t)NM * RB * kRows;
   static constexpr size_t slot_off = colsum_off + 4 * (size_t)kLv * N;
+  static constexpr size_t lim_off = slot_off + 8;
   static constexpr size_t bytes = slot_off + 16;
   static_assert(RB * LCOLS <= TSTRIDE && NTM * TSTRIDE <= 512, "tensor memory");
   static_assert(bytes <= 227 * 1024, "shared memory");
@@ -374,10 +408,11 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
   int* meta_ex = reinterpret_cast<int*>(smem + W::ex_off);
   int* colsum = reinterpret_cast<int*>(smem + W::colsum_off);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + W::slot_off);
+  int* lim = reinterpret_cast<int*>(smem + W::lim_off);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + W::slot_off + 4);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  tile_constants<NT, kWsThreads>(p, b_dig, a_pre, b_pre, csc, colsum, toff, rowoff, tid);
+  tile_constants<NT, kWsThreads>(p, b_dig, a_pre, b_pre, csc, lim, colsum, toff, rowoff, tid);
   if (tid == 0) {
 #pragma unroll
     for (int j = 0; j < NA; ++j) {
@@ -434,6 +469,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
         break;
       }
       const int egs = meta_ex[(m * RB + r) * kRows + g];
+      const bool rare = egs < lim[0] || egs > lim[1];
       char* tp = reinterpret_cast<char*>(psi) + ((xb | p.ctrl_mask) << 4);
       if (wait_ring_warp(accfull + k, (uint32_t)(i / NTM) & 1u, abort_flag)) {
         *abort_flag = 1;
@@ -453,16 +489,8 @@ __global__ void __launch_bounds__(kWsThreads, 1) k_dense_ozaki_ws(double2* __res
           if (lane == 0) mbar_arrive(tempty + k);
         }
         if (row_ok) {
-          const int4 s0 = *reinterpret_cast<const int4*>(csc + 2 * l0 + cc);
-          const int scl[4] = {s0.x, s0.y, s0.z, s0.w};
           double o[4];
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) {
-            float u[kLv];
-#pragma unroll
-            for (int L = 0; L < kLv; ++L) u[L] = v[L][qq];
-            o[qq] = finish_output<K>(u, egs, scl[qq]);
-          }
+          finish_outputs<K>(v, egs, csc + 2 * l0 + cc, rare, o);
           if (PAIRS) {
             store_pair(tp + te[cc >> 1], o);
           } else {
@@ -675,11 +703,11 @@ __device__ __forceinline__ bool wait_or_abort_warp(uint64_t* bar, uint32_t parit
 }
 
 // Epilogue of one N block (32 columns, accumulators at tb): a thread's row, NC of
-// its columns from column c0 of the block on; csc0: their scales; addr(a): where
-// amplitude a of those goes.  Hands the accumulators back on tempty once read.
+// its columns from column c0 of the block on; csc0: their scales; rare: as for
+// finish_outputs; addr(a): where amplitude a of those goes.  Hands the accumulators back on tempty once read.
 template <int K, int NC, bool PAIRS, typename Addr>
-__device__ __forceinline__ void epilogue_block(uint32_t tb, uint64_t* tempty, const int* csc0, int egs, bool row_ok,
-                                               int lane, const Addr& addr) {
+__device__ __forceinline__ void epilogue_block(uint32_t tb, uint64_t* tempty, const int* csc0, int egs, bool rare,
+                                               bool row_ok, int lane, const Addr& addr) {
 #pragma unroll
   for (int cc = 0; cc < NC; cc += 4) {
     float v[kLv][4];
@@ -692,16 +720,8 @@ __device__ __forceinline__ void epilogue_block(uint32_t tb, uint64_t* tempty, co
       if (lane == 0) mbar_arrive(tempty);
     }
     if (row_ok) {
-      const int4 s0 = *reinterpret_cast<const int4*>(csc0 + cc);
-      const int scl[4] = {s0.x, s0.y, s0.z, s0.w};
       double o[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float u[kLv];
-#pragma unroll
-        for (int L = 0; L < kLv; ++L) u[L] = v[L][q];
-        o[q] = finish_output<K>(u, egs, scl[q]);
-      }
+      finish_outputs<K>(v, egs, csc0 + cc, rare, o);
       if (PAIRS) {
         store_pair(addr(cc >> 1), o);
       } else {
@@ -770,6 +790,7 @@ struct W5 {
   static constexpr size_t ex_off = max_off + 4 * 3 * kRows;
   static constexpr size_t colsum_off = ex_off + 4 * NM * kRows;
   static constexpr size_t slot_off = colsum_off + 4 * (size_t)kLv * K;
+  static constexpr size_t lim_off = slot_off + 8;
   static constexpr size_t bytes = slot_off + 16;
   static_assert(bytes <= 227 * 1024, "shared memory");
 };
@@ -793,12 +814,14 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
   int* rowmax = reinterpret_cast<int*>(smem + X::max_off);       // 3 x kRows
   int* meta_ex = reinterpret_cast<int*>(smem + X::ex_off);       // NM x kRows
   int* colsum = reinterpret_cast<int*>(smem + X::colsum_off);    // K x 8 (setup)
+  int* lim = reinterpret_cast<int*>(smem + X::lim_off);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + X::slot_off);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + X::slot_off + 4);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   fill_start_rows(a_pre, tid, X::THREADS);
   fill_offsets<5>(p, toff, rowoff, tid, X::THREADS);
+  if (tid == 0) start_row_limits(lim);
   // B's slices in blocks of 32 x 32: block (K block, N block) at (kb KB + nb) 16 KB
   slice_matrix<5, X::THREADS>(
       p, b_dig, 2048,
@@ -809,7 +832,8 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
     fill_start_column(b_pre + (n >> 5) * 8192, L * 32 + (n & 31), qsby::start_value(L, K, colsum + n * kLv));
   }
   for (int j = tid; j < D; j += X::THREADS) {
-    const int sc = column_scale((int)qsby::row_field((uint32_t)csc[2 * j]));
+    const int mx = csc[2 * j], sc = column_scale((int)qsby::row_field((uint32_t)mx));
+    limit_rows(lim, mx, sc);
     csc[2 * j] = sc;
     csc[2 * j + 1] = sc;
   }
@@ -854,6 +878,7 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
       const uint32_t m = it % X::NM;
       if (wait_or_abort_warp(mready + m, (it / X::NM) & 1u, abort_flag)) break;
       const int egs = meta_ex[m * kRows + g];
+      const bool rare = egs < lim[0] || egs > lim[1];
       const uint64_t rb = xb | roff;
 #pragma unroll
       for (int nb = 0; nb < 2; ++nb) {
@@ -861,7 +886,7 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
         if (bad) break;
         fence_after_sync();
         epilogue_block<K, 16, PAIRS>(tmem + (uint32_t)(256 * nb + 16 * h) + lane_addr, tempty + nb, csc + 32 * nb + 16 * h, egs,
-                              row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 8 * h + a]); });
+                              rare, row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 8 * h + a]); });
       }
     }
   } else if (warp < kE5 + kKnWarps) {
@@ -971,8 +996,8 @@ static cudaError_t dense_ozaki5(void* amps, const TcParams& p, cudaStream_t st) 
 namespace {
 // layout of the scratch that k_wide_matrix fills
 constexpr int kWideStart = 16 * kKnBlock;            // four start operands (N block) of 256 columns x 32 bytes
-constexpr int kWideScale = kWideStart + 4 * 8192;    // 128 column exponent increments
-static_assert(kWideScale + 4 * 128 <= (int)kWideScratch, "scratch of the six-target kernel");
+constexpr int kWideScale = kWideStart + 4 * 8192;    // of 128 columns: exponent increment, largest high word
+static_assert(kWideScale + 8 * 128 <= (int)kWideScratch, "scratch of the six-target kernel");
 
 struct W6 {
   static constexpr int D = 64, K = 128, KB = 4;
@@ -987,6 +1012,7 @@ struct W6 {
   static constexpr size_t csc_off = bar_off + 8 * 18;
   static constexpr size_t max_off = csc_off + 4 * K;
   static constexpr size_t slot_off = max_off + 4 * 3 * kRows;
+  static constexpr size_t lim_off = slot_off + 8;
   static constexpr size_t bytes = slot_off + 16;
   static_assert(bytes <= 227 * 1024, "shared memory");
 };
@@ -1027,7 +1053,11 @@ __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcP
   __syncthreads();
   if (k < kLv)
     fill_start_column(out + kWideStart + (n >> 5) * 8192, k * 32 + (n & 31), qsby::start_value(k, K, sums));
-  if (k == 0) reinterpret_cast<int*>(out + kWideScale)[n] = column_scale((int)ef);
+  if (k == 0) {
+    int* col = reinterpret_cast<int*>(out + kWideScale) + 2 * n;
+    col[0] = column_scale((int)ef);
+    col[1] = mx;
+  }
 }
 
 template <bool PAIRS>
@@ -1048,12 +1078,19 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
   int* csc = reinterpret_cast<int*>(smem + X::csc_off);
   int* rowmax = reinterpret_cast<int*>(smem + X::max_off);       // 3 x kRows
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + X::slot_off);
+  int* lim = reinterpret_cast<int*>(smem + X::lim_off);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + X::slot_off + 4);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint4* src = reinterpret_cast<const uint4*>(wide + kWideStart);
   for (int i = tid; i < KB * 8192 / 16; i += X::THREADS) reinterpret_cast<uint4*>(b_pre)[i] = src[i];
-  for (int n = tid; n < K; n += X::THREADS) csc[n] = reinterpret_cast<const int*>(wide + kWideScale)[n];
+  if (tid == 0) start_row_limits(lim);
+  __syncthreads();
+  for (int n = tid; n < K; n += X::THREADS) {
+    const int* col = reinterpret_cast<const int*>(wide + kWideScale) + 2 * n;
+    limit_rows(lim, col[1], col[0]);
+    csc[n] = col[0];
+  }
   fill_start_rows(a_pre, tid, X::THREADS);
   fill_offsets<6>(p, toff, rowoff, tid, X::THREADS);
   for (int g = tid; g < 3 * kRows; g += X::THREADS) rowmax[g] = 0;
@@ -1113,6 +1150,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
       // the previous tile's slot: read by every warp before this barrier, next
       // written after the following one
       if (cg == 0) rowmax[(slot == 0 ? 2 : slot - 1) * kRows + g] = 0;
+      const bool rare = (int)ef < lim[0] || (int)ef > lim[1];
       const bool has_next = c + grid < p.ntiles;
       xb = ((xb | hole) + gstep) & ~hole;
       const uint64_t rb_next = xb | roff;
@@ -1139,7 +1177,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
           ++reads[h];
           fence_after_sync();
           epilogue_block<K, 8, PAIRS>(tmem + (uint32_t)(256 * h + 8 * cg) + lane_addr, tempty + h, csc + 32 * nb + 8 * cg, (int)ef,
-                               row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 4 * cg + a]); });
+                               rare, row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 4 * cg + a]); });
         }
       }
       rb = rb_next;
