@@ -383,6 +383,44 @@ bool needs_device_matrix(const qs_state* s, int n, int nctrl) {
   return n > 1 && !(n == 2 && is_fx(s)) && small_route(s, n, nctrl) == SMALL_NO;
 }
 
+// Dense pass on the CUDA cores in the handle's floating-point arithmetic; when: as in
+// DenseParams.
+qs_status cuda_core_pass(qs_state* s, const std::vector<int>& ctrls, const std::vector<int>& targs,
+                         const void* dev_mat, int conj, const int* when) {
+  // Dense tile: P = targets u the lowest free qubits, |P| = min(kTileBits, free + n).
+  const int n = (int)targs.size(), nfree = s->ns - n - (int)ctrls.size();
+  uint64_t cmask = 0;
+  for (int c : ctrls) cmask |= 1ull << c;
+  uint64_t fixed = cmask;
+  for (int t : targs) fixed |= 1ull << t;
+  const int g = std::min(qsk::kTileBits - n, nfree) < 0 ? 0 : std::min(qsk::kTileBits - n, nfree);
+  std::vector<int> P(targs);
+  for (int q = 0, added = 0; q < s->ns && added < g; ++q)
+    if (!(fixed >> q & 1)) {
+      P.push_back(q);
+      ++added;
+    }
+  std::sort(P.begin(), P.end());
+  qsk::DenseParams p{};
+  p.mat = static_cast<const double*>(dev_mat);
+  p.when = when;
+  p.ctrl_mask = cmask;
+  p.n = n;
+  p.conj = conj;
+  p.tile_bits = (int)P.size();
+  for (int b = 0; b < p.tile_bits; ++b) p.P[b] = (int8_t)P[b];
+  for (int q = 0; q < n; ++q)
+    p.tslot[q] = (int8_t)(std::find(P.begin(), P.end(), targs[q]) - P.begin());
+  std::vector<int> hi(P);
+  hi.insert(hi.end(), ctrls.begin(), ctrls.end());
+  std::sort(hi.begin(), hi.end());
+  p.nhi = (int)hi.size();
+  for (int i = 0; i < p.nhi; ++i) p.hi_ins[i] = (int8_t)hi[i];
+  p.ntiles = 1ull << (s->ns - p.nhi);
+  if (s->prec == QS_C128 && s->arith == QS_ARITH_DF) return cuda_status(qsk::launch_dense_df(s->amps, p, s->stream));
+  return cuda_status(qsk::launch_dense(s->prec, s->amps, p, s->stream));
+}
+
 // One dense or one-target gate pass on storage positions (already shifted).
 qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vector<int>& targs, const double* host_mat,
                     const void* dev_mat, int conj, bool force_dense) {
@@ -563,44 +601,22 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
     p.ntiles = 1ull << (s->ns - p.nhi);
     if (tc64) return cuda_status(qsk::launch_dense_tc(s->amps, p, s->stream));
     if (n < 6) return cuda_status(qsk::launch_dense_ozaki(s->amps, p, nullptr, s->stream));
-    // six targets: the sliced matrix goes through scratch in the ring
+    // six targets: the sliced matrix goes through scratch in the ring; a matrix that does
+    // not mix its groups takes the CUDA cores (k_wide_matrix decides)
+    const int* when = nullptr;
     void* wide = nullptr;
     int first = -1, count = 0;
     qs_status st = ring_take_run(s, qsk::kWideScratch, &wide, &first, &count);
     if (st != QS_OK) return st;
-    st = cuda_status(qsk::launch_dense_ozaki(s->amps, p, wide, s->stream));
+    st = cuda_status(qsk::launch_dense_ozaki(s->amps, p, wide, s->stream, &when));
+    if (st == QS_OK) st = cuda_core_pass(s, ctrls, targs, dev_mat, conj, when);
     for (int j = 0; j < count; ++j) {
       const qs_status st2 = ring_done(s, first + j);
       if (st == QS_OK) st = st2;
     }
     return st;
   }
-  // Dense tile: P = targets u the lowest free qubits, |P| = min(kTileBits, free + n).
-  const int g = std::min(qsk::kTileBits - n, nfree) < 0 ? 0 : std::min(qsk::kTileBits - n, nfree);
-  std::vector<int> P(targs);
-  for (int q = 0, added = 0; q < s->ns && added < g; ++q)
-    if (!(fixed >> q & 1)) {
-      P.push_back(q);
-      ++added;
-    }
-  std::sort(P.begin(), P.end());
-  qsk::DenseParams p{};
-  p.mat = static_cast<const double*>(dev_mat);
-  p.ctrl_mask = cmask;
-  p.n = n;
-  p.conj = conj;
-  p.tile_bits = (int)P.size();
-  for (int b = 0; b < p.tile_bits; ++b) p.P[b] = (int8_t)P[b];
-  for (int q = 0; q < n; ++q)
-    p.tslot[q] = (int8_t)(std::find(P.begin(), P.end(), targs[q]) - P.begin());
-  std::vector<int> hi(P);
-  hi.insert(hi.end(), ctrls.begin(), ctrls.end());
-  std::sort(hi.begin(), hi.end());
-  p.nhi = (int)hi.size();
-  for (int i = 0; i < p.nhi; ++i) p.hi_ins[i] = (int8_t)hi[i];
-  p.ntiles = 1ull << (s->ns - p.nhi);
-  if (df) return cuda_status(qsk::launch_dense_df(s->amps, p, s->stream));
-  return cuda_status(qsk::launch_dense(s->prec, s->amps, p, s->stream));
+  return cuda_core_pass(s, ctrls, targs, dev_mat, conj, nullptr);
 }
 
 qs_status gadget_pass(qs_state* s, const std::vector<int>& targs, const int* paulis, double theta) {

@@ -93,4 +93,9 @@ inline unsigned grid_for(uint64_t work, int threads, int max_blocks) {
 
 int num_sms();  // cached cudaDevAttrMultiProcessorCount of the current device
 
+// Whether one of the flags that a pass waits for is set (blocks of at least kWideFlags threads).
+__device__ __forceinline__ bool any_flag(const int* flags) {
+  return __syncthreads_or(threadIdx.x < kWideFlags && flags[threadIdx.x]) != 0;
+}
+
 }  // namespace qsk

@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(256) k_dense(typename Cplx<R>::T* __restrict__
   constexpr int kTile = 1 << kTileBits;
   constexpr int EPT = kTile / 256;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (p.when && !any_flag(p.when)) return;
   T2* sm_mat = reinterpret_cast<T2*>(smem_raw);   // D x D
   T2* sm_tile = sm_mat + D * D;                    // up to kTile
   uint32_t* sm_toff = reinterpret_cast<uint32_t*>(sm_tile + kTile);  // D
@@ -276,6 +277,8 @@ static cudaError_t dense_nt(void* amps, const DenseParams& p, cudaStream_t st) {
   static bool attr_done = false;
   if (!attr_done) {
     cudaError_t e = cudaFuncSetAttribute(k_dense<R, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && NT == 6)       // as the kernels before it (qs_tc_ozaki.cu)
+      e = cudaFuncSetAttribute(k_dense<R, NT>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }

@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(256) k_dense_df(double2* __restrict__ psi, con
   constexpr int kTile = 1 << kTileBits;
   constexpr int EPT = kTile / 256;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (p.when && !any_flag(p.when)) return;
   cdf* sm_mat = reinterpret_cast<cdf*>(smem_raw);          // D x D
   cdf* sm_tile = sm_mat + D * D;                            // up to kTile
   uint32_t* sm_toff = reinterpret_cast<uint32_t*>(sm_tile + kTile);

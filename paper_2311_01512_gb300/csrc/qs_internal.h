@@ -21,7 +21,8 @@ constexpr int kTileBits = 10;        // amplitudes staged per tile of the dense 
 constexpr int kReduceBlocks = 1216;  // 152 SMs x 8: largest grid of the stage-one expectation and trace reductions
 constexpr int kNormBlocks = 4864;    // 152 SMs x 32: largest grid of the norm, a pure stream over the state
 constexpr int kPartials = kNormBlocks;  // partial sums a handle holds (the larger grid)
-constexpr size_t kWideScratch = 295936;  // bytes of scratch of a six-target gate (qs_tc_ozaki.cu)
+constexpr int kWideFlags = 128;      // flags of k_wide_matrix
+constexpr size_t kWideScratch = 296448;  // bytes of scratch of a six-target gate (qs_tc_ozaki.cu)
 constexpr int kTermChunk = 2048;     // Pauli terms per device upload
 constexpr int kCostFeatures = 64;    // cost-model network: input features
 constexpr int kCostHidden = 64;      // hidden units per layer (two layers)
@@ -65,6 +66,7 @@ struct Gate1DfParams {
 // qubits); the remaining free bits number the tile.
 struct DenseParams {
   const double* mat;     // device, 2^n x 2^n complex128 row-major (re, im)
+  const int* when;       // null, or kWideFlags ints on the device: the pass is made if one of them is set
   uint64_t ctrl_mask;
   uint64_t ntiles;
   int n;
@@ -401,8 +403,9 @@ cudaError_t launch_dense_tc(void* amps, const TcParams& p, cudaStream_t st);
 // test of the bounded-wait path: a wait on an mbarrier nothing arrives at, given up after `polls` polls (qs_tc.cu)
 cudaError_t launch_test_wait_timeout(int* err, uint32_t polls, cudaStream_t st);
 // complex128 dense gates on the fp16 tensor cores, exact byte slices, 3 <= n <= 6 kernel targets (qs_tc_ozaki.cu);
-// scratch: kWideScratch bytes of device memory used on st alone (six targets: the sliced matrix)
-cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st);
+// scratch: kWideScratch bytes of device memory used on st alone (six targets: the sliced matrix).  Six targets:
+// nothing is done if the matrix does not mix every group (k_wide_matrix); the flags at *when say so
+cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st, const int** when = nullptr);
 cudaError_t launch_block_compose(const ComposeBlock* blocks, int nblocks, const ComposeInstr* instrs,
                                  const double* data, double* out, cudaStream_t st);
 // cost-model network (qs_mlp.cu)

@@ -997,7 +997,11 @@ namespace {
 // layout of the scratch that k_wide_matrix fills
 constexpr int kWideStart = 16 * kKnBlock;            // four start operands (N block) of 256 columns x 32 bytes
 constexpr int kWideScale = kWideStart + 4 * 8192;    // of 128 columns: exponent increment, largest high word
-static_assert(kWideScale + 8 * 128 <= (int)kWideScratch, "scratch of the six-target kernel");
+constexpr int kWideFlag = kWideScale + 8 * 128;      // kWideFlags flags: the matrix does not mix the group
+static_assert(kWideFlag + 4 * kWideFlags <= (int)kWideScratch && kWideFlags == 128, "scratch of the six-target kernel");
+// An output whose coefficients all lie within 2^-kMixBits of the largest depends on
+// every amplitude of its group, the largest among them.
+constexpr uint32_t kMixBits = 16;
 
 struct W6 {
   static constexpr int D = 64, K = 128, KB = 4;
@@ -1030,6 +1034,18 @@ __device__ __forceinline__ int k_block(int np, int j) { return np ? W6::KB - 1 -
 
 // One block per column of the realified six-target matrix, one thread per row:
 // digits into the 32 x 32 blocks of the scratch, start operands, column scale.
+//
+// Also whether the byte slices may stand in for FP64.  They hold an amplitude to 2^-55
+// of the largest of its group.  Where every output depends on that largest one that is
+// what an output can be held to (rounding errors of FP64 sums are of its size too), but
+// a matrix with zeros (a permutation, a diagonal, a gate with controls of its own) keeps
+// small amplitudes apart from large ones, and FP64 then keeps all their bits.  So a
+// matrix with an entry below 2^-16 of its row's largest, or one that is not finite, raises
+// a flag: k_dense_ozaki6 returns, and the FP64 kernel (or the double-float one, by the
+// handle's arithmetic) that is launched after it, and returns otherwise, makes the
+// pass.  2^-16: of Haar matrices one in 130 thousand has such an entry.  28 qubits,
+// spread targets: 3.98 ms mixing, 111 ms in FP64; the kernel that returns takes 2 us and
+// a launch (calls at 2^7 to 2^18 amplitudes 38 to 42 us without it, 43 to 47 with it).
 __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcParams p, unsigned char* __restrict__ out) {
   constexpr int D = 64, K = 128;
   __shared__ int mx, sums[kLv];
@@ -1041,6 +1057,7 @@ __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcP
   const double v = (n & 1) ? ((k & 1) ? m.x : m.y) : ((k & 1) ? -m.y : m.x);
   atomicMax(&mx, __double2hiint(v) & 0x7FFFFFFF);
   __syncthreads();
+  const bool flag = __syncthreads_or(mx >= 0x7FF00000 || max(abs_hi(m.x), abs_hi(m.y)) + (kMixBits << 20) < (uint32_t)mx);
   const uint32_t ef = qsby::row_field((uint32_t)mx);
   int d[qsby::kB];
   qsby::digits_b((uint32_t)__double2hiint(v), (uint32_t)__double2loint(v), ef, d);
@@ -1057,6 +1074,7 @@ __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcP
     int* col = reinterpret_cast<int*>(out + kWideScale) + 2 * n;
     col[0] = column_scale((int)ef);
     col[1] = mx;
+    reinterpret_cast<int*>(out + kWideFlag)[n] = flag;
   }
 }
 
@@ -1064,6 +1082,7 @@ template <bool PAIRS>
 __global__ void __launch_bounds__(W6::THREADS, 1)
     k_dense_ozaki6(double2* __restrict__ psi, const __grid_constant__ TcParams p, const unsigned char* __restrict__ wide) {
   using X = W6;
+  if (any_flag(reinterpret_cast<const int*>(wide + kWideFlag))) return;
   constexpr int K = X::K, KB = X::KB, NPASS = 2;
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* a_dig = smem;
@@ -1248,6 +1267,9 @@ static cudaError_t dense_ozaki6(void* amps, const TcParams& p, void* scratch, cu
   static bool attr_done = false;
   if (!attr_done) {
     cudaError_t e = cudaFuncSetAttribute(k_dense_ozaki6<PAIRS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W6::bytes);
+    // the three kernels of a pass in one split of shared memory and L1 (changing it
+    // between them took 3 us a call)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wide_matrix, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
@@ -1275,7 +1297,8 @@ static cudaError_t dense_ozaki(void* amps, const TcParams& p, void* scratch, cud
 // pairs: 3, 4, 5, 6 targets on qubits 0, 1, ...: 2.50 / 2.27, 3.01 / 2.34, 3.32 / 2.73, 5.03 / 4.33; on
 // qubit 0 and high ones: 1.94 / 1.71, 1.99 / 1.77, 2.25 / 2.20, 3.92 / 3.86.  Other
 // passes keep the plain form: the exchange costs the producers up to 8% there.
-cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st) {
+cudaError_t launch_dense_ozaki(void* amps, const TcParams& p, void* scratch, cudaStream_t st, const int** when) {
+  if (when) *when = p.n == 6 ? reinterpret_cast<const int*>(static_cast<unsigned char*>(scratch) + kWideFlag) : nullptr;
   if (p.tpos[0] == 0 && p.tile_bits > p.n) return dense_ozaki<true>(amps, p, scratch, st);
   return dense_ozaki<false>(amps, p, scratch, st);
 }

@@ -1,0 +1,128 @@
+"""Six-target complex128 gates whose matrix keeps amplitudes of a group apart
+(permutations, diagonals, gates with controls of their own, entries at rounding level):
+every amplitude keeps the bits that FP64 keeps, however small it is beside the others
+of its group.  The bound is per output: the rounding of a sum of K products,
+K 2^-53 sum_l |m_jl| |x_l| (a permutation is exact), in every way that such a pass is
+made."""
+
+import numpy as np
+import pytest
+
+from oracle import qsim_oracle as orc
+from paper_2311_01512_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def matrix(kind, rng):
+    if kind == "identity":
+        return np.eye(64, dtype=np.complex128)
+    if kind == "permutation":
+        return np.eye(64, dtype=np.complex128)[rng.permutation(64)]
+    if kind == "diagonal":
+        return np.diag(np.exp(1j * rng.uniform(0, 6, 64)))
+    m = np.eye(64, dtype=np.complex128)
+    if kind == "controlled":
+        m[32:, 32:] = wl.haar_unitary(32, rng)
+    if kind == "noise":                         # zeros of a composed block at rounding level
+        m[:32, :32] = wl.haar_unitary(32, rng)
+        m += 1e-17 * (rng.standard_normal((64, 64)) + 1j * rng.standard_normal((64, 64)))
+    return m
+
+
+def spread_state(size, rng):
+    v = (rng.standard_normal(size) + 1j * rng.standard_normal(size)) * 2.0 ** -rng.integers(0, 70, size=size)
+    v[rng.integers(0, size, size=size // 8)] = 0.0
+    return v
+
+
+def check(got, psi, ops, density, unit):
+    """Each pass of ops within 2 K units of sum |m| |x|, per output."""
+    want = orc.run_ops(psi, ops, is_density=density)
+    mags = [dict(op, mat=np.abs(op["mat"]).astype(np.complex128)) for op in ops]
+    size = orc.run_ops(np.abs(psi).astype(np.complex128), mags, is_density=density).real
+    passes = len(ops) * (2 if density else 1)
+    assert np.all(np.abs(got - want) <= passes * 2 * 128 * unit * size)
+
+
+@pytest.mark.parametrize("kind", ["identity", "permutation", "diagonal", "controlled", "noise"])
+@pytest.mark.parametrize("nq,density", [(6, False), (7, False), (9, False), (14, False), (20, False), (6, True), (7, True)])
+def test_passes(kind, nq, density):
+    import torch
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(660 + nq)
+    psi = spread_state(1 << (2 * nq if density else nq), rng)
+    mat = np.ascontiguousarray(matrix(kind, rng))
+    exact = kind in ("identity", "permutation")
+    for ctrls in ([], [0]) if nq > 6 else ([],):
+        targs = [int(t) for t in rng.permutation(nq) if t not in ctrls][:6]
+        op = {"op": "unitary", "ctrls": ctrls, "targs": targs, "mat": mat}
+        st = qs.State(nq, density=density, stream=torch.cuda.Stream())
+        for way in ("call", "block", "program"):
+            if way == "block" and ctrls:
+                continue
+            st.set_amps(psi)
+            if way == "call":
+                qs.apply_op(st.handle, op)
+            elif way == "block":
+                qs.qs_apply_dense_block(st.handle, targs, mat)
+            else:
+                qs.qs_record_begin(st.handle)
+                qs.apply_op(st.handle, op)
+                prog = qs.qs_record_end(st.handle)
+                qs.qs_program_run(prog)
+            qs.qs_synchronize(st.handle)
+            got = st.get_amps()
+            if way == "program":
+                qs.qs_program_destroy(prog)
+            if exact:
+                assert np.array_equal(got, orc.run_ops(psi, [op], is_density=density)), way
+            check(got, psi, [op], density, 2.0 ** -53)
+        st.close()
+
+
+@pytest.mark.parametrize("kind", ["permutation", "controlled"])
+def test_double_float(kind):
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(67)
+    psi = spread_state(1 << 13, rng)
+    op = {"op": "unitary", "ctrls": [], "targs": [int(t) for t in rng.permutation(13)[:6]],
+          "mat": np.ascontiguousarray(matrix(kind, rng))}
+    st = qs.State(13)
+    qs.qs_set_arithmetic(st.handle, qs.QS_ARITH_DF)
+    st.set_amps(psi)
+    qs.apply_op(st.handle, op)
+    qs.qs_synchronize(st.handle)
+    got = st.get_amps()
+    st.close()
+    check(got, psi, [op], False, 2.0 ** -46)
+
+
+def test_composed_block_and_channel():
+    """A fused block of NOTs with controls, and a three-qubit Kraus map of one
+    permutation: both keep every bit."""
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(68)
+    x = np.array([[0, 1], [1, 0]], dtype=np.complex128)
+    ops = []
+    for _ in range(12):
+        q = [int(t) for t in rng.permutation(6)]
+        ops.append({"op": "unitary", "ctrls": q[1:1 + int(rng.integers(0, 3))], "targs": q[:1], "mat": x})
+    psi = spread_state(1 << 12, rng)
+    st = qs.State(12)
+    st.set_amps(psi)
+    circ = qs.Circuit(12, ops)
+    circ.plan(qs.QS_PLAN_GREEDY, 6)
+    circ.apply(st.handle)
+    qs.qs_synchronize(st.handle)
+    assert np.array_equal(st.get_amps(), orc.run_ops(psi, ops, is_density=False))
+    circ.close()
+    st.close()
+    rho = spread_state(1 << 10, rng)
+    kraus = [np.eye(8, dtype=np.complex128)[rng.permutation(8)]]
+    dm = qs.State(5, density=True)
+    dm.set_amps(rho)
+    qs.qs_apply_kraus(dm.handle, [3, 0, 2], kraus)
+    got = dm.get_amps()
+    dm.close()
+    assert np.array_equal(got, orc.run_ops(rho, [{"op": "kraus", "targs": [3, 0, 2], "kraus": kraus}], is_density=True))
