@@ -990,6 +990,9 @@ static cudaError_t dense_ozaki5(void* amps, const TcParams& p, cudaStream_t st) 
 // caller's scratch, and another warp streams the 16 KB block of each (K, N) pair
 // from L2 into a ring of four slots with bulk copies.  Hand-offs as for five
 // targets, with bfull (bulk copy) and bempty (MMA completion) for B's slots.
+// Rows that the slices cannot hold as FP64 did (an infinity or NaN, amplitudes all below
+// 2^-965, results near the ends of the exponent range) are left alone and then made in
+// FP64, one warp a row.
 // Bound by the tensor cores (53% busy, two fifths of each tile's time being the
 // epilogues and slicing that share its 16 warps): 34.7 thousand cycles per tile.
 // ---------------------------------------------------------------------------
@@ -1030,6 +1033,34 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 
 // K block of step j of pass np over K: the second pass goes back
 __device__ __forceinline__ int k_block(int np, int j) { return np ? W6::KB - 1 - j : j; }
+
+// One group (amplitudes at base | target bits) in FP64 by one warp, with the sums of the
+// FP64 kernel: a lane holds two amplitudes and two outputs.
+__device__ __noinline__ void group_f64(double2* psi, uint64_t base, const TcParams& p, int lane) {
+  uint64_t at[2] = {base, base};
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    for (int q = 0; q < 6; ++q)
+      if ((lane + 32 * e) >> p.mbit[q] & 1) at[e] |= 1ull << p.tpos[q];
+  const double2 x[2] = {psi[at[0]], psi[at[1]]};
+  const double2* m = reinterpret_cast<const double2*>(p.mat) + 64 * lane;
+  double2 y[2] = {make_double2(0.0, 0.0), make_double2(0.0, 0.0)};
+  for (int l = 0; l < 64; ++l) {
+    const double xr = __shfl_sync(0xFFFFFFFFu, l < 32 ? x[0].x : x[1].x, l & 31);
+    const double xi = __shfl_sync(0xFFFFFFFFu, l < 32 ? x[0].y : x[1].y, l & 31);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      double2 c = m[2048 * e + l];
+      if (p.conj) c.y = -c.y;
+      y[e].x = fma(c.x, xr, y[e].x);
+      y[e].x = fma(-c.y, xi, y[e].x);
+      y[e].y = fma(c.x, xi, y[e].y);
+      y[e].y = fma(c.y, xr, y[e].y);
+    }
+  }
+  psi[at[0]] = y[0];
+  psi[at[1]] = y[1];
+}
 }  // namespace
 
 // One block per column of the realified six-target matrix, one thread per row:
@@ -1044,7 +1075,7 @@ __device__ __forceinline__ int k_block(int np, int j) { return np ? W6::KB - 1 -
 // a flag: k_dense_ozaki6 returns, and the FP64 kernel (or the double-float one, by the
 // handle's arithmetic) that is launched after it, and returns otherwise, makes the
 // pass.  2^-16: of Haar matrices one in 130 thousand has such an entry.  28 qubits,
-// spread targets: 3.98 ms mixing, 111 ms in FP64; the kernel that returns takes 2 us and
+// spread targets: 3.96 ms mixing, 111 ms in FP64; the kernel that returns takes 2 us and
 // a launch (calls at 2^7 to 2^18 amplitudes 38 to 42 us without it, 43 to 47 with it).
 __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcParams p, unsigned char* __restrict__ out) {
   constexpr int D = 64, K = 128;
@@ -1165,11 +1196,15 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
       for (int i = 0; i < KB * 4; ++i) mx = max_abs(mx, R[i]);
       atomicMax(rowmax + slot * kRows + g, (int)mx);   // the four threads of a row are in different warps
       if (compute_barrier_or(bad || *abort_flag)) break;
-      const uint32_t ef = qsby::row_field((uint32_t)rowmax[slot * kRows + g]);   // exponent field of the row
+      const uint32_t mr = (uint32_t)rowmax[slot * kRows + g];
+      const uint32_t ef = qsby::row_field(mr);   // exponent field of the row
       // the previous tile's slot: read by every warp before this barrier, next
       // written after the following one
       if (cg == 0) rowmax[(slot == 0 ? 2 : slot - 1) * kRows + g] = 0;
-      const bool rare = (int)ef < lim[0] || (int)ef > lim[1];
+      // a row that is not finite, below the slices' range, or whose results may be: its
+      // amplitudes stay as they are until the tile is done
+      const bool far = row_ok && mr != 0 && (mr >= 0x7FF00000u || mr < (uint32_t)qsby::kFloor << 20 ||
+                                             (int)ef < lim[0] || (int)ef > lim[1]);
       const bool has_next = c + grid < p.ntiles;
       xb = ((xb | hole) + gstep) & ~hole;
       const uint64_t rb_next = xb | roff;
@@ -1196,9 +1231,12 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
           ++reads[h];
           fence_after_sync();
           epilogue_block<K, 8, PAIRS>(tmem + (uint32_t)(256 * h + 8 * cg) + lane_addr, tempty + h, csc + 32 * nb + 8 * cg, (int)ef,
-                               rare, row_ok, lane, [&](int a) { return psi + (rb | toff[16 * nb + 4 * cg + a]); });
+                               false, row_ok && !far, lane, [&](int a) { return psi + (rb | toff[16 * nb + 4 * cg + a]); });
         }
       }
+      if (cg == 0)
+        for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, far); todo != 0; todo &= todo - 1)
+          group_f64(psi, __shfl_sync(0xFFFFFFFFu, rb, __ffs(todo) - 1), p, lane);
       rb = rb_next;
     }
   } else if (warp == kKnWarps && lane == 0) {

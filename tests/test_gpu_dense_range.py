@@ -52,7 +52,9 @@ def test_small_results(n, nq, density, e_amp, e_mat):
     assert diff.max() <= np.ldexp(tol, e) + K * 2.0 ** -1021
 
 
-@pytest.mark.parametrize("n,nq,density", [(3, 20, False), (4, 18, False), (5, 18, False), (6, 9, False), (3, 5, True)])
+# (Six targets take FP64 sums there, whose partial sums may overflow before the result
+# does: test_gpu_six_targets.py holds them to native FP64 bit for bit.)
+@pytest.mark.parametrize("n,nq,density", [(3, 20, False), (4, 18, False), (5, 18, False), (3, 5, True)])
 def test_large_results(n, nq, density):
     rng = np.random.default_rng(190 + 10 * n + nq)
     size = 1 << (2 * nq if density else nq)

@@ -126,3 +126,70 @@ def test_composed_block_and_channel():
     got = dm.get_amps()
     dm.close()
     assert np.array_equal(got, orc.run_ops(rho, [{"op": "kraus", "targs": [3, 0, 2], "kraus": kraus}], is_density=True))
+
+
+def gate(arith, nq, targs, ctrls, mat, psi, density=False):
+    from paper_2311_01512_gb300 import qs
+    st = qs.State(nq, density=density)
+    qs.qs_set_arithmetic(st.handle, arith)
+    st.set_amps(psi)
+    qs.qs_apply_ctrl_multi_target(st.handle, ctrls, targs, mat)
+    qs.qs_synchronize(st.handle)
+    got = st.get_amps()
+    st.close()
+    return got
+
+
+@pytest.mark.parametrize("nq", [6, 7, 12, 13, 14, 20])
+def test_groups_out_of_range(nq):
+    """With a matrix that mixes: groups that hold an infinity or a NaN, are far too
+    small, or have such results come out as in native FP64, bit for bit, the others as
+    without them."""
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(670 + nq)
+    mat = np.ascontiguousarray(wl.haar_unitary(64, rng))
+    perm = [int(t) for t in rng.permutation(nq)]
+    targs = perm[:6]
+    ctrls = perm[6:7] if nq > 7 else []
+    size = 1 << nq
+    psi = rng.standard_normal(size) + 1j * rng.standard_normal(size)
+    idx = np.arange(size)
+    group = idx.copy()
+    for t in targs:
+        group &= ~(1 << t)
+    groups = np.unique(group[[(i & sum(1 << c for c in ctrls)) == sum(1 << c for c in ctrls) for i in idx]])
+    values = [complex(np.inf, 1.0), complex(0.0, -np.inf), complex(np.nan, 0.0), "tiny", "large", "zero", "subnormal"]
+    odd = rng.permutation(groups)[:min(len(groups), 64)]
+    changed = psi.copy()
+    for k, g in enumerate(odd):
+        v = values[k % len(values)]
+        members = idx[group == g]
+        if isinstance(v, complex):
+            changed[rng.choice(members)] = v
+        else:
+            changed[members] *= {"tiny": 2.0 ** -1000, "large": 2.0 ** 1018, "zero": 0.0, "subnormal": 2.0 ** -1030}[v]
+    got = gate(qs.QS_ARITH_FX, nq, targs, ctrls, mat, changed)
+    plain = gate(qs.QS_ARITH_FX, nq, targs, ctrls, mat, psi)
+    native = gate(qs.QS_ARITH_F64, nq, targs, ctrls, mat, changed)
+    rest = ~np.isin(group, odd)
+    assert np.array_equal(got[rest].view(np.uint64), plain[rest].view(np.uint64))
+    for k, g in enumerate(odd):
+        if values[k % len(values)] != "large":
+            m = group == g
+            assert np.array_equal(got[m].view(np.float64), native[m].view(np.float64), equal_nan=True), values[k % len(values)]
+    large = np.isin(group, odd[4::len(values)])
+    g, w = got[large].view(np.float64), native[large].view(np.float64)
+    assert np.array_equal(np.isfinite(g), np.isfinite(w))
+    assert np.all(np.abs(g - w)[np.isfinite(w)] <= 1e-13 * np.float64(2.0) ** 1021)
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan, complex(0, np.inf)])
+def test_matrix_not_finite(value):
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(69)
+    mat = np.ascontiguousarray(wl.haar_unitary(64, rng))
+    mat[5, 9] = value
+    psi = rng.standard_normal(1 << 9) + 1j * rng.standard_normal(1 << 9)
+    args = (9, [4, 0, 7, 2, 8, 5], [], mat, psi)
+    got, want = gate(qs.QS_ARITH_FX, *args), gate(qs.QS_ARITH_F64, *args)
+    assert np.array_equal(got.view(np.float64), want.view(np.float64), equal_nan=True)
