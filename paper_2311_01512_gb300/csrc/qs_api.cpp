@@ -206,6 +206,7 @@ struct qs_program {
   qs_state* state = nullptr;
   std::vector<void*> chunks;      // device arena, never moved (the graph holds its addresses)
   size_t used = 0, cap = 0;       // in the last chunk
+  void* wide = nullptr;           // scratch of its six-target gates, which run one after another
   cudaStream_t side = nullptr;    // uploads during recording (outside the capture)
   std::vector<std::vector<unsigned char>> staged;  // their host copies, until the recording ends
   cudaGraph_t graph = nullptr;
@@ -292,14 +293,17 @@ qs_status ring_take(qs_state* s, size_t bytes, void** dev, int* slot) {
   return QS_OK;
 }
 
-// The same over as many consecutive slots as `bytes` needs, [*first, *first + *count).
-qs_status ring_take_run(qs_state* s, size_t bytes, void** dev, int* first, int* count) {
+// Scratch of a six-target gate: as many consecutive slots as it needs, [*first, *first +
+// *count), or while recording the program's own, shared by its gates.
+qs_status take_wide(qs_state* s, void** dev, int* first, int* count) {
   if (s->rec) {
     *first = -1;
     *count = 0;
-    *dev = rec_alloc(s->rec, bytes);
+    if (!s->rec->wide) s->rec->wide = rec_alloc(s->rec, qsk::kWideScratch);
+    *dev = s->rec->wide;
     return *dev ? QS_OK : QS_ERR_OOM;
   }
+  const size_t bytes = qsk::kWideScratch;
   const int n = (int)((bytes + kSlotBytes - 1) / kSlotBytes);
   if (n > kRingSlots) return QS_ERR_ARG;
   const int k = s->ring_next + n <= kRingSlots ? s->ring_next : 0;
@@ -606,7 +610,7 @@ qs_status gate_pass(qs_state* s, const std::vector<int>& ctrls, const std::vecto
     const int* when = nullptr;
     void* wide = nullptr;
     int first = -1, count = 0;
-    qs_status st = ring_take_run(s, qsk::kWideScratch, &wide, &first, &count);
+    qs_status st = take_wide(s, &wide, &first, &count);
     if (st != QS_OK) return st;
     st = cuda_status(qsk::launch_dense_ozaki(s->amps, p, wide, s->stream, &when));
     if (st == QS_OK) st = cuda_core_pass(s, ctrls, targs, dev_mat, conj, when);

@@ -193,3 +193,33 @@ def test_matrix_not_finite(value):
     args = (9, [4, 0, 7, 2, 8, 5], [], mat, psi)
     got, want = gate(qs.QS_ARITH_FX, *args), gate(qs.QS_ARITH_F64, *args)
     assert np.array_equal(got.view(np.float64), want.view(np.float64), equal_nan=True)
+
+
+def test_recorded_gates_share_their_scratch():
+    """Sixty recorded six-target gates need the memory of their matrices (3.8 MB, two
+    chunks of the program's 4 MB with its scratch), not a scratch each (18 MB more)."""
+    import torch
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(70)
+    nq = 8
+    psi = wl.random_statevector(nq, rng)
+    ops = [{"op": "unitary", "ctrls": [], "targs": [int(t) for t in rng.permutation(nq)[:6]],
+            "mat": wl.haar_unitary(64, rng) if k % 3 else matrix("controlled", rng)} for k in range(60)]
+    st = qs.State(nq, stream=torch.cuda.Stream())
+    st.set_amps(psi)
+    qs.qs_record_begin(st.handle)
+    try:
+        qs.qs_test_fail_allocations(1, 100)
+        for op in ops:
+            qs.apply_op(st.handle, op)
+    finally:
+        qs.qs_test_fail_allocations(0, 0)
+    prog = qs.qs_record_end(st.handle)
+    want = psi
+    for _ in range(2):
+        qs.qs_program_run(prog)
+        want = orc.run_ops(want, ops, is_density=False)
+    qs.qs_synchronize(st.handle)
+    assert np.max(np.abs(st.get_amps() - want)) < 1e-13
+    qs.qs_program_destroy(prog)
+    st.close()
