@@ -20,6 +20,7 @@
 // can take those instead: launch k runs the k-th pass of every such state, one block
 // per tile, while a second branch of the graph runs the other states.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -446,8 +447,8 @@ qs_status qs_batch_add_two_qubit_depolarising(qs_batch* b, int state, int t1, in
   return add_channel2(b, state, t1, t2, true, p);
 }
 
-qs_status qs_batch_compile(qs_batch* b, int autotune) {
-  if (!b || !b->pool) return QS_ERR_ARG;
+// with_passes: complex64 states whose operations fit may take tile passes.
+static qs_status compile(qs_batch* b, int autotune, bool with_passes) {
   free_device(b);
   const int S = (int)b->nq.size();
   std::vector<qsk::BatchState> states(S);
@@ -489,7 +490,7 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
   std::vector<char> tiled(S, 0);
   std::vector<unsigned char> passes;         // packed
   std::vector<qstile::TileItem> items;
-  if (b->prec == QS_C64) {
+  if (with_passes) {
     try {
       std::vector<std::vector<uint32_t>> of(S);   // where a state's passes start
       size_t levels = 0;
@@ -504,6 +505,7 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
           if (k < of[s].size())
             for (uint32_t t = 0; t < 1u << (b->nq[s] - qstile::kPassBits); ++t)
               items.push_back(qstile::TileItem{b->offset[s], of[s][k], t});
+        if (items.size() > INT_MAX) throw std::bad_alloc();   // more than a launch numbers
       }
       b->level.push_back((int)items.size());
     } catch (const std::bad_alloc&) {             // without tile passes
@@ -693,6 +695,14 @@ qs_status qs_batch_compile(qs_batch* b, int autotune) {
   }
   b->compiled = true;
   return QS_OK;
+}
+
+qs_status qs_batch_compile(qs_batch* b, int autotune) {
+  if (!b || !b->pool) return QS_ERR_ARG;
+  const bool c64 = b->prec == QS_C64;
+  const qs_status st = compile(b, autotune, c64);
+  // no device memory beside the tile passes' descriptors: the persistent launch alone
+  return st == QS_ERR_OOM && c64 ? compile(b, autotune, false) : st;
 }
 
 qs_status qs_batch_run(qs_batch* b) {

@@ -47,3 +47,41 @@ def test_tiled_states(sizes, dens):
         # 20 2^-24 of the norm a gate (a density matrix's gates are two operations each)
         bound = (2 * len(ops) * (2 if d else 1) + 1) * 20 * 2.0 ** -24 * max(1.0, np.linalg.norm(want))
         assert np.linalg.norm(batch.view(s).cpu().numpy() - want) <= bound, s
+
+
+@pytest.mark.parametrize("autotune", [False, True])
+def test_without_memory_for_the_passes(autotune):
+    """A batch whose descriptors do not fit into device memory beside those of its tile
+    passes, whichever allocation finds that out, runs in the persistent launch alone; if
+    that does not fit either, it is reported and the batch compiles afterwards."""
+    import torch
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(31)
+    sizes = [13, 12, 9]
+    batch = qs.Batch(sizes, prec=qs.QS_C64)
+    circuits = [wl.unitary_circuit(nq, 20, rng) for nq in sizes]
+    for s, ops in enumerate(circuits):
+        for op in ops:
+            batch.add(s, op)
+    inits = [wl.random_statevector(nq, rng) for nq in sizes]
+    for skip in range(8):
+        try:
+            qs.qs_test_fail_allocations(skip, 1)
+            batch.compile(autotune=autotune)
+        finally:
+            qs.qs_test_fail_allocations(0, 0)
+        for s, psi in enumerate(inits):
+            batch.view(s).copy_(torch.from_numpy(psi.astype(np.complex64)))
+        batch.run()
+        torch.cuda.synchronize()
+        for s, (psi, ops) in enumerate(zip(inits, circuits)):
+            want = orc.run_ops(psi, ops, is_density=False)
+            assert np.linalg.norm(batch.view(s).cpu().numpy() - want) <= (len(ops) + 1) * 20 * 2.0 ** -24, (skip, s)
+    try:
+        qs.qs_test_fail_allocations(0, 100)
+        with pytest.raises(qs.QSError) as ei:
+            batch.compile(autotune=autotune)
+        assert "QS_ERR_OOM" in str(ei.value)
+    finally:
+        qs.qs_test_fail_allocations(0, 0)
+    batch.compile(autotune=autotune)
