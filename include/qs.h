@@ -442,8 +442,8 @@ qs_status qs_batch_info(const qs_batch* batch, int* threads, int* ctas, int* sme
  * staging ring, recorded-program arenas, circuit matrices, batch tables)
  * succeed and the `count` after them fail as if out of memory, without
  * calling CUDA.  The caller then returns QS_ERR_OOM having freed what it had
- * taken.  count = 0 turns the injection off.  Process-wide; QS_ERR_ARG for
- * negative arguments. */
+ * taken (a complex64 batch after trying without its tile passes).  count = 0
+ * turns the injection off.  Process-wide; QS_ERR_ARG for negative arguments. */
 qs_status qs_test_fail_allocations(int skip, int count);
 
 /* Set the handle's device error word, as a tensor-core kernel does when one
@@ -457,6 +457,10 @@ qs_status qs_test_set_error_word(qs_state* state);
  * out.  Queued on the handle's stream; the next qs_synchronize reports
  * QS_ERR_TIMEOUT once.  Nothing faults or hangs. */
 qs_status qs_test_bounded_wait(qs_state* state, unsigned polls);
+
+/* Tile passes of a planned circuit, over all its runs of blocks that complex64
+ * statevectors take in them; -1 before the plan has met such a state. */
+qs_status qs_test_circuit_passes(qs_circuit* circuit, int* num_passes);
 
 /* Largest number of terms qs_expec_pauli_sum_noalloc accepts. */
 #define QS_NOALLOC_MAX_TERMS 256

@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -58,7 +59,11 @@ struct qs_circuit {
   std::vector<CGate> gates;
   std::vector<CBlock> blocks;
   bool planned = false;
-  std::vector<TileRun> runs;    // of a plan with fused blocks, in order
+  // tile passes of a plan with fused blocks, in order; formed for the first complex64
+  // statevector (form_runs)
+  std::vector<TileRun> runs;
+  bool runs_formed = false;
+  std::mutex runs_mutex;
   double* d_mats = nullptr;
   size_t mats_bytes = 0;
   // lazy relabelling (qs_circuit_plan_relabel): physical SWAPs before each
@@ -236,6 +241,21 @@ void find_runs(qs_circuit* c) {
   }
 }
 
+// The runs, formed once a plan: when it is made for a complex64 statevector, or first
+// applied to one (in any thread).  Other states have no use for them: scheduling takes
+// 0.1 s for 100,000 gates.
+void form_runs(qs_circuit* c) {
+  std::lock_guard<std::mutex> lock(c->runs_mutex);
+  if (c->runs_formed) return;
+  try {
+    find_runs(c);
+  } catch (const std::bad_alloc&) {
+    c->runs.clear();                 // block by block
+  }
+  c->runs_formed = true;
+}
+bool takes_runs(const qs_state* s) { return s->prec == QS_C64 && !s->is_density; }
+
 void close_block(qs_circuit* c, int first, int last, uint64_t mask) {
   CBlock b;
   b.first = first;
@@ -265,11 +285,8 @@ qs_status qs_circuit_set_blocks_internal(qs_circuit* c, const std::vector<int>& 
   }
   qs_status st = compose(c);
   c->planned = st == QS_OK;
-  try {
-    find_runs(c);
-  } catch (const std::bad_alloc&) {
-    c->runs.clear();                 // block by block
-  }
+  c->runs.clear();
+  c->runs_formed = false;
   return st;
 }
 
@@ -418,7 +435,9 @@ qs_status qs_circuit_plan_cost(qs_circuit* c, qs_costmodel* model, const qs_stat
   std::vector<int> starts;
   for (int j = G; j > 0; j = from[j]) starts.push_back(from[j]);
   std::reverse(starts.begin(), starts.end());
-  return qs_circuit_set_blocks_internal(c, starts, max_block_qubits);
+  st = qs_circuit_set_blocks_internal(c, starts, max_block_qubits);
+  if (st == QS_OK && takes_runs(s)) form_runs(c);
+  return st;
 }
 
 qs_status qs_circuit_plan_relabel(qs_circuit* c, qs_costmodel* model, const qs_state* s, int low_qubits,
@@ -535,6 +554,15 @@ qs_status qs_circuit_get_relabel(const qs_circuit* c, int* num_swaps) {
   return QS_OK;
 }
 
+qs_status qs_test_circuit_passes(qs_circuit* c, int* num_passes) {
+  if (!c || !num_passes) return QS_ERR_ARG;
+  std::lock_guard<std::mutex> lock(c->runs_mutex);
+  int n = 0;
+  for (const TileRun& r : c->runs) n += (int)r.at.size();
+  *num_passes = c->runs_formed ? n : -1;
+  return QS_OK;
+}
+
 qs_status qs_circuit_get_plan(const qs_circuit* c, int* num_gates, int* num_blocks, int* num_fused) {
   if (!c) return QS_ERR_ARG;
   int fused = 0;
@@ -573,8 +601,9 @@ qs_status qs_circuit_apply(qs_circuit* c, qs_state* s) {
   };
   // tile passes: complex64 statevectors; a relabelled plan only as a whole (its
   // passes need no swaps)
+  if (takes_runs(s)) form_runs(c);
   const bool whole = c->runs.size() == 1 && c->runs[0].first == 0 && c->runs[0].last == c->blocks.size();
-  const bool tiles = s->prec == QS_C64 && !s->is_density && (!rl || whole);
+  const bool tiles = takes_runs(s) && (!rl || whole);
   size_t run = 0;
   for (size_t bi = 0; bi < c->blocks.size(); ++bi) {
     if (tiles && run < c->runs.size() && c->runs[run].first == bi) {

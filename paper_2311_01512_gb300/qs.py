@@ -46,6 +46,7 @@ SIGNATURES = {
     "qs_test_fail_allocations": (_I, [_I, _I]),
     "qs_test_set_error_word": (_I, [_P]),
     "qs_test_bounded_wait": (_I, [_P, ctypes.c_uint]),
+    "qs_test_circuit_passes": (_I, [_P, _IP]),
     "qs_device_ptr": (_I, [_P, ctypes.POINTER(_P)]),
     "qs_set_arithmetic": (_I, [_P, _I, _I]),
     "qs_set_tensor_cores": (_I, [_P, _I]),
@@ -334,6 +335,14 @@ def qs_test_bounded_wait(h, polls):
     """Test hook: a device wait that nothing ends runs out after `polls`
     polls and sets the handle's error word (see include/qs.h)."""
     _check(_lib.qs_test_bounded_wait(h, int(polls)), "qs_test_bounded_wait")
+
+
+def qs_test_circuit_passes(circuit):
+    """Test hook: tile passes of a planned Circuit, -1 before it has met a
+    complex64 statevector (see include/qs.h)."""
+    n = _I(0)
+    _check(_lib.qs_test_circuit_passes(circuit.handle, ctypes.byref(n)), "qs_test_circuit_passes")
+    return n.value
 
 
 def qs_calc_norm_or_trace(h):

@@ -73,3 +73,35 @@ def test_circuits(nq, mode):
     c.close()
     st.close()
     assert np.linalg.norm(got - want) <= (len(ops) + 1) * 20 * 2.0 ** -24 * np.linalg.norm(want)
+
+
+def test_passes_are_formed_for_the_states_that_take_them():
+    """A plan forms its tile passes when it first meets a complex64 statevector (of at
+    least 12 qubits, with fused blocks), not for other states; and again for a new plan."""
+    from paper_2311_01512_gb300 import costmodel, qs
+    rng = np.random.default_rng(77)
+    nq = 13
+    ops = wl.unitary_circuit(nq, 60, rng)
+    psi = wl.random_statevector(nq, rng)
+    single, double = qs.State(nq, prec=qs.QS_C64), qs.State(nq)
+    model, _ = costmodel.load()
+    c = qs.Circuit(nq, ops)
+    c.plan(qs.QS_PLAN_GREEDY, 4)
+    double.set_amps(psi)
+    c.apply(double.handle)
+    assert qs.qs_test_circuit_passes(c) == -1
+    single.set_amps(psi)
+    c.apply(single.handle)
+    assert qs.qs_test_circuit_passes(c) > 0
+    c.plan_cost(model, double.handle, max_block_qubits=4, window=24)
+    assert qs.qs_test_circuit_passes(c) == -1
+    c.plan_cost(model, single.handle, max_block_qubits=4, window=24)
+    assert qs.qs_test_circuit_passes(c) > 0
+    c.plan(qs.QS_PLAN_NONE, 1)
+    c.apply(single.handle)
+    assert qs.qs_test_circuit_passes(c) == 0
+    qs.qs_synchronize(single.handle)
+    model.close()
+    c.close()
+    single.close()
+    double.close()
