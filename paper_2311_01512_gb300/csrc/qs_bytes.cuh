@@ -10,10 +10,14 @@
 //   V_b = m 2^(62 - Eb) rounded, |V_b| < 2^63: V_b = sum_{t<8} b_t 2^(8 (7 - t))
 // The products a_s b_t with L = s + t <= 7 are summed exactly, one accumulator
 // per level L, and
-//   y = Q 2^(Ea + Eb - 52),  Q = round(sum_L level_L 2^(8 (7 - L)) / 2^16).
+//   y = Q 2^(Ea + Eb - 52 - X),  Q = round(sum_L level_L 2^(8 (7 - L)) / 2^(16 - X)),
+// with X = 2 extra bits where they fit (K <= 64; |Q| < K 2^(54 + X)): a unit of Q is then
+// one of V_a times a power-of-two matrix entry, and a row with one nonzero entry (a
+// permutation, a diagonal) gives back what V_a holds: every bit of amplitudes within
+// 2^-2 of the row's largest.
 // Errors: half a unit of V_a per amplitude (2^-55 2^Ea), nothing from entries of
 // B within 2^10 of their column's largest, half a unit of Q, and the dropped
-// products (below 6 K 2^14 2^-24 units of Q, 0.4 for K = 64).
+// products (below 6 K 2^14 2^-24 2^X units of Q, 0.4 2^X for K = 64).
 //
 // Amplitude digits as bytes.  The integer V_a 2^8 is shifted into place with
 // eight guard bits (truncated) and one 64-bit addition of 128 in every byte
@@ -44,8 +48,9 @@ constexpr int kB = 8;        // digits of a matrix entry
 constexpr int kLevels = 8;   // levels kept
 constexpr uint32_t kMagicBits = 0x3F400000u;   // 0.75
 constexpr int kMagicInt = 12582912;            // 0.75 2^24
-constexpr int kRoundQ = 32768;                 // half a unit of Q, in units of level 7
-constexpr int kScale = 52;                     // y = Q 2^(Ea + Eb - kScale)
+constexpr int kRoundQ = 32768;                 // half a unit of Q at X = 0, in units of level 7
+constexpr int kScale = 52;                     // y = Q 2^(Ea + Eb - kScale - X)
+QS_HD constexpr int extra_bits(int K) { return K <= 64 ? 2 : 0; }   // X
 
 // Lower bound of a row's biased exponent: zeros and subnormals, whose implicit
 // bit is wrongly set below, are then shifted below half a unit.
@@ -133,15 +138,15 @@ QS_HD void digits_b(uint32_t hw, uint32_t lw, uint32_t ef, int* d) {
 QS_HD constexpr int level_bound(int L, int K) { return (L < kA ? L + 1 : kA) * 16384 * K; }
 QS_HD constexpr bool magic_level(int L, int K) { return level_bound(L, K) <= (1 << 22); }
 // Levels 6 and 7 hold less than one unit of Q in their low bits: above 2^22 they
-// are read divided by 2 or 4.
+// are read divided by 2 or 4 (2^-5 of a unit of Q at X = 2).
 QS_HD constexpr int low_shift(int K) { return level_bound(7, K) <= (1 << 22) ? 0 : (level_bound(7, K) <= (1 << 23) ? 1 : 2); }
 
 // Start of level L: minus the offset's share, the magic where it fits, half a
 // unit of Q in level 7.  colsum[t] = sum_k b_t(k).
-QS_HD int start_value(int L, int K, const int* colsum) {
+QS_HD int start_value(int L, int K, const int* colsum, int X = 0) {
   int c = 0;
   for (int t = L < kA ? 0 : L - kA + 1; t <= L; ++t) c += colsum[t];
-  return (magic_level(L, K) ? kMagicInt : 0) + (L == kLevels - 1 ? kRoundQ : 0) - 128 * c;
+  return (magic_level(L, K) ? kMagicInt : 0) + (L == kLevels - 1 ? kRoundQ >> X : 0) - 128 * c;
 }
 
 // P = p[0] + 256 p[1] + 65536 p[2] with |p[i]| <= 256 (exact in fp16), for
@@ -176,15 +181,16 @@ QS_HD int to_int(float v) { return (int)v; }   // exact integers
 // bits; r = 256 b_L + b_(L+1) is then 0x7F400000 + 256 level_L + level_(L+1)
 // mod 2^32, without a wrap for levels of at most 2^22 (257 2^22 < 0x7F400000),
 // so the offsets leave as constants.
-template <int K>
+template <int K, int X = 0>
 QS_HD int64_t combine(const float* v) {
   constexpr uint32_t off = 0x7F400000u;
   const uint32_t r0 = fbits(v[0]) * 256u + fbits(v[1]);
   if constexpr (K <= 32) {
     const uint32_t r1 = fbits(v[2]) * 256u + fbits(v[3]), r2 = fbits(v[4]) * 256u + fbits(v[5]);
     const uint32_t r3 = fbits(v[6]) * 256u + fbits(v[7]);
-    constexpr uint64_t C = ((uint64_t)off << 32) + ((uint64_t)off << 16) + off + (off >> 16);
-    return (int64_t)(((uint64_t)r0 << 32) + ((uint64_t)r1 << 16) + (uint64_t)r2 + (uint64_t)(r3 >> 16) - C);
+    constexpr uint64_t C = ((((uint64_t)off << 32) + ((uint64_t)off << 16) + off) << X) + (off >> (16 - X));
+    return (int64_t)(((uint64_t)r0 << (32 + X)) + ((uint64_t)r1 << (16 + X)) + ((uint64_t)r2 << X) +
+                     (uint64_t)(r3 >> (16 - X)) - C);
   } else {
     constexpr int ls = low_shift(K);
     constexpr float lf = ls == 1 ? 0.5f : 0.25f;
@@ -195,9 +201,12 @@ QS_HD int64_t combine(const float* v) {
       const uint32_t l4 = (uint32_t)to_int(qsdf::fmaf_(v[4], 16777216.0f, 8388608.0f));
       const uint32_t l5 = (uint32_t)to_int(qsdf::fmaf_(v[5], 16777216.0f, 8388608.0f));
       const uint32_t r2 = l4 * 256u + l5;
-      constexpr uint64_t C = ((uint64_t)off << 32) + ((uint64_t)off << 16) + 257ull * 8388608ull + (off >> (16 - ls));
-      return (int64_t)(((uint64_t)r0 << 32) + ((uint64_t)r1 << 16) + (uint64_t)r2 + (uint64_t)(r3 >> (16 - ls)) - C);
+      constexpr uint64_t C = ((((uint64_t)off << 32) + ((uint64_t)off << 16) + 257ull * 8388608ull) << X) +
+                             (off >> (16 - ls - X));
+      return (int64_t)(((uint64_t)r0 << (32 + X)) + ((uint64_t)r1 << (16 + X)) + ((uint64_t)r2 << X) +
+                       (uint64_t)(r3 >> (16 - ls - X)) - C);
     } else {                                       // levels 2 to 5
+      static_assert(X == 0, "no room for more bits");
       const int32_t q1 = to_int(v[2] * 16777216.0f) * 256 + to_int(v[3] * 16777216.0f);
       const int64_t q2 = (int64_t)to_int(v[4] * 16777216.0f) * 256 + to_int(v[5] * 16777216.0f);
       constexpr uint64_t C = ((uint64_t)off << 32) + (off >> (16 - ls));

@@ -215,17 +215,19 @@ __device__ __forceinline__ void fill_offsets(const TcParams& p, uint64_t* toff, 
   }
 }
 
-// column exponent field -> the increment it adds to a result's exponent field
+// column exponent field -> the increment it adds to a result's exponent field (K terms)
+template <int K>
 __host__ __device__ constexpr int column_scale(int field) {
-  return (field - (1024 << 20)) - ((1022 + qsby::kScale) << 20);   // in steps within 32 bits
+  return (field - (1024 << 20)) - ((1022 + qsby::kScale + qsby::extra_bits(K)) << 20);   // in steps within 32 bits
 }
 
 // Row exponent fields [lim[0], lim[1]] whose results can have their exponent fields
 // added (qsby::add_inc) in every column that is not all zeros.  The limits start at
 // those of a column of exponent 0; limit_rows takes in a column's (csc: its largest
 // high word, scale: its increment).
+template <int K>
 __device__ __forceinline__ void start_row_limits(int* lim) {
-  constexpr int one = column_scale(1023 << 20);
+  constexpr int one = column_scale<K>(1023 << 20);
   lim[0] = qsby::kMinInc - one;
   lim[1] = qsby::kMaxInc - one;
 }
@@ -242,16 +244,16 @@ template <int NT, int NTHR>
 __device__ void tile_constants(const TcParams& p, unsigned char* b_dig, unsigned char* a_pre, unsigned char* b_pre,
                                int* csc, int* lim, int* colsum, uint64_t* toff, uint64_t* rowoff, int tid) {
   constexpr int D = 1 << NT, K = 2 * D, N = 2 * D;
-  if (tid == 0) start_row_limits(lim);
+  if (tid == 0) start_row_limits<K>(lim);
   fill_start_rows(a_pre, tid, NTHR);
   fill_offsets<NT>(p, toff, rowoff, tid, NTHR);
   slice_matrix<NT, NTHR>(p, b_dig, N * K * 2, [](int n, int k) { return canon_off16(n, k, K); }, csc, colsum, tid);
   for (int idx = tid; idx < kLv * N; idx += NTHR) {
     const int L = idx / N, n = idx % N;
-    fill_start_column(b_pre, L * N + n, qsby::start_value(L, K, colsum + n * kLv));
+    fill_start_column(b_pre, L * N + n, qsby::start_value(L, K, colsum + n * kLv, qsby::extra_bits(K)));
   }
   for (int j = tid; j < D; j += NTHR) {
-    const int mx = csc[2 * j], sc = column_scale((int)qsby::row_field((uint32_t)mx));
+    const int mx = csc[2 * j], sc = column_scale<K>((int)qsby::row_field((uint32_t)mx));
     limit_rows(lim, mx, sc);
     csc[2 * j] = sc;
     csc[2 * j + 1] = sc;
@@ -269,7 +271,7 @@ __device__ __forceinline__ void finish_outputs(const float (*v)[4], int egs, con
     float u[kLv];
 #pragma unroll
     for (int L = 0; L < kLv; ++L) u[L] = v[L][q];
-    o[q] = __ll2double_rn(qsby::combine<K>(u));
+    o[q] = __ll2double_rn(qsby::combine<K, qsby::extra_bits(K)>(u));
   }
   if (rare) {
 #pragma unroll
@@ -821,7 +823,7 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   fill_start_rows(a_pre, tid, X::THREADS);
   fill_offsets<5>(p, toff, rowoff, tid, X::THREADS);
-  if (tid == 0) start_row_limits(lim);
+  if (tid == 0) start_row_limits<K>(lim);
   // B's slices in blocks of 32 x 32: block (K block, N block) at (kb KB + nb) 16 KB
   slice_matrix<5, X::THREADS>(
       p, b_dig, 2048,
@@ -829,10 +831,10 @@ __global__ void __launch_bounds__(W5::THREADS, 1)
       colsum, tid);
   for (int idx = tid; idx < kLv * K; idx += X::THREADS) {
     const int L = idx / K, n = idx % K;
-    fill_start_column(b_pre + (n >> 5) * 8192, L * 32 + (n & 31), qsby::start_value(L, K, colsum + n * kLv));
+    fill_start_column(b_pre + (n >> 5) * 8192, L * 32 + (n & 31), qsby::start_value(L, K, colsum + n * kLv, qsby::extra_bits(K)));
   }
   for (int j = tid; j < D; j += X::THREADS) {
-    const int mx = csc[2 * j], sc = column_scale((int)qsby::row_field((uint32_t)mx));
+    const int mx = csc[2 * j], sc = column_scale<K>((int)qsby::row_field((uint32_t)mx));
     limit_rows(lim, mx, sc);
     csc[2 * j] = sc;
     csc[2 * j + 1] = sc;
@@ -1100,10 +1102,10 @@ __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcP
   }
   __syncthreads();
   if (k < kLv)
-    fill_start_column(out + kWideStart + (n >> 5) * 8192, k * 32 + (n & 31), qsby::start_value(k, K, sums));
+    fill_start_column(out + kWideStart + (n >> 5) * 8192, k * 32 + (n & 31), qsby::start_value(k, K, sums, qsby::extra_bits(K)));
   if (k == 0) {
     int* col = reinterpret_cast<int*>(out + kWideScale) + 2 * n;
-    col[0] = column_scale((int)ef);
+    col[0] = column_scale<K>((int)ef);
     col[1] = mx;
     reinterpret_cast<int*>(out + kWideFlag)[n] = flag;
   }
@@ -1134,7 +1136,7 @@ __global__ void __launch_bounds__(W6::THREADS, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint4* src = reinterpret_cast<const uint4*>(wide + kWideStart);
   for (int i = tid; i < KB * 8192 / 16; i += X::THREADS) reinterpret_cast<uint4*>(b_pre)[i] = src[i];
-  if (tid == 0) start_row_limits(lim);
+  if (tid == 0) start_row_limits<K>(lim);
   __syncthreads();
   for (int n = tid; n < K; n += X::THREADS) {
     const int* col = reinterpret_cast<const int*>(wide + kWideScale) + 2 * n;
