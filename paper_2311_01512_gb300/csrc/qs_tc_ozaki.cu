@@ -29,9 +29,10 @@
 // top digit, one addition for rounding and balancing, and about 65.
 // Measured at 28 qubits, spread targets, per pass (the copy rate would take 1.27
 // ms): 3 targets 1.95 -> 1.50 ms, 4 targets 1.94 -> 1.50, 5 targets 3.32 -> 2.30,
-// 6 targets (native FP64 before) 110.6 -> 3.9.  Against extended precision the
-// relative error of an output vector fell from 7.7, 6.6, 7.6 and 37.5 to 6.7,
-// 6.1, 6.3 and 6.4 e-17.
+// 6 targets (native FP64 before) 110.6 -> 4.0 with a matrix that mixes its groups (any
+// other stays in FP64, see k_wide_matrix).  Against extended precision the relative
+// error of an output vector is 5.4, 5.4, 5.6 and 6.4e-17 (7-bit digits 7.7, 6.6 and 7.6,
+// FP64 at six targets 37.5).
 //
 // Three kernels share these pieces: k_dense_ozaki_ws (two to four targets) and
 // k_dense_ozaki5 give gathering and slicing, MMA issue and the epilogue to

@@ -70,6 +70,8 @@ def test_circuits(nq, mode):
         c.apply(st.handle)
         qs.qs_synchronize(st.handle)
         got = st.get_amps()
+    passes = qs.qs_test_circuit_passes(c)
+    assert passes > 0 if nq >= 12 else passes == 0        # the runs were tile passes
     c.close()
     st.close()
     assert np.linalg.norm(got - want) <= (len(ops) + 1) * 20 * 2.0 ** -24 * np.linalg.norm(want)
