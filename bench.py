@@ -37,7 +37,7 @@ DTYPE = {
     "fx": ("c128 storage; arithmetic at least FP64: one- and two-target gates, diagonals and gadgets in 60-bit "
            "block fixed point with exact integer products and one rounding per output (error <= 2^-53 |y| + "
            "2^-55 max|x| max|m|, 2^-54 for the two-target gates' eight terms), 3-6-target gates as exact "
-           "byte slices (55-bit amplitudes, 62-bit matrices) on the fp16 tensor cores"),
+           "byte slices (55-bit amplitudes, 63-bit matrices) on the fp16 tensor cores"),
     "df": "c128 storage, double-float (2xf32, 47-bit) arithmetic",
     "f64": "c128 storage, native f64 arithmetic",
 }

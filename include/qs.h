@@ -90,13 +90,29 @@ typedef enum { QS_C64 = 0, QS_C128 = 1 } qs_prec;
  *     conj(U) (x) U or of its superoperator on (t, t + N).
  *   - Dense gates with 3..6 targets (and two-target fused blocks) run on the
  *     fp16 tensor cores with exact 8-bit integer slices: 55-bit amplitudes
- *     (rows scaled by their largest exponent), 63-bit matrix entries (columns
- *     scaled by theirs), exact FP32 level sums, one rounding.
+ *     (scaled by the largest exponent of their group), 63-bit matrix entries
+ *     (by that of their matrix row), exact FP32 level sums, one rounding: half a
+ *     unit of each amplitude, 2^-55 of the group's scale, times its entry, plus
+ *     half a unit of the sum, 2^-55 of the product of the scales (2^-53 at six
+ *     targets).  Groups must be finite.
+ *     With six targets that holds for matrices whose entries all lie within
+ *     2^-16 of the largest of their row.  Other six-target matrices, and groups
+ *     that hold an infinity or NaN or lie outside the slices' exponent range, are
+ *     computed in native FP64.
+ *     Passes that change few amplitudes run on the CUDA cores: statevectors of at
+ *     most 2^20, 2^19, 2^17 and 2^17 amplitudes (2 to 5 targets, two in fused
+ *     blocks) in block fixed point, at most 2^-53 |y| + (2^(n+4) + 2^(2n-2))
+ *     2^-60 max|x_k| max|m_k| (64 2^-60 for n = 2); density matrices of at most
+ *     2^16, 2^16, 2^14 and 2^14 (2 to 5 targets of a pass) in eight 7-bit digits,
+ *     at most 2^-53 |y| + (2^(n+1) + 1) 2^-53 of the product of the scales.
+ *     Results below 2^-1022 become subnormal numbers or zero, results from 2^1024
+ *     on infinities.
  *   - Everything else (dephasing, superoperators,
  *     norm, trace, expectation values, partial traces) is native FP64.
  * QS_ARITH_DF: double-float.  Amplitudes are split into float pairs (47-bit
  *   significands) and combined with error-free FP32 transformations; dense
- *   gates take the tensor-core path above.  Relative error per operation: a
+ *   gates take the paths above (six targets in double-float where the above is
+ *   in FP64; small density matrices as statevectors).  Relative error per operation: a
  *   few units of 2^-46 for moduli in [2^-80, 2^128): narrower than IEEE double.
  * QS_ARITH_F64: native FP64 throughout (FP64-pipe bound on GB300).
  * complex64 states ignore the setting. */
@@ -137,9 +153,11 @@ qs_status qs_get_info(const qs_state* state, int* num_qubits, int* storage_qubit
  * otherwise idle); 0 = none. */
 qs_status qs_set_arithmetic(qs_state* state, qs_arith arith, int f64_share_16ths);
 
-/* complex64 dense gates with 3..5 targets run on the tensor cores (tcgen05,
- * 3xTF32 with FP32 accumulation: FP32-level accuracy) unless disabled here
- * (enable = 0: CUDA-core FP32 kernels).  complex128 states ignore it. */
+/* complex64 dense gates with 2..6 targets run on the tensor cores (tcgen05,
+ * 3xTF32, or three bf16 slices at six, with FP32 accumulation: FP32-level
+ * accuracy) unless disabled here (enable = 0: CUDA-core FP32 kernels).  So do
+ * complex128 ones as qs_set_arithmetic says (enable = 0: FP64, double-float under
+ * QS_ARITH_DF, for all passes of 2 to 6 targets but the two-target gates). */
 qs_status qs_set_tensor_cores(qs_state* state, int enable);
 
 /* Device address of the wrapped amplitudes. */

@@ -24,7 +24,7 @@ struct qs_state {
   qs_prec prec = QS_C128;
   qs_arith arith = QS_ARITH_FX;
   int f64_share = 0;     // sixteenths of one-target-gate chunks run in native FP64
-  int tensor_cores = 1;  // complex64 dense gates with 3..5 targets on tcgen05
+  int tensor_cores = 1;  // dense gates on tcgen05 (complex64 2..6 targets, complex128 as qs_set_arithmetic says)
   int* d_err = nullptr;  // device error word (bounded waits that ran out)
   cudaStream_t stream = nullptr;
   int device = 0;

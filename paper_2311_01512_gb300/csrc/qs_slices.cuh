@@ -1,5 +1,5 @@
-// Integer slicing of FP64 operands for exact products on the bf16 tensor cores
-// (the Ozaki scheme: Ozaki, Ogita, Oishi and Rump, "Error-free transformations
+// Integer slicing of FP64 operands into balanced 7-bit digits, for exact products of
+// digits in FP32 (the Ozaki scheme: Ozaki, Ogita, Oishi and Rump, "Error-free transformations
 // of matrix multiplication by using fast routines of matrix multiplication and
 // its applications", Numer. Algorithms 59 (2012)).
 //
@@ -19,6 +19,11 @@
 // exact and adding 1.5 * 2^23 puts the level's integer in the low significand
 // bits.  The levels L = 0..6 are recombined modulo 2^64 from those bit
 // patterns; the true value fits in 63 bits, so the wrap-around is exact.
+//
+// The kernel of small density matrices (qs_gates_digits.cu) takes eight digits:
+// biased_exp, fixed_t8, digit_floats_t8 and combine_pairs_u<8>.  The seven-digit form, the
+// packed bf16 words and the level-by-level recombinations are their checks' references
+// (tests/host/slices_check.cpp) and run on the host only.
 //
 // Host and device code (the host build is checked on the CPU).
 #pragma once

@@ -94,7 +94,7 @@ __device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double
 // one, so two sets of digits and 16 stores of a pair serve four entries (a
 // negated digit stays within 128).  Leaves the column scales in csc and the digit
 // column sums in colsum (2D x 8).  off(n, k): byte offset of entry (k, n) in a
-// slice; slices are tstride bytes apart.  Ends without a barrier.
+// slice; slices are tstride bytes apart.  Ends with a barrier.
 template <int NT, int NTHR, typename Off>
 __device__ __forceinline__ void slice_matrix(const TcParams& p, unsigned char* b_dig, uint32_t tstride, const Off& off,
                                              int* csc, int* colsum, int tid) {

@@ -6,8 +6,8 @@
 // qubits), and for 16 amplitudes a sweep adds 16 shared loads, 16 stores and some 50
 // index instructions a thread, a one-target gate 64 packed multiply-adds and 32 moves,
 // a two-target gate 128 and 32, a gadget 64 (32 with an odd number of Y) and 15 for
-// signs.  150 random gates at 29 qubits, 17 passes: 44.6 ms, 48.0 with one operation an
-// instruction, against 97 (blocks of six qubits) to 127 (of three) in dense blocks.
+// signs.  150 random gates at 29 qubits, 17 passes: 44 ms, 48 with one operation an
+// instruction, against 94 in dense blocks of at most six qubits.
 // Four 256-thread blocks a multiprocessor (64 registers a thread): one block's
 // sweeps run while the others' loads and stores are in flight (tiles of 2^13 with
 // two 512-thread blocks, 15 passes: 49.7 against 48.0 ms).  Matrices come from shared
