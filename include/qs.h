@@ -91,10 +91,11 @@ typedef enum { QS_C64 = 0, QS_C128 = 1 } qs_prec;
  *   - Dense gates with 3..6 targets (and two-target fused blocks) run on the
  *     fp16 tensor cores with exact 8-bit integer slices: 55-bit amplitudes
  *     (scaled by the largest exponent of their group), 63-bit matrix entries
- *     (by that of their matrix row), exact FP32 level sums, one rounding: half a
- *     unit of each amplitude, 2^-55 of the group's scale, times its entry, plus
- *     half a unit of the sum, 2^-55 of the product of the scales (2^-53 at six
- *     targets).  Groups must be finite.
+ *     (by that of their matrix row), exact FP32 level sums, one rounding.  Error:
+ *     half a unit of each amplitude (2^-55 of the group's scale) times its entry,
+ *     at most two units of the sum (2^-54 of the product of the scales, 2^-52 at
+ *     six targets) and 2^-53 |y|.  Groups must be finite; results below 2^-1022
+ *     become subnormal numbers or zero, results from 2^1024 on infinities.
  *     With six targets that holds for matrices whose entries all lie within
  *     2^-16 of the largest of their row.  Other six-target matrices, and groups
  *     that hold an infinity or NaN or lie outside the slices' exponent range, are
@@ -105,15 +106,14 @@ typedef enum { QS_C64 = 0, QS_C128 = 1 } qs_prec;
  *     2^-60 max|x_k| max|m_k| (64 2^-60 for n = 2); density matrices of at most
  *     2^16, 2^16, 2^14 and 2^14 (2 to 5 targets of a pass) in eight 7-bit digits,
  *     at most 2^-53 |y| + (2^(n+1) + 1) 2^-53 of the product of the scales.
- *     Results below 2^-1022 become subnormal numbers or zero, results from 2^1024
- *     on infinities.
  *   - Everything else (dephasing, superoperators,
  *     norm, trace, expectation values, partial traces) is native FP64.
  * QS_ARITH_DF: double-float.  Amplitudes are split into float pairs (47-bit
  *   significands) and combined with error-free FP32 transformations; dense
- *   gates take the paths above (six targets in double-float where the above is
- *   in FP64; small density matrices as statevectors).  Relative error per operation: a
- *   few units of 2^-46 for moduli in [2^-80, 2^128): narrower than IEEE double.
+ *   gates take the paths above (matrices that six targets take in FP64 above: in
+ *   double-float; small density matrices: as statevectors).  Relative error per
+ *   operation: a few units of 2^-46 for moduli in [2^-80, 2^128): narrower than
+ *   IEEE double.
  * QS_ARITH_F64: native FP64 throughout (FP64-pipe bound on GB300).
  * complex64 states ignore the setting. */
 typedef enum { QS_ARITH_DF = 0, QS_ARITH_F64 = 1, QS_ARITH_FX = 2 } qs_arith;
