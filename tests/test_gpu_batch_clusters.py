@@ -47,3 +47,33 @@ def test_heavy_states(sizes, dens, autotune, prec):
     for s, (psi, ops, d) in enumerate(zip(inits, circuits, density)):
         want = orc.run_ops(orc.run_ops(psi, ops, d), ops, d)
         assert np.max(np.abs(batch.view(s).cpu().numpy() - want)) <= TOL[prec], s
+
+
+@pytest.mark.parametrize("nq,dens", [(12, False), (6, True)])
+def test_segments_cost_no_bits(nq, dens):
+    """A complex128 state gives the same bits whether it stays in shared memory (one of
+    many) or is shared by a cluster, in small tiles that go through global memory between
+    segments (alone, it is heavy).  (Gadgets that pair too many qubits for a small tile
+    are left out: they run on the doubles in global memory.)"""
+    import torch
+    from paper_2311_01512_gb300 import qs
+    rng = np.random.default_rng(5 + nq)
+    ops = (wl.small_densmatr_circuit if dens else wl.unitary_circuit)(nq, 80, rng)
+    ops = [op for op in ops if op["op"] != "gadget" or len(op["targs"]) <= 4]
+    psi = wl.random_statevector(nq, rng)
+    init = torch.from_numpy(orc.densmatr_from_pure(psi) if dens else psi)
+    got = []
+    for count in (1, 400):
+        batch = qs.Batch([nq] * count, prec=qs.QS_C128, density=[dens] * count)
+        for s in range(count):
+            for op in ops:
+                batch.add(s, op)
+        batch.compile(autotune=False)
+        for s in range(count):
+            batch.view(s).copy_(init)
+        batch.run()
+        torch.cuda.synchronize()
+        got.append(batch.view(0).cpu().numpy().copy())
+    assert np.array_equal(got[0], got[1])
+    want = orc.run_ops(init.numpy(), ops, is_density=dens)
+    assert np.max(np.abs(got[0] - want)) <= len(ops) * 2.0 ** -46
