@@ -1077,7 +1077,7 @@ __device__ __noinline__ void group_f64(double2* psi, uint64_t base, const TcPara
 // matrix with an entry below 2^-16 of its row's largest, or one that is not finite, raises
 // a flag: k_dense_ozaki6 returns, and the FP64 kernel (or the double-float one, by the
 // handle's arithmetic) that is launched after it, and returns otherwise, makes the
-// pass.  2^-16: of Haar matrices one in 130 thousand has such an entry.  28 qubits,
+// pass.  2^-16: of Haar matrices one in 200 thousand has such an entry.  28 qubits,
 // spread targets: 3.96 ms mixing, 111 ms in FP64; the kernel that returns takes 2 us and
 // a launch (calls at 2^7 to 2^18 amplitudes 38 to 42 us without it, 43 to 47 with it).
 __global__ void __launch_bounds__(128) k_wide_matrix(const __grid_constant__ TcParams p, unsigned char* __restrict__ out) {
